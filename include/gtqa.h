@@ -90,22 +90,20 @@ typedef struct gtqa_stats_t {
     double last_bp_dist;     /* dist/|E| after the last sweep (max over instances), App. B */
     double discarded_weight; /* sum over gates of sum_{dropped} s^2 / sum s^2 */
     double log_fidelity;     /* sum over gates of log f, f = (1 - discarded)^2, Eq. (gate_fidelity) */
-    int64_t svd_pairs;       /* column pairs examined by the gate-core FP64 Jacobi sweeps (the polish
-                                in GTQA_MIXED; work counter) */
-    int64_t svd_rotations;   /* rotations applied by the gate-core Jacobi SVDs (work counter) */
+    int64_t svd_pairs;       /* column pairs examined in FP64 by the gate-core SVDs (refinement passes over
+                                all pairs, and Jacobi steps; work counter) */
+    int64_t svd_rotations;   /* FP64 Jacobi rotations of the gate-core SVDs (work counter) */
     int64_t bp_sweeps;       /* BP sweeps run since creation (sum over calls, max over instances) */
     int64_t launches;        /* kernels launched by the library since creation */
     int64_t bp_calls;        /* BP runs since creation (one per layer in gtqa_anneal) */
     int64_t bp_not_converged_calls; /* BP runs in which some instance reached max_iter */
     int64_t bp_exact_passes; /* separate passes computing the exact trace-norm distance of a sweep
                                 (persistent path: when a sweep's lower bound falls under tol) */
-    int64_t regauge_svd_sweeps; /* Jacobi sweeps of the regauge's eigen-decompositions and SVDs
+    int64_t regauge_svd_sweeps; /* FP64 refinement passes of the regauge's eigen-decompositions and SVDs
                                    (persistent path; work counter) */
-    int32_t gate_svd_sweeps_max;      /* most FP64 Jacobi sweeps of one gate-core SVD since creation
-                                         (the FP64 polish sweeps in GTQA_MIXED, whose sweeps after
-                                         the first run only the schedule steps that still rotate
-                                         by more than the stop threshold; persistent path) */
-    int32_t gate_svd_sweeps32_max;    /* GTQA_MIXED: most FP32 preconditioning sweeps of one gate-core SVD */
+    int32_t gate_svd_sweeps_max;      /* most FP64 refinement passes (and sweeps of a closing Jacobi polish)
+                                         of one gate-core SVD since creation (persistent path) */
+    int32_t gate_svd_sweeps32_max;    /* most FP32 Jacobi sweeps of one gate-core SVD */
     int32_t regauge_svd_sweeps_max;   /* the same two maxima for the regauge's decompositions */
     int32_t regauge_svd_sweeps32_max;
 } gtqa_stats_t;

@@ -164,9 +164,8 @@ struct GateSm {
     double tau[4][CHI];        // square roots of the reflector coefficients
     cd M[4 * CHI * CHI];
     cd V[4 * CHI * CHI];
-    cd G[4 * CHI * CHI];       // mixed: V^H V, then M V
-    cd Vn[4 * CHI * CHI];      // mixed: Newton-Schulz update of V
-    cf M32[4 * CHI * CHI];     // mixed: FP32 copy of M for the preconditioning sweeps
+    cd G[4 * CHI * CHI];       // scratch of the refinement
+    cf M32[4 * CHI * CHI];     // FP32 copy of M for the first stage
     cf V32[4 * CHI * CHI];
     double w[2][CHI * CHI];
     double lab[CHI];
@@ -175,7 +174,7 @@ struct GateSm {
     cd ph[4];
     int perm[2 * CHI];
     int keep;
-    unsigned relmask;          // mixed: columns that decide the polish's stop
+    unsigned relmask;          // columns that decide the stop of a closing polish
     int flag;
     int nrot;
 };
@@ -287,90 +286,24 @@ __device__ void gate_edge(const Ctx& c, int e, int tid, int team, GateSm<CHI>& s
     if constexpr (TEAM <= 32) prune_noise<NM>(sm.M, tid, WarpGroup{group_mask<TEAM>()});
     else prune_noise<NM>(sm.M, tid, TeamGroup<TEAM>{team, &sm.flag});
 
-    // ---- SVD of M ----
-    // FP64 mode: one-sided Jacobi in FP64 from V = I.
-    // Mixed mode: Jacobi sweeps in FP32 on a copy of M give V32; one FP64 Newton-Schulz
-    // step V <- V (3I - V^H V)/2 makes it unitary to ~1e-14; the FP64 Jacobi then polishes
-    // W = M V (typically two sweeps; the confirming sweep is skipped by the quadratic
-    // stop).  The result is an FP64 SVD of M with a fraction of the FP64 instructions.
-    int nrot = 0, sweeps, nsteps = 0;
-    // FP32 rotation angles with FP64-exact rotations; the confirming sweep is skipped
-    // once a sweep's rotations are all below sqrt(tol) (quadratic convergence)
-    auto svd64 = [&](bool init_v, double tol, double quad) {
-        if constexpr (TEAM <= 32) {
-            WarpGroup grp{group_mask<TEAM>()};
-            return jacobi_svd<NM, double, WarpGroup, true, true>(sm.M, sm.V, tid, grp, group_mask<NM>(), tol, 60,
-                                                                 init_v, &nrot, quad);
-        } else {
-            TeamGroup<TEAM> grp{team, &sm.flag};
-            return jacobi_svd<NM, double, TeamGroup<TEAM>, true, true>(sm.M, sm.V, tid, grp, group_mask<NM>(), tol,
-                                                                       60, init_v, &nrot, quad);
-        }
+    // ---- SVD of M: an FP32 Jacobi solve brought to FP64 accuracy by refinement passes ----
+    // (refined_svd; before it, FP64 mode ran 6 to 11 FP64 Jacobi sweeps, and the mixed mode one or
+    // two FP64 polish sweeps)
+    SvdCount done;
+    auto svd = [&](const auto& grp) {
+        return refined_svd<NM, !Mode::mixed>(sm.M, sm.V, sm.M32, sm.V32, sm.G, sm.sig, &sm.relmask, tid, grp,
+                                             group_mask<NM>(), c.svd_cut, c.chi, Mode::mixed ? 1e-5f : 1e-8f,
+                                             Mode::mixed ? 1e-12 : 1e-15);
     };
-    if constexpr (!Mode::mixed) {
-        sweeps = svd64(true, 1e-15, 3e-8);
-    } else {
-        for (int t = tid; t < NM * NM; t += TEAM) sm.M32[t] = ccast<float>(sm.M[t]);
-        team_bar<TEAM>(team);
-        int sw32;
-        if constexpr (TEAM <= 32) {
-            WarpGroup grp{group_mask<TEAM>()};
-            sw32 = jacobi_svd<NM, float>(sm.M32, sm.V32, tid, grp, group_mask<NM>(), 1e-6f, 40, true, nullptr, 1e-3f);
-        } else {
-            TeamGroup<TEAM> grp{team, &sm.flag};
-            sw32 = jacobi_svd<NM, float>(sm.M32, sm.V32, tid, grp, group_mask<NM>(), 1e-6f, 40, true, nullptr, 1e-3f);
-        }
-        if (tid == 0) atomicMax(&c.ctl->gate_sw32_max, sw32);
-        team_bar<TEAM>(team);
-        for (int t = tid; t < NM * NM; t += TEAM) sm.V[t] = ccast<double>(sm.V32[t]);
-        team_bar<TEAM>(team);
-        // G = V^H V (column-major: G[p][q] at q*NM + p)
-        for (int t = tid; t < NM * NM; t += TEAM) {
-            const int q = t / NM, p = t % NM;
-            cd acc = cd{0.0, 0.0};
-            for (int r = 0; r < NM; ++r) acc = cfmac(sm.V[p * NM + r], sm.V[q * NM + r], acc);
-            sm.G[t] = acc;
-        }
-        team_bar<TEAM>(team);
-        // Vn = V (1.5 I - 0.5 G)
-        for (int t = tid; t < NM * NM; t += TEAM) {
-            const int q = t / NM, r = t % NM;
-            cd acc = 1.5 * sm.V[q * NM + r];
-            for (int p = 0; p < NM; ++p) acc = cfma(-0.5 * sm.V[p * NM + r], sm.G[q * NM + p], acc);
-            sm.Vn[t] = acc;
-        }
-        team_bar<TEAM>(team);
-        // W = M Vn into G, then M <- W, V <- Vn
-        for (int t = tid; t < NM * NM; t += TEAM) {
-            const int q = t / NM, r = t % NM;
-            cd acc = cd{0.0, 0.0};
-            for (int p = 0; p < NM; ++p) acc = cfma(sm.M[p * NM + r], sm.Vn[q * NM + p], acc);
-            sm.G[t] = acc;
-        }
-        team_bar<TEAM>(team);
-        for (int t = tid; t < NM * NM; t += TEAM) {
-            sm.M[t] = sm.G[t];
-            sm.V[t] = sm.Vn[t];
-        }
-        team_bar<TEAM>(team);
-        if constexpr (TEAM <= 32) {
-            WarpGroup grp{group_mask<TEAM>()};
-            sweeps = jacobi_polish<NM, decltype(grp), true>(sm.M, sm.V, sm.sig, tid, grp, group_mask<NM>(), 1e-12,
-                                                            1e-5, 60, &nrot, c.chi, &sm.relmask, &nsteps);
-        } else {
-            TeamGroup<TEAM> grp{team, &sm.flag};
-            sweeps = jacobi_polish<NM, decltype(grp), true>(sm.M, sm.V, sm.sig, tid, grp, group_mask<NM>(), 1e-12,
-                                                            1e-5, 60, &nrot, c.chi, &sm.relmask, &nsteps);
-        }
-    }
-    if (nrot) atomicAdd(&sm.nrot, nrot);
+    if constexpr (TEAM <= 32) done = svd(WarpGroup{group_mask<TEAM>()});
+    else done = svd(TeamGroup<TEAM>{team, &sm.flag});
+    if (done.rot) atomicAdd(&sm.nrot, done.rot);
     team_bar<TEAM>(team);
-    for (int cc = tid; cc < NM; cc += TEAM) {
-        double s2 = 0.0;
-        for (int r = 0; r < NM; ++r) s2 += norm2(sm.M[cc * NM + r]);
-        const double sv = nr_sqrt(s2);
-        sm.sig[cc] = sv;
-        sm.isig[cc] = sv > 0.0 ? nr_rcp(sv) : 0.0;
+    for (int cc = tid; cc < NM; cc += TEAM) {   // sm.sig holds the squared column norms
+        const double s2 = sm.sig[cc];
+        const double is = s2 > 1e-300 ? nr_rsqrt(s2) : 0.0;
+        sm.sig[cc] = s2 * is;
+        sm.isig[cc] = is;
     }
     team_bar<TEAM>(team);
     for (int cc = tid; cc < NM; cc += TEAM) sm.perm[desc_rank(sm.sig, NM, cc)] = cc;
@@ -393,10 +326,10 @@ __device__ void gate_edge(const Ctx& c, int e, int tid, int team, GateSm<CHI>& s
             atomicAdd(&c.stats[0], disc);
             // log of the gate fidelity (1 - disc)^2, Eq. (gate_fidelity); a float log in the mixed mode
             atomicAdd(&c.stats[1], Mode::mixed ? 2.0 * (double)log1pf(-(float)disc) : 2.0 * log1p(-disc));
-            // Jacobi pairs examined (the mixed polish runs partial sweeps)
-            atomicAdd(&c.stats[2], (double)(Mode::mixed ? nsteps : sweeps * (NM - 1)) * (NM / 2));
+            atomicAdd(&c.stats[2], (double)done.pairs);
             atomicAdd(&c.stats[3], (double)sm.nrot);
-            atomicMax(&c.ctl->gate_sw_max, sweeps);
+            atomicMax(&c.ctl->gate_sw_max, done.passes);
+            atomicMax(&c.ctl->gate_sw32_max, done.sweeps32);
             sm.keep = keep;
         }
     }
@@ -1051,11 +984,10 @@ struct RGSm {
     double isig[CHI];   // 1 / sig (0 for a zero singular value)
     int perm[CHI];
     double scal[2];
-    // mixed mode: scratch of the FP32-preconditioned SVDs
+    // scratch of the decompositions
     cf A32[2][CHI * CHI];
     cf V32[2][CHI * CHI];
     cd T1[2][CHI * CHI];
-    cd T2[2][CHI * CHI];
     double nrm[2][CHI];
 };
 
@@ -1088,22 +1020,17 @@ __device__ void regauge_edge(const Ctx& c, int e, int tid, int team, int cur, RG
     team_bar<TEAM>(team);
     {
         // FP64 eigen-decompositions of the two Hermitian messages (the singular values of a
-        // Hermitian matrix are the moduli of its eigenvalues); the mixed mode takes the
-        // FP32-preconditioned path, whose result is FP64-accurate as well
+        // Hermitian matrix are the moduli of its eigenvalues)
         const int x = tid / GJ, g = tid % GJ;
         WarpGroup grp{group_mask<GJ>()};
         prune_noise<CHI>(sm.Am[x], g, grp);
-        int sw, sw32 = 0;
-        if constexpr (Mode::mixed)
-            sw = mixed_svd<CHI>(sm.Am[x], sm.Vm[x], sm.A32[x], sm.V32[x], sm.T1[x], sm.T2[x], sm.nrm[x], g, grp,
-                                group_mask<CHI>(), 1e-13, 3e-7, nullptr, &sw32);
-        else
-            sw = jacobi_svd<CHI, double, WarpGroup, true, true>(sm.Am[x], sm.Vm[x], g, grp, group_mask<CHI>(), 1e-15, 60,
-                                                                true, nullptr, 3e-8);
+        const SvdCount cnt = refined_svd<CHI, !Mode::mixed>(
+            sm.Am[x], sm.Vm[x], sm.A32[x], sm.V32[x], sm.T1[x], sm.nrm[x], nullptr, g, grp, group_mask<CHI>(), c.eig_cut,
+            CHI, Mode::mixed ? 3e-7f : 1e-8f, Mode::mixed ? 1e-13 : 1e-15);
         if (g == 0) {
-            atomicAdd(&c.stats[4], (double)sw);
-            atomicMax(&c.ctl->reg_sw_max, sw);
-            atomicMax(&c.ctl->reg_sw32_max, sw32);
+            atomicAdd(&c.stats[4], (double)cnt.passes);
+            atomicMax(&c.ctl->reg_sw_max, cnt.passes);
+            atomicMax(&c.ctl->reg_sw32_max, cnt.sweeps32);
         }
     }
     team_bar<TEAM>(team);
@@ -1157,17 +1084,13 @@ __device__ void regauge_edge(const Ctx& c, int e, int tid, int team, int cur, RG
     if (tid < GJ) {
         WarpGroup grp{group_mask<GJ>()};
         prune_noise<CHI>(sm.M, tid, grp);
-        int sw, sw32 = 0;
-        if constexpr (Mode::mixed)
-            sw = mixed_svd<CHI>(sm.M, sm.VM, sm.A32[0], sm.V32[0], sm.T1[0], sm.T2[0], sm.nrm[0], tid, grp,
-                                group_mask<CHI>(), 1e-13, 3e-7, nullptr, &sw32);
-        else
-            sw = jacobi_svd<CHI, double, WarpGroup, true, true>(sm.M, sm.VM, tid, grp, group_mask<CHI>(), 1e-15, 60, true,
-                                                                nullptr, 3e-8);
+        const SvdCount cnt = refined_svd<CHI, !Mode::mixed>(
+            sm.M, sm.VM, sm.A32[0], sm.V32[0], sm.T1[0], sm.nrm[0], nullptr, tid, grp, group_mask<CHI>(), c.svd_cut, CHI,
+            Mode::mixed ? 3e-7f : 1e-8f, Mode::mixed ? 1e-13 : 1e-15);
         if (tid == 0) {
-            atomicAdd(&c.stats[4], (double)sw);
-            atomicMax(&c.ctl->reg_sw_max, sw);
-            atomicMax(&c.ctl->reg_sw32_max, sw32);
+            atomicAdd(&c.stats[4], (double)cnt.passes);
+            atomicMax(&c.ctl->reg_sw_max, cnt.passes);
+            atomicMax(&c.ctl->reg_sw32_max, cnt.sweeps32);
         }
     }
     team_bar<TEAM>(team);

@@ -318,12 +318,13 @@ __device__ __forceinline__ bool norm_collapsed(double x, double ref) {
 // times the largest rotation of that sweep (the rotations of its columns with the others
 // reintroduce only products of their sizes), which is the accuracy of the quadratic stop, so
 // those steps need no second pass.  Otherwise every pair is rotated in each sweep that runs.
+// first_steps: the steps that the first sweep runs (all by default).
 // Returns the sweeps run (partial ones included); *nsteps (if given, group lane 0) counts the
 // steps run, of N / 2 pairs each.
 template <int N, typename Group, bool PARTIAL = false>
 __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, const Group& grp, unsigned pair_mask,
                              double tol, double quad_tol, int max_sweeps, int* nrot, int keep_rank = N,
-                             unsigned* relmask = nullptr, int* nsteps = nullptr) {
+                             unsigned* relmask = nullptr, int* nsteps = nullptr, unsigned first_steps = ~0u) {
     using CD = C<double>;
     const int k = g / N;
     const int r = g % N;
@@ -356,8 +357,8 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
     }
     const unsigned rel = partial ? *relmask : 0xffffffffu;
     const double tol2 = tol * tol, quad2 = quad_tol * quad_tol;
-    static_assert(N - 1 <= 32, "one bit per step");
-    unsigned steps = N - 1 == 32 ? 0xffffffffu : (1u << (N - 1)) - 1u;   // steps this sweep runs
+    static_assert(N - 1 < 32, "one bit per step");
+    unsigned steps = ((1u << (N - 1)) - 1u) & first_steps;   // steps this sweep runs
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
         int big = 0;
@@ -446,51 +447,306 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
     return sweep;
 }
 
-// FP64 SVD of an N x N complex matrix A (column-major, shared memory) by the mixed path:
-// one-sided Jacobi sweeps on an FP32 copy give V32; one FP64 Newton-Schulz step
-// V <- V (3I - V^H V)/2 makes V unitary to ~1e-14; W = A V (FP64) then goes through the
-// FP64 polish (jacobi_polish) to orthogonality `tol`.  On exit A holds U S (columns unsorted)
-// and V the right singular vectors, as after jacobi_svd<N, double>.  A32, V32 (N^2 complex
-// floats), T1, T2 (N^2 complex) and nrm (N) are scratch.  The group has N^2/2 lanes.
+// ---------------------------------------------------------------------------
+// FP64 SVD of an N x N complex matrix (column-major, shared memory) from an FP32 one.
+//
+// What bounds it: the FP64 pipe (one warp instruction per 64 cycles and sub-partition, whatever
+// its active lanes).  An FP64 Jacobi sweep costs N - 1 dependent steps of about 57 FP64
+// instructions per warp (N = 8: 400), and a decomposition needs 6 to 11 of them; a pass of the
+// refinement below costs two or three N^3 products (N = 8: 130 to 200), all lanes busy and no
+// chain of steps, and one or two passes suffice:
+//   1. one-sided Jacobi on an FP32 copy (scaled by the exponent of its largest entry) gives V32;
+//   2. V = V32 is made unitary: V <- V (I - E/2), E = V^H V - I from an FP64 Gram product, the
+//      correction's product in FP32 (|E| ~ 1e-6, so its rounding lies near 1e-13); F64: twice,
+//      which leaves rounding level;
+//   3. W = A V in FP64;
+//   4. passes: the Gram matrix of W in FP64, every pair's rotation parameter (as in
+//      jacobi_polish: K_pq = tau gamma_pq) at once, and W <- W (I + K + K^2/2), V likewise, for
+//      all pairs with |K_pq| <= 1e-4.  K is antihermitian, so the factor is unitary up to
+//      |K|^4/4 < 3e-17, and the off-diagonals shrink to products of their sizes.  The passes
+//      end once every pair was below `stop` (relative to its columns) before its pass.
+//      A pair with a larger K (nearly equal or not yet resolved columns) is rotated by
+//      FP64 Jacobi steps (only the steps of the schedule that hold such a pair) or, for N >= 16
+//      with many of them, by FP32 Jacobi on those columns of W rescaled to the largest of them,
+//      which resolves the columns that lay below the FP32 resolution of the first stage.
+//   A decomposition that is still open after MAXP passes goes to jacobi_polish.
+// Cores of whole anneals (n = 300, chi = 4): 1.3 passes on average in the mixed mode, 2.1 with
+// F64, Jacobi steps in 2 % of the gates; slow early anneals with spectra graded over 12 orders:
+// 3.3 and 3.9.  Orthogonality of the kept columns after it: 2e-10 (stop 1e-5) and 1e-15 (F64).
+// ---------------------------------------------------------------------------
+// The pair of columns of lane g: the N (N - 1) / 2 pairs in the order of the Jacobi schedule
+// (lane g: pair g % (N / 2) of step g / (N / 2)); false for the lanes that are left over.
+template <int N>
+__device__ __forceinline__ bool lane_pair(int g, int& step, int& p, int& q) {
+    step = g / (N / 2);
+    p = 0;
+    q = N > 1 ? 1 : 0;
+    if (step >= N - 1) return false;
+    round_robin_pair(N, step, g % (N / 2), p, q);
+    return true;
+}
+// Squared column norms into nrm[N] (N / 2 lanes per column, two rows each); no synchronisation.
+template <int N>
+__device__ __forceinline__ void column_norms(const C<double>* A, double* nrm, int g) {
+    constexpr int H = N / 2;
+    const int c = g / H, r = g % H;
+    double s = norm2(A[c * N + r]) + norm2(A[c * N + r + H]);
+    s = group_sum<H>(s, group_mask<(H < 32 ? H : 32)>());
+    if (r == 0) nrm[c] = s;
+}
+// Column norms into nrm, and a_p^H a_q of the lane's pair.  The rows start at the lane's own, so
+// that the lanes of a warp read different banks.
 template <int N, typename Group>
-__device__ int mixed_svd(C<double>* A, C<double>* V, C<float>* A32, C<float>* V32, C<double>* T1, C<double>* T2,
-                         double* nrm, int g, const Group& grp, unsigned pair_mask, double tol, double quad_tol,
-                         int* nrot, int* sweeps32 = nullptr) {
+__device__ __forceinline__ C<double> gram(const C<double>* A, double* nrm, int g, const Group& grp, bool has, int p,
+                                          int q) {
+    column_norms<N>(A, nrm, g);
+    C<double> gam = C<double>{0.0, 0.0};
+    if (has)
+        for (int i = 0; i < N; ++i) {
+            const int r = (i + g) & (N - 1);
+            gam = cfmac(A[p * N + r], A[q * N + r], gam);
+        }
+    grp.sync();
+    return gam;
+}
+// V <- V + V32 L with the product in FP32, and V32 <- V rounded.
+template <int N, typename Group>
+__device__ __forceinline__ void add_product32(C<double>* V, C<float>* V32, const C<float>* L, int g, const Group& grp) {
+    constexpr int LN = N * N / 2;
+    C<float> acc[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int t = g + j * LN, q = t / N, r = t % N;
+        acc[j] = C<float>{0.f, 0.f};
+        for (int p = 0; p < N; ++p) acc[j] = cfma(V32[p * N + r], L[q * N + p], acc[j]);
+    }
+    grp.sync();
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int t = g + j * LN;
+        const C<double> v = V[t] + ccast<double>(acc[j]);
+        V[t] = v;
+        V32[t] = ccast<float>(v);
+    }
+    grp.sync();
+}
+// X <- X B (ADD: X + X B) in FP64, in place.
+template <int N, bool ADD, typename Group>
+__device__ __forceinline__ void mul64(C<double>* X, const C<double>* B, int g, const Group& grp) {
+    constexpr int LN = N * N / 2;
+    C<double> acc[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int t = g + j * LN, q = t / N, r = t % N;
+        acc[j] = ADD ? X[t] : C<double>{0.0, 0.0};
+        for (int p = 0; p < N; ++p) acc[j] = cfma(X[p * N + r], B[q * N + p], acc[j]);
+    }
+    grp.sync();
+#pragma unroll
+    for (int j = 0; j < 2; ++j) X[g + j * LN] = acc[j];
+    grp.sync();
+}
+// 2^-e for the exponent field `bits` of a normal double; 0 for a zero, subnormal or non-finite one
+__device__ __forceinline__ double inv_exp2(int bits) {
+    return bits > 0 && bits < 2046 ? __longlong_as_double((long long)(2046 - bits) << 52) : 0.0;
+}
+
+struct SvdCount {       // work of one decomposition
+    int passes = 0;     // refinement passes (and sweeps of a closing jacobi_polish)
+    int sweeps32 = 0;   // FP32 sweeps
+    int pairs = 0;      // pairs examined in FP64: N (N - 1) / 2 per pass, N / 2 per Jacobi step
+    int rot = 0;        // FP64 Jacobi rotations of this lane's pairs
+};
+
+// V32's Jacobi run on the FP32 copy in A32, and V (FP64) from it, unitary to ~1e-12 (F64: to
+// rounding).  V32 holds V rounded afterwards.
+template <int N, bool F64, typename Group>
+__device__ int svd32_unitary(C<double>* V, C<float>* A32, C<float>* V32, double* nrm, int g, const Group& grp,
+                             unsigned pair_mask) {
+    constexpr int LN = N * N / 2;
+    int step, p, q;
+    const bool has = lane_pair<N>(g, step, p, q);
+    const int sw = jacobi_svd<N, float>(A32, V32, g, grp, pair_mask, 1e-6f, 40, true, nullptr, 1e-3f);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) V[g + j * LN] = ccast<double>(V32[g + j * LN]);
+    grp.sync();
+    for (int pass = 0; pass < (F64 ? 2 : 1); ++pass) {
+        const C<double> e = gram<N>(V, nrm, g, grp, has, p, q);
+        if (has) {
+            const C<float> ef = ccast<float>(-0.5 * e);
+            A32[q * N + p] = ef;
+            A32[p * N + q] = conj(ef);
+        }
+        if (g < N) A32[g * N + g] = C<float>{(float)fma(-0.5, nrm[g], 0.5), 0.f};
+        grp.sync();
+        add_product32<N>(V, V32, A32, g, grp);
+    }
+    return sw;
+}
+
+// On exit A holds U S (columns unsorted), V the right singular vectors and nrm the squared
+// column norms of A.  keep_rank, cut: the caller keeps at most keep_rank singular triplets and
+// drops those at or below cut times the largest; only pairs with a column among the keep_rank
+// largest (norms within a factor 4 of the keep_rank-th count) and above cut / 2 are brought to
+// orthogonality, judged against the larger column when the other one is not kept.  A32, V32
+// (N^2 complex floats), T (N^2 complex) and relmask (one word) are scratch; the group has
+// N^2 / 2 lanes.
+template <int N, bool F64, typename Group>
+__device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<float>* V32, C<double>* T, double* nrm,
+                                unsigned* relmask, int g, const Group& grp, unsigned pair_mask, double cut,
+                                int keep_rank, float stop, double tol) {
     using CD = C<double>;
-    constexpr int NN = N * N, L = NN / 2;
-    for (int t = g; t < NN; t += L) A32[t] = ccast<float>(A[t]);
-    grp.sync();
-    const int sw32 = jacobi_svd<N, float>(A32, V32, g, grp, pair_mask, 1e-6f, 40, true, nullptr, 1e-3f);
-    if (sweeps32) *sweeps32 = sw32;
-    for (int t = g; t < NN; t += L) V[t] = ccast<double>(V32[t]);
-    grp.sync();
-    for (int t = g; t < NN; t += L) {   // T1 = V^H V
-        const int q = t / N, p = t % N;
-        CD acc = CD{0.0, 0.0};
-        for (int r = 0; r < N; ++r) acc = cfmac(V[p * N + r], V[q * N + r], acc);
-        T1[t] = acc;
+    using CF = C<float>;
+    constexpr int LN = N * N / 2, NP = N * (N - 1) / 2, MAXP = 8;
+    constexpr float KMAX2 = 1e-8f;   // |K|^2 limit of the simultaneous rotations
+    SvdCount cnt;
+    int step, p, q;
+    const bool has = lane_pair<N>(g, step, p, q);
+    {
+        int e = 0;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const CD a = A[g + j * LN];
+            e = max(e, max(exp_bits(a.x), exp_bits(a.y)));
+        }
+        const double sc = inv_exp2(grp.max_int(e));
+#pragma unroll
+        for (int j = 0; j < 2; ++j) A32[g + j * LN] = ccast<float>(sc * A[g + j * LN]);
+        grp.sync();
     }
-    grp.sync();
-    for (int t = g; t < NN; t += L) {   // T2 = V (1.5 I - 0.5 T1)
-        const int q = t / N, r = t % N;
-        CD acc = 1.5 * V[q * N + r];
-        for (int p = 0; p < N; ++p) acc = cfma(-0.5 * V[p * N + r], T1[q * N + p], acc);
-        T2[t] = acc;
+    cnt.sweeps32 = svd32_unitary<N, F64>(V, A32, V32, nrm, g, grp, pair_mask);
+    mul64<N, false>(A, V, g, grp);
+    const float stop2 = stop * stop, cut2 = (float)(0.25 * cut * cut);
+    int second = 0;   // FP32 runs on a part of the columns
+    for (int pass = 0;; ++pass) {
+        const CD gam = gram<N>(A, nrm, g, grp, has, p, q);
+        ++cnt.passes;
+        cnt.pairs += NP;
+        CF K = CF{0.f, 0.f};
+        unsigned flags = 0u;   // 1: a pair above stop, 2: one of those with a large K, 4: |K| > 1e-8, 8: any K
+        if (has) {
+            const double al = nrm[p], be = nrm[q];
+            const long long la = __double_as_longlong(al), lb = __double_as_longlong(be);
+            // positive doubles compare as integers; + 2 in the exponent: times 4
+            const long long a4 = la + (2ll << 52), b4 = lb + (2ll << 52);
+            long long lmax = 0;
+            int ca = 0, cb = 0;
+            for (int j = 0; j < N; ++j) {
+                const long long x = __double_as_longlong(nrm[j]);
+                ca += x > a4;
+                cb += x > b4;
+                lmax = x > lmax ? x : lmax;
+            }
+            const double sc = inv_exp2((int)((la > lb ? la : lb) >> 52));
+            const float an = (float)(al * sc), bn = (float)(be * sc);
+            const float top = (float)(__longlong_as_double(lmax) * sc);
+            const bool rp = ca < keep_rank && an >= cut2 * top, rq = cb < keep_rank && bn >= cut2 * top;
+            if ((rp || rq) && sc > 0.0) {
+                const float dn = (float)((be - al) * sc);
+                const double gsc = sc * 1073741824.0;   // gamma times 2^30: |gamma|^2 stays in the FP32 range
+                const float gx = (float)(gam.x * gsc), gy = (float)(gam.y * gsc);
+                const float g2 = fmaf(gx, gx, gy * gy);
+                const float lim = rp && rq ? an * bn : fmaxf(an, bn) * fmaxf(an, bn);
+                const bool open = g2 > stop2 * 1.152921504606847e18f * lim;
+                if (open) flags |= 1u;
+                if (g2 > 0.f) {
+                    const float g2n = g2 * 8.673617379884035e-19f;
+                    const float tn = 2.f * 9.313225746154785e-10f * __frcp_rn(fabsf(dn) + sqrtf(fmaf(dn, dn, 4.f * g2n)));
+                    const float t = dn >= 0.f ? tn : -tn;
+                    K = CF{t * gx, t * gy};
+                    const float k2 = norm2(K);
+                    if (!(k2 <= KMAX2)) {
+                        K = CF{0.f, 0.f};
+                        if (open) flags |= 2u;
+                    } else {
+                        flags |= 8u;
+                        if (k2 > 1e-16f) flags |= 4u;
+                    }
+                }
+            }
+        }
+        const unsigned mine = flags;
+        flags = grp.or_bits(flags);
+        if (flags & 8u) {
+            // I + K + K^2/2 on W (FP64) and V (FP64, or the correction in FP32)
+            if (has) {
+                A32[q * N + p] = K;
+                A32[p * N + q] = CF{-K.x, K.y};
+            }
+            if (g < N) A32[g * N + g] = CF{0.f, 0.f};
+            grp.sync();
+            CF l[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int t = g + j * LN, c = t / N, r = t % N;
+                CD x = ccast<double>(A32[t]);
+                CF k2 = CF{0.f, 0.f};
+                if (flags & 4u) {
+                    for (int s = 0; s < N; ++s) k2 = cfma(A32[s * N + r], A32[c * N + s], k2);
+                    x = x + ccast<double>(0.5f * k2);
+                }
+                l[j] = A32[t] + 0.5f * k2;
+                T[t] = x;
+            }
+            grp.sync();
+            mul64<N, true>(A, T, g, grp);
+            if (F64 && (flags & 4u)) {
+                mul64<N, true>(V, T, g, grp);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    A32[g + j * LN] = l[j];
+                    if constexpr (F64) V32[g + j * LN] = ccast<float>(V[g + j * LN]);
+                }
+                grp.sync();
+                add_product32<N>(V, V32, A32, g, grp);
+            }
+        }
+        if (!(flags & 1u)) break;
+        if (pass + 1 >= MAXP) {
+            int nsteps = 0;
+            cnt.passes += jacobi_polish<N, Group, true>(A, V, nrm, g, grp, pair_mask, tol, stop, 60, &cnt.rot, keep_rank,
+                                                        relmask, &nsteps);
+            cnt.pairs += nsteps * (N / 2);
+            break;
+        }
+        if (!(flags & 2u) || pass == 0) continue;   // the first pass only clears what it can
+        const unsigned steps = grp.or_bits((mine & 2u) ? 1u << step : 0u);
+        const int nst = __popc(steps);
+        bool part = false;
+        if constexpr (N >= 16) part = nst > N / 4 && second < 3;
+        if (!part) {
+            jacobi_polish<N, Group, true>(A, V, nrm, g, grp, pair_mask, tol, stop, 1, &cnt.rot, N, nullptr, nullptr, steps);
+            cnt.pairs += nst * (N / 2);
+        } else if constexpr (N >= 16) {
+            ++second;
+            const unsigned cols = grp.or_bits((mine & 2u) ? (1u << p) | (1u << q) : 0u);
+            int e = 0;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const CD a = A[g + j * LN];
+                if ((cols >> ((g + j * LN) / N)) & 1u) e = max(e, max(exp_bits(a.x), exp_bits(a.y)));
+            }
+            const double sc = inv_exp2(grp.max_int(e));
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int t = g + j * LN;
+                A32[t] = ((cols >> (t / N)) & 1u) ? ccast<float>(sc * A[t]) : CF{0.f, 0.f};
+            }
+            grp.sync();
+            cnt.sweeps32 += svd32_unitary<N, F64>(T, A32, V32, nrm, g, grp, pair_mask);
+            mul64<N, false>(A, T, g, grp);
+            mul64<N, false>(V, T, g, grp);
+        }
+        if constexpr (!F64) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) V32[g + j * LN] = ccast<float>(V[g + j * LN]);
+            grp.sync();
+        }
     }
+    column_norms<N>(A, nrm, g);
     grp.sync();
-    for (int t = g; t < NN; t += L) {   // T1 = A T2
-        const int q = t / N, r = t % N;
-        CD acc = CD{0.0, 0.0};
-        for (int p = 0; p < N; ++p) acc = cfma(A[p * N + r], T2[q * N + p], acc);
-        T1[t] = acc;
-    }
-    grp.sync();
-    for (int t = g; t < NN; t += L) {
-        A[t] = T1[t];
-        V[t] = T2[t];
-    }
-    grp.sync();
-    return jacobi_polish<N, Group>(A, V, nrm, g, grp, pair_mask, tol, quad_tol, 60, nrot);
+    return cnt;
 }
 
 // Rank of value i among n values, descending, ties by index (used to sort
