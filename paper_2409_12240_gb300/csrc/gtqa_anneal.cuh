@@ -78,11 +78,9 @@ struct Ctx {
     const int4* vert_edges;   // edge at slots 0..2 (-1 phantom), degree
     const int* vert_inst;
     const double* J;
-    const double* h;
-    const int* colour_edges;
+    const double* hd;         // h_a / degree of a
+    const struct GateMeta* gates;   // [m], colour by colour
     const int* colour_off;    // [ncol + 1]
-    const int* last_colour;   // per vertex: colour of its last gate in a layer (-1: none)
-    const int* first_colour;  // per vertex: colour of its first gate in a layer (-1: none)
     const int* iso;           // vertices of degree 0
     int n_iso;
     int ncol;
@@ -156,18 +154,30 @@ template <int CHI, int V = 0> struct Shape {
 
 // ===========================================================================
 // gates: simple update of one edge (team of 2 CHI^2 threads)
+//
+// The FP64 pipe bounds it (64 cycles per warp instruction and sub-partition): at n = 1000,
+// chi = 4 every sub-partition holds one gate of a colour, so the time of a phase is the FP64
+// instruction count of a gate plus the latencies in between.  Hence: the four QRs keep their rows
+// in registers, all inner products of a reflector are summed at once (group_sums), scalars are
+// formed once per group of lanes, and the reflectors go to shared memory already scaled, in the
+// type of the back-application.
 // ===========================================================================
-template <int CHI>
+// One gate of the schedule, in the order the colours run: everything a team has to know before it
+// touches the state.
+struct GateMeta {
+    int4 a;   // edge, u, v, bits: slot in u, slot in v (two each); first gate of u, of v; last of u, of v
+    int4 b;   // edges at the other slots of u and of v, ascending (-1: none)
+};
+
+template <int CHI, class Mode>
 struct GateSm {
-    cd X[4][CHI][CHI * CHI];   // [block][col][row]: (a,0) (a,1) (b,0) (b,1); reused for staging
-    cd vk[4][CHI];
-    double tau[4][CHI];        // square roots of the reflector coefficients
+    using TS = typename Mode::TS;
+    C<TS> U[4][CHI][CHI * CHI];   // [block][col][row]: scaled reflectors, then the new tensors
     cd M[4 * CHI * CHI];
-    cd V[4 * CHI * CHI];
+    cd V[4 * CHI * CHI];       // first the R factors [block][row][col], then V
     cd G[4 * CHI * CHI];       // scratch of the refinement
     cf M32[4 * CHI * CHI];     // FP32 copy of M for the first stage
     cf V32[4 * CHI * CHI];
-    double w[2][CHI * CHI];
     double lab[CHI];
     double sig[2 * CHI];
     double isig[2 * CHI];      // 1 / sig
@@ -179,108 +189,203 @@ struct GateSm {
     int nrot;
 };
 
+// Householder steps K .. CHI - 1 of a (2 G) x CHI block, rows l and l + G of a lane in y0, y1.
+// The reflector of step k is stored as u = sqrt(tau) v (|u| = sqrt 2) in the type of the
+// back-application, [col][row]; y0 of the lanes l < CHI ends as the rows of R.
+template <int CHI, int G, int K, typename R, typename RB>
+__device__ __forceinline__ void qr_steps(C<R> (&y0)[CHI], C<R> (&y1)[CHI], C<RB>* U, int l, unsigned gm) {
+    if constexpr (K < CHI) {
+        using CR = C<R>;
+        constexpr int NC = CHI - 1 - K;   // later columns
+        const CR z = CR{(R)0, (R)0};
+        const CR x0 = l >= K ? y0[K] : z, x1 = y1[K];
+        // |x|^2 and x^H y of every later column
+        R s[1 + 2 * NC];
+        s[0] = fma(x0.x, x0.x, fma(x0.y, x0.y, fma(x1.x, x1.x, x1.y * x1.y)));
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const CR d = cfmac(x0, y0[K + 1 + c], cfmac(x1, y1[K + 1 + c], z));
+            s[1 + 2 * c] = d.x;
+            s[2 + 2 * c] = d.y;
+        }
+        group_sums<G>(s, gm);
+        const CR xkk = CR{__shfl_sync(gm, y0[K].x, K, G), __shfl_sync(gm, y0[K].y, K, G)};
+        const R a2 = norm2(xkk);
+        // 1 / |x| on the even lanes and 1 / |x_K| on the odd ones, in one pass of the pipe
+        const R arg = (l & 1) ? a2 : s[0];
+        const R rs = arg > (R)1e-300 ? nr_rsqrt(arg) : (R)0;
+        const R r0 = __shfl_sync(gm, rs, 0, G), ra = __shfl_sync(gm, rs, 1, G);
+        const R nrm = s[0] * r0, axkk = a2 * ra;
+        const CR ph = nonzero(ra) ? CR{xkk.x * ra, xkk.y * ra} : CR{(R)1, (R)0};
+        const R stau = nonzero(nrm) ? nr_rsqrt(nrm * (nrm + axkk)) : (R)0;
+        const CR pv = nrm * ph;
+        const CR vkk = xkk + pv;
+        // tau v^H y = tau (x^H y + conj(|x| ph) y_K), column K + 1 + c on lane c
+        CR sx = z, yk = z;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const R yx = __shfl_sync(gm, y0[K + 1 + c].x, K, G), yy = __shfl_sync(gm, y0[K + 1 + c].y, K, G);
+            if (l % CHI == c) {
+                sx = CR{s[1 + 2 * c], s[2 + 2 * c]};
+                yk = CR{yx, yy};
+            }
+        }
+        const R tau = stau * stau;
+        const CR w = tau * cfmac(pv, yk, sx);
+        const CR v0 = l == K ? vkk : x0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const CR wc = CR{__shfl_sync(gm, w.x, c, G), __shfl_sync(gm, w.y, c, G)};
+            if (l >= K) y0[K + 1 + c] = cfms(v0, wc, y0[K + 1 + c]);
+            y1[K + 1 + c] = cfms(x1, wc, y1[K + 1 + c]);
+        }
+        U[K * 2 * G + l] = ccast<RB>(stau * v0);
+        U[K * 2 * G + l + G] = ccast<RB>(stau * x1);
+        if (l == K) y0[K] = CR{-pv.x, -pv.y};
+        qr_steps<CHI, G, K + 1>(y0, y1, U, l, gm);
+    }
+}
+
+// Back-application of NK reflectors, last first: E <- (I - u u^H) E for CHI columns, rows l and
+// l + G of a lane.
+template <int CHI, int G, int NK = CHI, typename RB>
+__device__ __forceinline__ void apply_reflectors(C<RB> (&E0)[CHI], C<RB> (&E1)[CHI], const C<RB>* U, int l,
+                                                 unsigned gm) {
+    for (int k = NK - 1; k >= 0; --k) {
+        const C<RB> v0 = U[k * 2 * G + l], v1 = U[k * 2 * G + l + G];
+        RB s[2 * CHI];
+#pragma unroll
+        for (int c = 0; c < CHI; ++c) {
+            const C<RB> d = cfmac(v0, E0[c], cfmac(v1, E1[c], C<RB>{(RB)0, (RB)0}));
+            s[2 * c] = d.x;
+            s[2 * c + 1] = d.y;
+        }
+        group_sums<G>(s, gm);
+#pragma unroll
+        for (int c = 0; c < CHI; ++c) {
+            const C<RB> d = C<RB>{s[2 * c], s[2 * c + 1]};
+            E0[c] = cfms(v0, d, E0[c]);
+            E1[c] = cfms(v1, d, E1[c]);
+        }
+    }
+}
+
+// 2 log(1 - d), Eq. (gate_fidelity); the series drops terms below 1e-20
+__device__ __forceinline__ double log_fidelity(double d) {
+    return d < 1e-5 ? -2.0 * d * fma(d, fma(d, 1.0 / 3.0, 0.5), 1.0) : 2.0 * log1p(-d);
+}
+
+// Truncation of a core to chi (App. D "Truncation") by its first NM lanes: n2 the squared column
+// norms of A = U S, perm their order (descending).  Lane r takes the r-th largest: writes lambda_e
+// and isig[r] = 1 / sigma_r for the first CHI, adds the discarded weight and the log-fidelity, and
+// returns the number of triplets kept.
+template <int NM, int CHI, bool LOG32>
+__device__ __forceinline__ int truncate_core(const double* n2, const int* perm, double* isig, double* lam_e,
+                                             double* stats, int chi, double cut, int r) {
+    const unsigned mk = group_mask<NM>();
+    const double s2 = n2[perm[r]];
+    const double is = s2 > 1e-300 ? nr_rsqrt(s2) : 0.0;
+    const double sv = s2 * is;
+    const double smax = __shfl_sync(mk, sv, 0, NM);
+    const int cnt = __popc(__ballot_sync(mk, sv > cut * smax) & mk);
+    int keep = cnt < chi ? cnt : chi;
+    if (keep < 1) keep = 1;
+    double kd[2] = {r < keep ? s2 : 0.0, r < keep ? 0.0 : s2};
+    group_sums<NM>(kd, mk);
+    const double kept = kd[0], drop = kd[1];
+    const double inv = kept > 0.0 ? nr_rsqrt(kept) : 0.0;
+    if (r < CHI) {
+        lam_e[r] = r < keep ? sv * inv : 0.0;
+        isig[r] = is;
+    }
+    if (r == 0) {
+        const double tot = kept + drop;
+        const double disc = tot > 0.0 ? drop * nr_rcp(tot) : 0.0;
+        atomicAdd(&stats[0], disc);
+        // log of the gate fidelity (1 - disc)^2, Eq. (gate_fidelity); a float log in the mixed mode
+        atomicAdd(&stats[1], LOG32 ? 2.0 * (double)log1pf(-(float)disc) : log_fidelity(disc));
+    }
+    return keep;
+}
+
 template <int CHI, class Mode>
-__device__ void gate_edge(const Ctx& c, int e, int tid, int team, GateSm<CHI>& sm, double tZ, double cX, double sX,
-                          int colour, bool pre, double cXp, double sXp) {
+__device__ void gate_edge(const Ctx& c, const GateMeta& gm_, int tid, int team, GateSm<CHI, Mode>& sm, double tZ,
+                          double cX, double sX, bool pre, double cXp, double sXp) {
     using TS = typename Mode::TS;
-    constexpr int NM = 2 * CHI, NR = CHI * CHI, G = NR / 2, TEAM = 2 * CHI * CHI;
-    C<TS>* Gam = (C<TS>*)c.Gamma;
-    const int4 ei = c.edge_info[e];
-    const int vtx[2] = {ei.x, ei.y};
-    const int slot[2] = {ei.z, ei.w};
-    int oe[2][2], os[2][2];
-    for (int x = 0; x < 2; ++x) {
-        const int4 ve = c.vert_edges[vtx[x]];
-        const int es[3] = {ve.x, ve.y, ve.z};
-        others_of(slot[x], os[x][0], os[x][1]);
-        oe[x][0] = es[os[x][0]];
-        oe[x][1] = es[os[x][1]];
-    }
-    for (int t = tid; t < 2 * NR; t += TEAM) {
-        const int x = t / NR, J = t % NR;
-        sm.w[x][J] = lam_get(c.lam, CHI, oe[x][0], J / CHI) * lam_get(c.lam, CHI, oe[x][1], J % CHI);
-    }
-    for (int t = tid; t < CHI; t += TEAM) sm.lab[t] = __ldcg(c.lam + (size_t)e * CHI + t);
-    team_bar<TEAM>(team);
-    // both physical components of one element per thread, so that the leading mixing
-    // gate [[c, -i s], [-i s, c]] can act on a vertex before its first gate of the layer
-    for (int t = tid; t < 2 * CHI * NR; t += TEAM) {
-        const int x = t / (CHI * NR), rem = t % (CHI * NR);
-        const int col = rem / NR, row = rem % NR;
-        const size_t off = (size_t)vtx[x] * (2 * CHI * CHI * CHI) + col * sstride<CHI>(slot[x]) +
-                           (row / CHI) * sstride<CHI>(os[x][0]) + (row % CHI) * sstride<CHI>(os[x][1]);
-        cd g0 = ccast<double>(ldcg(Gam + off));
-        cd g1 = ccast<double>(ldcg(Gam + off + CHI * CHI * CHI));
-        if (pre && c.first_colour[vtx[x]] == colour) {
-            const cd a0 = g0, a1 = g1;
-            g0 = cd{cXp * a0.x + sXp * a1.y, cXp * a0.y - sXp * a1.x};
-            g1 = cd{sXp * a0.y + cXp * a1.x, -sXp * a0.x + cXp * a1.y};
-        }
-        sm.X[2 * x][col][row] = sm.w[x][row] * g0;
-        sm.X[2 * x + 1][col][row] = sm.w[x][row] * g1;
-    }
-    team_bar<TEAM>(team);
-
-    // ---- Householder QR of the four CHI^2 x CHI blocks, G threads per block ----
-    const int blk = tid / G, l = tid % G;
+    using CT = C<TS>;
+    constexpr int NM = 2 * CHI, NR = CHI * CHI, G = NR / 2, TEAM = 2 * CHI * CHI, H = CHI * CHI * CHI;
+    CT* Gam = (CT*)c.Gamma;
+    const int e = gm_.a.x, bits = gm_.a.w;
+    const int blk = tid / G, l = tid % G, x = blk >> 1, i = blk & 1;
     const unsigned gm = group_mask<G>();
-    const int r0 = l, r1 = l + G;
-    for (int k = 0; k < CHI; ++k) {
-        cd* Xk = sm.X[blk][k];
-        const cd z = cd{0.0, 0.0};
-        const cd x0 = (r0 >= k) ? Xk[r0] : z;
-        const cd x1 = (r1 >= k) ? Xk[r1] : z;
-        const double nrm2 = group_sum<G>(norm2(x0) + norm2(x1), gm);
-        const cd xkk = Xk[k];
-        const double nrm = nr_sqrt(nrm2);
-        const double a2 = norm2(xkk);
-        const double ra = a2 > 0.0 ? nr_rsqrt(a2) : 0.0;
-        const double axkk = a2 * ra;
-        const cd ph = a2 > 0.0 ? cd{xkk.x * ra, xkk.y * ra} : cd{1.0, 0.0};
-        const double stau = nrm > 0.0 ? nr_rsqrt(nrm * (nrm + axkk)) : 0.0;   // sqrt(tau)
-        const double tau = stau * stau;
-        const cd vkk = (axkk + nrm) * ph;
-        const cd v0 = (r0 == k) ? vkk : x0;
-        const cd v1 = x1;
-        for (int cc = k + 1; cc < CHI; ++cc) {
-            cd* Xc = sm.X[blk][cc];
-            const cd y0 = Xc[r0], y1 = Xc[r1];
-            cd d = cfmac(v0, y0, cfmac(v1, y1, z));
-            d.x = group_sum<G>(d.x, gm);
-            d.y = group_sum<G>(d.y, gm);
-            const cd td = tau * d;
-            if (r0 >= k) Xc[r0] = y0 - v0 * td;
-            Xc[r1] = y1 - v1 * td;
+    auto stride = [](int k) { return k == 0 ? CHI * CHI : (k == 1 ? CHI : 1); };
+
+    // ---- rows l and l + G of the lane's block, weighted with the other bonds ----
+    cd y0[CHI], y1[CHI];
+    double w0, w1;
+    {
+        const int slot = (bits >> (2 * x)) & 3, vtx = x ? gm_.a.z : gm_.a.y;
+        const int e0 = x ? gm_.b.z : gm_.b.x, e1 = x ? gm_.b.w : gm_.b.y;
+        int o0, o1;
+        others_of(slot, o0, o1);
+        const int ss = stride(slot), s0 = stride(o0), s1 = stride(o1);
+        const CT* g = Gam + (size_t)vtx * (2 * H) + l / CHI * s0 + l % CHI * s1;
+        const int d1 = G / CHI * s0;   // G is a multiple of CHI: row l + G lies G / CHI further along slot o0
+        CT t0[CHI], t1[CHI];
+        const bool lead = pre && ((bits >> (4 + x)) & 1);
+#pragma unroll
+        for (int cc = 0; cc < CHI; ++cc) {
+            t0[cc] = ldcg(g + i * H + cc * ss);
+            t1[cc] = ldcg(g + i * H + cc * ss + d1);
         }
-        __syncwarp(gm);
-        if (r0 == k) Xk[k] = (-nrm) * ph;
-        if (l == 0) {
-            sm.vk[blk][k] = vkk;
-            sm.tau[blk][k] = stau;
+        w0 = lam_get(c.lam, CHI, e0, l / CHI) * lam_get(c.lam, CHI, e1, l % CHI);
+        w1 = lam_get(c.lam, CHI, e0, (l + G) / CHI) * lam_get(c.lam, CHI, e1, l % CHI);
+        if (tid < CHI) sm.lab[tid] = __ldcg(c.lam + (size_t)e * CHI + tid);
+        // the four diagonal gate phases
+        if (tid < 4) {
+            const double ha = c.hd[gm_.a.y], hb = c.hd[gm_.a.z], Je = c.J[e];
+            const double za = 1.0 - 2.0 * (tid >> 1), zb = 1.0 - 2.0 * (tid & 1);
+            double sn, cs;
+            sincos(-tZ * (Je * za * zb + ha * za + hb * zb), &sn, &cs);
+            sm.ph[tid] = cd{cs, sn};
         }
-        __syncwarp(gm);
+#pragma unroll
+        for (int cc = 0; cc < CHI; ++cc) {
+            y0[cc] = ccast<double>(t0[cc]);
+            y1[cc] = ccast<double>(t1[cc]);
+            if (lead) {   // the leading mixing gate [[c, -i s], [-i s, c]]
+                const cd p0 = ccast<double>(ldcg(g + (i ^ 1) * H + cc * ss));
+                const cd p1 = ccast<double>(ldcg(g + (i ^ 1) * H + cc * ss + d1));
+                y0[cc] = cd{cXp * y0[cc].x + sXp * p0.y, cXp * y0[cc].y - sXp * p0.x};
+                y1[cc] = cd{cXp * y1[cc].x + sXp * p1.y, cXp * y1[cc].y - sXp * p1.x};
+            }
+            y0[cc] = w0 * y0[cc];
+            y1[cc] = w1 * y1[cc];
+        }
+        if (tid == 0) sm.nrot = 0;
+        team_bar<TEAM>(team);   // lab and the phases; the previous edge's readers of sm are done
+    }
+
+    // ---- Householder QR of the four CHI^2 x CHI blocks; R (side a times lambda) goes to sm.V ----
+    qr_steps<CHI, G, 0>(y0, y1, &sm.U[blk][0][0], l, gm);
+    if (l < CHI) {
+#pragma unroll
+        for (int cc = 0; cc < CHI; ++cc)
+            if (cc >= l) sm.V[(blk * CHI + l) * CHI + cc] = x == 0 ? sm.lab[cc] * y0[cc] : y0[cc];
     }
     team_bar<TEAM>(team);
 
-    // ---- core matrix M (column-major NM x NM); the 4 diagonal gate phases first ----
-    if (tid < 4) {
-        const int Da = c.vert_edges[vtx[0]].w, Db = c.vert_edges[vtx[1]].w;
-        const double ha = c.h[vtx[0]] * nr_rcp((double)Da), hb = c.h[vtx[1]] * nr_rcp((double)Db), Je = c.J[e];
-        const double za = 1.0 - 2.0 * (tid >> 1), zb = 1.0 - 2.0 * (tid & 1);
-        double sn, cs;
-        sincos(-tZ * (Je * za * zb + ha * za + hb * zb), &sn, &cs);
-        sm.ph[tid] = cd{cs, sn};
-    }
-    team_bar<TEAM>(team);
+    // ---- core matrix M (column-major NM x NM) ----
     for (int t = tid; t < NM * NM; t += TEAM) {
         const int col = t / NM, row = t % NM;
         const int ia = row / CHI, r = row % CHI, ib = col / CHI, rp = col % CHI;
+        const cd* Ra = sm.V + (ia * CHI + r) * CHI;
+        const cd* Rb = sm.V + ((2 + ib) * CHI + rp) * CHI;
         cd acc = cd{0.0, 0.0};
         const int j0 = r > rp ? r : rp;
-        for (int j = j0; j < CHI; ++j) acc = cfma(sm.lab[j] * sm.X[ia][j][r], sm.X[2 + ib][j][rp], acc);
+        for (int j = j0; j < CHI; ++j) acc = cfma(Ra[j], Rb[j], acc);
         sm.M[t] = sm.ph[2 * ia + ib] * acc;
     }
-    if (tid == 0) sm.nrot = 0;
     team_bar<TEAM>(team);
     // rounding-level entries of the core (graded spectra of the early anneal) are zeroed first
     if constexpr (TEAM <= 32) prune_noise<NM>(sm.M, tid, WarpGroup{group_mask<TEAM>()});
@@ -298,39 +403,17 @@ __device__ void gate_edge(const Ctx& c, int e, int tid, int team, GateSm<CHI>& s
     if constexpr (TEAM <= 32) done = svd(WarpGroup{group_mask<TEAM>()});
     else done = svd(TeamGroup<TEAM>{team, &sm.flag});
     if (done.rot) atomicAdd(&sm.nrot, done.rot);
-    team_bar<TEAM>(team);
-    for (int cc = tid; cc < NM; cc += TEAM) {   // sm.sig holds the squared column norms
-        const double s2 = sm.sig[cc];
-        const double is = s2 > 1e-300 ? nr_rsqrt(s2) : 0.0;
-        sm.sig[cc] = s2 * is;
-        sm.isig[cc] = is;
-    }
-    team_bar<TEAM>(team);
-    for (int cc = tid; cc < NM; cc += TEAM) sm.perm[desc_rank(sm.sig, NM, cc)] = cc;
+    if (tid < NM) sm.perm[desc_rank_bits(sm.sig, NM, tid)] = tid;   // sm.sig: squared column norms
     team_bar<TEAM>(team);
     if (tid < NM) {   // lane r holds the r-th largest singular value
-        const unsigned mk = group_mask<NM>();
-        const double sv = sm.sig[sm.perm[tid]];
-        const double smax = sm.sig[sm.perm[0]];
-        const int cnt = __popc(__ballot_sync(mk, sv > c.svd_cut * smax));
-        int keep = cnt < c.chi ? cnt : c.chi;
-        if (keep < 1) keep = 1;
-        const double s2 = sv * sv;
-        const double kept = group_sum<NM>(tid < keep ? s2 : 0.0, mk);
-        const double drop = group_sum<NM>(tid < keep ? 0.0 : s2, mk);
-        const double inv = kept > 0.0 ? nr_rsqrt(kept) : 0.0;
-        if (tid < CHI) c.lam[(size_t)e * CHI + tid] = (tid < keep) ? sv * inv : 0.0;
+        const int k = truncate_core<NM, CHI, Mode::mixed>(sm.sig, sm.perm, sm.isig, c.lam + (size_t)e * CHI, c.stats, c.chi,
+                                                          c.svd_cut, tid);
         if (tid == 0) {
-            const double tot = kept + drop;
-            const double disc = tot > 0.0 ? drop * nr_rcp(tot) : 0.0;
-            atomicAdd(&c.stats[0], disc);
-            // log of the gate fidelity (1 - disc)^2, Eq. (gate_fidelity); a float log in the mixed mode
-            atomicAdd(&c.stats[1], Mode::mixed ? 2.0 * (double)log1pf(-(float)disc) : 2.0 * log1p(-disc));
             atomicAdd(&c.stats[2], (double)done.pairs);
             atomicAdd(&c.stats[3], (double)sm.nrot);
             atomicMax(&c.ctl->gate_sw_max, done.passes);
             atomicMax(&c.ctl->gate_sw32_max, done.sweeps32);
-            sm.keep = keep;
+            sm.keep = k;
         }
     }
     team_bar<TEAM>(team);
@@ -338,63 +421,47 @@ __device__ void gate_edge(const Ctx& c, int e, int tid, int team, GateSm<CHI>& s
 
     // ---- new Gamma: reflectors of each block applied to U (side a) / V^* (side b) ----
     // FP64 mode in double, mixed mode in float (the result is stored in complex64).
-    using RB = typename Mode::TS;
-    C<RB> E0[CHI], E1[CHI];
-    const int x = blk >> 1, i = blk & 1;
+    CT E0[CHI], E1[CHI];
 #pragma unroll
     for (int cc = 0; cc < CHI; ++cc) {
-        E0[cc] = C<RB>{(RB)0, (RB)0};
-        E1[cc] = C<RB>{(RB)0, (RB)0};
-        if (r0 < CHI && cc < keep) {
+        E0[cc] = CT{(TS)0, (TS)0};
+        E1[cc] = CT{(TS)0, (TS)0};
+        if (l < CHI && cc < keep) {
             const int pc = sm.perm[cc];
-            const int row = i * CHI + r0;
-            const cd u = (x == 0) ? sm.isig[pc] * sm.M[pc * NM + row] : conj(sm.V[pc * NM + row]);
-            E0[cc] = ccast<RB>(u);
+            const int row = i * CHI + l;
+            const cd u = (x == 0) ? sm.isig[cc] * sm.M[pc * NM + row] : conj(sm.V[pc * NM + row]);
+            E0[cc] = ccast<TS>(u);
         }
     }
-    // H_k = I - tau v v^H is applied as I - u u^H with u = sqrt(tau) v (|u| = sqrt 2), so
-    // neither factor over- or underflows when the reflector is tiny (matters in float).
-    for (int k = CHI - 1; k >= 0; --k) {
-        const double st = sm.tau[blk][k];
-        const C<RB> v0 = ccast<RB>(st * ((r0 == k) ? sm.vk[blk][k] : ((r0 > k) ? sm.X[blk][k][r0] : cd{0.0, 0.0})));
-        const C<RB> v1 = ccast<RB>(st * sm.X[blk][k][r1]);
-#pragma unroll
-        for (int cc = 0; cc < CHI; ++cc) {
-            C<RB> d = cfmac(v0, E0[cc], cfmac(v1, E1[cc], C<RB>{(RB)0, (RB)0}));
-            d.x = group_sum<G>(d.x, gm);
-            d.y = group_sum<G>(d.y, gm);
-            E0[cc] = E0[cc] - v0 * d;
-            E1[cc] = E1[cc] - v1 * d;
-        }
-    }
-    const double w0 = sm.w[x][r0], w1 = sm.w[x][r1];
-    const RB iw0 = w0 > 0.0 ? (RB)nr_rcp(w0) : (RB)0, iw1 = w1 > 0.0 ? (RB)nr_rcp(w1) : (RB)0;
-    team_bar<TEAM>(team);   // everyone is done reading the reflectors in sm.X
-    // stage Gamma~ (rounded to storage) in sm.X as [x*2+i][col][row]
+    apply_reflectors<CHI, G>(E0, E1, &sm.U[blk][0][0], l, gm);
+    const TS iw0 = w0 > 0.0 ? (TS)(Mode::mixed ? nr_rcp1(w0) : nr_rcp(w0)) : (TS)0;
+    const TS iw1 = w1 > 0.0 ? (TS)(Mode::mixed ? nr_rcp1(w1) : nr_rcp(w1)) : (TS)0;
+    team_bar<TEAM>(team);   // everyone is done reading the reflectors
 #pragma unroll
     for (int cc = 0; cc < CHI; ++cc) {
-        sm.X[blk][cc][r0] = ccast<double>(ccast<TS>(iw0 * E0[cc]));
-        sm.X[blk][cc][r1] = ccast<double>(ccast<TS>(iw1 * E1[cc]));
+        sm.U[blk][cc][l] = iw0 * E0[cc];
+        sm.U[blk][cc][l + G] = iw1 * E1[cc];
     }
     team_bar<TEAM>(team);
     // write back, applying the mixing gate to a vertex after its last gate of the layer
+    const TS cs = (TS)cX, sn = (TS)sX;
     for (int t = tid; t < 2 * CHI * NR; t += TEAM) {
         const int xx = t / (CHI * NR), rem = t % (CHI * NR);
         const int col = rem / NR, row = rem % NR;
-        C<TS> g0 = ccast<TS>(sm.X[2 * xx][col][row]);
-        C<TS> g1 = ccast<TS>(sm.X[2 * xx + 1][col][row]);
-        if (c.last_colour[vtx[xx]] == colour) {
-            const C<TS> a0 = g0, a1 = g1;
-            const TS cs = (TS)cX, sn = (TS)sX;
+        const int slot = (bits >> (2 * xx)) & 3, vtx = xx ? gm_.a.z : gm_.a.y;
+        int o0, o1;
+        others_of(slot, o0, o1);
+        CT g0 = sm.U[2 * xx][col][row];
+        CT g1 = sm.U[2 * xx + 1][col][row];
+        if ((bits >> (6 + xx)) & 1) {
+            const CT a0 = g0, a1 = g1;
             // [[c, -i s], [-i s, c]]
-            g0 = C<TS>{cs * a0.x + sn * a1.y, cs * a0.y - sn * a1.x};
-            g1 = C<TS>{sn * a0.y + cs * a1.x, -sn * a0.x + cs * a1.y};
+            g0 = CT{cs * a0.x + sn * a1.y, cs * a0.y - sn * a1.x};
+            g1 = CT{sn * a0.y + cs * a1.x, -sn * a0.x + cs * a1.y};
         }
-        const size_t base = (size_t)vtx[xx] * (2 * CHI * CHI * CHI);
-        const size_t off = col * sstride<CHI>(slot[xx]) + (row / CHI) * sstride<CHI>(os[xx][0]) +
-                           (row % CHI) * sstride<CHI>(os[xx][1]);
-        Gam[base + off] = g0;
-        Gam[base + CHI * CHI * CHI + off] = g1;
+        CT* g = Gam + (size_t)vtx * (2 * H) + col * stride(slot) + (row / CHI) * stride(o0) + (row % CHI) * stride(o1);
+        g[0] = g0;
+        g[H] = g1;
     }
 }
 
@@ -1187,7 +1254,7 @@ template <int CHI, class Mode, unsigned PH, int V = 0>
 struct SmemSize {
     using S = Shape<CHI, V>;
     static constexpr int TPB = S::TPB;
-    static constexpr size_t gate = sizeof(GateSm<CHI>) * (TPB / S::TG);
+    static constexpr size_t gate = sizeof(GateSm<CHI, Mode>) * (TPB / S::TG);
     // per-team caches, block sums (64 doubles), scratch of the exact-distance pass
     static constexpr size_t bp = sizeof(BPSm<CHI, Mode, S::TB>) * (TPB / S::TB) + 64 * sizeof(double) +
                                  sizeof(C<typename Mode::TS>) * 2 * TPB;
@@ -1231,15 +1298,23 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
                 sincos(tX + tXp, &sXi, &cXi);   // vertices without gates: both mixing gates at once
             }
             const int team = threadIdx.x / S::TG, tid = threadIdx.x % S::TG;
-            GateSm<CHI>& sm = reinterpret_cast<GateSm<CHI>*>(smem)[team];
+            GateSm<CHI, Mode>& sm = reinterpret_cast<GateSm<CHI, Mode>*>(smem)[team];
             const int gteam = team * c.nblocks + blockIdx.x;
+            GateMeta next = {};
+            if (c.ncol > 0 && c.colour_off[0] + gteam < c.colour_off[1]) next = c.gates[c.colour_off[0] + gteam];
             for (int col = 0; col < c.ncol; ++col) {
                 const int beg = c.colour_off[col], end = c.colour_off[col + 1];
-                for (int idx = beg + gteam; idx < end; idx += nteams_total_g)
-                    gate_edge<CHI, Mode>(c, c.colour_edges[idx], tid, team, sm, tZ, cX, sX, col, pre, cXp, sXp);
+                for (int idx = beg + gteam; idx < end; idx += nteams_total_g) {
+                    const GateMeta gm = next;
+                    if (idx + nteams_total_g < end) next = c.gates[idx + nteams_total_g];
+                    gate_edge<CHI, Mode>(c, gm, tid, team, sm, tZ, cX, sX, pre, cXp, sXp);
+                }
                 if (col == c.ncol - 1)
                     for (int q = gteam; q < c.n_iso; q += nteams_total_g)
                         mixing_vertex<CHI, Mode>(c, c.iso[q], tid, S::TG, cXi, sXi);
+                // the next colour's first gate is known before the barrier
+                else if (end + gteam < c.colour_off[col + 2])
+                    next = c.gates[end + gteam];
                 if (!grid_sync(gb, c.spin_limit)) return;
             }
             if (c.ncol == 0) {

@@ -78,8 +78,7 @@ struct gtqa_state {
     double* h = nullptr;
     int* colour_edges = nullptr;
     int* colour_off = nullptr;
-    int* last_colour = nullptr;
-    int* first_colour = nullptr;
+    GateMeta* gates_meta = nullptr;
     int* iso = nullptr;
     int n_iso = 0;
     int* inst_vbeg = nullptr;
@@ -512,7 +511,7 @@ void free_state(gtqa_state* s) {
     for (cudaEvent_t e : s->gev)
         if (e) cudaEventDestroy(e);
     void* ptrs[] = {s->kdev, s->Gamma, s->lam, s->T, s->msg[0], s->msg[1], s->D0, s->t0, s->X, s->edge_info,
-                    s->vert_edges, s->vert_inst, s->J, s->h, s->colour_edges, s->colour_off, s->last_colour, s->first_colour,
+                    s->vert_edges, s->vert_inst, s->J, s->h, s->colour_edges, s->colour_off, s->gates_meta,
                     s->iso, s->inst_vbeg, s->inst_m, s->acc, s->inst_done, s->inst_iters, s->inst_dist,
                     s->stats, s->ctl, s->rho, s->sign, s->flags, s->rbuf, s->cutbuf, s->xs, s->ps,
                     s->gate_edge, s->gate_U, s->sq_vertex, s->sq_W, s->vslots4, s->allv, s->pscratch, s->dm};
@@ -536,11 +535,9 @@ Ctx make_ctx(const gtqa_state* s) {
     c.vert_edges = s->vert_edges;
     c.vert_inst = s->vert_inst;
     c.J = s->J;
-    c.h = s->h;
-    c.colour_edges = s->colour_edges;
+    c.hd = s->h;
+    c.gates = s->gates_meta;
     c.colour_off = s->colour_off;
-    c.last_colour = s->last_colour;
-    c.first_colour = s->first_colour;
     c.iso = s->iso;
     c.n_iso = s->n_iso;
     c.ncol = s->ncol;
@@ -803,8 +800,7 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
         (rc = dalloc(s, &s->X, (size_t)s->m * 2 * CHI * CHI)) || (rc = dalloc(s, &s->edge_info, s->m)) ||
         (rc = dalloc(s, &s->vert_edges, s->n)) || (rc = dalloc(s, &s->vert_inst, s->n)) ||
         (rc = dalloc(s, &s->J, s->m)) || (rc = dalloc(s, &s->h, s->n)) || (rc = dalloc(s, &s->colour_edges, s->m)) ||
-        (rc = dalloc(s, &s->colour_off, ncol + 1)) || (rc = dalloc(s, &s->last_colour, s->n)) ||
-        (rc = dalloc(s, &s->first_colour, s->n)) ||
+        (rc = dalloc(s, &s->colour_off, ncol + 1)) || (rc = dalloc(s, &s->gates_meta, s->m)) ||
         (rc = dalloc(s, &s->iso, iso.size())) || (rc = dalloc(s, &s->inst_vbeg, B + 1)) ||
         (rc = dalloc(s, &s->inst_m, B)) || (rc = dalloc(s, &s->acc, 6 * (size_t)B)) ||
         (rc = dalloc(s, &s->inst_done, B)) || (rc = dalloc(s, &s->inst_iters, B)) ||
@@ -842,7 +838,24 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
     std::vector<double> l0((size_t)s->m * CHI, 0.0);
     for (long long e = 0; e < Mtot; ++e) l0[e * CHI] = 1.0;
     std::vector<double> Jv(J ? J : (const double*)nullptr, J ? J + Mtot : (const double*)nullptr);
-    std::vector<double> hv(h, h + N);
+    std::vector<double> hv(N);   // h_a / degree of a, the share of every gate at a (App. F)
+    for (long long a = 0; a < N; ++a) hv[a] = deg[a] > 0 ? h[a] / deg[a] : h[a];
+    // the gates in the order they run, with what a gate needs to know of the graph
+    std::vector<GateMeta> gmeta(s->plain ? 0 : Mtot);
+    for (size_t q = 0; q < gmeta.size(); ++q) {
+        const int ed = cedges[q], v[2] = {ge[2 * ed], ge[2 * ed + 1]};
+        int bits = 0, other[4];
+        for (int x = 0; x < 2; ++x) {
+            const int es[3] = {vedges[v[x]].x, vedges[v[x]].y, vedges[v[x]].z}, sl = x ? einfo[ed].w : einfo[ed].z;
+            int o0, o1;
+            others_of(sl, o0, o1);
+            other[2 * x] = es[o0];
+            other[2 * x + 1] = es[o1];
+            bits |= sl << (2 * x) | (firstc[v[x]] == gcol[ed]) << (4 + x) | (lastc[v[x]] == gcol[ed]) << (6 + x);
+        }
+        gmeta[q].a = make_int4(ed, v[0], v[1], bits);
+        gmeta[q].b = make_int4(other[0], other[1], other[2], other[3]);
+    }
     Control ctl0;
     std::memset(&ctl0, 0, sizeof(ctl0));
     cudaStream_t st = s->stream;
@@ -858,8 +871,7 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
               cuda_ok(s, cudaMemcpyAsync(s->h, hv.data(), sizeof(double) * N, cudaMemcpyHostToDevice, st)) &&
               cuda_ok(s, cudaMemcpyAsync(s->colour_edges, cedges.data(), sizeof(int) * Mtot, cudaMemcpyHostToDevice, st)) &&
               cuda_ok(s, cudaMemcpyAsync(s->colour_off, coff.data(), sizeof(int) * (ncol + 1), cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->last_colour, lastc.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->first_colour, firstc.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st)) &&
+              cuda_ok(s, cudaMemcpyAsync(s->gates_meta, gmeta.data(), sizeof(GateMeta) * Mtot, cudaMemcpyHostToDevice, st)) &&
               (iso.empty() || cuda_ok(s, cudaMemcpyAsync(s->iso, iso.data(), sizeof(int) * iso.size(), cudaMemcpyHostToDevice, st))) &&
               cuda_ok(s, cudaMemcpyAsync(s->inst_vbeg, vbeg.data(), sizeof(int) * (B + 1), cudaMemcpyHostToDevice, st)) &&
               cuda_ok(s, cudaMemcpyAsync(s->inst_m, minst.data(), sizeof(int) * B, cudaMemcpyHostToDevice, st)) &&

@@ -40,6 +40,12 @@ template <typename R> __device__ __forceinline__ C<R> cfmac(C<R> a, C<R> b, C<R>
     acc.y = fma(a.x, b.y, fma(-a.y, b.x, acc.y));
     return acc;
 }
+// acc - a * b
+template <typename R> __device__ __forceinline__ C<R> cfms(C<R> a, C<R> b, C<R> acc) {
+    acc.x = fma(-a.x, b.x, fma(a.y, b.y, acc.x));
+    acc.y = fma(-a.x, b.y, fma(-a.y, b.x, acc.y));
+    return acc;
+}
 template <typename To, typename From> __device__ __forceinline__ C<To> ccast(C<From> a) {
     return C<To>{(To)a.x, (To)a.y};
 }
@@ -64,6 +70,55 @@ __device__ __forceinline__ T group_sum(T v, unsigned mask) {
 #pragma unroll
     for (int off = G / 2; off > 0; off >>= 1) v += __shfl_xor_sync(mask, v, off);
     return v;
+}
+
+// Sums of NV values at once over aligned groups of G lanes.  At each butterfly level a lane hands
+// the half of the values it gives up to its partner, so NV values take about NV + log2 G
+// additions instead of NV log2 G (8 values over 8 lanes: 7 FP64 additions instead of 24); the
+// finished sums then go to every lane by shuffles, which cost no FP64 instruction.
+template <int OFF, int N, int NV, typename T>
+__device__ __forceinline__ void rs_level(T (&v)[NV], unsigned mask, unsigned lane) {
+    if constexpr (OFF > 0) {
+        if constexpr (N == 1) {
+            v[0] += __shfl_xor_sync(mask, v[0], OFF);
+            rs_level<OFF / 2, 1>(v, mask, lane);
+        } else {
+            constexpr int H = (N + 1) / 2;
+            const bool up = (lane & OFF) != 0;
+#pragma unroll
+            for (int i = 0; i < H; ++i) {
+                const T lo = v[i], hi = H + i < N ? v[H + i < N ? H + i : i] : (T)0;
+                v[i] = (up ? hi : lo) + __shfl_xor_sync(mask, up ? lo : hi, OFF);
+            }
+            rs_level<OFF / 2, H>(v, mask, lane);
+        }
+    }
+}
+// lane of the group and place there that hold the sum of value i
+__host__ __device__ constexpr int rs_lane(int off, int n, int i) {
+    return off == 0 || n == 1 ? 0
+                              : (i < (n + 1) / 2 ? rs_lane(off / 2, (n + 1) / 2, i)
+                                                 : off + rs_lane(off / 2, (n + 1) / 2, i - (n + 1) / 2));
+}
+__host__ __device__ constexpr int rs_place(int off, int n, int i) {
+    return off == 0 || n == 1 ? i
+                              : (i < (n + 1) / 2 ? rs_place(off / 2, (n + 1) / 2, i)
+                                                 : rs_place(off / 2, (n + 1) / 2, i - (n + 1) / 2));
+}
+template <int G, int I, int NV, typename T>
+__device__ __forceinline__ void rs_collect(const T (&v)[NV], T (&out)[NV], unsigned mask) {
+    if constexpr (I < NV) {
+        out[I] = __shfl_sync(mask, v[rs_place(G / 2, NV, I)], rs_lane(G / 2, NV, I), G);
+        rs_collect<G, I + 1>(v, out, mask);
+    }
+}
+template <int G, int NV, typename T>
+__device__ __forceinline__ void group_sums(T (&v)[NV], unsigned mask) {
+    rs_level<G / 2, NV>(v, mask, threadIdx.x & (G - 1));
+    T out[NV];
+    rs_collect<G, 0>(v, out, mask);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = out[i];
 }
 
 // Synchronisation policy for a group that lives inside one warp.
@@ -108,18 +163,17 @@ struct BlockGroup {
 // ---------------------------------------------------------------------------
 // Reciprocal and (reciprocal) square root without the FP64 divide/sqrt sequences,
 // which cost ~10-15 FP64 pipe instructions each on this part.  A hardware seed
-// (PTX rcp.approx.ftz.f64 / rsqrt.approx.ftz.f64, ~2^-22 relative error) is refined by
-// two Newton-Raphson steps (quadratic convergence: error ~2^-88, i.e. FP64 rounding).
+// (PTX rcp.approx.ftz.f64 / rsqrt.approx.ftz.f64, ~2^-22 relative error) is refined by one
+// third-order step (error e -> O(e^3) ~ 2^-63, i.e. FP64 rounding): 3 and 5 FP64 instructions,
+// against 4 and 8 for two Newton steps.
 // Float versions use the single-precision hardware approximations directly.
 // Inputs must be finite and positive (callers guard zero).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double nr_rcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);   // r (1 + e + e^2)
 }
 // one refinement step only: relative error ~2^-44, for results that are rounded to FP32
 __device__ __forceinline__ double nr_rcp1(double x) {
@@ -130,11 +184,8 @@ __device__ __forceinline__ double nr_rcp1(double x) {
 __device__ __forceinline__ double nr_rsqrt(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    // y <- y + y (1 - x y^2) / 2
-    double e = fma(-x * y, y, 1.0);
-    y = fma(0.5 * y, e, y);
-    e = fma(-x * y, y, 1.0);
-    return fma(0.5 * y, e, y);
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);   // y (1 + e/2 + 3 e^2/8)
 }
 __device__ __forceinline__ double nr_sqrt(double x) {
     if (!(x > 0.0)) return 0.0;
@@ -280,6 +331,101 @@ __device__ int jacobi_svd(C<R>* A, C<R>* V, int g, const Group& grp, unsigned pa
         }
     }
     return sweep;   // sweeps run, including the final one (without rotations unless quad_tol stopped it)
+}
+
+// hardware approximations (about 2^-22), for rotation angles
+__device__ __forceinline__ float fast_sqrt(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float fast_rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// The right singular vectors of an FP32 N x N matrix by one-sided Jacobi (the stopping rule of
+// jacobi_svd with tol 1e-6 and quad_tol 1e-3), for a group of N^2 / 2 <= 32 lanes: lane (k, r)
+// keeps row r of the two columns of pair k, and of V, in registers.  The circle ordering
+// moves one column of every pair to each neighbouring pair per step, by shuffles, so a step has
+// no shared-memory round trip and no index arithmetic: it is the latency of three shuffle
+// levels, the angle (one square root, one reciprocal, one reciprocal square root) and the move
+// (460 cycles per step of N = 8, against about 700 through shared memory).  keep < N: pairs without
+// a column among the keep largest (norms within a factor 4 of the keep-th count) do not ask for
+// another sweep, and a kept column with a smaller one is judged by the kept column's norm, as in
+// refined_svd; that saves 0.6 to 1 of 4.6 to 5.3 sweeps of the gates.
+template <int N>
+__device__ int jacobi_v32(const C<float>* A, C<float>* V, int g, unsigned gmask, unsigned pair_mask, int keep) {
+    using CF = C<float>;
+    constexpr int LN = N * N / 2, LAST = N / 2 - 1;
+    static_assert(LN <= 32, "the group lives in one warp");
+    const int k = g / N, r = g % N;
+    CF a = A[k * N + r], b = A[(N - 1 - k) * N + r];
+    CF va = CF{k == r ? 1.f : 0.f, 0.f}, vb = CF{N - 1 - k == r ? 1.f : 0.f, 0.f};
+    int sweep = 0;
+    for (; sweep < 40; ++sweep) {
+        int big = 0;
+        float thr = 0.f;   // a quarter of the keep-th largest squared norm
+        for (int step = 0; step < N - 1; ++step) {
+            float s[4] = {norm2(a), norm2(b), fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x)};
+#pragma unroll
+            for (int o = N / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s[i] += __shfl_xor_sync(pair_mask, s[i], o);
+            const float g2 = fmaf(s[2], s[2], s[3] * s[3]), ab = s[0] * s[1];
+            const bool rot = g2 > 1e-36f && g2 > 1e-12f * ab;
+            if (N > 2 && step == 0 && keep < N) {
+                int ca = 0, cb = 0;   // columns at least as long as this pair's two
+                for (int j = 0; j < N / 2; ++j) {
+                    const float x = __shfl_sync(gmask, s[0], j * N, LN), y = __shfl_sync(gmask, s[1], j * N, LN);
+                    ca += (x >= s[0]) + (y >= s[0]);
+                    cb += (x >= s[1]) + (y >= s[1]);
+                }
+                const float x = fmaxf(ca >= keep ? s[0] : 0.f, cb >= keep ? s[1] : 0.f);
+                thr = 0.25f * __int_as_float(__reduce_max_sync(gmask, __float_as_int(x)));
+            }
+            const float mx = fmaxf(s[0], s[1]), lim = fminf(s[0], s[1]) >= thr ? ab : mx * mx;
+            if (rot && mx >= thr && g2 > 1e-6f * lim) big = 1;
+            const float d = s[1] - s[0];
+            const float tn = 2.f * fast_rcp(fabsf(d) + fast_sqrt(fmaf(d, d, 4.f * g2)));
+            const float tau = rot ? (d >= 0.f ? tn : -tn) : 0.f;
+            const float c = rot ? rsqrtf(fmaf(tau * tau, g2, 1.f)) : 1.f;
+            const CF se = CF{c * tau * s[2], c * tau * s[3]};
+            const CF na = CF{fmaf(-se.x, b.x, fmaf(-se.y, b.y, c * a.x)), fmaf(-se.x, b.y, fmaf(se.y, b.x, c * a.y))};
+            const CF nb = CF{fmaf(se.x, a.x, fmaf(-se.y, a.y, c * b.x)), fmaf(se.x, a.y, fmaf(se.y, a.x, c * b.y))};
+            const CF ma = CF{fmaf(-se.x, vb.x, fmaf(-se.y, vb.y, c * va.x)), fmaf(-se.x, vb.y, fmaf(se.y, vb.x, c * va.y))};
+            const CF mb = CF{fmaf(se.x, va.x, fmaf(-se.y, va.y, c * vb.x)), fmaf(se.x, va.y, fmaf(se.y, va.x, c * vb.y))};
+            if constexpr (N > 2) {
+                // first column: from pair k + 1 (the last pair: its own second one); second column:
+                // from pair k - 1 (pair 1: the first one of pair 0; pair 0 keeps its own)
+                auto first = [&](float x, float y) {
+                    const float t = __shfl_down_sync(gmask, x, N, LN);
+                    return k == LAST ? y : t;
+                };
+                auto second = [&](float x, float y) {
+                    const float t = __shfl_up_sync(gmask, k == 0 ? x : y, N, LN);
+                    return k == 0 ? y : t;
+                };
+                a = CF{first(na.x, nb.x), first(na.y, nb.y)};
+                b = CF{second(na.x, nb.x), second(na.y, nb.y)};
+                va = CF{first(ma.x, mb.x), first(ma.y, mb.y)};
+                vb = CF{second(ma.x, mb.x), second(ma.y, mb.y)};
+            } else {
+                a = na;
+                b = nb;
+                va = ma;
+                vb = mb;
+            }
+        }
+        if (!__any_sync(gmask, big)) {
+            ++sweep;
+            break;
+        }
+    }
+    // after a whole sweep every column is back at its pair
+    V[k * N + r] = va;
+    V[(N - 1 - k) * N + r] = vb;
+    return sweep;
 }
 
 // True if x (an updated squared norm) is negative, zero or below about half of ref, from the
@@ -551,6 +697,10 @@ __device__ __forceinline__ double inv_exp2(int bits) {
     return bits > 0 && bits < 2046 ? __longlong_as_double((long long)(2046 - bits) << 52) : 0.0;
 }
 
+// whether a non-negative value is not zero, from its bits (no FP64 compare)
+__device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.f; }
+
 struct SvdCount {       // work of one decomposition
     int passes = 0;     // refinement passes (and sweeps of a closing jacobi_polish)
     int sweeps32 = 0;   // FP32 sweeps
@@ -562,11 +712,17 @@ struct SvdCount {       // work of one decomposition
 // rounding).  V32 holds V rounded afterwards.
 template <int N, bool F64, typename Group>
 __device__ int svd32_unitary(C<double>* V, C<float>* A32, C<float>* V32, double* nrm, int g, const Group& grp,
-                             unsigned pair_mask) {
+                             unsigned pair_mask, int keep) {
     constexpr int LN = N * N / 2;
     int step, p, q;
     const bool has = lane_pair<N>(g, step, p, q);
-    const int sw = jacobi_svd<N, float>(A32, V32, g, grp, pair_mask, 1e-6f, 40, true, nullptr, 1e-3f);
+    int sw;
+    if constexpr (LN <= 32) {
+        sw = jacobi_v32<N>(A32, V32, g, group_mask<LN>(), pair_mask, keep);
+        grp.sync();
+    } else {
+        sw = jacobi_svd<N, float>(A32, V32, g, grp, pair_mask, 1e-6f, 40, true, nullptr, 1e-3f);
+    }
 #pragma unroll
     for (int j = 0; j < 2; ++j) V[g + j * LN] = ccast<double>(V32[g + j * LN]);
     grp.sync();
@@ -614,7 +770,7 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         for (int j = 0; j < 2; ++j) A32[g + j * LN] = ccast<float>(sc * A[g + j * LN]);
         grp.sync();
     }
-    cnt.sweeps32 = svd32_unitary<N, F64>(V, A32, V32, nrm, g, grp, pair_mask);
+    cnt.sweeps32 = svd32_unitary<N, F64>(V, A32, V32, nrm, g, grp, pair_mask, keep_rank);
     mul64<N, false>(A, V, g, grp);
     const float stop2 = stop * stop, cut2 = (float)(0.25 * cut * cut);
     int second = 0;   // FP32 runs on a part of the columns
@@ -734,7 +890,7 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                 A32[t] = ((cols >> (t / N)) & 1u) ? ccast<float>(sc * A[t]) : CF{0.f, 0.f};
             }
             grp.sync();
-            cnt.sweeps32 += svd32_unitary<N, F64>(T, A32, V32, nrm, g, grp, pair_mask);
+            cnt.sweeps32 += svd32_unitary<N, F64>(T, A32, V32, nrm, g, grp, pair_mask, N);
             mul64<N, false>(A, T, g, grp);
             mul64<N, false>(V, T, g, grp);
         }
@@ -760,6 +916,19 @@ __device__ __forceinline__ int desc_rank(const R* v, int n, int i) {
     for (int j = 0; j < n; ++j) {
         const R y0 = v[j];
         const R y = (y0 == y0) ? y0 : (R)-INFINITY;
+        rk += (y > x) || (y == x && j < i);
+    }
+    return rk;
+}
+
+// desc_rank for non-negative doubles on the integer pipe (their bits order as integers; a NaN
+// ranks below every number).
+__device__ __forceinline__ int desc_rank_bits(const double* v, int n, int i) {
+    constexpr long long inf = 0x7ff0000000000000ll;
+    const long long x0 = __double_as_longlong(v[i]), x = x0 >= 0 && x0 <= inf ? x0 : -1;
+    int rk = 0;
+    for (int j = 0; j < n; ++j) {
+        const long long y0 = __double_as_longlong(v[j]), y = y0 >= 0 && y0 <= inf ? y0 : -1;
         rk += (y > x) || (y == x && j < i);
     }
     return rk;
