@@ -871,7 +871,7 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
               cuda_ok(s, cudaMemcpyAsync(s->h, hv.data(), sizeof(double) * N, cudaMemcpyHostToDevice, st)) &&
               cuda_ok(s, cudaMemcpyAsync(s->colour_edges, cedges.data(), sizeof(int) * Mtot, cudaMemcpyHostToDevice, st)) &&
               cuda_ok(s, cudaMemcpyAsync(s->colour_off, coff.data(), sizeof(int) * (ncol + 1), cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->gates_meta, gmeta.data(), sizeof(GateMeta) * Mtot, cudaMemcpyHostToDevice, st)) &&
+              cuda_ok(s, cudaMemcpyAsync(s->gates_meta, gmeta.data(), sizeof(GateMeta) * gmeta.size(), cudaMemcpyHostToDevice, st)) &&
               (iso.empty() || cuda_ok(s, cudaMemcpyAsync(s->iso, iso.data(), sizeof(int) * iso.size(), cudaMemcpyHostToDevice, st))) &&
               cuda_ok(s, cudaMemcpyAsync(s->inst_vbeg, vbeg.data(), sizeof(int) * (B + 1), cudaMemcpyHostToDevice, st)) &&
               cuda_ok(s, cudaMemcpyAsync(s->inst_m, minst.data(), sizeof(int) * B, cudaMemcpyHostToDevice, st)) &&
