@@ -213,7 +213,7 @@ __device__ __forceinline__ void qr_steps(C<R> (&y0)[CHI], C<R> (&y1)[CHI], C<RB>
         const R a2 = norm2(xkk);
         // 1 / |x| on the even lanes and 1 / |x_K| on the odd ones, in one pass of the pipe
         const R arg = (l & 1) ? a2 : s[0];
-        const R rs = arg > (R)1e-300 ? nr_rsqrt(arg) : (R)0;
+        const R rs = arg > tiny_norm2<R>() ? nr_rsqrt(arg) : (R)0;
         const R r0 = __shfl_sync(gm, rs, 0, G), ra = __shfl_sync(gm, rs, 1, G);
         const R nrm = s[0] * r0, axkk = a2 * ra;
         const CR ph = nonzero(ra) ? CR{xkk.x * ra, xkk.y * ra} : CR{(R)1, (R)0};

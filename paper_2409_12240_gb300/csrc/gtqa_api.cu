@@ -110,9 +110,8 @@ struct gtqa_state {
     cd* pscratch = nullptr;     // plain path: per-block tensor buffers in global memory
     cd* dm = nullptr;           // plain path: new - old of every message of a sweep
     int4* vslots4 = nullptr;
-    int* allv = nullptr;
-    std::vector<int> h_deg, h_cedges, h_coff;
-    std::vector<double> h_J, h_h;
+    int* gate_bits = nullptr;   // per gate in colour order: first and last gates of its vertices
+    std::vector<int> h_coff;    // first gate of every colour
     int cur4 = 0;               // message buffer holding the latest messages (degree 4)
     // gtqa_anneal_graph: one captured layer (gates, BP, regauge) whose layer index is read from
     // *kdev, and what it was captured for; with profiling on, events between the launches
@@ -514,7 +513,7 @@ void free_state(gtqa_state* s) {
                     s->vert_edges, s->vert_inst, s->J, s->h, s->colour_edges, s->colour_off, s->gates_meta,
                     s->iso, s->inst_vbeg, s->inst_m, s->acc, s->inst_done, s->inst_iters, s->inst_dist,
                     s->stats, s->ctl, s->rho, s->sign, s->flags, s->rbuf, s->cutbuf, s->xs, s->ps,
-                    s->gate_edge, s->gate_U, s->sq_vertex, s->sq_W, s->vslots4, s->allv, s->pscratch, s->dm};
+                    s->gate_edge, s->gate_U, s->sq_vertex, s->sq_W, s->vslots4, s->gate_bits, s->pscratch, s->dm};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& p : s->pending) {
@@ -783,12 +782,22 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
             if (gcol[e] == c) cedges.push_back((int)e);
     }
     coff[ncol] = (int)cedges.size();
+    std::vector<int> gbits;
     if (s->plain) {
-        s->h_cedges = cedges;
         s->h_coff = coff;
-        s->h_J.assign(J ? J : (const double*)nullptr, J ? J + Mtot : (const double*)nullptr);
-        s->h_h.assign(h, h + N);
-        s->h_deg.assign(deg.begin(), deg.end());
+        gbits.resize(Mtot);
+        for (long long q = 0; q < Mtot; ++q) {
+            const int ed = cedges[q];
+            for (int x = 0; x < 2; ++x) {
+                const int v = ge[2 * (size_t)ed + x];
+                gbits[q] |= (firstc[v] == gcol[ed]) << x | (lastc[v] == gcol[ed]) << (2 + x);
+            }
+        }
+        if (plain_ising_launch(s->CHI, s->D, pmode, nullptr, nullptr) != cudaSuccess) {
+            cudaGetLastError();
+            delete s;
+            return GTQA_ERR_CUDA;
+        }
     }
     const int CHI = s->CHI;
     const size_t gel = gamma_elems(s), mel = msg_elems(s), eb = elem_bytes(s);
@@ -809,17 +818,15 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
         (rc = dalloc(s, &s->flags, 4)) || (rc = dalloc(s, &s->rbuf, 1)) ||
         (rc = dalloc(s, &s->cutbuf, std::max(s->m, 1))) || (rc = dalloc(s, &s->xs, s->n)) ||
         (rc = dalloc(s, &s->ps, s->n)) || (s->plain && (rc = dalloc(s, &s->vslots4, s->n))) ||
-        (s->plain && (rc = dalloc(s, &s->allv, s->n))) ||
+        (s->plain && (rc = dalloc(s, &s->gate_bits, s->m))) ||
         (s->plain && (rc = dalloc(s, &s->pscratch, plain_scratch_entries(s->CHI, s->D, s->n, s->m)))) ||
         (s->plain && (rc = dalloc(s, &s->dm, (size_t)2 * s->m * CHI * CHI)))) {
         free_state(s);
         return rc;
     }
     if (s->plain) {
-        std::vector<int> all(N);
-        for (long long a = 0; a < N; ++a) all[a] = (int)a;
         if (!cuda_ok(s, cudaMemcpyAsync(s->vslots4, v4.data(), sizeof(int4) * N, cudaMemcpyHostToDevice, s->stream)) ||
-            !cuda_ok(s, cudaMemcpyAsync(s->allv, all.data(), sizeof(int) * N, cudaMemcpyHostToDevice, s->stream)) ||
+            !cuda_ok(s, cudaMemcpyAsync(s->gate_bits, gbits.data(), sizeof(int) * Mtot, cudaMemcpyHostToDevice, s->stream)) ||
             !cuda_ok(s, cudaStreamSynchronize(s->stream))) {
             free_state(s);
             return GTQA_ERR_CUDA;
@@ -1022,87 +1029,42 @@ int d4_fail(gtqa_state* s) {
     return GTQA_ERR_CUDA;
 }
 
-// exp(-i t X) on every vertex (Sec. II D)
-int d4_mixing(gtqa_state* s, double t) {
-    if (t == 0.0 || s->n == 0) return GTQA_OK;
-    std::vector<double> W(8 * (size_t)s->n);
-    const double c = std::cos(t), sn = std::sin(t);
-    for (int a = 0; a < s->n; ++a) {
-        double* w = &W[8 * (size_t)a];
-        w[0] = c; w[1] = 0.0; w[2] = 0.0; w[3] = -sn;
-        w[4] = 0.0; w[5] = -sn; w[6] = c; w[7] = 0.0;
-    }
-    int rc;
-    if ((rc = grow_pair(s, &s->sq_vertex, &s->sq_W, 4, s->sq_cap, (size_t)s->n))) return rc;
-    if (!cuda_ok(s, cudaMemcpyAsync(s->sq_W, W.data(), sizeof(double) * W.size(), cudaMemcpyHostToDevice, s->stream)))
-        return GTQA_ERR_CUDA;
-    if (plain_single_gates_launch(s->CHI, s->D, pm(s), s->Gamma, s->allv, s->sq_W, s->n, s->stream) != cudaSuccess)
-        return d4_fail(s);
-    s->launches += 1;
-    return GTQA_OK;
-}
-
-// Edge gates of U_Z(t_Z) by colour class (App. F; App. E through the whole-side update).
-int d4_interaction(gtqa_state* s, double tZ) {
-    const int m = s->m;
-    if (m == 0) return GTQA_OK;
-    std::vector<double> U(32 * (size_t)m, 0.0);
-    for (int q = 0; q < m; ++q) {
-        const int e = s->h_cedges[q];
-        const int a = s->h_edges[2 * (size_t)e], b = s->h_edges[2 * (size_t)e + 1];
-        const double ha = s->h_h[a] / s->h_deg[a], hb = s->h_h[b] / s->h_deg[b], Je = s->h_J.empty() ? 0.0 : s->h_J[e];
-        for (int ia = 0; ia < 2; ++ia)
-            for (int ib = 0; ib < 2; ++ib) {
-                const double za = 1.0 - 2.0 * ia, zb = 1.0 - 2.0 * ib;
-                const double ph = -tZ * (Je * za * zb + ha * za + hb * zb);
-                const int d = 2 * ia + ib;
-                U[32 * (size_t)q + 2 * (4 * d + d)] = std::cos(ph);
-                U[32 * (size_t)q + 2 * (4 * d + d) + 1] = std::sin(ph);
-            }
-    }
-    int rc;
-    if ((rc = grow_pair(s, &s->gate_edge, &s->gate_U, 16, s->gate_cap, (size_t)m))) return rc;
-    if (!cuda_ok(s, cudaMemcpyAsync(s->gate_U, U.data(), sizeof(double) * U.size(), cudaMemcpyHostToDevice, s->stream)))
-        return GTQA_ERR_CUDA;
+// One layer U_X(tXpost) U_Z(tZ) U_X(tXpre): the edge gates by colour class, which apply the mixing
+// gates of their vertices (Sec. II D); vertices without edges get both mixing angles at once.
+int d4_trotter(gtqa_state* s, double tZ, double tXpre, double tXpost) {
+    PlainGateArgs g;
+    g.Gamma = s->Gamma;
+    g.lam = s->lam;
+    g.edge_info = s->edge_info;
+    g.vslots = s->vslots4;
+    g.J = s->J;
+    g.hd = s->h;
+    g.scratch = s->pscratch;
+    g.stats = s->stats;
+    g.ctl = s->ctl;
+    g.chi = s->chi;
+    g.svd_cut = s->svd_cutoff;
+    g.tZ = tZ;
+    g.cX = std::cos(tXpost);
+    g.sX = std::sin(tXpost);
+    g.pre = tXpre != 0.0;
+    g.cXp = std::cos(tXpre);
+    g.sXp = std::sin(tXpre);
     for (int c = 0; c < s->ncol; ++c) {
-        cudaError_t e;
-        if (s->CHI == 16) {
-            Gate16Args g;
-            g.Gamma = s->Gamma;
-            g.lam = s->lam;
-            g.edge_info = s->edge_info;
-            g.vslots = s->vslots4;
-            g.gate_edge = s->colour_edges + s->h_coff[c];
-            g.gate_U = s->gate_U + 16 * (size_t)s->h_coff[c];
-            g.scratch = s->pscratch;
-            g.count = s->h_coff[c + 1] - s->h_coff[c];
-            g.stats = s->stats;
-            g.chi = s->chi;
-            g.svd_cut = s->svd_cutoff;
-            e = ising16_gates_launch(g, pm(s), s->stream);
-        } else {
-            GenArgs g;
-            g.Gamma = s->Gamma;
-            g.lam = s->lam;
-            g.edge_info = s->edge_info;
-            g.vert_edges = s->vslots4;
-            g.gate_edge = s->colour_edges + s->h_coff[c];
-            g.gate_U = s->gate_U + 16 * (size_t)s->h_coff[c];
-            g.count = s->h_coff[c + 1] - s->h_coff[c];
-            g.stats = s->stats;
-            g.chi = s->chi;
-            g.svd_cut = s->svd_cutoff;
-            e = plain_general_gates_launch(s->CHI, s->D, pm(s), g, s->stream);
-        }
-        if (e != cudaSuccess) return d4_fail(s);
+        g.gate_edge = s->colour_edges + s->h_coff[c];
+        g.gate_bits = s->gate_bits + s->h_coff[c];
+        g.count = s->h_coff[c + 1] - s->h_coff[c];
+        if (g.count <= 0) continue;
+        if (plain_ising_launch(s->CHI, s->D, pm(s), &g, s->stream) != cudaSuccess) return d4_fail(s);
         s->launches += 1;
     }
-    return GTQA_OK;
-}
-
-int d4_trotter(gtqa_state* s, double tZ, double tXpre, double tXpost) {
-    int rc;
-    if ((rc = d4_mixing(s, tXpre)) || (rc = d4_interaction(s, tZ)) || (rc = d4_mixing(s, tXpost))) return rc;
+    if (s->n_iso > 0 && tXpre + tXpost != 0.0) {
+        const double t = tXpre + tXpost;
+        if (plain_mixing_launch(s->CHI, s->D, pm(s), s->Gamma, s->iso, s->n_iso, std::cos(t), std::sin(t), s->stream) !=
+            cudaSuccess)
+            return d4_fail(s);
+        s->launches += 1;
+    }
     s->layers += 1;
     s->gates += s->m;
     return GTQA_OK;

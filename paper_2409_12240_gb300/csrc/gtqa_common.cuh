@@ -697,6 +697,9 @@ __device__ __forceinline__ double inv_exp2(int bits) {
     return bits > 0 && bits < 2046 ? __longlong_as_double((long long)(2046 - bits) << 52) : 0.0;
 }
 
+// squared norms at or below this count as zero (their reciprocal roots leave the range)
+template <typename R> __host__ __device__ constexpr R tiny_norm2() { return 1e-300; }
+template <> __host__ __device__ constexpr float tiny_norm2<float>() { return 0.f; }
 // whether a non-negative value is not zero, from its bits (no FP64 compare)
 __device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) != 0; }
 __device__ __forceinline__ bool nonzero(float x) { return x != 0.f; }

@@ -48,30 +48,60 @@ struct GenShape {
 template <int CHI, int D = 3, typename R = double>
 struct GenSm {
     using S = GenShape<CHI, D>;
-    C<R> X[2][S::NC][S::NR];   // [side][column (i, j)][row J]; reflectors after the QR
-    C<R> vk[2][S::NC];
-    R tau[2][S::NC];
+    C<R> X[2][S::NC][S::NR];   // [side][column (i, j)][row J]; scaled reflectors after the QR
+    C<R> Rf[2][S::NC][S::NC];  // R factors, [side][row][column]
     C<R> M[S::NM * S::NM];
     C<R> V[S::NM * S::NM];
+    C<R> T[sizeof(R) == 8 ? S::NM * S::NM : 1];   // scratch of refined_svd
+    cf M32[sizeof(R) == 8 ? S::NM * S::NM : 1];
+    cf V32[sizeof(R) == 8 ? S::NM * S::NM : 1];
     C<R> U[16];
     R w[2][S::NR];
     R lab[CHI];
-    R sig[S::NM];
+    double n2[S::NM], isig[CHI];
     int perm[S::NM];
     int keep;
     int flag;
     int nrot;
+    unsigned relmask;
 };
+
+// The SVD of a core: FP64 by refined_svd, FP32 by one-sided Jacobi.  n2: squared column norms.
+template <int NM, typename Group>
+__device__ __forceinline__ SvdCount core_svd(C<double>* M, C<double>* V, C<float>* M32, C<float>* V32, C<double>* T,
+                                             double* n2, unsigned* relmask, int g, const Group& grp, double cut, int chi) {
+    prune_noise<NM>(M, g, grp);
+    return refined_svd<NM, true>(M, V, M32, V32, T, n2, relmask, g, grp, group_mask<NM>(), cut, chi, 1e-8f, 1e-15);
+}
+template <int NM, typename Group>
+__device__ __forceinline__ SvdCount core_svd(C<float>* M, C<float>* V, C<float>*, C<float>*, C<float>*, double* n2,
+                                             unsigned*, int g, const Group& grp, double, int) {
+    SvdCount cnt;
+    int rot = 0;
+    cnt.sweeps32 = jacobi_svd<NM, float>(M, V, g, grp, group_mask<NM>(), 1e-6f, 60, true, &rot, 1e-3f);
+    cnt.passes = cnt.sweeps32;
+    cnt.pairs = cnt.sweeps32 * (NM - 1) * (NM / 2);
+    cnt.rot = rot;
+    grp.sync();
+    if (g < NM) {
+        float s = 0.f;
+        for (int r = 0; r < NM; ++r) s += norm2(M[g * NM + r]);
+        n2[g] = (double)s;
+    }
+    grp.sync();
+    return cnt;
+}
 
 template <int CHI, int D, class Mode>
 __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kernel(GenArgs c) {
     using TS = typename Mode::TS;
     using R = typename Mode::RC;   // FP64, or FP32 in the complex64 mode
     using CR = C<R>;
-    constexpr bool R64 = sizeof(R) == 8;
     using S = GenShape<CHI, D>;
     constexpr int NR = S::NR, NC = S::NC, NM = S::NM, G = S::G, TEAM = S::TEAM, HV = ipow(CHI, D);
     static_assert(G <= 32, "a Householder group must fit in one warp");
+    // rows in registers: every pivot row is some lane's first row, and 2 NC complex values fit
+    constexpr bool QREG = NC <= G && NC <= 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GenSm<CHI, D, R>& sm = *reinterpret_cast<GenSm<CHI, D, R>*>(smem_raw);
     const int g = threadIdx.x;
@@ -135,40 +165,57 @@ __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kerne
     if (g < 2 * G) {
         const int x = g / G;
         const unsigned gm = group_mask<G>();
-        for (int k = 0; k < NC; ++k) {
-            CR* Xk = sm.X[x][k];
-            const CR z = CR{(R)0, (R)0};
-            const CR x0 = (r0 >= k) ? Xk[r0] : z;
-            const CR x1 = (r1 >= k) ? Xk[r1] : z;
-            const R nrm2 = group_sum<G>(norm2(x0) + norm2(x1), gm);
-            const CR xkk = Xk[k];
-            const R nrm = nr_sqrt(nrm2);
-            const R a2 = norm2(xkk);
-            const R ra = a2 > 0.0 ? nr_rsqrt(a2) : 0.0;
-            const R axkk = a2 * ra;
-            const CR ph = a2 > 0.0 ? CR{xkk.x * ra, xkk.y * ra} : CR{(R)1, (R)0};
-            const R tau = nrm > 0.0 ? nr_rcp(nrm * (nrm + axkk)) : 0.0;
-            const CR vkk = (axkk + nrm) * ph;
-            const CR v0 = (r0 == k) ? vkk : x0;
-            const CR v1 = (r1 == k) ? vkk : x1;
-            for (int cc = k + 1; cc < NC; ++cc) {
-                CR* Xc = sm.X[x][cc];
-                const CR y0 = Xc[r0], y1 = Xc[r1];
-                CR d = cfmac(v0, y0, cfmac(v1, y1, z));
-                d.x = group_sum<G>(d.x, gm);
-                d.y = group_sum<G>(d.y, gm);
-                const CR td = tau * d;
-                if (r0 >= k) Xc[r0] = y0 - v0 * td;
-                if (r1 >= k) Xc[r1] = y1 - v1 * td;
+        if constexpr (QREG) {
+            // rows in registers, as in the Ising gates; the reflectors stay scaled (sqrt(tau) v) in
+            // sm.X, R in sm.R
+            CR y0[NC], y1[NC];
+#pragma unroll
+            for (int cc = 0; cc < NC; ++cc) {
+                y0[cc] = sm.X[x][cc][r0];
+                y1[cc] = sm.X[x][cc][r1];
             }
-            __syncwarp(gm);
-            if (r0 == k) Xk[k] = (-nrm) * ph;
-            if (r1 == k) Xk[k] = (-nrm) * ph;
-            if (l == 0) {
-                sm.vk[x][k] = vkk;
-                sm.tau[x][k] = tau;
+            qr_steps<NC, G, 0>(y0, y1, &sm.X[x][0][0], l, gm);
+            if (l < NC) {
+#pragma unroll
+                for (int cc = 0; cc < NC; ++cc)
+                    if (cc >= l) sm.Rf[x][l][cc] = y0[cc];
             }
-            __syncwarp(gm);
+        } else {
+            for (int k = 0; k < NC; ++k) {
+                CR* Xk = sm.X[x][k];
+                const CR z = CR{(R)0, (R)0};
+                const CR x0 = (r0 >= k) ? Xk[r0] : z;
+                const CR x1 = (r1 >= k) ? Xk[r1] : z;
+                const R nrm2 = group_sum<G>(norm2(x0) + norm2(x1), gm);
+                const CR xkk = Xk[k];
+                const R nrm = nr_sqrt(nrm2);
+                const R a2 = norm2(xkk);
+                const R ra = a2 > tiny_norm2<R>() ? nr_rsqrt(a2) : (R)0;
+                const R axkk = a2 * ra;
+                const CR ph = ra > (R)0 ? CR{xkk.x * ra, xkk.y * ra} : CR{(R)1, (R)0};
+                const R stau = nrm > (R)0 ? nr_rsqrt(nrm * (nrm + axkk)) : (R)0;   // sqrt(tau)
+                const CR vkk = (axkk + nrm) * ph;
+                const CR u0 = stau * ((r0 == k) ? vkk : x0);
+                const CR u1 = stau * ((r1 == k) ? vkk : x1);
+                for (int cc = k + 1; cc < NC; ++cc) {
+                    CR* Xc = sm.X[x][cc];
+                    const CR y0 = Xc[r0], y1 = Xc[r1];
+                    CR d = cfmac(u0, y0, cfmac(u1, y1, z));
+                    d.x = group_sum<G>(d.x, gm);
+                    d.y = group_sum<G>(d.y, gm);
+                    Xc[r0] = cfms(u0, d, y0);
+                    Xc[r1] = cfms(u1, d, y1);
+                }
+                __syncwarp(gm);
+                // column k: R above the diagonal and on it, the scaled reflector below and in sm.Rf's
+                // column for the diagonal entry
+                for (int r = l; r < NC; r += G)
+                    if (r <= k) sm.Rf[x][r][k] = r < k ? Xk[r] : CR{-nrm * ph.x, -nrm * ph.y};
+                __syncwarp(gm);
+                Xk[r0] = u0;
+                Xk[r1] = u1;
+                __syncwarp(gm);
+            }
         }
     }
     bar();
@@ -184,7 +231,7 @@ __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kerne
                 CR acc = CR{(R)0, (R)0};
                 for (int j = 0; j < CHI; ++j) {
                     const int ca = ia * CHI + j, cb = ib * CHI + j;
-                    if (r <= ca && rp <= cb) acc = cfma(sm.lab[j] * sm.X[0][ca][r], sm.X[1][cb][rp], acc);
+                    if (r <= ca && rp <= cb) acc = cfma(sm.lab[j] * sm.Rf[0][r][ca], sm.Rf[1][rp][cb], acc);
                 }
                 B[ia][ib] = acc;
             }
@@ -203,51 +250,27 @@ __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kerne
     if (g == 0) sm.nrot = 0;
     bar();
 
-    // ---- FP64 one-sided Jacobi SVD of M (FP32 angles, FP64-unitary rotations) ----
-    int nrot = 0, sweeps;
-    if constexpr (TEAM <= 32) {
-        WarpGroup grp{group_mask<TEAM>()};
-        sweeps = jacobi_svd<NM, R, WarpGroup, true, R64>(sm.M, sm.V, g, grp, group_mask<NM>(), (R)(R64 ? 1e-15 : 1e-6), 60, true,
-                                                               &nrot, (R)(R64 ? 3e-8 : 1e-3));
-    } else {
-        BlockGroup grp{&sm.flag};
-        sweeps = jacobi_svd<NM, R, BlockGroup, true, R64>(sm.M, sm.V, g, grp, group_mask<NM>(), (R)(R64 ? 1e-15 : 1e-6), 60, true,
-                                                                &nrot, (R)(R64 ? 3e-8 : 1e-3));
-    }
-    if (nrot) atomicAdd(&sm.nrot, nrot);
-    bar();
-    for (int cc = g; cc < NM; cc += TEAM) {
-        R s2 = 0.0;
-        for (int r = 0; r < NM; ++r) s2 += norm2(sm.M[cc * NM + r]);
-        sm.sig[cc] = nr_sqrt(s2);
-    }
-    bar();
-    for (int cc = g; cc < NM; cc += TEAM) sm.perm[desc_rank(sm.sig, NM, cc)] = cc;
-    bar();
-    if (g == 0) {
-        const R smax = sm.sig[sm.perm[0]];
-        int cnt = 0;
-        R tot = 0.0;
-        for (int r = 0; r < NM; ++r) {
-            const R s = sm.sig[sm.perm[r]];
-            tot += s * s;
-            cnt += (s > c.svd_cut * smax) ? 1 : 0;
+    // ---- SVD of M and truncation ----
+    // (before refined_svd, FP64 one-sided Jacobi: 7 to 9 sweeps of NM - 1 steps)
+    {
+        SvdCount done;
+        auto run = [&](const auto& grp) {
+            done = core_svd<NM>(sm.M, sm.V, sm.M32, sm.V32, sm.T, sm.n2, &sm.relmask, g, grp, c.svd_cut, c.chi);
+            if (done.rot) atomicAdd(&sm.nrot, done.rot);
+            if (g < NM) sm.perm[desc_rank_bits(sm.n2, NM, g)] = g;
+            grp.sync();
+        };
+        if constexpr (TEAM <= 32) run(WarpGroup{group_mask<TEAM>()});
+        else run(BlockGroup{&sm.flag});
+        if (g < NM) {
+            const int k = truncate_core<NM, CHI, false>(sm.n2, sm.perm, sm.isig, c.lam + (size_t)e * CHI, c.stats, c.chi,
+                                                        c.svd_cut, g);
+            if (g == 0) {
+                atomicAdd(&c.stats[2], (double)done.pairs);
+                atomicAdd(&c.stats[3], (double)sm.nrot);
+                sm.keep = k;
+            }
         }
-        int keep = cnt < c.chi ? cnt : c.chi;
-        if (keep < 1) keep = 1;
-        R kept = 0.0, drop = 0.0;
-        for (int r = 0; r < NM; ++r) {
-            const R s = sm.sig[sm.perm[r]];
-            if (r < keep) kept += s * s; else drop += s * s;
-        }
-        const R inv = kept > 0.0 ? nr_rsqrt(kept) : 0.0;
-        for (int r = 0; r < CHI; ++r) c.lam[(size_t)e * CHI + r] = (r < keep) ? sm.sig[sm.perm[r]] * inv : 0.0;
-        const R disc = tot > 0.0 ? drop * nr_rcp(tot) : 0.0;
-        atomicAdd(&c.stats[0], disc);
-        atomicAdd(&c.stats[1], 2.0 * log1p(-disc));   // Eq. (gate_fidelity)
-        atomicAdd(&c.stats[2], (double)sweeps * (NM - 1) * (NM / 2));
-        atomicAdd(&c.stats[3], (double)sm.nrot);
-        sm.keep = keep;
     }
     bar();
     const int keep = sm.keep;
@@ -263,7 +286,7 @@ __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kerne
             E1[cc] = CR{(R)0, (R)0};
             if (cc < keep) {
                 const int pc = sm.perm[cc];
-                const R is = sm.sig[pc] > 0.0 ? nr_rcp(sm.sig[pc]) : 0.0;
+                const R is = (R)sm.isig[cc];
                 if (r0 < NC) {
                     const int row = i * NC + r0;
                     E0[cc] = (x == 0) ? is * sm.M[pc * NM + row] : conj(sm.V[pc * NM + row]);
@@ -274,20 +297,7 @@ __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kerne
                 }
             }
         }
-        // H_k = I - tau v v^H applied as I - u u^H with u = sqrt(tau) v, last reflector first
-        for (int k = NC - 1; k >= 0; --k) {
-            const R st = nr_sqrt(sm.tau[x][k]);
-            const CR v0 = st * ((r0 == k) ? sm.vk[x][k] : ((r0 > k) ? sm.X[x][k][r0] : CR{(R)0, (R)0}));
-            const CR v1 = st * ((r1 == k) ? sm.vk[x][k] : ((r1 > k) ? sm.X[x][k][r1] : CR{(R)0, (R)0}));
-#pragma unroll
-            for (int cc = 0; cc < CHI; ++cc) {
-                CR d = cfmac(v0, E0[cc], cfmac(v1, E1[cc], CR{(R)0, (R)0}));
-                d.x = group_sum<G>(d.x, gm);
-                d.y = group_sum<G>(d.y, gm);
-                E0[cc] = E0[cc] - v0 * d;
-                E1[cc] = E1[cc] - v1 * d;
-            }
-        }
+        apply_reflectors<CHI, G, NC>(E0, E1, &sm.X[x][0][0], l, gm);
         const R w0 = sm.w[x][r0], w1 = sm.w[x][r1];
         const R iw0 = w0 > 0.0 ? nr_rcp(w0) : 0.0, iw1 = w1 > 0.0 ? nr_rcp(w1) : 0.0;
         const size_t base = (size_t)vtx[x] * (2 * HV) + (size_t)i * HV;

@@ -73,6 +73,8 @@ cudaError_t plain_sample_launch(int CHI, int D, int pm, void* Gamma, const doubl
 cudaError_t plain_general_gates_launch(int CHI, int D, int pm, const GenArgs& a, cudaStream_t st);
 cudaError_t plain_single_gates_launch(int CHI, int D, int pm, void* Gamma, const int* vertex, const cd* W, int count,
                                       cudaStream_t st);
-cudaError_t ising16_gates_launch(const Gate16Args& a, int pm, cudaStream_t st);
+cudaError_t plain_ising_launch(int CHI, int D, int pm, const PlainGateArgs* a, cudaStream_t st);
+cudaError_t plain_mixing_launch(int CHI, int D, int pm, void* Gamma, const int* vertex, int count, double c, double s,
+                                cudaStream_t st);
 
 }  // namespace gtqa

@@ -174,12 +174,41 @@ cudaError_t plain_single_gates_launch(int CHI, int D, int pm, void* G, const int
     }
     return cudaErrorInvalidValue;
 }
-cudaError_t ising16_gates_launch(const Gate16Args& a, int pm, cudaStream_t st) {
-    if (a.count <= 0) return cudaSuccess;
-    if (pm == 0) ising16_gate_kernel<16, double, double><<<a.count, 512, 0, st>>>(a);
-    else if (pm == 1) ising16_gate_kernel<16, float, double><<<a.count, 512, 0, st>>>(a);
-    else ising16_gate_kernel<16, float, float><<<a.count, 512, 0, st>>>(a);
+
+namespace {
+template <int CHI, int D, typename TS, typename R>
+cudaError_t ising_t(const PlainGateArgs* a, cudaStream_t st) {
+    if constexpr (CHI == 16) {
+        constexpr size_t smem = sizeof(Gate16Sm<R>);
+        if (!a) return raise_smem_limit(ising16_gate_kernel<TS, R>, smem);
+        ising16_gate_kernel<TS, R><<<a->count, 512, smem, st>>>(*a);
+    } else {
+        constexpr size_t smem = sizeof(PlainGateSm<CHI, D, TS, R>);
+        if (!a) return raise_smem_limit(plain_ising_kernel<CHI, D, TS, R>, smem);
+        plain_ising_kernel<CHI, D, TS, R><<<a->count, PlainGateShape<CHI, D>::TEAM, smem, st>>>(*a);
+    }
     return cudaGetLastError();
+}
+template <int CHI, int D, typename TS>
+cudaError_t mixing_t(void* G, const int* v, int count, double c, double s, cudaStream_t st) {
+    plain_mixing_kernel<CHI, D, TS><<<count, 64, 0, st>>>(G, v, c, s);
+    return cudaGetLastError();
+}
+}  // namespace
+
+// a = nullptr: only raises the kernel's shared-memory limit (once per state, at creation)
+cudaError_t plain_ising_launch(int CHI, int D, int pm, const PlainGateArgs* a, cudaStream_t st) {
+    if (a && a->count <= 0) return cudaSuccess;
+#define C_(c, d, r, rc) ising_t<c, d, r, rc>(a, st)
+    GTQA_PLAIN_DISPATCH(C_)
+#undef C_
+}
+cudaError_t plain_mixing_launch(int CHI, int D, int pm, void* G, const int* v, int count, double cs, double sn,
+                                cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+#define C_(c, d, r, rc) mixing_t<c, d, r>(G, v, count, cs, sn, st)
+    GTQA_PLAIN_DISPATCH(C_)
+#undef C_
 }
 
 }  // namespace gtqa

@@ -14,10 +14,9 @@
 // CHI^(D-1-k); phantom slots of vertices with fewer edges have dimension 1 with lambda = e_0);
 // lambda [m][CHI]; messages [2m][CHI][CHI] as in the persistent path.
 // The steps are those of the persistent path, in plain launches:
-//   gates    degree 4: general_gates_kernel<CHI, 4> with the diagonal Ising gate (App. E);
-//            CHI = 16: ising16_gate_kernel, the per-physical-index QR-reduced simple update
-//            with a 2 CHI x 2 CHI core (App. E, App. D "Truncation"); one launch per colour
-//            class; mixing gates through single_gates_kernel (Sec. II D);
+//   gates    one launch per colour: plain_ising_kernel (CHI <= 8), ising16_gate_kernel
+//            (CHI = 16), the per-physical-index QR-reduced simple update with a 2 CHI x 2 CHI
+//            core (App. E, App. D "Truncation"), the mixing gates (Sec. II D) fused;
 //   bp       T = Gamma prod lambda^{1/2} (Eq. (symmetric_gauge)), warm start
 //            diag(lambda)/sum(lambda) (Eq. (reconstructed_messages)); per flooding sweep of
 //            Eq. (local_consistency) one launch over vertices and one over messages for the
@@ -29,6 +28,8 @@
 //              Sec. II C reads it on the host);
 //   sampling   the projection step of Sec. IV A for one vertex, then BP and the regauge.
 #pragma once
+
+#include <type_traits>
 
 #include "gtqa_general.cuh"
 
@@ -676,238 +677,495 @@ __global__ void plain_sample_kernel(C<R>* Gamma, const double* lam, const int4* 
 }
 
 // ---------------------------------------------------------------------------
-// CHI = 16, degree 3: the simple update of a diagonal gate (App. E) in QR-reduced form, one
-// block of 512 threads per edge.  The four blocks A_{x,i}[J, j] = w_x[J] Gamma_x[i][j][J]
-// (CHI^2 x CHI) live in global scratch; each gets a Householder QR from a group of 128 threads
-// (two rows each) whose sums go through shared memory.  The core
-//   M[(i_a r), (i_b r')] = U[(i_a i_b), (i_a i_b)] sum_j R_{a,i_a}[r, j] lambda_j R_{b,i_b}[r', j]
-// (2 CHI x 2 CHI) has the same singular values as Theta; one-sided Jacobi (512 threads),
-// truncation to chi as in App. D "Truncation", and the new Gamma from the reflectors.
+// The simple update of a diagonal gate (App. E) in QR-reduced form, as on the persistent path: each
+// side and physical index is one block A_{x,i}[J, j] = w_x[J] Gamma_x[i][j][J] (CHI^(D-1) x CHI),
+//   M[(i_a r), (i_b r')] = ph(i_a, i_b) sum_j R_{a,i_a}[r, j] lambda_j R_{b,i_b}[r', j]
+// (2 CHI x 2 CHI) has the singular values of Theta, and the new tensors come from the reflectors.
+// One block of threads per edge, one launch per colour.  Against the whole-side update of
+// gtqa_general.cuh, which takes any 4 x 4 gate, the core has half the order, so an eighth of the
+// SVD work.  The last gate of a vertex in the layer applies the mixing gate exp(-i t_X X) to it,
+// the first one the leading mixing gate.
 // ---------------------------------------------------------------------------
-struct Gate16Args {
+struct PlainGateArgs {
     void* Gamma;
     double* lam;
     const int4* edge_info;
     const int4* vslots;
-    const int* gate_edge;
-    const cd* gate_U;         // [gates][16], diagonal used
-    cd* scratch;              // [gates in launch][4][CHI][CHI^2]
+    const int* gate_edge;     // edges of this launch
+    const int* gate_bits;     // first gate of u, of v; last gate of u, of v
     int count;
+    const double* J;
+    const double* hd;         // h_a / degree of a
     double* stats;
+    Control* ctl;
     int chi;
     double svd_cut;
+    double tZ, cX, sX;        // mixing gate after a vertex's last gate
+    int pre;                  // leading mixing gate before its first one
+    double cXp, sXp;
+    void* scratch;            // CHI = 16: reflectors, [gates in launch][4][CHI^2][CHI]
 };
 
-template <int CHI, typename R>
-struct Gate16Sm {
-    using CR = C<R>;
-    static constexpr int NM = 2 * CHI, NR = CHI * CHI;
-    CR M[NM * NM];
-    CR V[NM * NM];
-    CR vk[4][CHI];
-    R st[4][CHI];             // square roots of the reflector coefficients
-    R w[2][NR];
-    R lab[CHI];
-    CR ph[4];
-    R sig[NM];
-    int perm[NM];
-    CR red[4][4][CHI];        // [group][warp][value] partial sums
-    int keep, flag, nrot;
-};
-
-// sum over the 128 threads of group grp of vals[0..nv) (complex), returned to every thread;
-// red is [4 warps][nv]; named barrier 1 + grp
-template <int NV, typename CR>
-__device__ __forceinline__ void group128_sum(CR (&vals)[NV], int nv, CR (*red)[16], int grp) {
-    const int lane = threadIdx.x & 31, wig = (threadIdx.x / 32) & 3;
-    for (int q = 0; q < nv; ++q) {
-        vals[q].x = group_sum<32>(vals[q].x, 0xffffffffu);
-        vals[q].y = group_sum<32>(vals[q].y, 0xffffffffu);
-        if (lane == 0) red[wig][q] = vals[q];
-    }
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
-    for (int q = 0; q < nv; ++q) vals[q] = red[0][q] + red[1][q] + red[2][q] + red[3][q];
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
+// The four diagonal gate phases of edge e: lane d = 2 i_a + i_b < 4.
+__device__ __forceinline__ cd ising_phase(double tZ, double J, double ha, double hb, int d) {
+    const double za = 1.0 - 2.0 * (d >> 1), zb = 1.0 - 2.0 * (d & 1);
+    double sn, cs;
+    sincos(-tZ * (J * za * zb + ha * za + hb * zb), &sn, &cs);
+    return cd{cs, sn};
+}
+// [[c, -i s], [-i s, c]] on the pair (g0, g1)
+template <typename TS>
+__device__ __forceinline__ void mix_pair(C<TS>& g0, C<TS>& g1, double c, double s) {
+    const cd a0 = ccast<double>(g0), a1 = ccast<double>(g1);
+    g0 = ccast<TS>(cd{c * a0.x + s * a1.y, c * a0.y - s * a1.x});
+    g1 = ccast<TS>(cd{s * a0.y + c * a1.x, -s * a0.x + c * a1.y});
 }
 
-// TS is the storage type of Gamma, R the arithmetic type: (double, double) is the FP64
-// precision mode, (float, float) the complex64 mode (QR, Jacobi SVD and the new Gamma in FP32)
-// and (float, double) the mixed mode (FP64 QR and SVD on complex64 Gamma).  lambda is always
-// written as float64.
-template <int CHI, typename TS, typename R>
-__global__ void __launch_bounds__(512, 1) ising16_gate_kernel(Gate16Args c) {
+template <int CHI, int D>
+struct PlainGateShape {
+    static constexpr int NR = ipow(CHI, D - 1), G = NR / 2, TEAM = 4 * G, NM = 2 * CHI, LS = NM * NM / 2;
+    static_assert(G <= 32 && LS <= TEAM, "one warp per block at most");
+};
+
+template <int CHI, int D, typename TS, typename R>
+struct PlainGateSm {
+    using S = PlainGateShape<CHI, D>;
+    C<R> U[4][CHI][S::NR];     // scaled reflectors, then the new tensors
+    C<R> M[S::NM * S::NM];
+    C<R> V[S::NM * S::NM];     // first the R factors [block][row][col]
+    C<R> T[sizeof(R) == 8 ? S::NM * S::NM : 1];
+    cf M32[sizeof(R) == 8 ? S::NM * S::NM : 1];
+    cf V32[sizeof(R) == 8 ? S::NM * S::NM : 1];
+    double lab[CHI];
+    double n2[S::NM], isig[CHI];
+    C<R> ph[4];
+    int perm[S::NM];
+    int keep, flag, nrot;
+    unsigned relmask;
+};
+
+template <int CHI, int D, typename TS, typename R>
+__global__ void __launch_bounds__(PlainGateShape<CHI, D>::TEAM) plain_ising_kernel(PlainGateArgs c) {
+    using S = PlainGateShape<CHI, D>;
     using CR = C<R>;
-    constexpr bool R64 = sizeof(R) == 8;
-    constexpr int NM = 2 * CHI, NR = CHI * CHI, H = CHI * CHI * CHI;
-    static_assert(NR == 2 * 128, "the 128-thread groups hold two rows each");
-    __shared__ Gate16Sm<CHI, R> sm;
-    const int tid = threadIdx.x;
-    const int e = c.gate_edge[blockIdx.x];
+    using CT = C<TS>;
+    constexpr int NM = S::NM, NR = S::NR, G = S::G, TEAM = S::TEAM, LS = S::LS, H = ipow(CHI, D);
+    extern __shared__ __align__(16) unsigned char plain_smem[];
+    PlainGateSm<CHI, D, TS, R>& sm = *reinterpret_cast<PlainGateSm<CHI, D, TS, R>*>(plain_smem);
+    auto bar = [&]() {
+        if constexpr (TEAM < 32) __syncwarp(group_mask<TEAM>());
+        else __syncthreads();
+    };
+    const int tid = threadIdx.x, blk = tid / G, l = tid % G, x = blk >> 1, i = blk & 1;
+    const unsigned gm = group_mask<G>();
+    const int e = c.gate_edge[blockIdx.x], bits = c.gate_bits[blockIdx.x];
     const int4 ei = c.edge_info[e];
-    const int vtx[2] = {ei.x, ei.y};
-    const int slot[2] = {ei.z, ei.w};
-    int oe[2][2], os[2][2];
-    for (int x = 0; x < 2; ++x) {
-        const int4 ve = c.vslots[vtx[x]];
-        const int es[3] = {ve.x, ve.y, ve.z};
-        others_of(slot[x], os[x][0], os[x][1]);
-        oe[x][0] = es[os[x][0]];
-        oe[x][1] = es[os[x][1]];
-    }
-    CR* Xg = reinterpret_cast<CR*>(c.scratch) + (size_t)blockIdx.x * 4 * CHI * NR;   // [blk][col][row]
-    C<TS>* Gam = (C<TS>*)c.Gamma;
-    for (int t = tid; t < 2 * NR; t += 512) {
-        const int x = t / NR, J = t % NR;
-        sm.w[x][J] = (R)(lam_get(c.lam, CHI, oe[x][0], J / CHI) * lam_get(c.lam, CHI, oe[x][1], J % CHI));
-    }
-    for (int t = tid; t < CHI; t += 512) sm.lab[t] = (R)c.lam[(size_t)e * CHI + t];
-    if (tid < 4) sm.ph[tid] = ccast<R>(c.gate_U[(size_t)blockIdx.x * 16 + 5 * tid]);
-    if (tid == 0) sm.nrot = 0;
-    __syncthreads();
-    for (int t = tid; t < 4 * CHI * NR; t += 512) {
-        const int blk = t / (CHI * NR), rem = t % (CHI * NR);
-        const int col = rem / NR, row = rem % NR;
-        const int x = blk >> 1, i = blk & 1;
-        const size_t off = (size_t)vtx[x] * 2 * H + (size_t)i * H + col * sstride<CHI>(slot[x]) +
-                           (row / CHI) * sstride<CHI>(os[x][0]) + (row % CHI) * sstride<CHI>(os[x][1]);
-        Xg[((size_t)blk * CHI + col) * NR + row] = sm.w[x][row] * ccast<R>(Gam[off]);
-    }
-    __syncthreads();
-    // ---- Householder QR of the four blocks, 128 threads per block, rows l and l + 128 ----
-    const int blk = tid / 128, l = tid % 128;
-    CR* Xb = Xg + (size_t)blk * CHI * NR;
-    for (int k = 0; k < CHI; ++k) {
-        CR* Xk = Xb + (size_t)k * NR;
-        const CR z = CR{(R)0, (R)0};
-        CR x0 = (l >= k) ? Xk[l] : z;
-        CR x1 = Xk[l + 128];
-        CR nv[1] = {CR{norm2(x0) + norm2(x1), (R)0}};
-        group128_sum<1>(nv, 1, sm.red[blk], blk);
-        const R nrm = nr_sqrt(nv[0].x);
-        const CR xkk = Xk[k];
-        const R a2 = norm2(xkk);
-        const R ra = a2 > (R)0 ? nr_rsqrt(a2) : (R)0;
-        const R axkk = a2 * ra;
-        const CR ph = a2 > (R)0 ? CR{xkk.x * ra, xkk.y * ra} : CR{(R)1, (R)0};
-        const R stau = nrm > (R)0 ? nr_rsqrt(nrm * (nrm + axkk)) : (R)0;
-        const R tau = stau * stau;
-        const CR vkk = (axkk + nrm) * ph;
-        const CR v0 = (l == k) ? vkk : x0;
-        const CR v1 = x1;
-        CR d[CHI];
-#pragma unroll
-        for (int cc = 0; cc < CHI; ++cc) {
-            d[cc] = z;
-            if (cc > k) {
-                const CR* Xc = Xb + (size_t)cc * NR;
-                d[cc] = cfmac(v0, Xc[l], cfmac(v1, Xc[l + 128], z));
+    const int slot2[2] = {ei.z, ei.w}, vtx2[2] = {ei.x, ei.y};
+    // offset of row J (the other slots, last one fastest) inside a vertex tensor, side x
+    auto row_off = [&](int slot, int J) {
+        int off = 0;
+        for (int k = D - 1; k >= 0; --k)
+            if (k != slot) {
+                off += (J % CHI) * ipow(CHI, D - 1 - k);
+                J /= CHI;
             }
-        }
-        group128_sum<CHI>(d, CHI, sm.red[blk], blk);
+        return off;
+    };
+    CT* Gam = (CT*)c.Gamma;
+    CR y0[CHI], y1[CHI];
+    double w0 = 1.0, w1 = 1.0;
+    {
+        const int slot = slot2[x], ss = ipow(CHI, D - 1 - slot);
+        const int4 sl = c.vslots[vtx2[x]];
+        const int es[4] = {sl.x, sl.y, sl.z, sl.w};
+        int J0 = l, J1 = l + G;
+        for (int k = D - 1; k >= 0; --k)
+            if (k != slot) {
+                w0 *= lam_get(c.lam, CHI, es[k], J0 % CHI);
+                w1 *= lam_get(c.lam, CHI, es[k], J1 % CHI);
+                J0 /= CHI;
+                J1 /= CHI;
+            }
+        const CT* g = Gam + (size_t)vtx2[x] * 2 * H;
+        const int f0 = row_off(slot, l), f1 = row_off(slot, l + G);
+        const bool lead = c.pre && ((bits >> x) & 1);
 #pragma unroll
         for (int cc = 0; cc < CHI; ++cc) {
-            if (cc <= k) continue;
-            CR* Xc = Xb + (size_t)cc * NR;
-            const CR td = tau * d[cc];
-            if (l >= k) Xc[l] = Xc[l] - v0 * td;
-            Xc[l + 128] = Xc[l + 128] - v1 * td;
+            CT a = g[i * H + f0 + cc * ss], b = g[i * H + f1 + cc * ss];
+            if (lead) {   // own component of the mixed pair; mix_pair is symmetric in the two
+                CT a2 = g[(i ^ 1) * H + f0 + cc * ss], b2 = g[(i ^ 1) * H + f1 + cc * ss];
+                mix_pair(a, a2, c.cXp, c.sXp);
+                mix_pair(b, b2, c.cXp, c.sXp);
+            }
+            y0[cc] = (R)w0 * ccast<R>(a);
+            y1[cc] = (R)w1 * ccast<R>(b);
         }
-        if (l == k) Xk[k] = (-nrm) * ph;
-        if (l == 0) {
-            sm.vk[blk][k] = vkk;
-            sm.st[blk][k] = stau;
-        }
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + blk) : "memory");
+        if (tid < CHI) sm.lab[tid] = c.lam[(size_t)e * CHI + tid];
+        if (tid < 4) sm.ph[tid] = ccast<R>(ising_phase(c.tZ, c.J[e], c.hd[ei.x], c.hd[ei.y], tid));
+        if (tid == 0) sm.nrot = 0;
+        bar();
     }
-    __syncthreads();
-    // ---- core M (column-major NM x NM) with the diagonal gate ----
-    for (int t = tid; t < NM * NM; t += 512) {
+    qr_steps<CHI, G, 0>(y0, y1, &sm.U[blk][0][0], l, gm);
+    // rows l and, where the group is smaller than CHI, l + G of R
+#pragma unroll
+    for (int cc = 0; cc < CHI; ++cc) {
+        const R lb = x == 0 ? (R)sm.lab[cc] : (R)1;
+        if (l < CHI && cc >= l) sm.V[(blk * CHI + l) * CHI + cc] = lb * y0[cc];
+    }
+    bar();
+    for (int t = tid; t < NM * NM; t += TEAM) {
         const int col = t / NM, row = t % NM;
         const int ia = row / CHI, r = row % CHI, ib = col / CHI, rp = col % CHI;
-        const CR* Ra = Xg + (size_t)ia * CHI * NR;          // block (a, ia)
-        const CR* Rb = Xg + (size_t)(2 + ib) * CHI * NR;    // block (b, ib)
+        const CR* Ra = sm.V + (ia * CHI + r) * CHI;
+        const CR* Rb = sm.V + ((2 + ib) * CHI + rp) * CHI;
         CR acc = CR{(R)0, (R)0};
-        const int j0 = r > rp ? r : rp;
-        for (int j = j0; j < CHI; ++j) acc = cfma(sm.lab[j] * Ra[(size_t)j * NR + r], Rb[(size_t)j * NR + rp], acc);
+        for (int j = r > rp ? r : rp; j < CHI; ++j) acc = cfma(Ra[j], Rb[j], acc);
         sm.M[t] = sm.ph[2 * ia + ib] * acc;
     }
-    __syncthreads();
-    int nrot = 0;
-    BlockGroup grp{&sm.flag};
-    const int sweeps = jacobi_svd<NM, R, BlockGroup, true, R64>(sm.M, sm.V, tid, grp, group_mask<NM>(),
-                                                                (R)(R64 ? 1e-15 : 1e-6), 60, true, &nrot,
-                                                                (R)(R64 ? 3e-8 : 1e-3));
-    if (nrot) atomicAdd(&sm.nrot, nrot);
-    __syncthreads();
-    for (int cc = tid; cc < NM; cc += 512) {
-        R s2 = (R)0;
-        for (int r = 0; r < NM; ++r) s2 += norm2(sm.M[cc * NM + r]);
-        sm.sig[cc] = nr_sqrt(s2);
-    }
-    __syncthreads();
-    for (int cc = tid; cc < NM; cc += 512) sm.perm[desc_rank(sm.sig, NM, cc)] = cc;
-    __syncthreads();
-    if (tid < NM) {   // lane r holds the r-th largest singular value (NM = 32: one warp)
-        const unsigned mk = group_mask<NM>();
-        const R sv = sm.sig[sm.perm[tid]];
-        const R smax = sm.sig[sm.perm[0]];
-        const int cnt = __popc(__ballot_sync(mk, sv > (R)c.svd_cut * smax));
-        int keep = cnt < c.chi ? cnt : c.chi;
-        if (keep < 1) keep = 1;
-        const R s2 = sv * sv;
-        const R kept = group_sum<NM>(tid < keep ? s2 : (R)0, mk);
-        const R drop = group_sum<NM>(tid < keep ? (R)0 : s2, mk);
-        const R inv = kept > (R)0 ? nr_rsqrt(kept) : (R)0;
-        if (tid < CHI) c.lam[(size_t)e * CHI + tid] = (tid < keep) ? (double)(sv * inv) : 0.0;
-        if (tid == 0) {
-            const R tot = kept + drop;
-            const R disc = tot > (R)0 ? drop * nr_rcp(tot) : (R)0;
-            atomicAdd(&c.stats[0], (double)disc);
-            atomicAdd(&c.stats[1], 2.0 * log1p(-(double)disc));   // Eq. (gate_fidelity)
-            atomicAdd(&c.stats[2], (double)sweeps * (NM - 1) * (NM / 2));
-            atomicAdd(&c.stats[3], (double)sm.nrot);
-            sm.keep = keep;
+    bar();
+    if (tid < LS) {
+        SvdCount done;
+        auto run = [&](const auto& grp) {
+            done = core_svd<NM>(sm.M, sm.V, sm.M32, sm.V32, sm.T, sm.n2, &sm.relmask, tid, grp, c.svd_cut, c.chi);
+            if (done.rot) atomicAdd(&sm.nrot, done.rot);
+            if (tid < NM) sm.perm[desc_rank_bits(sm.n2, NM, tid)] = tid;
+            grp.sync();
+        };
+        if constexpr (LS <= 32) run(WarpGroup{group_mask<LS>()});
+        else run(TeamGroup<LS>{0, &sm.flag});
+        if (tid < NM) {
+            const int k = truncate_core<NM, CHI, false>(sm.n2, sm.perm, sm.isig, c.lam + (size_t)e * CHI, c.stats, c.chi,
+                                                        c.svd_cut, tid);
+            if (tid == 0) {
+                atomicAdd(&c.stats[2], (double)done.pairs);
+                atomicAdd(&c.stats[3], (double)sm.nrot);
+                sm.keep = k;
+            }
         }
     }
-    __syncthreads();
+    bar();
     const int keep = sm.keep;
-    // ---- new Gamma: the reflectors of each block applied to U (side a) / V^* (side b) ----
-    const int x = blk >> 1, i = blk & 1;
     CR E0[CHI], E1[CHI];
 #pragma unroll
     for (int cc = 0; cc < CHI; ++cc) {
-        E0[cc] = CR{(R)0, (R)0};
-        E1[cc] = CR{(R)0, (R)0};
+        E0[cc] = E1[cc] = CR{(R)0, (R)0};
         if (l < CHI && cc < keep) {
-            const int pc = sm.perm[cc];
-            const int row = i * CHI + l;
-            E0[cc] = (x == 0) ? nr_rcp(sm.sig[pc]) * sm.M[pc * NM + row] : conj(sm.V[pc * NM + row]);
+            const int pc = sm.perm[cc], row = i * CHI + l;
+            E0[cc] = x == 0 ? (R)sm.isig[cc] * sm.M[pc * NM + row] : conj(sm.V[pc * NM + row]);
         }
     }
-    for (int k = CHI - 1; k >= 0; --k) {
-        const R st = sm.st[blk][k];
-        const CR* Xk = Xb + (size_t)k * NR;
-        const CR v0 = st * ((l == k) ? sm.vk[blk][k] : ((l > k) ? Xk[l] : CR{(R)0, (R)0}));
-        const CR v1 = st * Xk[l + 128];
-        CR d[CHI];
-#pragma unroll
-        for (int cc = 0; cc < CHI; ++cc) d[cc] = cfmac(v0, E0[cc], cfmac(v1, E1[cc], CR{(R)0, (R)0}));
-        group128_sum<CHI>(d, CHI, sm.red[blk], blk);
-#pragma unroll
-        for (int cc = 0; cc < CHI; ++cc) {
-            E0[cc] = E0[cc] - v0 * d[cc];
-            E1[cc] = E1[cc] - v1 * d[cc];
-        }
-    }
-    const R w0 = sm.w[x][l], w1 = sm.w[x][l + 128];
-    const R iw0 = w0 > (R)0 ? nr_rcp(w0) : (R)0, iw1 = w1 > (R)0 ? nr_rcp(w1) : (R)0;
-    const size_t base = (size_t)vtx[x] * 2 * H + (size_t)i * H;
-    const size_t o0 = (l / CHI) * sstride<CHI>(os[x][0]) + (l % CHI) * sstride<CHI>(os[x][1]);
-    const size_t o1 = ((l + 128) / CHI) * sstride<CHI>(os[x][0]) + ((l + 128) % CHI) * sstride<CHI>(os[x][1]);
+    apply_reflectors<CHI, G>(E0, E1, &sm.U[blk][0][0], l, gm);
+    const R iw0 = w0 > 0.0 ? (R)nr_rcp(w0) : (R)0, iw1 = w1 > 0.0 ? (R)nr_rcp(w1) : (R)0;
+    bar();   // everyone is done reading the reflectors
 #pragma unroll
     for (int cc = 0; cc < CHI; ++cc) {
-        Gam[base + cc * sstride<CHI>(slot[x]) + o0] = ccast<TS>(iw0 * E0[cc]);
-        Gam[base + cc * sstride<CHI>(slot[x]) + o1] = ccast<TS>(iw1 * E1[cc]);
+        sm.U[blk][cc][l] = iw0 * E0[cc];
+        sm.U[blk][cc][l + G] = iw1 * E1[cc];
+    }
+    bar();
+    for (int t = tid; t < 2 * CHI * NR; t += TEAM) {
+        const int xx = t / (CHI * NR), rem = t % (CHI * NR), col = rem / NR, row = rem % NR;
+        CT g0 = ccast<TS>(sm.U[2 * xx][col][row]), g1 = ccast<TS>(sm.U[2 * xx + 1][col][row]);
+        if ((bits >> (2 + xx)) & 1) mix_pair(g0, g1, c.cX, c.sX);
+        CT* g = Gam + (size_t)vtx2[xx] * 2 * H + row_off(slot2[xx], row) + col * ipow(CHI, D - 1 - slot2[xx]);
+        g[0] = g0;
+        g[H] = g1;
+    }
+}
+
+// exp(-i t X) on the vertices of a list (those without edges)
+template <int CHI, int D, typename TS>
+__global__ void plain_mixing_kernel(void* Gamma, const int* vertex, double c, double s) {
+    constexpr int H = ipow(CHI, D);
+    C<TS>* g = (C<TS>*)Gamma + (size_t)vertex[blockIdx.x] * 2 * H;
+    for (int r = threadIdx.x; r < H; r += blockDim.x) {
+        C<TS> g0 = g[r], g1 = g[H + r];
+        mix_pair(g0, g1, c, s);
+        g[r] = g0;
+        g[H + r] = g1;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// CHI = 16, degree 3: the same update, one block of 512 threads per edge.
+//
+// What bounds it: the FP64 pipe.  The useful products of one gate are, per block of
+// CHI^2 x CHI, 30k complex products each for the QR's inner products, its updates and the
+// reflectors' Gram matrix, and 64k for the back-application.  So:
+//  * one side at a time, 256 lanes per block of it, each with its row of 16 columns in registers
+//    (the panel of both sides, 256 KB in FP64, fits neither shared memory nor the registers);
+//    finished reflectors go to global scratch once and are read back once;
+//  * the inner products of a step with all other columns (later ones for the QR, earlier ones for
+//    the Gram matrix of the reflectors) are summed together, 31 values by one reduce-scatter per
+//    warp; the scalars of a step are formed by one warp of the block, not by all;
+//  * the back-application is one product E - U Z per row with Z from (I + strict upper(U^H U)) Z =
+//    U^H E (compact WY form), instead of 16 reductions over 256 rows;
+//  * columns beyond the bond's current dimension (lambda = 0) are skipped, and the core is
+//    decomposed at the order (8, 16 or 32) that holds both of its halves.
+// ---------------------------------------------------------------------------
+template <typename R>
+struct Gate16Sm {
+    using CR = C<R>;
+    static constexpr int CHI = 16, NM = 32, NR = 256;
+    CR M[NM * NM];
+    CR V[NM * NM];            // first the R factors [block][row][col]
+    CR T[NM * NM];            // scratch of the SVD; then Z [block][j][col]
+    cf M32[sizeof(R) == 8 ? NM * NM : 1];
+    cf V32[sizeof(R) == 8 ? NM * NM : 1];
+    CR SU[4][CHI][CHI];       // u_j^H u_k, j < k
+    CR top[4][CHI][CHI];      // rows 0 .. 15 of the reflectors, [block][k][row]
+    R red[2][8][32];          // partial sums, [block of the side][warp][value]
+    CR wv[2][CHI];            // tau v^H y of the later columns
+    R st[2];
+    CR vkk[2];
+    double lab[CHI];
+    double n2[NM], isig[CHI];
+    CR ph[4];
+    int perm[NM];
+    int keep, flag, nrot;
+    unsigned relmask;
+};
+
+// Step K of the QR of the two blocks of one side: lane `row` of block i holds y[0 .. 15].  nc: the
+// columns in use.  vd: this row's diagonal reflector entry (row < CHI).
+template <int K, typename R>
+__device__ __forceinline__ void qr16_steps(C<R> (&y)[16], C<R>& vd, Gate16Sm<R>& sm, C<R>* U, int blk, int i, int row,
+                                           int nc) {
+    if constexpr (K < 16) {
+        using CR = C<R>;
+        if (K >= nc) return;
+        const int lane = threadIdx.x & 31, warp = row / 32;
+        const CR z = CR{(R)0, (R)0};
+        const CR x = row >= K ? y[K] : z;
+        // |x|^2 and the inner products of x with the 15 other columns, in two groups of 16 values
+        // (registers); value v of a group ends on lane 2 v
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            R s[16];
+            s[0] = half == 0 ? norm2(x) : (R)0;
+            s[15] = (R)0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int c = half == 0 ? q - 1 : 7 + q;   // other column, skipping K
+                if (c < 0) continue;
+                const int col = c < K ? c : c + 1, at = half == 0 ? 2 * q - 1 : 2 * q;
+                CR d = z;
+                if (col < nc) {
+                    // an earlier column: its reflector, below the diagonal and vd on it
+                    const CR a = c < K ? (row > c ? y[c] : (row == c ? vd : z)) : y[col];
+                    d = c < K ? cfmac(a, x, z) : cfmac(x, a, z);
+                }
+                s[at] = d.x;
+                s[at + 1] = d.y;
+            }
+            rs_level<16, 16>(s, 0xffffffffu, lane);
+            if ((lane & 1) == 0) sm.red[i][warp][16 * half + lane / 2] = s[0];
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // value v on lane v
+            R t = (R)0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) t += sm.red[i][w][lane];
+            const R x2 = __shfl_sync(0xffffffffu, t, 0);
+            const CR xkk = CR{__shfl_sync(0xffffffffu, y[K].x, K), __shfl_sync(0xffffffffu, y[K].y, K)};
+            const R a2 = norm2(xkk);
+            const R arg = (lane & 1) ? a2 : x2;
+            const R rs = arg > tiny_norm2<R>() ? nr_rsqrt(arg) : (R)0;
+            const R r0 = __shfl_sync(0xffffffffu, rs, 0), ra = __shfl_sync(0xffffffffu, rs, 1);
+            const R nrm = x2 * r0, axkk = a2 * ra;
+            const CR ph = nonzero(ra) ? CR{xkk.x * ra, xkk.y * ra} : CR{(R)1, (R)0};
+            const R stau = nonzero(nrm) ? nr_rsqrt(nrm * (nrm + axkk)) : (R)0;
+            const CR pv = nrm * ph;
+            // lane c < 15: the sum of column c (earlier) or c + 1 (later), and row K of that column
+            const int at = lane < 7 ? 1 + 2 * lane : 2 + 2 * (lane % 15);
+            const CR sum = CR{__shfl_sync(0xffffffffu, t, at), __shfl_sync(0xffffffffu, t, at + 1)};
+            CR yk = z;
+#pragma unroll
+            for (int c = 0; c < 15; ++c) {
+                const CR a = y[c < K ? c : c + 1];
+                const R bx = __shfl_sync(0xffffffffu, a.x, K), by = __shfl_sync(0xffffffffu, a.y, K);
+                if (lane == c) yk = CR{bx, by};
+            }
+            if (lane < K) {
+                // v_c^H v_K = v_c^H x + conj(v_c[K]) pv, scaled to u
+                const CR g = cfmac(yk, pv, sum);
+                sm.SU[blk][lane][K] = (stau * sm.SU[blk][lane][lane].x) * g;
+            } else if (lane < 15) {
+                sm.wv[i][lane + 1] = (stau * stau) * cfmac(pv, yk, sum);   // tau (x^H y + conj(pv) y_K)
+            }
+            if (lane == K) {
+                sm.SU[blk][K][K] = CR{stau, (R)0};   // kept for the scaling of later columns
+                sm.st[i] = stau;
+                sm.vkk[i] = xkk + pv;
+                y[K] = CR{-pv.x, -pv.y};
+                vd = xkk + pv;
+            }
+        }
+        __syncthreads();
+        const R stau = sm.st[i];
+        const CR v = row == K ? sm.vkk[i] : x;
+#pragma unroll
+        for (int c = K + 1; c < 16; ++c)
+            if (c < nc && row >= K) y[c] = cfms(v, sm.wv[i][c], y[c]);
+        const CR u = stau * v;
+        U[K * 256 + row] = u;
+        if (row < 16) sm.top[blk][K][row] = u;
+        qr16_steps<K + 1>(y, vd, sm, U, blk, i, row, nc);
+    }
+}
+
+template <typename TS, typename R>
+__global__ void __launch_bounds__(512, 1) ising16_gate_kernel(PlainGateArgs c) {
+    using CR = C<R>;
+    using CT = C<TS>;
+    constexpr int CHI = 16, NR = 256, H = CHI * CHI * CHI;
+    extern __shared__ __align__(16) unsigned char plain_smem[];
+    Gate16Sm<R>& sm = *reinterpret_cast<Gate16Sm<R>*>(plain_smem);
+    const int tid = threadIdx.x, i = tid / NR, row = tid % NR;
+    const int e = c.gate_edge[blockIdx.x], bits = c.gate_bits[blockIdx.x];
+    const int4 ei = c.edge_info[e];
+    CT* Gam = (CT*)c.Gamma;
+    CR* Us = reinterpret_cast<CR*>(c.scratch) + (size_t)blockIdx.x * 4 * CHI * NR;   // [blk][k][row]
+    if (tid < CHI) sm.lab[tid] = c.lam[(size_t)e * CHI + tid];
+    if (tid >= 32 && tid < 36) sm.ph[tid - 32] = ccast<R>(ising_phase(c.tZ, c.J[e], c.hd[ei.x], c.hd[ei.y], tid - 32));
+    if (tid == 0) sm.nrot = 0;
+    __syncthreads();
+    int nc = 0;   // the bond's current dimension
+    for (int j = 0; j < CHI; ++j) nc = sm.lab[j] > 0.0 ? j + 1 : nc;
+    nc = nc > 0 ? nc : 1;
+    double w2[2];
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int slot = x ? ei.w : ei.z, vtx = x ? ei.y : ei.x, blk = 2 * x + i;
+        const int4 ve = c.vslots[vtx];
+        int o0, o1;
+        others_of(slot, o0, o1);
+        const int e0 = plain_slot_edge(ve, o0), e1 = plain_slot_edge(ve, o1);
+        const double w = lam_get(c.lam, CHI, e0, row / CHI) * lam_get(c.lam, CHI, e1, row % CHI);
+        if (x == 0) w2[0] = w;
+        else w2[1] = w;
+        auto stride = [](int k) { return k == 0 ? CHI * CHI : (k == 1 ? CHI : 1); };
+        const int ss = stride(slot);
+        const CT* g = Gam + (size_t)vtx * 2 * H + row / CHI * stride(o0) + row % CHI * stride(o1);
+        const bool lead = c.pre && ((bits >> x) & 1);
+        CR y[CHI];
+        CR vd = CR{(R)0, (R)0};
+#pragma unroll
+        for (int cc = 0; cc < CHI; ++cc) {
+            CT a = g[i * H + cc * ss];
+            if (lead) {
+                CT b = g[(i ^ 1) * H + cc * ss];
+                mix_pair(a, b, c.cXp, c.sXp);
+            }
+            y[cc] = (R)w * ccast<R>(a);
+        }
+        qr16_steps<0>(y, vd, sm, Us + (size_t)blk * CHI * NR, blk, i, row, nc);
+        if (row < CHI) {
+#pragma unroll
+            for (int cc = 0; cc < CHI; ++cc)
+                if (cc >= row) sm.V[(blk * CHI + row) * CHI + cc] = x == 0 ? (R)sm.lab[cc] * y[cc] : y[cc];
+        }
+        __syncthreads();
+    }
+    // ---- core with the diagonal gate at order 2 hc, column-major ----
+    const int hc = nc <= 4 ? 4 : (nc <= 8 ? 8 : 16), NM = 2 * hc;
+    for (int t = tid; t < NM * NM; t += 512) {
+        const int col = t / NM, rw = t % NM;
+        const int ia = rw / hc, r = rw % hc, ib = col / hc, rp = col % hc;
+        const CR* Ra = sm.V + (ia * CHI + r) * CHI;
+        const CR* Rb = sm.V + ((2 + ib) * CHI + rp) * CHI;
+        CR acc = CR{(R)0, (R)0};
+        for (int j = r > rp ? r : rp; j < nc; ++j) acc = cfma(Ra[j], Rb[j], acc);
+        sm.M[t] = sm.ph[2 * ia + ib] * acc;
+    }
+    __syncthreads();
+    auto solve = [&](auto order, const auto& grp) {
+        constexpr int N = decltype(order)::value;
+        SvdCount done = core_svd<N>(sm.M, sm.V, sm.M32, sm.V32, sm.T, sm.n2, &sm.relmask, tid, grp, c.svd_cut, c.chi);
+        if (done.rot) atomicAdd(&sm.nrot, done.rot);
+        if (tid < N) sm.perm[desc_rank_bits(sm.n2, N, tid)] = tid;
+        grp.sync();
+        if (tid < N) {
+            const int k = truncate_core<N, (N < CHI ? N : CHI), false>(sm.n2, sm.perm, sm.isig, c.lam + (size_t)e * CHI, c.stats,
+                                                                       c.chi, c.svd_cut, tid);
+            if (tid == 0) {
+                atomicAdd(&c.stats[2], (double)done.pairs);
+                atomicAdd(&c.stats[3], (double)sm.nrot);
+                sm.keep = k;
+            }
+        }
+        // a core of order 8 has no more than 8 triplets; the bond's other weights are zero
+        if (N < CHI && tid < CHI - N) c.lam[(size_t)e * CHI + N + tid] = 0.0;
+    };
+    if (hc == 4) {
+        if (tid < 32) solve(std::integral_constant<int, 8>{}, WarpGroup{0xffffffffu});
+    } else if (hc == 8) {
+        if (tid < 128) solve(std::integral_constant<int, 16>{}, TeamGroup<128>{0, &sm.flag});
+    } else {
+        solve(std::integral_constant<int, 32>{}, BlockGroup{&sm.flag});
+    }
+    __syncthreads();
+    const int keep = sm.keep;
+    // ---- Z of every block: Y = U^H E (E has its first nc rows only), then back substitution ----
+    auto etop = [&](int blk, int r, int cc) {   // row r < nc of column cc < keep
+        const int pc = sm.perm[cc], rw = (blk & 1) * hc + r;
+        return blk < 2 ? (R)sm.isig[cc] * sm.M[pc * NM + rw] : conj(sm.V[pc * NM + rw]);
+    };
+    for (int t = tid; t < 4 * CHI * CHI; t += 512) {
+        const int blk = t / (CHI * CHI), j = (t / CHI) % CHI, cc = t % CHI;
+        CR acc = CR{(R)0, (R)0};
+        if (j < nc && cc < keep)
+            for (int r = j; r < nc; ++r) acc = cfmac(sm.top[blk][j][r], etop(blk, r, cc), acc);
+        sm.T[t] = acc;
+    }
+    __syncthreads();
+    if (tid % 128 < CHI) {   // one lane per column, the blocks on different warps
+        const int blk = tid / 128, cc = tid % 128;
+        if (cc < keep) {
+            CR* Z = sm.T + blk * CHI * CHI + cc;
+            for (int j = nc - 2; j >= 0; --j) {
+                CR acc = Z[j * CHI];
+                for (int k = j + 1; k < nc; ++k) acc = cfms(sm.SU[blk][j][k], Z[k * CHI], acc);
+                Z[j * CHI] = acc;
+            }
+        }
+    }
+    __syncthreads();
+    // ---- new tensors, row by row ----
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) {
+        const int slot = x ? ei.w : ei.z, vtx = x ? ei.y : ei.x, blk = 2 * x + i;
+        int o0, o1;
+        others_of(slot, o0, o1);
+        CR E[CHI];
+#pragma unroll
+        for (int cc = 0; cc < CHI; ++cc) E[cc] = row < nc && cc < keep ? etop(blk, row, cc) : CR{(R)0, (R)0};
+        const CR* Ub = Us + (size_t)blk * CHI * NR + row;
+        for (int j = 0; j < nc; ++j) {
+            const CR u = Ub[j * NR];
+            const CR* Z = sm.T + (blk * CHI + j) * CHI;
+#pragma unroll
+            for (int cc = 0; cc < CHI; ++cc)
+                if (cc < keep) E[cc] = cfms(u, Z[cc], E[cc]);
+        }
+        const double w = x ? w2[1] : w2[0];
+        const R iw = w > 0.0 ? (R)nr_rcp(w) : (R)0;
+        auto stride = [](int k) { return k == 0 ? CHI * CHI : (k == 1 ? CHI : 1); };
+        const int ss = stride(slot);
+        CT* gv = Gam + (size_t)vtx * 2 * H;
+        CT* g = gv + (size_t)i * H + row / CHI * stride(o0) + row % CHI * stride(o1);
+#pragma unroll
+        for (int cc = 0; cc < CHI; ++cc) g[cc * ss] = ccast<TS>(iw * E[cc]);
+        if ((bits >> (2 + x)) & 1) {   // the mixing gate after the vertex's last gate
+            __syncthreads();
+            for (int r = tid; r < H; r += 512) {
+                CT g0 = gv[r], g1 = gv[H + r];
+                mix_pair(g0, g1, c.cX, c.sX);
+                gv[r] = g0;
+                gv[H + r] = g1;
+            }
+        }
     }
 }
 
