@@ -109,10 +109,10 @@ struct gtqa_state {
     bool plain = false;         // degree 4 or CHI = 16: the plain kernels
     cd* pscratch = nullptr;     // plain path: per-block tensor buffers in global memory
     cd* dm = nullptr;           // plain path: new - old of every message of a sweep
+    cd* Fp = nullptr;           // plain path: the two halves of every message of a sweep
     int4* vslots4 = nullptr;
     int* gate_bits = nullptr;   // per gate in colour order: first and last gates of its vertices
     std::vector<int> h_coff;    // first gate of every colour
-    int cur4 = 0;               // message buffer holding the latest messages (degree 4)
     // gtqa_anneal_graph: one captured layer (gates, BP, regauge) whose layer index is read from
     // *kdev, and what it was captured for; with profiling on, events between the launches
     cudaGraph_t graph = nullptr;
@@ -513,7 +513,7 @@ void free_state(gtqa_state* s) {
                     s->vert_edges, s->vert_inst, s->J, s->h, s->colour_edges, s->colour_off, s->gates_meta,
                     s->iso, s->inst_vbeg, s->inst_m, s->acc, s->inst_done, s->inst_iters, s->inst_dist,
                     s->stats, s->ctl, s->rho, s->sign, s->flags, s->rbuf, s->cutbuf, s->xs, s->ps,
-                    s->gate_edge, s->gate_U, s->sq_vertex, s->sq_W, s->vslots4, s->gate_bits, s->pscratch, s->dm};
+                    s->gate_edge, s->gate_U, s->sq_vertex, s->sq_W, s->vslots4, s->gate_bits, s->pscratch, s->dm, s->Fp};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& p : s->pending) {
@@ -783,6 +783,7 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
     }
     coff[ncol] = (int)cedges.size();
     std::vector<int> gbits;
+    int max_gates = 0;   // of one colour
     if (s->plain) {
         s->h_coff = coff;
         gbits.resize(Mtot);
@@ -793,7 +794,9 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
                 gbits[q] |= (firstc[v] == gcol[ed]) << x | (lastc[v] == gcol[ed]) << (2 + x);
             }
         }
-        if (plain_ising_launch(s->CHI, s->D, pmode, nullptr, nullptr) != cudaSuccess) {
+        for (int q = 0; q < ncol; ++q) max_gates = std::max(max_gates, coff[q + 1] - coff[q]);
+        if (plain_ising_launch(s->CHI, s->D, pmode, nullptr, nullptr) != cudaSuccess ||
+            plain_prepare(s->CHI, s->D, pmode) != cudaSuccess) {
             cudaGetLastError();
             delete s;
             return GTQA_ERR_CUDA;
@@ -819,7 +822,8 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
         (rc = dalloc(s, &s->cutbuf, std::max(s->m, 1))) || (rc = dalloc(s, &s->xs, s->n)) ||
         (rc = dalloc(s, &s->ps, s->n)) || (s->plain && (rc = dalloc(s, &s->vslots4, s->n))) ||
         (s->plain && (rc = dalloc(s, &s->gate_bits, s->m))) ||
-        (s->plain && (rc = dalloc(s, &s->pscratch, plain_scratch_entries(s->CHI, s->D, s->n, s->m)))) ||
+        (s->plain && (rc = dalloc(s, &s->pscratch, plain_scratch_entries(s->CHI, s->D, max_gates)))) ||
+        (s->plain && (rc = dalloc(s, &s->Fp, (size_t)4 * s->m * CHI * CHI))) ||
         (s->plain && (rc = dalloc(s, &s->dm, (size_t)2 * s->m * CHI * CHI)))) {
         free_state(s);
         return rc;
@@ -1000,26 +1004,25 @@ void tridiag_min_eigvec(const std::vector<double>& a, const std::vector<double>&
 }
 
 // ---------------------------------------------------------------------------
-// degree-4 graphs: host orchestration of the plain kernels of gtqa_deg4.cuh
+// the plain path: host orchestration of the kernels of gtqa_plain.cuh
 // ---------------------------------------------------------------------------
-PlainArgs d4_args(gtqa_state* s, int cur) {
+PlainArgs d4_args(gtqa_state* s) {
     PlainArgs a;
     a.Gamma = s->Gamma;
     a.T = s->T;
     a.lam = s->lam;
-    a.msg_cur = s->msg[cur];
-    a.msg_nxt = s->msg[cur ^ 1];
+    a.msg[0] = s->msg[0];
+    a.msg[1] = s->msg[1];
     a.X = s->X;
     a.dm = s->dm;
-    a.scratch = s->pscratch;
     a.vslots = s->vslots4;
     a.edge_info = s->edge_info;
     a.n = s->n;
     a.m = s->m;
-    a.acc = s->acc;
     a.warm = 0;
     a.D0 = s->D0;
     a.t0 = s->t0;
+    a.ctl = s->ctl;
     return a;
 }
 
@@ -1071,64 +1074,37 @@ int d4_trotter(gtqa_state* s, double tZ, double tXpre, double tXpost) {
 }
 
 int d4_regauge(gtqa_state* s) {
-    if (plain_regauge_launch(s->CHI, s->D, pm(s), d4_args(s, s->cur4), s->msg[s->cur4], s->eig_cutoff,
-                             s->svd_cutoff, s->stream) != cudaSuccess)
+    if (plain_regauge_launch(s->CHI, s->D, pm(s), d4_args(s), s->eig_cutoff, s->svd_cutoff, s->stream) != cudaSuccess)
         return d4_fail(s);
     s->launches += 2;
     return GTQA_OK;
 }
 
-// Flooding BP (App. B): one launch per sweep; the host reads the trace-norm distance after
-// each sweep and stops after the sweep where dist/|E| < tol, or after max_iter sweeps.
-int d4_bp(gtqa_state* s, double tol, int max_iter, uint32_t flags, int32_t* iters_out, double* dist_out) {
-    int cur = s->cur4;
-    PlainArgs a = d4_args(s, cur);
-    a.warm = (flags & GTQA_BP_WARM_START) ? 1 : 0;
-    a.msg_nxt = s->msg[cur];   // the init kernel writes the warm start where the first sweep reads
-    if (s->n > 0 && plain_bp_init_launch(s->CHI, s->D, pm(s), a, s->stream) != cudaSuccess) return d4_fail(s);
-    s->launches += 1;
-    int it = 0;
-    double dist = 0.0;
-    bool conv = false;
-    for (; it < max_iter;) {
-        if (!cuda_ok(s, cudaMemsetAsync(s->acc, 0, sizeof(double), s->stream))) return GTQA_ERR_CUDA;
-        PlainArgs w = d4_args(s, cur);
-        if (plain_bp_sweep_launch(s->CHI, s->D, pm(s), w, s->stream) != cudaSuccess) return d4_fail(s);
-        s->launches += 2;
-        double acc = 0.0;
-        if (!cuda_ok(s, cudaMemcpyAsync(&acc, s->acc, sizeof(double), cudaMemcpyDeviceToHost, s->stream)) ||
-            !cuda_ok(s, cudaStreamSynchronize(s->stream)))
-            return GTQA_ERR_CUDA;
-        cur ^= 1;
-        ++it;
-        dist = s->m > 0 ? acc / s->m : 0.0;
-        if (!(dist == dist)) {
-            s->sticky = GTQA_ERR_NUMERIC;
-            return GTQA_ERR_NUMERIC;
-        }
-        if (dist < tol) {
-            conv = true;
-            break;
-        }
-    }
-    s->cur4 = cur;
+// Flooding BP (App. B), and with GTQA_BP_REGAUGE the regauge: asynchronous, the sweeps and the
+// stopping rule run on the device.
+int d4_bp(gtqa_state* s, double tol, int max_iter, uint32_t flags) {
+    PlainBPArgs b;
+    b.p = d4_args(s);
+    b.p.warm = (flags & GTQA_BP_WARM_START) ? 1 : 0;
+    if (plain_bp_init_launch(s->CHI, s->D, pm(s), b.p, s->stream) != cudaSuccess) return d4_fail(s);
+    if (!cuda_ok(s, cudaMemsetAsync(s->acc, 0, 6 * sizeof(double), s->stream))) return GTQA_ERR_CUDA;
+    b.tol = tol;
+    b.max_iter = max_iter;
+    b.Fp = s->Fp;
+    b.acc = s->acc;
+    b.bar = &s->ctl->bar_pk[PK_BP];
+    b.nblocks = s->grid[PK_BP];
+    b.bar_expect = s->grid[PK_BP] + s->bar_extra;
+    b.spin_limit = s->spin_limit;
+    if (plain_bp_launch(s->CHI, s->D, pm(s), b, s->stream) != cudaSuccess) return d4_fail(s);
+    s->launches += 2;
+    return (flags & GTQA_BP_REGAUGE) ? d4_regauge(s) : GTQA_OK;
+}
+
+// The layers' errors (a NaN distance, a barrier that gave up), once per call.
+int d4_finish(gtqa_state* s) {
     Control ctl;
-    int rc;
-    if ((rc = read_ctl(s, &ctl))) return rc;
-    ctl.cur = cur;
-    ctl.last_iters = it;
-    ctl.last_dist = dist;
-    ctl.not_conv = conv ? 0 : 1;
-    ctl.sweeps_total += it;
-    ctl.bp_calls += 1;
-    ctl.nc_calls += conv ? 0 : 1;
-    if (!cuda_ok(s, cudaMemcpyAsync(s->ctl, &ctl, sizeof(Control), cudaMemcpyHostToDevice, s->stream)) ||
-        !cuda_ok(s, cudaStreamSynchronize(s->stream)))
-        return GTQA_ERR_CUDA;
-    if (iters_out) *iters_out = it;
-    if (dist_out) *dist_out = dist;
-    if ((flags & GTQA_BP_REGAUGE) && (rc = d4_regauge(s))) return rc;
-    return conv ? GTQA_OK : GTQA_ERR_NOT_CONVERGED;
+    return read_ctl(s, &ctl);
 }
 
 // Unnormalised residual sum of App. C over the 2m directed bonds, added to s->rbuf.
@@ -1161,8 +1137,7 @@ int d4_anneal_policy(gtqa_state* s, int k_begin, int k_end, int K, double dt, do
             return GTQA_ERR_NUMERIC;
         }
         if (sum > thr_sum) {
-            rc = d4_bp(s, tol, max_iter, GTQA_BP_DEFAULT, nullptr, nullptr);
-            if (rc && rc != GTQA_ERR_NOT_CONVERGED) return rc;
+            if ((rc = d4_bp(s, tol, max_iter, GTQA_BP_DEFAULT))) return rc;
             ++reg;
         } else {
             ++skip;
@@ -1477,14 +1452,17 @@ int gtqa_bp_sweep(gtqa_state* s, double tol, int32_t max_iter, uint32_t flags, i
     int rc = check_state(s);
     if (rc) return rc;
     if (max_iter < 1 || !(tol >= 0.0) || (flags & ~3u)) return GTQA_ERR_INVALID_ARG;
-    if (s->plain) return d4_bp(s, tol, max_iter, flags, iters_out, dist_out);
-    Ctx c = make_ctx(s);
-    c.phases = PH_BP | ((flags & GTQA_BP_WARM_START) ? PH_WARM : 0u);
-    c.k0 = c.k1 = 0;
-    c.tol = tol;
-    c.max_iter = max_iter;
-    if ((rc = run(s, c, PK_BP, GTQA_K_BP, s->n))) return rc;
-    if ((flags & GTQA_BP_REGAUGE) && (rc = run(s, c, PK_REGAUGE, GTQA_K_REGAUGE, s->m))) return rc;
+    if (s->plain) {
+        if ((rc = d4_bp(s, tol, max_iter, flags))) return rc;
+    } else {
+        Ctx c = make_ctx(s);
+        c.phases = PH_BP | ((flags & GTQA_BP_WARM_START) ? PH_WARM : 0u);
+        c.k0 = c.k1 = 0;
+        c.tol = tol;
+        c.max_iter = max_iter;
+        if ((rc = run(s, c, PK_BP, GTQA_K_BP, s->n))) return rc;
+        if ((flags & GTQA_BP_REGAUGE) && (rc = run(s, c, PK_REGAUGE, GTQA_K_REGAUGE, s->m))) return rc;
+    }
     Control ctl;
     if ((rc = read_ctl(s, &ctl))) return rc;
     if (iters_out) *iters_out = ctl.last_iters;
@@ -1520,8 +1498,7 @@ int gtqa_sample(gtqa_state* s, int32_t k, const int32_t* order, const double* u,
             return d4_fail(s);
         s->launches += 1;
         // the projection leaves the Vidal gauge: BP from the warm start, then the regauge
-        rc = d4_bp(s, tol, max_iter, GTQA_BP_WARM_START | GTQA_BP_REGAUGE, nullptr, nullptr);
-        if (rc && rc != GTQA_ERR_NOT_CONVERGED) return rc;
+        if ((rc = d4_bp(s, tol, max_iter, GTQA_BP_WARM_START | GTQA_BP_REGAUGE))) return rc;
     }
     for (int q = 0; q < k && !s->plain; ++q) {
         const cudaError_t e = mixed(s) ? AuxUnit<ModeMixed>::sample(s->CHI, s->Gamma, s->lam, s->vert_edges, order[q], u[q], q,
@@ -1672,10 +1649,9 @@ int gtqa_anneal(gtqa_state* s, int32_t k_begin, int32_t k_end, int32_t K, double
         for (int k = k_begin; k <= k_end; ++k) {
             const double tau = (double)k / (double)K;
             if ((rc = d4_trotter(s, dt * tau, 0.0, dt * (1.0 - tau)))) return rc;
-            rc = d4_bp(s, tol, max_iter, GTQA_BP_DEFAULT, nullptr, nullptr);
-            if (rc && rc != GTQA_ERR_NOT_CONVERGED) return rc;
+            if ((rc = d4_bp(s, tol, max_iter, GTQA_BP_DEFAULT))) return rc;
         }
-        return GTQA_OK;
+        return d4_finish(s);
     }
     return anneal_launches(s, k_begin, k_end, K, dt, tol, max_iter);
 }
@@ -1825,10 +1801,9 @@ int gtqa_anneal_ex(gtqa_state* s, int32_t k_begin, int32_t k_end, int32_t K, dou
             const double pre = order == GTQA_TROTTER_SYMMETRIC ? 0.5 * tX : (rev ? tX : 0.0);
             const double post = order == GTQA_TROTTER_SYMMETRIC ? 0.5 * tX : (rev ? 0.0 : tX);
             if ((rc = d4_trotter(s, tZ, pre, post))) return rc;
-            rc = d4_bp(s, tol, max_iter, GTQA_BP_DEFAULT, nullptr, nullptr);
-            if (rc && rc != GTQA_ERR_NOT_CONVERGED) return rc;
+            if ((rc = d4_bp(s, tol, max_iter, GTQA_BP_DEFAULT))) return rc;
         }
-        return GTQA_OK;
+        return d4_finish(s);
     }
     Ctx c = make_ctx(s);
     c.phases = PH_GATES | PH_BP | PH_WARM | PH_REGAUGE;

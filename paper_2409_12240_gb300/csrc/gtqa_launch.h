@@ -59,11 +59,12 @@ struct GeneralUnit {
 // degree 3 with CHI = 16 for both) or 2 complex64 (degree 3 with CHI in {2, 4, 8, 16}, degree 4
 // with CHI in {2, 4})
 bool plain_supported(int CHI, int D, int pm);
-size_t plain_scratch_entries(int CHI, int D, int n, int m);
+size_t plain_scratch_entries(int CHI, int D, int gates);
+cudaError_t plain_prepare(int CHI, int D, int pm);
 cudaError_t plain_bp_init_launch(int CHI, int D, int pm, const PlainArgs& a, cudaStream_t st);
-cudaError_t plain_bp_sweep_launch(int CHI, int D, int pm, const PlainArgs& a, cudaStream_t st);
-cudaError_t plain_regauge_launch(int CHI, int D, int pm, const PlainArgs& a, const void* msg, double eig_cut,
-                                 double svd_cut, cudaStream_t st);
+cudaError_t plain_bp_launch(int CHI, int D, int pm, const PlainBPArgs& a, cudaStream_t st);
+cudaError_t plain_regauge_launch(int CHI, int D, int pm, const PlainArgs& a, double eig_cut, double svd_cut,
+                                 cudaStream_t st);
 cudaError_t plain_marginals_launch(int CHI, int D, int pm, const void* Gamma, const double* lam, const int4* vslots,
                                    int n, cd* rho, int8_t* sign, int* flag, cudaStream_t st);
 cudaError_t plain_residual_launch(int CHI, int D, int pm, const void* Gamma, const double* lam, const int4* vslots,

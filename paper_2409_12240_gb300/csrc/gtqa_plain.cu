@@ -8,46 +8,39 @@ namespace gtqa {
 
 namespace {
 template <int CHI, int D, typename R, typename RC>
-size_t sweep_smem() {
-    using S = PlainShape<CHI, D, R>;
-    // the mixed mode adds m0 and delta of the incoming messages
-    const int mix = sizeof(R) != sizeof(RC) ? 2 * D * S::CC : 0;
-    return sizeof(C<R>) * ((D + 1) * S::CC + (S::SMEM ? 3 * S::H2 : 0) + mix);
-}
-template <int CHI, int D, typename R>
-size_t vertex_smem() {
-    using S = PlainShape<CHI, D, R>;
-    return sizeof(C<R>) * (D * S::CC + (S::SMEM ? 2 * S::H2 : 0));
-}
-template <int CHI, int D, typename R, typename RC>
 cudaError_t init_t(const PlainArgs& a, cudaStream_t st) {
     if (a.n <= 0) return cudaSuccess;
-    plain_bp_init_kernel<CHI, D, R, RC><<<a.n, 256, 0, st>>>(a);
+    plain_bp_init_kernel<CHI, D, R, RC><<<a.n, 256, PlainShape<CHI, D, R, RC>::init_smem, st>>>(a);
     return cudaGetLastError();
 }
 template <int CHI, int D, typename R, typename RC>
-cudaError_t sweep_t(const PlainArgs& a, cudaStream_t st) {
-    using S = PlainShape<CHI, D, R>;
-    if (a.n > 0) {
-        plain_bp_sweep_kernel<CHI, D, R, RC><<<a.n, S::NT, sweep_smem<CHI, D, R, RC>(), st>>>(a);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    if (a.m > 0) plain_trace_norm_kernel<CHI, R, RC><<<2 * a.m, S::CC / 2, 0, st>>>((const C<R>*)a.dm, a.acc);
-    return cudaGetLastError();
+cudaError_t bp_t(const PlainBPArgs& a, cudaStream_t st) {
+    PlainBPArgs copy = a;
+    void* args[] = {&copy};
+    return cudaLaunchCooperativeKernel((const void*)plain_bp_kernel<CHI, D, R, RC>, dim3(a.nblocks), dim3(512), args,
+                                       PlainShape<CHI, D, R, RC>::bp_smem, st);
 }
 template <int CHI, int D, typename R, typename RC>
-cudaError_t regauge_t(const PlainArgs& a, const void* msg, double eig_cut, double svd_cut, cudaStream_t st) {
-    using S = PlainShape<CHI, D, R>;
+cudaError_t regauge_t(const PlainArgs& a, double eig_cut, double svd_cut, cudaStream_t st) {
+    using S = PlainShape<CHI, D, R, R>;
     if (a.m > 0) {
-        plain_regauge_edge_kernel<CHI, R, RC><<<a.m, S::CC / 2, 0, st>>>((const C<R>*)msg, a.lam, (C<R>*)a.X,
-                                                                         eig_cut, svd_cut);
+        plain_regauge_edge_kernel<CHI, R, RC><<<a.m, S::CC, sizeof(PlainEdgeSm<CHI, RC>), st>>>(a, eig_cut, svd_cut);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     if (a.n <= 0) return cudaSuccess;
-    plain_regauge_vertex_kernel<CHI, D, R><<<a.n, 256, vertex_smem<CHI, D, R>(), st>>>(a);
+    plain_regauge_vertex_kernel<CHI, D, R><<<2 * a.n, S::NT, S::vertex_smem, st>>>(a);
     return cudaGetLastError();
+}
+// the shared-memory limits of the kernels of one shape
+template <int CHI, int D, typename R, typename RC>
+cudaError_t prepare_t() {
+    using S = PlainShape<CHI, D, R, RC>;
+    cudaError_t e = raise_smem_limit(plain_bp_init_kernel<CHI, D, R, RC>, S::init_smem);
+    if (e == cudaSuccess) e = raise_smem_limit(plain_bp_kernel<CHI, D, R, RC>, S::bp_smem);
+    if (e == cudaSuccess) e = raise_smem_limit(plain_regauge_edge_kernel<CHI, R, RC>, sizeof(PlainEdgeSm<CHI, RC>));
+    if (e == cudaSuccess) e = raise_smem_limit(plain_regauge_vertex_kernel<CHI, D, R>, PlainShape<CHI, D, R, R>::vertex_smem);
+    return e;
 }
 template <int CHI, int D, typename R>
 cudaError_t marg_t(const void* G, const double* lam, const int4* vs, int n, cd* rho, int8_t* sign, int* flag,
@@ -97,26 +90,29 @@ bool plain_supported(int CHI, int D, int pm) {
     return (D == 3 && (CHI == 2 || CHI == 4 || CHI == 8 || CHI == 16)) || (D == 4 && (CHI == 2 || CHI == 4));
 }
 
-size_t plain_scratch_entries(int CHI, int D, int n, int m) {
-    // complex entries (sized for complex128; the complex64 mode uses half of each entry)
-    if (D == 3 && CHI == 16)
-        return std::max((size_t)n * PlainShape<16, 3, double>::scratch_per_block, (size_t)m * 4 * 16 * 256);
-    return 0;
+size_t plain_scratch_entries(int CHI, int D, int gates) {
+    // complex entries: the reflectors of the largest launch of CHI = 16 gates
+    return D == 3 && CHI == 16 ? (size_t)gates * 4 * 16 * 256 : 0;
 }
 
+cudaError_t plain_prepare(int CHI, int D, int pm) {
+#define C_(c, d, r, rc) prepare_t<c, d, r, rc>()
+    GTQA_PLAIN_DISPATCH(C_)
+#undef C_
+}
 cudaError_t plain_bp_init_launch(int CHI, int D, int pm, const PlainArgs& a, cudaStream_t st) {
 #define C_(c, d, r, rc) init_t<c, d, r, rc>(a, st)
     GTQA_PLAIN_DISPATCH(C_)
 #undef C_
 }
-cudaError_t plain_bp_sweep_launch(int CHI, int D, int pm, const PlainArgs& a, cudaStream_t st) {
-#define C_(c, d, r, rc) sweep_t<c, d, r, rc>(a, st)
+cudaError_t plain_bp_launch(int CHI, int D, int pm, const PlainBPArgs& a, cudaStream_t st) {
+#define C_(c, d, r, rc) bp_t<c, d, r, rc>(a, st)
     GTQA_PLAIN_DISPATCH(C_)
 #undef C_
 }
-cudaError_t plain_regauge_launch(int CHI, int D, int pm, const PlainArgs& a, const void* msg, double eig_cut,
-                                 double svd_cut, cudaStream_t st) {
-#define C_(c, d, r, rc) regauge_t<c, d, r, rc>(a, msg, eig_cut, svd_cut, st)
+cudaError_t plain_regauge_launch(int CHI, int D, int pm, const PlainArgs& a, double eig_cut, double svd_cut,
+                                 cudaStream_t st) {
+#define C_(c, d, r, rc) regauge_t<c, d, r, rc>(a, eig_cut, svd_cut, st)
     GTQA_PLAIN_DISPATCH(C_)
 #undef C_
 }

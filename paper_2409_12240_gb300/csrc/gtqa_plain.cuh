@@ -18,9 +18,8 @@
 //            (CHI = 16), the per-physical-index QR-reduced simple update with a 2 CHI x 2 CHI
 //            core (App. E, App. D "Truncation"), the mixing gates (Sec. II D) fused;
 //   bp       T = Gamma prod lambda^{1/2} (Eq. (symmetric_gauge)), warm start
-//            diag(lambda)/sum(lambda) (Eq. (reconstructed_messages)); per flooding sweep of
-//            Eq. (local_consistency) one launch over vertices and one over messages for the
-//            exact trace-norm distance (App. B); the host reads the distance after every sweep;
+//            diag(lambda)/sum(lambda) (Eq. (reconstructed_messages)); then one cooperative launch
+//            runs the flooding sweeps of Eq. (local_consistency) and their stopping rule (App. B);
 //   regauge  per edge the Vidal gauge transforms from the two messages (App. D "Vidal gauge
 //            finding"), then per vertex the transforms applied to T;
 //   marginals  Eq. (partial_dens) with the environment of Eq. (bp_approx);
@@ -39,27 +38,41 @@ struct PlainArgs {
     void* Gamma;
     void* T;
     double* lam;
-    const void* msg_cur;      // incoming and previous outgoing messages
-    void* msg_nxt;            // new outgoing messages
+    void* msg[2];             // the message buffers; ctl->cur is the current one
     void* X;                  // regauge transforms [m][2][CHI^2]
-    void* dm;                 // [2m][CHI^2]: new - old of every outgoing message of a sweep
-    void* scratch;            // per-block tensor buffers when shared memory is too small
+    void* dm;                 // [2m][CHI^2]: new - old of every message of a sweep
     const int4* vslots;       // slots per vertex (x, y, z, w; -1 phantom)
     const int4* edge_info;    // (u, v, slot at u, slot at v)
     int n, m;
-    double* acc;              // distance accumulator (one double)
     int warm;
     void* D0;                 // mixed mode: [2m][CHI^2] warm-start defect F(m0) - tr F(m0) m0 (storage type)
     cd* t0;                   // mixed mode: [2m] tr F(m0)
+    Control* ctl;
 };
 
-template <int CHI, int D, typename R = double>
+template <int CHI, int D, typename R, typename RC = R>
 struct PlainShape {
     static constexpr int H = ipow(CHI, D), H2 = 2 * H, CC = CHI * CHI;
-    static constexpr int NT = 16 * CC < 1024 ? 16 * CC : 1024;    // threads of the sweep kernel
-    static constexpr int TPO = NT / CC;                           // threads per message entry
-    static constexpr bool SMEM = 3 * H2 * (int)sizeof(C<R>) <= 48 * 1024;   // tensor buffers in shared memory
-    static constexpr size_t scratch_per_block = SMEM ? 0 : (size_t)3 * H2;   // complex entries
+    static constexpr bool MIX = sizeof(R) != sizeof(RC);
+    // team of one (vertex, physical index) item, and the outputs of a fiber per lane
+    static constexpr int NT = CHI == 16 ? 512 : (CHI == 8 || (D == 4 && CHI == 4) ? 128 : (CHI == 4 ? 64 : 32));
+    static constexpr int XO = H > NT ? H / NT : 1;
+    static constexpr int ITEMS = H / XO, PARTS = NT / CC;
+    static constexpr int TPB = 512, TEAMS = TPB / NT;
+    static constexpr int PH = H + H / CC;                // one padding element per CHI^2 plane
+    static constexpr int NB = D == 4 ? 4 : 3;            // T, prefix, suffix (and one more)
+    static constexpr bool RANK = CHI >= 8;               // skip indices beyond the bonds' dimensions
+    static constexpr size_t team_smem = sizeof(C<R>) * (NB * PH + (MIX ? 2 : 1) * D * CC) + sizeof(R) * D * CHI +
+                                        sizeof(int) * 16;
+    static constexpr int GL = CC / 2 > 1 ? CC / 2 : 1;   // lanes of a trace norm
+    static constexpr int GROUPS = TPB / GL < 64 ? TPB / GL : 64;
+    static constexpr size_t group_smem =
+        sizeof(RC) == 8 ? (size_t)CC * (3 * sizeof(cd) + 2 * sizeof(cf)) + 2 * CHI * sizeof(double) : (size_t)CC * sizeof(cf) + 16;
+    static constexpr size_t bp_smem = (TEAMS * ((team_smem + 15) / 16 * 16) > GROUPS * ((group_smem + 15) / 16 * 16)
+                                           ? TEAMS * ((team_smem + 15) / 16 * 16)
+                                           : GROUPS * ((group_smem + 15) / 16 * 16));
+    static constexpr size_t init_smem = MIX ? sizeof(cd) * (H2 + H2 / CC) : 0;
+    static constexpr size_t vertex_smem = sizeof(C<R>) * (PH + CC);
 };
 
 __device__ __forceinline__ int plain_slot_edge(const int4& v, int k) {
@@ -67,12 +80,19 @@ __device__ __forceinline__ int plain_slot_edge(const int4& v, int k) {
 }
 
 // T = Gamma prod_k lambda_k^{1/2}; with warm, the vertex's outgoing messages are set to
-// diag(lambda)/sum(lambda) in msg_nxt (the buffer the first sweep reads).  One block per vertex.
+// diag(lambda)/sum(lambda) (mixed: delta = 0) in the current message buffer.  One block per vertex.
+// Mixed: F0 = F(m0) of every outgoing message in FP64 from the stored T (so that F(m0 + delta) =
+// F0 + F_delta holds for the T that the sweeps contract), kept as D0 = F0 - tr(F0) m0 and t0.  As on
+// the persistent path the weights are folded into T~ = T prod m0^{1/2} once, so that a term is one
+// complex product (4 FP64 instructions instead of 12), and only j <= j' is summed.
 template <int CHI, int D, typename R, typename RC = R>
-__global__ void plain_bp_init_kernel(PlainArgs a) {
-    using S = PlainShape<CHI, D, R>;
+__global__ void __launch_bounds__(256) plain_bp_init_kernel(PlainArgs a) {
+    using S = PlainShape<CHI, D, R, RC>;
+    constexpr bool MIX = S::MIX;
+    constexpr int CC = S::CC, H = S::H, H2 = S::H2;
+    extern __shared__ __align__(16) unsigned char plain_smem[];
     const int v = blockIdx.x;
-    __shared__ RC sq[D][CHI], m0[D][CHI];
+    __shared__ RC sq[D][CHI], m0[D][CHI], rt[D][CHI];
     const int4 sl = a.vslots[v];
     if (threadIdx.x < D * CHI) {
         const int k = threadIdx.x / CHI, j = threadIdx.x % CHI;
@@ -82,467 +102,697 @@ __global__ void plain_bp_init_kernel(PlainArgs a) {
         RC s = 0.0;
         for (int q = 0; q < CHI; ++q) s += lam_get(a.lam, CHI, e, q);
         m0[k][j] = s > 0.0 ? lj / s : 0.0;
+        if constexpr (MIX) rt[k][j] = s > 0.0 ? sqrt(lj / s) : 0.0;
     }
     __syncthreads();
-    const C<R>* g = (const C<R>*)a.Gamma + (size_t)v * S::H2;
-    C<R>* T = (C<R>*)a.T + (size_t)v * S::H2;
-    for (int t = threadIdx.x; t < S::H2; t += blockDim.x) {
-        int r = t % S::H;
-        RC f = 1.0;
+    const C<R>* g = (const C<R>*)a.Gamma + (size_t)v * H2;
+    C<R>* T = (C<R>*)a.T + (size_t)v * H2;
+    cd* Tm = reinterpret_cast<cd*>(plain_smem);
+    for (int t = threadIdx.x; t < H2; t += blockDim.x) {
+        int r = t % H;
+        RC f = 1.0, w = 1.0;
+#pragma unroll
         for (int k = D - 1; k >= 0; --k) {
             f *= sq[k][r % CHI];
+            if constexpr (MIX) w *= rt[k][r % CHI];
             r /= CHI;
         }
-        T[t] = ccast<R>(f * ccast<RC>(g[t]));
+        const C<R> tv = ccast<R>(f * ccast<RC>(g[t]));
+        T[t] = tv;
+        if constexpr (MIX) Tm[t + t / CC] = w * ccast<double>(tv);
     }
-    constexpr bool MIX = sizeof(R) != sizeof(RC);
     if (a.warm) {
-        // the mixed mode holds delta = m - m0, which the warm start sets to 0
-        C<R>* out = (C<R>*)a.msg_nxt;
-        for (int t = threadIdx.x; t < D * S::CC; t += blockDim.x) {
-            const int k = t / S::CC, r = t % S::CC;
+        C<R>* out = (C<R>*)a.msg[a.ctl->cur];
+        for (int t = threadIdx.x; t < D * CC; t += blockDim.x) {
+            const int k = t / CC, r = t % CC;
             const int e = plain_slot_edge(sl, k);
             if (e < 0) continue;
             const int o = 2 * e + (a.edge_info[e].x == v ? 0 : 1);
             const int j = r / CHI, jp = r % CHI;
-            out[(size_t)o * S::CC + r] = C<R>{(!MIX && j == jp) ? (R)m0[k][j] : (R)0, (R)0};
+            out[(size_t)o * CC + r] = C<R>{(!MIX && j == jp) ? (R)m0[k][j] : (R)0, (R)0};
         }
     }
     if constexpr (MIX) {
-        // F0 = F(m0) of every outgoing message in RC from the stored T (so that F(m0 + delta) =
-        // F0 + F_delta holds for the T the sweeps contract), kept as D0 = F0 - tr(F0) m0 and t0
-        __shared__ C<RC> F0[D][S::CC];
-        __shared__ C<RC> tr0[D];
-        __syncthreads();   // this block's T is written
-        constexpr int NO = S::H / CHI;
-        for (int t = threadIdx.x; t < D * S::CC; t += blockDim.x) {
-            const int k = t / S::CC, r = t % S::CC;
-            if (plain_slot_edge(sl, k) < 0) continue;
-            const int j = r / CHI, jp = r % CHI;
-            int sk = 1;
-            for (int l = D - 1; l > k; --l) sk *= CHI;
-            C<RC> f = C<RC>{(RC)0, (RC)0};
-            for (int i = 0; i < 2; ++i)
-                for (int q = 0; q < NO; ++q) {
-                    int rem = q, base = 0, stride = 1;
-                    RC w = 1.0;
-                    for (int l = D - 1; l >= 0; --l) {
-                        if (l != k) {
-                            const int idx = rem % CHI;
-                            rem /= CHI;
-                            w *= m0[l][idx];
-                            base += idx * stride;
-                        }
-                        stride *= CHI;
-                    }
-                    const C<RC> x = ccast<RC>(T[i * S::H + base + j * sk]), y = ccast<RC>(T[i * S::H + base + jp * sk]);
-                    f = cfmac(y, w * x, f);
+        __shared__ cd F0[D][CC];
+        __shared__ double tr0[D];
+        __syncthreads();
+        // PN lanes per entry (j <= j') of a slot
+        constexpr int NU = CHI * (CHI + 1) / 2, PN = CHI == 16 ? 1 : (CHI == 4 ? 8 : 16), NO = H / CHI;
+        for (int item = threadIdx.x / PN; item < D * NU; item += blockDim.x / PN) {
+            const int k = item / NU, part = threadIdx.x % PN;
+            int u = item % NU, j = 0;
+            while (u >= CHI - j) { u -= CHI - j; ++j; }
+            const int jp = j + u;
+            cd f = cd{0.0, 0.0};
+            if (plain_slot_edge(sl, k) >= 0 && m0[k][j] > 0.0 && m0[k][jp] > 0.0) {
+                const int sk = ipow(CHI, D - 1 - k);
+                for (int q = part; q < 2 * NO; q += PN) {
+                    const int i = q / NO, c = q % NO;
+                    const int base = i * H + (c / sk) * sk * CHI + c % sk;
+                    const int tj = base + j * sk, tp = base + jp * sk;
+                    f = cfmac(Tm[tp + tp / CC], Tm[tj + tj / CC], f);
                 }
-            F0[k][r] = f;
+            }
+            f.x = group_sum<PN>(f.x, group_mask<PN>());
+            f.y = group_sum<PN>(f.y, group_mask<PN>());
+            if (part == 0) {
+                const double d = m0[k][j] * m0[k][jp];
+                f = d > 0.0 ? (1.0 / sqrt(d)) * f : cd{0.0, 0.0};
+                F0[k][j * CHI + jp] = f;
+                F0[k][jp * CHI + j] = conj(f);
+            }
         }
         __syncthreads();
         if (threadIdx.x < D) {
-            C<RC> tr = C<RC>{(RC)0, (RC)0};
-            for (int j = 0; j < CHI; ++j) tr = tr + F0[threadIdx.x][j * CHI + j];
+            double tr = 0.0;
+            for (int j = 0; j < CHI; ++j) tr += F0[threadIdx.x][j * CHI + j].x;
             tr0[threadIdx.x] = tr;
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < D * S::CC; t += blockDim.x) {
-            const int k = t / S::CC, r = t % S::CC;
+        for (int t = threadIdx.x; t < D * CC; t += blockDim.x) {
+            const int k = t / CC, r = t % CC;
             const int e = plain_slot_edge(sl, k);
             if (e < 0) continue;
             const int o = 2 * e + (a.edge_info[e].x == v ? 0 : 1);
             const int j = r / CHI, jp = r % CHI;
-            C<RC> d = F0[k][r];
-            if (j == jp) d = d - m0[k][j] * tr0[k];
-            ((C<R>*)a.D0)[(size_t)o * S::CC + r] = ccast<R>(d);
-            if (r == 0) a.t0[o] = ccast<double>(tr0[k]);
+            cd d = F0[k][r];
+            if (j == jp) d.x -= m0[k][j] * tr0[k];
+            ((C<R>*)a.D0)[(size_t)o * CC + r] = ccast<R>(d);
+            if (r == 0) a.t0[o] = cd{tr0[k], 0.0};
         }
     }
 }
 
-// One flooding sweep for one vertex: every outgoing message
-//   m_{v->b}[j][j'] = sum T[.., j@s, ..] conj(T[.., j'@s, ..]) prod_{o != s} m_o[x_o][x'_o]
-// (Eq. (local_consistency)), divided by its complex trace; new - old goes to dm for the
-// trace-norm kernel.
-// R is the storage and contraction type; RC the type of the trace and the normalisation
-// (FP64 in the mixed mode).
-template <int CHI, int D, typename R, typename RC = R>
-__global__ void __launch_bounds__(PlainShape<CHI, D, R>::NT) plain_bp_sweep_kernel(PlainArgs a) {
-    using S = PlainShape<CHI, D, R>;
-    constexpr int H2 = S::H2, CC = S::CC, NT = S::NT, TPO = S::TPO;
-    extern __shared__ __align__(16) unsigned char plain_smem[];
-    C<R>* min = reinterpret_cast<C<R>*>(plain_smem);   // [D][CC]
-    C<R>* F = min + D * CC;                          // [CC]
-    C<R>* T;
-    C<R>* P0;
-    C<R>* P1;
-    if constexpr (S::SMEM) {
-        T = F + CC;
-        P0 = T + H2;
-        P1 = P0 + H2;
+// ---------------------------------------------------------------------------
+// Flooding BP (App. B) of the plain path in one cooperative launch: sweeps of Eq.
+// (local_consistency) until dist/|E| < tol or max_iter, decided on the device.
+//
+// Per sweep: (A) an item is one physical index i of one vertex.  With L_s = T x_0 m_0 .. x_{s-1}
+// m_{s-1} and R_s = T x_{s+1} m_{s+1}^H .. x_{D-1} m_{D-1}^H the message out of slot s is
+// F_s[j][j'] = sum L_s[.. j@s ..] conj(R_s[.. j'@s ..]), so that 2 (D - 1) contractions along one slot
+// serve all D messages (instead of D (D - 1)).  A lane contracts (part of) a fiber: it
+// reads the fiber's CHI elements once into registers and writes its outputs in place; the
+// message's entries are shared-memory broadcasts.  Mixed mode (messages m = m0 + delta): the same
+// with dL_{s+1} = dL_s x m_s + (T prod m0) x delta_s, likewise dR, and
+// F_s - F_s(m0) = sum dL conj(R) + (L - dL) conj(dR).  The halves i = 0, 1 are added in (B), one
+// warp per message: trace, normalisation (reading R10), new - old and its Frobenius norm, a lower
+// bound of the trace norm; only a sweep whose sum of bounds falls under tol |E| (or the last one)
+// is followed by (C), the exact trace norms.  Two grid barriers per sweep; the host is not
+// involved.
+//
+// chi = 16 in FP64 is bound by the FP64 pipe (7 contraction-sized products of 2 CHI^4 per vertex);
+// splitting a vertex by i lets three 64 KB buffers fit shared memory and balances 2n items over
+// the SMs; indices beyond a bond's current dimension are skipped there.
+// ---------------------------------------------------------------------------
+struct PlainBPArgs {
+    PlainArgs p;
+    double tol;
+    int max_iter;
+    void* Fp;                 // [2][2m][CC] partial messages
+    double* acc;              // [6]: bounds and exact distances, cycled over three sweeps
+    unsigned long long* bar;
+    int nblocks, bar_expect;
+    long long spin_limit;
+};
+
+template <int CHI, int D, typename R, typename RC>
+struct PlainTeam {   // shared memory of one team
+    using S = PlainShape<CHI, D, R, RC>;
+    C<R>* buf[4];
+    C<R>* m;      // [D][CC] incoming messages
+    C<R>* dm;     // mixed: incoming delta
+    R* m0;        // [D][CHI]: mixed, warm-start diagonals
+    int* dim;     // [D] dimensions of the bonds, [4 ..] outgoing message of each slot (-1)
+    __device__ PlainTeam(unsigned char* base) {
+        C<R>* p = reinterpret_cast<C<R>*>(base);
+        for (int k = 0; k < 4; ++k) buf[k] = p + (k < S::NB ? k : 0) * S::PH;
+        m = p + S::NB * S::PH;
+        dm = m + (S::MIX ? D * S::CC : 0);
+        m0 = reinterpret_cast<R*>(dm + D * S::CC);
+        dim = reinterpret_cast<int*>(m0 + D * CHI);
+    }
+};
+
+// product of the warm-start weights of the slots before (SUF: after) K at element index r
+template <int CHI, int D, int K, bool SUF, typename R>
+__device__ __forceinline__ R plain_weight(const R* m0, int r) {
+    R w = (R)1;
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+        if (SUF ? k > K : k < K) w *= m0[k * CHI + (r / ipow(CHI, D - 1 - k)) % CHI];
+    return w;
+}
+
+// dst = src contracted along slot K with m_K (SUF: m_K^H); mixed: + weight (T contracted with
+// delta_K); FIRST: src is T (mixed: the first term is absent).  dst may be src.
+template <int CHI, int D, typename R, typename RC, int K, bool SUF, bool FIRST>
+__device__ __forceinline__ void plain_contract(const PlainTeam<CHI, D, R, RC>& tm, C<R>* dst, const C<R>* src, int tid,
+                                               int team) {
+    using S = PlainShape<CHI, D, R, RC>;
+    constexpr int ST = ipow(CHI, D - 1 - K), NP = CHI / S::XO, CC = S::CC;
+    const int fib = tid / NP, part = tid % NP;
+    const int base = (fib / ST) * ST * CHI + fib % ST;
+    const C<R>* T = tm.buf[0];
+    bool on = tid < S::ITEMS;
+    int rk = CHI;
+    if constexpr (S::RANK) {   // degree 3: the two other indices of the fiber
+        constexpr int o0 = K == 0 ? 1 : 0, o1 = K == 2 ? 1 : 2;
+        rk = tm.dim[K];
+        on = on && (base / ipow(CHI, D - 1 - o0)) % CHI < tm.dim[o0] && (base / ipow(CHI, D - 1 - o1)) % CHI < tm.dim[o1];
+    }
+    C<R> in[CHI], tin[S::MIX ? CHI : 1];
+    if (on) {
+#pragma unroll
+        for (int q = 0; q < CHI; ++q) {
+            const int r = base + q * ST;
+            if (!(S::MIX && FIRST)) in[q] = src[r + r / CC];
+            if constexpr (S::MIX) tin[q] = T[r + r / CC];
+        }
+    }
+    team_bar<S::NT>(team);
+    if (on) {
+        const C<R>* m = tm.m + K * CC;
+        const C<R>* dl = tm.dm + K * CC;
+        R w = (R)1;
+        if constexpr (S::MIX && !FIRST) w = plain_weight<CHI, D, K, SUF>(tm.m0, base);
+        for (int xo = 0; xo < S::XO; ++xo) {
+            const int x = part * S::XO + xo;
+            if (S::RANK && x >= rk) break;
+            C<R> acc = C<R>{(R)0, (R)0};
+            if constexpr (S::MIX) {
+#pragma unroll
+                for (int q = 0; q < CHI; ++q) {
+                    if (S::RANK && q >= rk) break;
+                    acc = SUF ? cfmac(dl[x * CHI + q], tin[q], acc) : cfma(tin[q], dl[q * CHI + x], acc);
+                }
+                if constexpr (!FIRST) acc = w * acc;
+            }
+            if constexpr (!(S::MIX && FIRST)) {
+#pragma unroll
+                for (int q = 0; q < CHI; ++q) {
+                    if (S::RANK && q >= rk) break;
+                    acc = SUF ? cfmac(m[x * CHI + q], in[q], acc) : cfma(in[q], m[q * CHI + x], acc);
+                }
+            }
+            const int r = base + x * ST;
+            dst[r + r / CC] = acc;
+        }
+    }
+    team_bar<S::NT>(team);
+}
+
+// Partial message out of slot K into Fp: L (and R) may be absent at the ends (LAST: R_K = T, dR = 0;
+// K = 0: L_0 = T, dL = 0).
+template <int CHI, int D, typename R, typename RC, int K>
+__device__ __forceinline__ void plain_overlap(const PlainTeam<CHI, D, R, RC>& tm, const C<R>* L, const C<R>* Rt, int tid,
+                                              C<R>* Fp) {
+    using S = PlainShape<CHI, D, R, RC>;
+    constexpr int ST = ipow(CHI, D - 1 - K), CC = S::CC, NO = S::H / CHI, PARTS = S::PARTS;
+    const int out = tm.dim[4 + K];
+    if (out < 0) return;   // the same for the team
+    const int pr = tid / PARTS, part = tid % PARTS, j = pr / CHI, jp = pr % CHI;
+    const C<R>* T = tm.buf[0];
+    C<R> f = C<R>{(R)0, (R)0};
+    auto term = [&](int base) {
+        const int rj = base + j * ST, rp = base + jp * ST;
+        const int pj = rj + rj / CC, pp = rp + rp / CC;
+        if constexpr (!S::MIX) {
+            f = cfmac(K == D - 1 ? T[pp] : Rt[pp], K == 0 ? T[pj] : L[pj], f);
+        } else {
+            if constexpr (K > 0) {
+                C<R> y = T[pp];
+                if constexpr (K < D - 1) y = plain_weight<CHI, D, K, true>(tm.m0, base) * y;
+                f = cfmac(y, L[pj], f);
+            }
+            if constexpr (K < D - 1) {
+                C<R> x = T[pj];
+                if constexpr (K > 0) x = L[pj] + plain_weight<CHI, D, K, false>(tm.m0, base) * x;
+                f = cfmac(Rt[pp], x, f);
+            }
+        }
+    };
+    if constexpr (S::RANK) {
+        constexpr int o0 = K == 0 ? 1 : 0, o1 = K == 2 ? 1 : 2;
+        constexpr int s0 = ipow(CHI, D - 1 - o0), s1 = ipow(CHI, D - 1 - o1);
+        const int n0 = tm.dim[o0], n1 = tm.dim[o1], rk = tm.dim[K];
+        if (j < rk && jp < rk)
+            for (int u = part; u < n0; u += PARTS)
+                for (int v = 0; v < n1; ++v) term(u * s0 + v * s1);
     } else {
-        T = (C<R>*)a.scratch + (size_t)blockIdx.x * S::scratch_per_block;
-        P0 = T + H2;
-        P1 = P0 + H2;
+        for (int c = part; c < NO; c += PARTS) term((c / ST) * ST * CHI + c % ST);
     }
-    __shared__ int es[4], in_idx[4], out_idx[4];
-    __shared__ C<RC> itr;
-    // mixed mode (the delta form of the persistent path): the messages hold delta = m - m0 with
-    // m0 = diag(lambda)/sum(lambda); mz and md hold m0 and delta of the incoming messages
-    constexpr bool MIX = sizeof(R) != sizeof(RC);
-    C<R>* mz = min + (D + 1) * CC + (S::SMEM ? 3 * H2 : 0);   // [D][CC], mixed mode only
-    C<R>* md = mz + D * CC;                                  // [D][CC], mixed mode only
-    __shared__ RC m0d[D][CHI];
-    __shared__ C<RC> tau;
-    const int v = blockIdx.x, tid = threadIdx.x;
-    const C<R>* src_msg = (const C<R>*)a.msg_cur;
-    C<R>* dst_msg = (C<R>*)a.msg_nxt;
+    f.x = group_sum<PARTS>(f.x, group_mask<PARTS>());
+    f.y = group_sum<PARTS>(f.y, group_mask<PARTS>());
+    if (part == 0) Fp[(size_t)out * CC + pr] = f;
+}
+
+// (A): the three or four partial messages of item (v, i)
+template <int CHI, int D, typename R, typename RC>
+__device__ void plain_bp_item(const PlainBPArgs& a, int item, int cur, int tid, int team,
+                              const PlainTeam<CHI, D, R, RC>& tm) {
+    using S = PlainShape<CHI, D, R, RC>;
+    constexpr int CC = S::CC, NT = S::NT;
+    const int v = item >> 1, i = item & 1;
+    const int4 sl = a.p.vslots[v];
+    const C<R>* src = (const C<R>*)a.p.msg[cur];
+    team_bar<NT>(team);   // the team may still read the previous item's buffers
     if (tid < D) {
-        const int e = plain_slot_edge(a.vslots[v], tid);
-        es[tid] = e;
+        const int e = plain_slot_edge(sl, tid);
+        int dim = 1;
         if (e >= 0) {
-            const bool first = a.edge_info[e].x == v;
-            out_idx[tid] = 2 * e + (first ? 0 : 1);
-            in_idx[tid] = 2 * e + (first ? 1 : 0);
-        } else {
-            out_idx[tid] = in_idx[tid] = -1;
+            dim = 0;
+            for (int q = 0; q < CHI; ++q) dim = __ldcg(a.p.lam + (size_t)e * CHI + q) > 0.0 ? q + 1 : dim;
         }
+        tm.dim[tid] = dim;
+        tm.dim[4 + tid] = e < 0 ? -1 : 2 * e + (a.p.edge_info[e].x == v ? 0 : 1);
     }
-    if (MIX && tid < D * CHI) {
-        const int k = tid / CHI, j = tid % CHI;
-        const int e = plain_slot_edge(a.vslots[v], k);
-        RC sum = 0.0;
-        for (int q = 0; q < CHI; ++q) sum += lam_get(a.lam, CHI, e, q);
-        m0d[k][j] = sum > 0.0 ? lam_get(a.lam, CHI, e, j) / sum : 0.0;
-    }
-    for (int t = tid; t < H2; t += NT) T[t] = ((const C<R>*)a.T)[(size_t)v * H2 + t];
-    __syncthreads();
+    const C<R>* Tg = (const C<R>*)a.p.T + (size_t)item * S::H;
+    for (int t = tid; t < S::H; t += NT) tm.buf[0][t + t / CC] = Tg[t];
     for (int t = tid; t < D * CC; t += NT) {
-        const int k = t / CC, r = t % CC;
-        if constexpr (MIX) {
-            const int j = r / CHI, jp = r % CHI;
-            const C<R> dv = in_idx[k] >= 0 ? src_msg[(size_t)in_idx[k] * CC + r] : C<R>{(R)0, (R)0};
-            const C<R> zv = C<R>{j == jp ? (R)m0d[k][j] : (R)0, (R)0};
-            md[t] = dv;
-            mz[t] = zv;
-            min[t] = zv + dv;
-        } else {
-            min[t] = in_idx[k] >= 0 ? src_msg[(size_t)in_idx[k] * CC + r] : C<R>{(R)(r == 0 ? 1 : 0), (R)0};
+        const int k = t / CC, r = t % CC, e = plain_slot_edge(sl, k), j = r / CHI, jp = r % CHI;
+        C<R> mv = e >= 0 ? ldcg(src + (size_t)(2 * e + (a.p.edge_info[e].x == v ? 1 : 0)) * CC + r)
+                         : C<R>{(R)(!S::MIX && r == 0 ? 1 : 0), (R)0};
+        if constexpr (S::MIX) {
+            tm.dm[t] = mv;
+            if (j == jp) {
+                RC s = 0.0;
+                for (int q = 0; q < CHI; ++q) s += lam_get(a.p.lam, CHI, e, q);
+                const R z = s > 0.0 ? (R)(lam_get(a.p.lam, CHI, e, j) * nr_rcp(s)) : (R)0;
+                tm.m0[k * CHI + j] = z;
+                mv.x += z;
+            }
+        }
+        tm.m[t] = mv;
+    }
+    team_bar<NT>(team);
+    C<R>* T = tm.buf[0];
+    C<R>* A = tm.buf[1];
+    C<R>* B = tm.buf[2];
+    C<R>* Fp = (C<R>*)a.Fp + (size_t)i * 2 * a.p.m * CC;
+    if constexpr (D == 3) {
+        plain_contract<CHI, D, R, RC, 0, false, true>(tm, A, T, tid, team);    // L_1
+        plain_contract<CHI, D, R, RC, 2, true, true>(tm, B, T, tid, team);     // R_1
+        plain_overlap<CHI, D, R, RC, 1>(tm, A, B, tid, Fp);
+        team_bar<NT>(team);
+        plain_contract<CHI, D, R, RC, 1, false, false>(tm, A, A, tid, team);   // L_2
+        plain_contract<CHI, D, R, RC, 1, true, false>(tm, B, B, tid, team);    // R_0
+        plain_overlap<CHI, D, R, RC, 2>(tm, A, T, tid, Fp);
+        plain_overlap<CHI, D, R, RC, 0>(tm, T, B, tid, Fp);
+    } else {
+        C<R>* E = tm.buf[3];
+        plain_contract<CHI, D, R, RC, 0, false, true>(tm, A, T, tid, team);    // L_1
+        plain_contract<CHI, D, R, RC, 3, true, true>(tm, B, T, tid, team);     // R_2
+        plain_contract<CHI, D, R, RC, 2, true, false>(tm, E, B, tid, team);    // R_1
+        plain_overlap<CHI, D, R, RC, 1>(tm, A, E, tid, Fp);
+        team_bar<NT>(team);
+        plain_contract<CHI, D, R, RC, 1, false, false>(tm, A, A, tid, team);   // L_2
+        plain_contract<CHI, D, R, RC, 1, true, false>(tm, E, E, tid, team);    // R_0
+        plain_overlap<CHI, D, R, RC, 2>(tm, A, B, tid, Fp);
+        plain_overlap<CHI, D, R, RC, 0>(tm, T, E, tid, Fp);
+        team_bar<NT>(team);
+        plain_contract<CHI, D, R, RC, 2, false, false>(tm, A, A, tid, team);   // L_3
+        plain_overlap<CHI, D, R, RC, 3>(tm, A, T, tid, Fp);
+    }
+}
+
+// (B): message o from its two halves; returns the Frobenius norm of new - old
+template <int CHI, typename R, typename RC>
+__device__ RC plain_bp_finish(const PlainBPArgs& a, int o, int cur, int lane) {
+    constexpr int CC = CHI * CHI, NE = (CC + 31) / 32;
+    constexpr bool MIX = sizeof(R) != sizeof(RC);
+    const C<R>* F0 = (const C<R>*)a.Fp + (size_t)o * CC;
+    const C<R>* F1 = F0 + (size_t)2 * a.p.m * CC;
+    const C<R>* old = (const C<R>*)a.p.msg[cur] + (size_t)o * CC;
+    C<R>* dst = (C<R>*)a.p.msg[cur ^ 1] + (size_t)o * CC;
+    C<RC> f[NE];
+    RC tr[3] = {(RC)0, (RC)0, (RC)0};   // trace, and sum(lambda)
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+        const int r = lane + 32 * q;
+        f[q] = C<RC>{(RC)0, (RC)0};
+        if (r < CC) {
+            f[q] = ccast<RC>(ldcg(F0 + r)) + ccast<RC>(ldcg(F1 + r));
+            if (r / CHI == r % CHI) {
+                tr[0] += f[q].x;
+                tr[1] += f[q].y;
+            }
         }
     }
-    __syncthreads();
+    RC lam = (RC)0;
     if constexpr (MIX) {
-        // F(m0 + delta) - F(m0) telescoped over the other slots o_1 < o_2 < ...: chain c takes
-        // m0 on the slots before its own, delta on its own and m after it (FP32 contractions);
-        // then delta' = (D0 + F_delta - m0 tr F_delta) / (t0 + tr F_delta) in RC
-        for (int s = 0; s < D; ++s) {
-            if (es[s] < 0) continue;   // uniform: es is shared
-            const int ss = ipow(CHI, D - 1 - s);
-            constexpr int NTERM = H2 / CHI;
-            for (int c = 0; c < D - 1; ++c) {
-                const C<R>* src = T;
-                C<R>* dst = P0;
-                int i = 0;
-                for (int o = 0; o < D; ++o) {
-                    if (o == s) continue;
-                    const C<R>* mo = (i < c ? mz : (i == c ? md : min)) + o * CC;
-                    ++i;
-                    const int so = ipow(CHI, D - 1 - o);
-                    for (int t = tid; t < H2; t += NT) {
-                        const int x = (t / so) % CHI, base = t - x * so;
-                        C<R> acc = C<R>{(R)0, (R)0};
-#pragma unroll 4
-                        for (int q = 0; q < CHI; ++q) acc = cfma(src[base + q * so], mo[q * CHI + x], acc);
-                        dst[t] = acc;
-                    }
-                    __syncthreads();
-                    src = dst;
-                    dst = (dst == P0) ? P1 : P0;
-                }
-                for (int rr = tid / TPO; rr < CC; rr += NT / TPO) {
-                    const int part = tid % TPO;
-                    const int j = rr / CHI, jp = rr % CHI;
-                    C<R> f = C<R>{(R)0, (R)0};
-                    for (int q = part; q < NTERM; q += TPO) {
-                        const int t = (q / ss) * (ss * CHI) + (q % ss);
-                        f = cfmac(T[t + jp * ss], src[t + j * ss], f);
-                    }
-                    f.x = group_sum<TPO>(f.x, group_mask<TPO>());
-                    f.y = group_sum<TPO>(f.y, group_mask<TPO>());
-                    if (part == 0) F[rr] = c == 0 ? f : F[rr] + f;
-                }
-                __syncthreads();
-            }
-            const int out = out_idx[s];
-            if (tid == 0) {
-                C<RC> tr = C<RC>{(RC)0, (RC)0};
-                for (int q = 0; q < CHI; ++q) tr = tr + ccast<RC>(F[q * CHI + q]);
-                tau = tr;
-                const C<RC> den = a.t0[out] + tr;
-                const RC d = den.x * den.x + den.y * den.y;
-                itr = d > 0.0 ? C<RC>{den.x / d, -den.y / d} : C<RC>{(RC)0, (RC)0};
-            }
-            __syncthreads();
-            for (int r = tid; r < CC; r += NT) {
-                const int j = r / CHI, jp = r % CHI;
-                C<RC> num = ccast<RC>(((const C<R>*)a.D0)[(size_t)out * CC + r]) + ccast<RC>(F[r]);
-                if (j == jp) num = num - m0d[s][j] * tau;
-                const C<RC> dn = num * itr;
-                const C<RC> dold = ccast<RC>(src_msg[(size_t)out * CC + r]);
-                dst_msg[(size_t)out * CC + r] = ccast<R>(dn);
-                ((C<R>*)a.dm)[(size_t)out * CC + r] = ccast<R>(dn - dold);
-            }
-            __syncthreads();
-        }
-        return;
+        if (lane < CHI) lam = __ldcg(a.p.lam + (size_t)(o >> 1) * CHI + lane);
+        tr[2] = lam;
     }
-    for (int s = 0; s < D; ++s) {
-        if (es[s] < 0) continue;   // uniform: es is shared
-        const C<R>* src = T;
-        C<R>* dst = P0;
-        for (int o = 0; o < D; ++o) {
-            if (o == s) continue;
-            const int so = ipow(CHI, D - 1 - o);
-            for (int t = tid; t < H2; t += NT) {
-                const int x = (t / so) % CHI, base = t - x * so;
-                C<R> acc = C<R>{(R)0, (R)0};
-#pragma unroll 4
-                for (int q = 0; q < CHI; ++q) acc = cfma(src[base + q * so], min[o * CC + q * CHI + x], acc);
-                dst[t] = acc;
+    group_sums<32>(tr, 0xffffffffu);
+    C<RC> den = C<RC>{tr[0], tr[1]};
+    if constexpr (MIX) den = den + ldcg(a.p.t0 + o);
+    const RC n2 = norm2(den);
+    const RC in = n2 > (RC)0 ? nr_rcp(n2) : (RC)0;
+    const C<RC> itr = C<RC>{den.x * in, -den.y * in};
+    const RC m0 = MIX && tr[2] > (RC)0 ? lam * nr_rcp(tr[2]) : (RC)0;   // lane j: m0_j
+    RC d2 = (RC)0;
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+        const int r = lane + 32 * q, j = r / CHI, jp = r % CHI;
+        C<RC> num = f[q];
+        if constexpr (MIX) {
+            const RC z = __shfl_sync(0xffffffffu, m0, j & 31);
+            if (r < CC) {
+                num = num + ccast<RC>(ldcg((const C<R>*)a.p.D0 + (size_t)o * CC + r));
+                if (j == jp) num = num - z * C<RC>{tr[0], tr[1]};
             }
-            __syncthreads();
-            src = dst;
-            dst = (dst == P0) ? P1 : P0;
         }
-        // F[j][j'] = sum over the entries with slot-s index j of conj(T[.. j' ..]) src[.. j ..]
-        const int ss = ipow(CHI, D - 1 - s);
-        constexpr int NTERM = H2 / CHI;
-        for (int rr = tid / TPO; rr < CC; rr += NT / TPO) {
-            const int part = tid % TPO;
-            const int j = rr / CHI, jp = rr % CHI;
-            C<R> f = C<R>{(R)0, (R)0};
-            for (int q = part; q < NTERM; q += TPO) {
-                const int t = (q / ss) * (ss * CHI) + (q % ss);
-                f = cfmac(T[t + jp * ss], src[t + j * ss], f);
+        if (r < CC) {
+            const C<RC> nv = num * itr;
+            const C<RC> d = nv - ccast<RC>(ldcg(old + r));
+            dst[r] = ccast<R>(nv);
+            ((C<R>*)a.p.dm)[(size_t)o * CC + r] = ccast<R>(d);
+            d2 += norm2(d);
+        }
+    }
+    d2 = group_sum<32>(d2, 0xffffffffu);
+    return nr_sqrt(d2);
+}
+
+// (C): trace norm of new - old of message o (group of CC / 2 lanes)
+template <int CHI, typename R, typename RC, typename Group>
+__device__ RC plain_trace_norm(const C<R>* dm, unsigned char* base, int g, const Group& grp) {
+    constexpr int CC = CHI * CHI, GL = CC / 2;
+    C<RC>* A = reinterpret_cast<C<RC>*>(base);
+    for (int t = g; t < CC; t += GL) A[t] = ccast<RC>(ldcg(dm + t));
+    grp.sync();
+    RC s = (RC)0;
+    if constexpr (sizeof(RC) == 8) {
+        cd* V = A + CC;
+        cd* T = V + CC;
+        cf* A32 = reinterpret_cast<cf*>(T + CC);
+        double* nrm = reinterpret_cast<double*>(A32 + 2 * CC);
+        prune_noise<CHI>(A, g, grp);
+        refined_svd<CHI, true>(A, V, A32, A32 + CC, T, nrm, nullptr, g, grp, group_mask<CHI>(), 1e-16, CHI, 1e-8f, 1e-15);
+        if (g == 0)
+            for (int q = 0; q < CHI; ++q) s += nr_sqrt(nrm[q]);
+    } else {
+        jacobi_svd<CHI, RC, Group, false>(A, nullptr, g, grp, group_mask<CHI>(), (RC)1e-6, 60, false);
+        grp.sync();
+        if (g == 0)
+            for (int q = 0; q < CHI; ++q) {
+                RC n2 = (RC)0;
+                for (int r = 0; r < CHI; ++r) n2 += norm2(A[q * CHI + r]);
+                s += nr_sqrt(n2);
             }
-            f.x = group_sum<TPO>(f.x, group_mask<TPO>());
-            f.y = group_sum<TPO>(f.y, group_mask<TPO>());
-            if (part == 0) F[rr] = f;
+    }
+    grp.sync();
+    return s;
+}
+
+template <int CHI, int D, typename R, typename RC>
+__global__ void __launch_bounds__(512, 1) plain_bp_kernel(PlainBPArgs a) {
+    using S = PlainShape<CHI, D, R, RC>;
+    constexpr int CC = S::CC, NT = S::NT, GL = S::GL;
+    extern __shared__ __align__(16) unsigned char plain_smem[];
+    __shared__ double bsum;
+    __shared__ int flags[8];
+    Control* ctl = a.p.ctl;
+    GridBarrier gb = grid_barrier_init(a.bar, &ctl->err, (unsigned)a.bar_expect);
+    int cur = *(volatile int*)&ctl->cur;
+    const int team = threadIdx.x / NT, tid = threadIdx.x % NT;
+    const PlainTeam<CHI, D, R, RC> tm(plain_smem + team * ((S::team_smem + 15) / 16 * 16));
+    const double E = (double)a.p.m, slack = sizeof(R) == 4 ? 1e-5 : 1e-12;
+    const double go = a.tol * E / (1.0 - slack);   // a bound at least this large cannot stop
+    double dist = 0.0;
+    bool conv = false;
+    int it = 0;
+    // the accumulators of sweep `it` are zeroed two barriers ahead (those of the first sweeps by the host)
+    while (it < a.max_iter) {
+        double* acc = a.acc + it % 3;
+        double* ex = a.acc + 3 + it % 3;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            a.acc[(it + 1) % 3] = 0.0;
+            a.acc[3 + (it + 1) % 3] = 0.0;
+        }
+        for (int item = team * a.nblocks + blockIdx.x; item < 2 * a.p.n; item += a.nblocks * S::TEAMS)
+            plain_bp_item<CHI, D, R, RC>(a, item, cur, tid, team, tm);
+        if (!grid_sync(gb, a.spin_limit)) return;
+        if (threadIdx.x == 0) bsum = 0.0;
+        __syncthreads();
+        double mine = 0.0;
+        for (int o = (threadIdx.x / 32) * a.nblocks + blockIdx.x; o < 2 * a.p.m; o += a.nblocks * (S::TPB / 32))
+            mine += (double)plain_bp_finish<CHI, R, RC>(a, o, cur, threadIdx.x & 31);
+        if ((threadIdx.x & 31) == 0 && mine != 0.0) atomicAdd(&bsum, mine);
+        __syncthreads();
+        if (threadIdx.x == 0 && bsum != 0.0) atomicAdd(acc, bsum);
+        if (!grid_sync(gb, a.spin_limit)) return;
+        cur ^= 1;
+        ++it;
+        const bool last = it >= a.max_iter;
+        const double bound = __ldcg(acc);
+        if (!(bound == bound)) {
+            dist = bound;
+            break;
+        }
+        if (!last && a.p.m > 0 && bound >= go) continue;
+        if (threadIdx.x == 0) bsum = 0.0;
+        __syncthreads();
+        const int gi = threadIdx.x / GL, g = threadIdx.x % GL;
+        if (gi < S::GROUPS) {
+            unsigned char* base = plain_smem + gi * ((S::group_smem + 15) / 16 * 16);
+            double t = 0.0;
+            for (int o = gi * a.nblocks + blockIdx.x; o < 2 * a.p.m; o += a.nblocks * S::GROUPS) {
+                const C<R>* dm = (const C<R>*)a.p.dm + (size_t)o * CC;
+                if constexpr (GL <= 32) t += (double)plain_trace_norm<CHI, R, RC>(dm, base, g, WarpGroup{group_mask<GL>()});
+                else t += (double)plain_trace_norm<CHI, R, RC>(dm, base, g, TeamGroup<GL>{gi, &flags[gi]});
+            }
+            if (g == 0 && t != 0.0) atomicAdd(&bsum, t);
         }
         __syncthreads();
-        if (tid == 0) {
-            C<RC> tr = C<RC>{(RC)0, (RC)0};
-            for (int q = 0; q < CHI; ++q) tr = tr + ccast<RC>(F[q * CHI + q]);
-            const RC d = tr.x * tr.x + tr.y * tr.y;
-            itr = d > 0.0 ? C<RC>{tr.x / d, -tr.y / d} : C<RC>{(RC)0, (RC)0};
+        if (threadIdx.x == 0 && bsum != 0.0) atomicAdd(ex, bsum);
+        if (blockIdx.x == 0 && threadIdx.x == 0) ++ctl->exact_passes;
+        if (!grid_sync(gb, a.spin_limit)) return;
+        dist = a.p.m > 0 ? __ldcg(ex) / E : 0.0;
+        if (!(dist == dist)) break;
+        if (dist < a.tol) {
+            conv = true;
+            break;
         }
-        __syncthreads();
-        for (int r = tid; r < CC; r += NT) {
-            const C<RC> mn = ccast<RC>(F[r]) * itr;
-            const C<RC> mo = ccast<RC>(src_msg[(size_t)out_idx[s] * CC + r]);
-            dst_msg[(size_t)out_idx[s] * CC + r] = ccast<R>(mn);
-            ((C<R>*)a.dm)[(size_t)out_idx[s] * CC + r] = ccast<R>(mn - mo);
-        }
-        __syncthreads();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (!(dist == dist)) ctl->err = 3;   // GTQA_ERR_NUMERIC
+        ctl->last_iters = it;
+        ctl->last_dist = dist;
+        ctl->not_conv = conv ? 0 : 1;
+        ctl->sweeps_total += it;
+        ctl->bp_calls += 1;
+        ctl->nc_calls += conv ? 0 : 1;
+        ctl->cur = cur;
     }
 }
 
-// Trace norm (sum of singular values, one-sided Jacobi in FP64) of every directed message's
-// new - old; block = CHI^2 / 2 threads, one message per block; the sum goes to *acc.
-template <int CHI, typename R, typename RC = R>
-__global__ void plain_trace_norm_kernel(const C<R>* dm, double* acc) {
-    constexpr int CC = CHI * CHI;
-    __shared__ C<RC> A[CC];
-    __shared__ RC tn;
-    __shared__ int flag;
-    const int g = threadIdx.x;
-    for (int t = g; t < CC; t += blockDim.x) A[t] = ccast<RC>(dm[(size_t)blockIdx.x * CC + t]);
-    if (g == 0) tn = 0.0;
-    __syncthreads();
-    BlockGroup grp{&flag};
-    jacobi_svd<CHI, RC, BlockGroup, false>(A, nullptr, g, grp, group_mask<CHI>(), (RC)(sizeof(RC) == 8 ? 1e-15 : 1e-6),
-                                           60, false);
-    __syncthreads();
-    if (g < CHI) {
-        RC c2 = 0.0;
-        for (int r = 0; r < CHI; ++r) c2 += norm2(A[g * CHI + r]);
-        atomicAdd(&tn, sqrt(c2));
-    }
-    __syncthreads();
-    if (g == 0) atomicAdd(acc, tn);
-}
-
-// Vidal gauge finding, edge part (App. D "Vidal gauge finding"), FP64, block = CHI^2 / 2
-// threads: Hermitian eigen-decompositions of m_{a->b} and m_{b->a} (as SVDs; signs from
-// v^H A v), principal square roots and pseudo-inverse square roots, the SVD of
+// Vidal gauge finding, edge part (App. D "Vidal gauge finding"), block = CHI^2 threads:
+// Hermitian eigen-decompositions of m_{a->b} and m_{b->a} (as SVDs, each by half of the block; signs
+// from v^H A v), principal square roots and pseudo-inverse square roots, the SVD of
 // M = (m_{a->b}^{1/2})^T m_{b->a}^{1/2}, lambda = S/||S||, X_a = conj(m_{a->b}^{-1/2}) U ||S||^{1/2}
 // and X_b = conj(m_{b->a}^{-1/2}) V^* ||S||^{1/2}.
+template <int CHI, typename RC>
+struct PlainEdgeSm {
+    static constexpr int CC = CHI * CHI;
+    C<RC> Am[2][CC], Vm[2][CC], sqm[2][CC], isq[2][CC], M[CC], VM[CC];
+    C<RC> T[2][sizeof(RC) == 8 ? CC : 1];
+    cf A32[2][sizeof(RC) == 8 ? CC : 1], V32[2][sizeof(RC) == 8 ? CC : 1];
+    double n2[2][CHI];
+    RC w[2][CHI], wq[2][CHI], wiq[2][CHI], sig[CHI], isig[CHI], m0[CHI], scal[2];
+    int perm[CHI], flag[2];
+};
+template <int CHI, typename RC, typename Group>
+__device__ __forceinline__ void plain_edge_svd(C<RC>* A, C<RC>* V, PlainEdgeSm<CHI, RC>& sm, int x, int g,
+                                               const Group& grp, double cut) {
+    if constexpr (sizeof(RC) == 8) {
+        prune_noise<CHI>(A, g, grp);
+        refined_svd<CHI, true>(A, V, sm.A32[x], sm.V32[x], sm.T[x], sm.n2[x], nullptr, g, grp, group_mask<CHI>(), cut, CHI,
+                               1e-8f, 1e-15);
+    } else {
+        jacobi_svd<CHI, RC>(A, V, g, grp, group_mask<CHI>(), (RC)1e-6, 60, true, nullptr, (RC)1e-3);
+    }
+}
 template <int CHI, typename R, typename RC = R>
-__global__ void plain_regauge_edge_kernel(const C<R>* msg, double* lam, C<R>* X, double eig_cut, double svd_cut) {
-    constexpr int CC = CHI * CHI;
-    __shared__ C<RC> Am[2][CC], Vm[2][CC], sqm[2][CC], isq[2][CC], M[CC], VM[CC];
-    __shared__ RC w[2][CHI], sig[CHI], scal[2];
-    __shared__ int perm[CHI], flag;
-    const int e = blockIdx.x, tid = threadIdx.x, NT = blockDim.x;
-    BlockGroup grp{&flag};
+__global__ void __launch_bounds__(CHI * CHI) plain_regauge_edge_kernel(PlainArgs a, double eig_cut, double svd_cut) {
+    constexpr int CC = CHI * CHI, GL = CC / 2, NT = CC;
+    constexpr bool MIX = sizeof(R) != sizeof(RC);
+    extern __shared__ __align__(16) unsigned char plain_smem[];
+    PlainEdgeSm<CHI, RC>& sm = *reinterpret_cast<PlainEdgeSm<CHI, RC>*>(plain_smem);
+    const int e = blockIdx.x, tid = threadIdx.x;
+    auto bar = [&]() {
+        if constexpr (NT < 32) __syncwarp(group_mask<NT>());
+        else __syncthreads();
+    };
+    auto half_svd = [&](C<RC>* A, C<RC>* V, int x, int g, double cut) {
+        if constexpr (GL <= 32) plain_edge_svd<CHI, RC>(A, V, sm, x, g, WarpGroup{group_mask<GL>()}, cut);
+        else plain_edge_svd<CHI, RC>(A, V, sm, x, g, TeamGroup<GL>{x, &sm.flag[x]}, cut);
+    };
+    const C<R>* msg = (const C<R>*)a.msg[a.ctl->cur];
     // mixed mode: the messages hold delta = m - m0, m0 = diag(lambda_e)/sum(lambda_e) (read before
     // this kernel overwrites lambda_e)
-    constexpr bool MIX = sizeof(R) != sizeof(RC);
-    __shared__ RC m0e[CHI];
     if (MIX && tid < CHI) {
         RC sum = 0.0;
-        for (int q = 0; q < CHI; ++q) sum += lam[(size_t)e * CHI + q];
-        m0e[tid] = sum > 0.0 ? lam[(size_t)e * CHI + tid] / sum : 0.0;
+        for (int q = 0; q < CHI; ++q) sum += a.lam[(size_t)e * CHI + q];
+        sm.m0[tid] = sum > 0.0 ? a.lam[(size_t)e * CHI + tid] / sum : 0.0;
     }
-    if (MIX) __syncthreads();
+    if (MIX) bar();
     for (int t = tid; t < 2 * CC; t += NT) {
         const int x = t / CC, r = t % CC;
         const int row = r % CHI, col = r / CHI;
         const C<R>* mm = msg + (size_t)(2 * e + x) * CC;
         C<RC> v = ccast<RC>(mm[row * CHI + col]), vt = ccast<RC>(mm[col * CHI + row]);
         if (MIX && row == col) {
-            v.x += m0e[row];
-            vt.x += m0e[row];
+            v.x += sm.m0[row];
+            vt.x += sm.m0[row];
         }
-        Am[x][col * CHI + row] = C<RC>{(RC)0.5 * (v.x + vt.x), (RC)0.5 * (v.y - vt.y)};
+        sm.Am[x][col * CHI + row] = C<RC>{(RC)0.5 * (v.x + vt.x), (RC)0.5 * (v.y - vt.y)};
     }
-    __syncthreads();
-    for (int x = 0; x < 2; ++x)
-        jacobi_svd<CHI, RC, BlockGroup, true, sizeof(RC) == 8>(Am[x], Vm[x], tid, grp, group_mask<CHI>(),
-                                                                  (RC)(sizeof(RC) == 8 ? 1e-15 : 1e-6), 60, true, nullptr,
-                                                                  (RC)(sizeof(RC) == 8 ? 3e-8 : 1e-3));
-    __syncthreads();
+    bar();
+    half_svd(sm.Am[tid / GL], sm.Vm[tid / GL], tid / GL, tid % GL, eig_cut);
+    bar();
     for (int t = tid; t < 2 * CHI; t += NT) {
         const int x = t / CHI, k = t % CHI;
         RC n2 = 0.0, sg = 0.0;
         for (int r = 0; r < CHI; ++r) {
-            const C<RC> av = Am[x][k * CHI + r], vv = Vm[x][k * CHI + r];
+            const C<RC> av = sm.Am[x][k * CHI + r], vv = sm.Vm[x][k * CHI + r];
             n2 += norm2(av);
             sg += vv.x * av.x + vv.y * av.y;
         }
         const RC wv = nr_sqrt(n2);
-        w[x][k] = sg >= 0.0 ? wv : -wv;
+        sm.w[x][k] = sg >= 0.0 ? wv : -wv;
     }
-    __syncthreads();
+    bar();
+    for (int t = tid; t < 2 * CHI; t += NT) {   // the roots of each kept eigenvalue once
+        const int x = t / CHI, k = t % CHI;
+        RC wmax = 0.0;
+        for (int q = 0; q < CHI; ++q) wmax = fmax(wmax, sm.w[x][q]);
+        const RC wk = sm.w[x][k];
+        const RC is = wk > eig_cut * wmax ? nr_rsqrt(wk) : (RC)0;
+        sm.wiq[x][k] = is;
+        sm.wq[x][k] = is > (RC)0 ? wk * is : (RC)0;
+    }
+    bar();
     for (int t = tid; t < 2 * CC; t += NT) {
         const int x = t / CC, r = t % CC;
         const int j = r / CHI, jp = r % CHI;
-        RC wmax = 0.0;
-        for (int k = 0; k < CHI; ++k) wmax = fmax(wmax, w[x][k]);
         C<RC> s1 = C<RC>{(RC)0, (RC)0}, s2 = C<RC>{(RC)0, (RC)0};
         for (int k = 0; k < CHI; ++k) {
-            const RC wk = w[x][k];
-            if (!(wk > eig_cut * wmax)) continue;
-            const RC is = nr_rsqrt(wk);
-            const RC sq = wk * is;
-            const C<RC> vv = Vm[x][k * CHI + j] * conj(Vm[x][k * CHI + jp]);
-            s1 = cfma(C<RC>{sq, (RC)0}, vv, s1);
-            s2 = cfma(C<RC>{is, (RC)0}, vv, s2);
+            const RC is = sm.wiq[x][k];
+            if (!(is > (RC)0)) continue;
+            const RC sq = sm.wq[x][k];
+            const C<RC> vv = sm.Vm[x][k * CHI + j] * conj(sm.Vm[x][k * CHI + jp]);
+            s1.x = fma(sq, vv.x, s1.x);
+            s1.y = fma(sq, vv.y, s1.y);
+            s2.x = fma(is, vv.x, s2.x);
+            s2.y = fma(is, vv.y, s2.y);
         }
-        sqm[x][r] = s1;
-        isq[x][r] = s2;
+        sm.sqm[x][r] = s1;
+        sm.isq[x][r] = s2;
     }
-    __syncthreads();
+    bar();
     for (int t = tid; t < CC; t += NT) {
         const int k = t % CHI, l = t / CHI;
         C<RC> acc = C<RC>{(RC)0, (RC)0};
-        for (int j = 0; j < CHI; ++j) acc = cfma(sqm[0][j * CHI + k], sqm[1][j * CHI + l], acc);
-        M[l * CHI + k] = acc;
+        for (int j = 0; j < CHI; ++j) acc = cfma(sm.sqm[0][j * CHI + k], sm.sqm[1][j * CHI + l], acc);
+        sm.M[l * CHI + k] = acc;
     }
-    __syncthreads();
-    jacobi_svd<CHI, RC, BlockGroup, true, sizeof(RC) == 8>(M, VM, tid, grp, group_mask<CHI>(),
-                                                         (RC)(sizeof(RC) == 8 ? 1e-15 : 1e-6), 60, true, nullptr,
-                                                         (RC)(sizeof(RC) == 8 ? 3e-8 : 1e-3));
-    __syncthreads();
+    bar();
+    if (tid < GL) half_svd(sm.M, sm.VM, 0, tid, svd_cut);
+    bar();
     for (int cc = tid; cc < CHI; cc += NT) {
         RC n2 = 0.0;
-        for (int r = 0; r < CHI; ++r) n2 += norm2(M[cc * CHI + r]);
-        sig[cc] = nr_sqrt(n2);
+        for (int r = 0; r < CHI; ++r) n2 += norm2(sm.M[cc * CHI + r]);
+        const RC sv = nr_sqrt(n2);
+        sm.sig[cc] = sv;
+        sm.isig[cc] = sv > (RC)0 ? nr_rcp(sv) : (RC)0;
     }
-    __syncthreads();
-    for (int cc = tid; cc < CHI; cc += NT) perm[desc_rank(sig, CHI, cc)] = cc;
-    __syncthreads();
+    bar();
+    for (int cc = tid; cc < CHI; cc += NT) sm.perm[desc_rank(sm.sig, CHI, cc)] = cc;
+    bar();
     if (tid == 0) {
         RC tot = 0.0;
-        for (int cc = 0; cc < CHI; ++cc) tot += sig[cc] * sig[cc];
+        for (int cc = 0; cc < CHI; ++cc) tot += sm.sig[cc] * sm.sig[cc];
         const RC nrm = nr_sqrt(tot);
-        scal[0] = nrm;
-        scal[1] = nr_sqrt(nrm);
+        sm.scal[0] = nrm;
+        sm.scal[1] = nr_sqrt(nrm);
         const RC inrm = nrm > 0.0 ? nr_rcp(nrm) : 0.0;
-        const RC smax = sig[perm[0]];
+        const RC smax = sm.sig[sm.perm[0]];
         for (int r = 0; r < CHI; ++r) {
-            const RC s = sig[perm[r]];
-            lam[(size_t)e * CHI + r] = (nrm > 0.0 && s > svd_cut * smax) ? s * inrm : 0.0;
+            const RC s = sm.sig[sm.perm[r]];
+            a.lam[(size_t)e * CHI + r] = (nrm > 0.0 && s > svd_cut * smax) ? s * inrm : 0.0;
         }
     }
-    __syncthreads();
+    bar();
     for (int t = tid; t < 2 * CC; t += NT) {
         const int x = t / CC, r = t % CC;
         const int jpp = r / CHI, j = r % CHI;
-        const int pc = perm[j];
-        const RC s = sig[pc];
+        const int pc = sm.perm[j];
         C<RC> acc = C<RC>{(RC)0, (RC)0};
-        const bool kept = scal[0] > 0.0 && s > svd_cut * sig[perm[0]];
-        if (kept) {
+        if (sm.scal[0] > 0.0 && sm.sig[pc] > svd_cut * sm.sig[sm.perm[0]]) {
             for (int jp = 0; jp < CHI; ++jp) {
-                const C<RC> u = (x == 0) ? nr_rcp(s) * M[pc * CHI + jp] : conj(VM[pc * CHI + jp]);
-                acc = cfma(isq[x][jp * CHI + jpp], u, acc);
+                const C<RC> u = (x == 0) ? sm.isig[pc] * sm.M[pc * CHI + jp] : conj(sm.VM[pc * CHI + jp]);
+                acc = cfma(sm.isq[x][jp * CHI + jpp], u, acc);
             }
-            acc = scal[1] * acc;
+            acc = sm.scal[1] * acc;
         }
-        X[((size_t)e * 2 + x) * CC + r] = ccast<R>(acc);
+        ((C<R>*)a.X)[((size_t)e * 2 + x) * CC + r] = ccast<R>(acc);
     }
 }
 
 // Vidal gauge finding, vertex part: Gamma[.., j@k, ..] = sum_q T[.., q@k, ..] X_k[q][j] for every
-// slot (X of the edge, from this vertex's side; identity on phantom slots).
-template <int CHI, int D, typename R>
-__global__ void plain_regauge_vertex_kernel(PlainArgs a) {
-    using S = PlainShape<CHI, D, R>;
-    constexpr int H2 = S::H2, CC = S::CC;
-    extern __shared__ __align__(16) unsigned char plain_smem[];
-    C<R>* Xs = reinterpret_cast<C<R>*>(plain_smem);   // [D][CC]
-    C<R>* b0;
-    C<R>* b1;
-    if constexpr (S::SMEM) {
-        b0 = Xs + D * CC;
-        b1 = b0 + H2;
-    } else {
-        b0 = (C<R>*)a.scratch + (size_t)blockIdx.x * S::scratch_per_block;
-        b1 = b0 + H2;
-    }
-    const int v = blockIdx.x;
-    const int4 sl = a.vslots[v];
-    for (int t = threadIdx.x; t < H2; t += blockDim.x) b0[t] = ((const C<R>*)a.T)[(size_t)v * H2 + t];
-    for (int t = threadIdx.x; t < D * CC; t += blockDim.x) {
-        const int k = t / CC, r = t % CC;
-        const int e = plain_slot_edge(sl, k);
-        if (e >= 0) {
+// slot (X of the edge, from this vertex's side; identity on phantom slots).  One block per (vertex,
+// physical index); a lane contracts (part of) a fiber in place.
+template <int CHI, int D, typename R, int K>
+__device__ __forceinline__ void plain_regauge_slot(C<R>* buf, C<R>* Xs, const PlainArgs& a, const int4& sl, int v, int tid) {
+    if constexpr (K < D) {
+        using S = PlainShape<CHI, D, R, R>;
+        constexpr int ST = ipow(CHI, D - 1 - K), NP = CHI / S::XO, CC = S::CC, NT = S::NT;
+        const int e = plain_slot_edge(sl, K);
+        if (e >= 0) {   // the same for the block
             const int side = a.edge_info[e].x == v ? 0 : 1;
-            Xs[t] = ((const C<R>*)a.X)[((size_t)e * 2 + side) * CC + r];
-        } else {
-            Xs[t] = C<R>{(R)((r / CHI == r % CHI) ? 1 : 0), (R)0};
+            for (int t = tid; t < CC; t += NT) Xs[t] = ((const C<R>*)a.X)[((size_t)e * 2 + side) * CC + t];
+            const int fib = tid / NP, part = tid % NP, base = (fib / ST) * ST * CHI + fib % ST;
+            C<R> in[CHI];
+            bool any = false;
+            if (tid < S::ITEMS) {
+#pragma unroll
+                for (int q = 0; q < CHI; ++q) {
+                    const int r = base + q * ST;
+                    in[q] = buf[r + r / CC];
+                    any |= in[q].x != (R)0 || in[q].y != (R)0;
+                }
+            }
+            __syncthreads();
+            if (any)   // a fiber of zeros stays one (indices beyond the bonds' dimensions)
+                for (int xo = 0; xo < S::XO; ++xo) {
+                    const int x = part * S::XO + xo;
+                    C<R> acc = C<R>{(R)0, (R)0};
+#pragma unroll
+                    for (int q = 0; q < CHI; ++q) acc = cfma(in[q], Xs[q * CHI + x], acc);
+                    const int r = base + x * ST;
+                    buf[r + r / CC] = acc;
+                }
+            __syncthreads();
         }
+        plain_regauge_slot<CHI, D, R, K + 1>(buf, Xs, a, sl, v, tid);
     }
+}
+template <int CHI, int D, typename R>
+__global__ void __launch_bounds__(PlainShape<CHI, D, R, R>::NT) plain_regauge_vertex_kernel(PlainArgs a) {
+    using S = PlainShape<CHI, D, R, R>;
+    constexpr int CC = S::CC, NT = S::NT;
+    extern __shared__ __align__(16) unsigned char plain_smem[];
+    C<R>* buf = reinterpret_cast<C<R>*>(plain_smem);
+    C<R>* Xs = buf + S::PH;
+    const int v = blockIdx.x >> 1;
+    const int4 sl = a.vslots[v];
+    const C<R>* T = (const C<R>*)a.T + (size_t)blockIdx.x * S::H;
+    for (int t = threadIdx.x; t < S::H; t += NT) buf[t + t / CC] = T[t];
     __syncthreads();
-    C<R>* cur = b0;
-    C<R>* nxt = b1;
-    for (int k = 0; k < D; ++k) {
-        const int st = ipow(CHI, D - 1 - k);
-        for (int t = threadIdx.x; t < H2; t += blockDim.x) {
-            const int jk = (t / st) % CHI, base = t - jk * st;
-            C<R> acc = C<R>{(R)0, (R)0};
-            for (int q = 0; q < CHI; ++q) acc = cfma(cur[base + q * st], Xs[k * CC + q * CHI + jk], acc);
-            nxt[t] = acc;
-        }
-        __syncthreads();
-        C<R>* tmp = cur;
-        cur = nxt;
-        nxt = tmp;
-    }
-    C<R>* g = (C<R>*)a.Gamma + (size_t)v * H2;
-    for (int t = threadIdx.x; t < H2; t += blockDim.x) g[t] = cur[t];
+    plain_regauge_slot<CHI, D, R, 0>(buf, Xs, a, sl, v, threadIdx.x);
+    C<R>* g = (C<R>*)a.Gamma + (size_t)blockIdx.x * S::H;
+    for (int t = threadIdx.x; t < S::H; t += NT) g[t] = buf[t + t / CC];
 }
 
 // rho_a = sum_J Gamma[i, J] conj(Gamma[i', J]) prod_k lambda_k[j_k]^2 / trace (Eqs. (partial_dens),
