@@ -629,6 +629,40 @@ struct BPSm {
     int cached;          // vertex held in the cache, -1 if none
 };
 
+// Trace norm (sum of singular values) of the CHI x CHI matrix A (column-major, CHI^2/2 lanes; A is
+// overwritten), on lane 0.  FP64 through refined_svd with the scratch after A (trace_norm_bytes in
+// all): 9 us for a 4 x 4 matrix against 22 us for FP64 Jacobi sweeps without V.  FP32 by Jacobi.
+template <int CHI, typename TS>
+__host__ __device__ constexpr size_t trace_norm_bytes() {
+    return CHI * CHI * (sizeof(TS) == 8 ? 3 * sizeof(cd) + 2 * sizeof(cf) : sizeof(cf)) + CHI * sizeof(double);
+}
+template <int CHI, typename TS>
+__device__ __forceinline__ TS trace_norm(C<TS>* A, int g, const WarpGroup& grp) {
+    constexpr int CC = CHI * CHI;
+    TS s = (TS)0;
+    if constexpr (sizeof(TS) == 8) {
+        cd* V = A + CC;
+        cd* T = V + CC;
+        cf* A32 = reinterpret_cast<cf*>(T + CC);
+        double* nrm = reinterpret_cast<double*>(A32 + 2 * CC);
+        grp.sync();
+        prune_noise<CHI>(A, g, grp);
+        refined_svd<CHI, true>(A, V, A32, A32 + CC, T, nrm, nullptr, g, grp, group_mask<CHI>(), 1e-16, CHI, 1e-8f, 1e-15);
+        if (g == 0)
+            for (int q = 0; q < CHI; ++q) s += nr_sqrt(nrm[q]);
+    } else {
+        jacobi_svd<CHI, TS, WarpGroup, false, false>(A, nullptr, g, grp, group_mask<CHI>(), (TS)1e-6, 60, false, nullptr,
+                                                     (TS)1e-3);
+        if (g == 0)
+            for (int cc = 0; cc < CHI; ++cc) {
+                TS n2 = (TS)0;
+                for (int r = 0; r < CHI; ++r) n2 += norm2(A[cc * CHI + r]);
+                s += nr_sqrt(n2);
+            }
+    }
+    return s;
+}
+
 template <int CHI, class Mode, int TB>
 __device__ void bp_prepare(const Ctx& c, int a, int tid, int team, int cur, BPSm<CHI, Mode, TB>& sm) {
     using TS = typename Mode::TS;
@@ -951,18 +985,14 @@ __device__ void bp_back(const Ctx& c, int tid, int team, int cur, bool exact, BP
     } else if (tid < 3 * GJ) {
         const int k = tid / GJ, g = tid % GJ;
         WarpGroup grp{group_mask<GJ>()};
-        jacobi_svd<CHI, TS, WarpGroup, false, !Mode::mixed>(sm.D[k], nullptr, g, grp, group_mask<CHI>(),
-                                                             Mode::mixed ? (TS)1e-6 : (TS)1e-15, 60, false, nullptr,
-                                                             Mode::mixed ? (TS)1e-3 : (TS)3e-8);
-        if (g == 0) {
-            TS sacc = (TS)0;
-            for (int cc = 0; cc < CHI; ++cc) {
-                TS n2 = (TS)0;
-                for (int r = 0; r < CHI; ++r) n2 += norm2(sm.D[k][cc * CHI + r]);
-                sacc += nr_sqrt(n2);
-            }
-            sm.dl[k] = sacc;
+        CT* A = sm.D[k];
+        if constexpr (!Mode::mixed) {   // with its scratch in P and Q, which are free here
+            static_assert(3 * trace_norm_bytes<CHI, TS>() <= sizeof(sm.P) + sizeof(sm.Q), "scratch of the trace norms");
+            A = reinterpret_cast<CT*>(reinterpret_cast<unsigned char*>(sm.P) + k * trace_norm_bytes<CHI, TS>());
+            for (int r = g; r < CC; r += GJ) A[r] = sm.D[k][r];
         }
+        const TS sacc = trace_norm<CHI, TS>(A, g, grp);
+        if (g == 0) sm.dl[k] = sacc;
     }
     team_bar<TEAM>(team);
     if (gacc) {
@@ -992,34 +1022,30 @@ __device__ void bp_copy_vertex(const Ctx& c, int a, int tid, int TEAM, int cur) 
 // Exact distance of the sweep that wrote msg[cur_new] for the instances with need[b]
 // set: trace norms of new - old for every directed message, one group of CHI^2/2
 // threads per message (whole block, after a grid barrier).  Accumulates into ex[b].
-template <int CHI, class Mode, int TPB>
-__device__ void bp_exact_pass(const Ctx& c, int cur_new, const int* need, C<typename Mode::TS>* scratch,
-                              double* bacc, double* ex) {
+template <int CHI, class Mode, int TPB, int TB>
+__device__ void bp_exact_pass(const Ctx& c, int cur_new, const int* need, BPSm<CHI, Mode, TB>& sm, double* bacc,
+                              double* ex) {
     using TS = typename Mode::TS;
     using CT = C<TS>;
-    constexpr int CC = CHI * CHI, GJ = CC / 2, NG = TPB / GJ;
-    const int gi = threadIdx.x / GJ, g = threadIdx.x % GJ;
-    CT* Dm = scratch + gi * CC;
+    // the groups of a team have their matrices and scratch in its P and Q buffers
+    constexpr int CC = CHI * CHI, GJ = CC / 2, FIT = (int)((sizeof(sm.P) + sizeof(sm.Q)) / trace_norm_bytes<CHI, TS>());
+    constexpr int NGT = TB / GJ < FIT ? TB / GJ : FIT, TEAMS = TPB / TB;
+    static_assert(NGT >= 1, "scratch of the trace norms");
+    const int team = threadIdx.x / TB, gi = (threadIdx.x % TB) / GJ, g = threadIdx.x % GJ;
+    CT* Dm = reinterpret_cast<CT*>(reinterpret_cast<unsigned char*>(sm.P) + (gi < NGT ? gi : 0) * trace_norm_bytes<CHI, TS>());
     const CT* nw = (const CT*)c.msg[cur_new];
     const CT* od = (const CT*)c.msg[cur_new ^ 1];
     if (threadIdx.x == 0) *bacc = 0.0;
     __syncthreads();
     const WarpGroup grp{group_mask<GJ>()};
     double mine = 0.0;
-    for (int mi = blockIdx.x * NG + gi; mi < 2 * c.m; mi += c.nblocks * NG) {
+    // consecutive messages go to different blocks, then to different teams
+    for (int mi = (gi * TEAMS + team) * c.nblocks + blockIdx.x; gi < NGT && mi < 2 * c.m; mi += c.nblocks * TEAMS * NGT) {
         const int inst = c.vert_inst[c.edge_info[mi >> 1].x];
         if (!need[inst]) continue;
         for (int r = g; r < CC; r += GJ) Dm[r] = ldcg(nw + (size_t)mi * CC + r) - ldcg(od + (size_t)mi * CC + r);
-        jacobi_svd<CHI, TS, WarpGroup, false, !Mode::mixed>(Dm, nullptr, g, grp, group_mask<CHI>(),
-                                                             Mode::mixed ? (TS)1e-6 : (TS)1e-15, 60, false, nullptr,
-                                                             Mode::mixed ? (TS)1e-3 : (TS)3e-8);
+        const TS sacc = trace_norm<CHI, TS>(Dm, g, grp);
         if (g == 0) {
-            TS sacc = (TS)0;
-            for (int cc = 0; cc < CHI; ++cc) {
-                TS n2 = (TS)0;
-                for (int r = 0; r < CHI; ++r) n2 += norm2(Dm[cc * CHI + r]);
-                sacc += nr_sqrt(n2);
-            }
             if (c.B == 1) mine += (double)sacc;
             else atomicAdd(ex + inst, (double)sacc);
         }
@@ -1255,9 +1281,8 @@ struct SmemSize {
     using S = Shape<CHI, V>;
     static constexpr int TPB = S::TPB;
     static constexpr size_t gate = sizeof(GateSm<CHI, Mode>) * (TPB / S::TG);
-    // per-team caches, block sums (64 doubles), scratch of the exact-distance pass
-    static constexpr size_t bp = sizeof(BPSm<CHI, Mode, S::TB>) * (TPB / S::TB) + 64 * sizeof(double) +
-                                 sizeof(C<typename Mode::TS>) * 2 * TPB;
+    // per-team caches, block sums (64 doubles)
+    static constexpr size_t bp = sizeof(BPSm<CHI, Mode, S::TB>) * (TPB / S::TB) + 64 * sizeof(double);
     static constexpr size_t rg = sizeof(RGSm<CHI>) * (TPB / S::TR);
     static constexpr size_t rv =
         sizeof(C<typename Mode::TS>) * (4 * CHI * CHI * CHI + 3 * CHI * CHI) * (TPB / S::TRV);
@@ -1364,7 +1389,6 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
                                                     (3 * sizeof(int) * (size_t)c.B + 7) / 8 * 8);
             double* thr_hi = thr + c.B;                               // bound that lets a sweep continue
             float* thr3 = reinterpret_cast<float*>(thr_hi + c.B);     // inline-exact trigger
-            CT_* scratch = reinterpret_cast<CT_*>(bsum + 64);
             const double slack = Mode::mixed ? 1e-5 : 1e-12;   // rounding of the lower bound
             for (int b = threadIdx.x; b < c.B; b += S::TPB) {
                 done[b] = 0;
@@ -1470,7 +1494,7 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
                 if (threadIdx.x == 0) sflag[(it + 1) & 1] = 0;
                 if (fl & 1) {
                     if (blockIdx.x == 0 && threadIdx.x == 0) ++c.ctl->exact_passes;
-                    bp_exact_pass<CHI, Mode, S::TPB>(c, cur, need, scratch, bsum + 32, ex);
+                    bp_exact_pass<CHI, Mode, S::TPB, S::TB>(c, cur, need, sm, bsum + 32, ex);
                     if (!grid_sync(gb, c.spin_limit)) return;
                     for (int b = threadIdx.x; b < c.B; b += S::TPB) {
                         if (!need[b]) continue;
