@@ -63,7 +63,8 @@ struct gtqa_state {
     int tpb[PK_COUNT] = {0, 0, 0};       // threads per block and team size of each kernel's variant
     int team[PK_COUNT] = {0, 0, 0};
     std::vector<int> h_inst_m;
-    // device buffers
+    // device buffers: parts of one allocation (arena), except the gate lists further down
+    void* arena = nullptr;
     void* Gamma = nullptr;
     double* lam = nullptr;
     void* T = nullptr;
@@ -509,11 +510,7 @@ void free_state(gtqa_state* s) {
     if (s->graph) cudaGraphDestroy(s->graph);
     for (cudaEvent_t e : s->gev)
         if (e) cudaEventDestroy(e);
-    void* ptrs[] = {s->kdev, s->Gamma, s->lam, s->T, s->msg[0], s->msg[1], s->D0, s->t0, s->X, s->edge_info,
-                    s->vert_edges, s->vert_inst, s->J, s->h, s->colour_edges, s->colour_off, s->gates_meta,
-                    s->iso, s->inst_vbeg, s->inst_m, s->acc, s->inst_done, s->inst_iters, s->inst_dist,
-                    s->stats, s->ctl, s->rho, s->sign, s->flags, s->rbuf, s->cutbuf, s->xs, s->ps,
-                    s->gate_edge, s->gate_U, s->sq_vertex, s->sq_W, s->vslots4, s->gate_bits, s->pscratch, s->dm, s->Fp};
+    void* ptrs[] = {s->arena, s->gate_edge, s->gate_U, s->sq_vertex, s->sq_W};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& p : s->pending) {
@@ -522,6 +519,14 @@ void free_state(gtqa_state* s) {
     }
     for (cudaEvent_t e : s->pool) cudaEventDestroy(e);
     delete s;
+}
+
+// |+>^N in zeroed memory: Gamma[a][i][0...] = 1/sqrt(2), lambda_e = (1, 0, ...)
+template <typename TS>
+__global__ void plus_state_kernel(C<TS>* Gamma, size_t H, int n, double* lam, int CHI, int m) {
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 2 * (size_t)n) Gamma[t * H] = C<TS>{(TS)0.70710678118654752440, (TS)0};
+    if (t < (size_t)m) lam[t * CHI] = 1.0;
 }
 
 // stores the first layer index of a run of graph replays (gtqa_anneal_graph)
@@ -650,7 +655,7 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
     if (N > (1LL << 28) || Mtot > (1LL << 28)) return GTQA_ERR_INVALID_ARG;
     if (Mtot > 0 && (!edges || !J)) return GTQA_ERR_INVALID_ARG;
     std::vector<int> ge((size_t)Mtot * 2), gcol((size_t)Mtot), vinst(N);
-    std::vector<int> deg(N, 0);
+    std::vector<int> deg(N, 0), nb(4 * (size_t)N);
     std::vector<int> vbeg(B + 1, 0), minst(B);
     int ncol = 0;
     {
@@ -658,22 +663,19 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
         for (int b = 0; b < B; ++b) {
             vbeg[b] = (int)voff;
             minst[b] = m[b];
-            std::vector<long long> keys;
-            keys.reserve(m[b]);
             for (int e = 0; e < m[b]; ++e) {
                 const int u = edges[2 * (eoff + e)], v = edges[2 * (eoff + e) + 1];
                 if (u < 0 || v < 0 || u >= n[b] || v >= n[b] || u == v) return GTQA_ERR_INVALID_ARG;
                 if (!std::isfinite(J[eoff + e])) return GTQA_ERR_INVALID_ARG;
-                const long long a = u < v ? u : v, c = u < v ? v : u;
-                keys.push_back(a * n[b] + c);
-                ge[2 * (eoff + e)] = (int)(u + voff);
-                ge[2 * (eoff + e) + 1] = (int)(v + voff);
-                if (++deg[u + voff] > 4 || ++deg[v + voff] > 4) return GTQA_ERR_INVALID_ARG;
+                const int gu = (int)(u + voff), gv = (int)(v + voff);
+                ge[2 * (eoff + e)] = gu;
+                ge[2 * (eoff + e) + 1] = gv;
+                if (deg[gu] >= 4 || deg[gv] >= 4) return GTQA_ERR_INVALID_ARG;
+                for (int q = 0; q < deg[gu]; ++q)
+                    if (nb[4 * (size_t)gu + q] == gv) return GTQA_ERR_INVALID_ARG;   // a repeated edge
+                nb[4 * (size_t)gu + deg[gu]++] = gv;
+                nb[4 * (size_t)gv + deg[gv]++] = gu;
             }
-            std::vector<long long> sk = keys;
-            std::sort(sk.begin(), sk.end());
-            for (size_t i = 1; i < sk.size(); ++i)
-                if (sk[i] == sk[i - 1]) return GTQA_ERR_INVALID_ARG;
             for (int a = 0; a < n[b]; ++a) {
                 if (!std::isfinite(h[voff + a])) return GTQA_ERR_INVALID_ARG;
                 vinst[voff + a] = b;
@@ -804,51 +806,6 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
     }
     const int CHI = s->CHI;
     const size_t gel = gamma_elems(s), mel = msg_elems(s), eb = elem_bytes(s);
-    int rc = GTQA_OK;
-    if ((rc = dalloc(s, (unsigned char**)&s->Gamma, gel * eb)) || (rc = dalloc(s, (unsigned char**)&s->T, gel * eb)) ||
-        (rc = dalloc(s, (unsigned char**)&s->msg[0], mel * eb)) ||
-        (rc = dalloc(s, (unsigned char**)&s->msg[1], mel * eb)) || (rc = dalloc(s, &s->lam, (size_t)s->m * CHI)) ||
-        (rc = dalloc(s, &s->D0, mixed(s) ? mel : 1)) || (rc = dalloc(s, &s->t0, mixed(s) ? (size_t)2 * s->m : 1)) ||
-        (rc = dalloc(s, &s->X, (size_t)s->m * 2 * CHI * CHI)) || (rc = dalloc(s, &s->edge_info, s->m)) ||
-        (rc = dalloc(s, &s->vert_edges, s->n)) || (rc = dalloc(s, &s->vert_inst, s->n)) ||
-        (rc = dalloc(s, &s->J, s->m)) || (rc = dalloc(s, &s->h, s->n)) || (rc = dalloc(s, &s->colour_edges, s->m)) ||
-        (rc = dalloc(s, &s->colour_off, ncol + 1)) || (rc = dalloc(s, &s->gates_meta, s->m)) ||
-        (rc = dalloc(s, &s->iso, iso.size())) || (rc = dalloc(s, &s->inst_vbeg, B + 1)) ||
-        (rc = dalloc(s, &s->inst_m, B)) || (rc = dalloc(s, &s->acc, 6 * (size_t)B)) ||
-        (rc = dalloc(s, &s->inst_done, B)) || (rc = dalloc(s, &s->inst_iters, B)) ||
-        (rc = dalloc(s, &s->inst_dist, B)) || (rc = dalloc(s, &s->stats, kStats)) || (rc = dalloc(s, &s->ctl, 1)) || (rc = dalloc(s, &s->kdev, 1)) ||
-        (rc = dalloc(s, &s->rho, (size_t)s->n * 4)) || (rc = dalloc(s, &s->sign, s->n)) ||
-        (rc = dalloc(s, &s->flags, 4)) || (rc = dalloc(s, &s->rbuf, 1)) ||
-        (rc = dalloc(s, &s->cutbuf, std::max(s->m, 1))) || (rc = dalloc(s, &s->xs, s->n)) ||
-        (rc = dalloc(s, &s->ps, s->n)) || (s->plain && (rc = dalloc(s, &s->vslots4, s->n))) ||
-        (s->plain && (rc = dalloc(s, &s->gate_bits, s->m))) ||
-        (s->plain && (rc = dalloc(s, &s->pscratch, plain_scratch_entries(s->CHI, s->D, max_gates)))) ||
-        (s->plain && (rc = dalloc(s, &s->Fp, (size_t)4 * s->m * CHI * CHI))) ||
-        (s->plain && (rc = dalloc(s, &s->dm, (size_t)2 * s->m * CHI * CHI)))) {
-        free_state(s);
-        return rc;
-    }
-    if (s->plain) {
-        if (!cuda_ok(s, cudaMemcpyAsync(s->vslots4, v4.data(), sizeof(int4) * N, cudaMemcpyHostToDevice, s->stream)) ||
-            !cuda_ok(s, cudaMemcpyAsync(s->gate_bits, gbits.data(), sizeof(int) * Mtot, cudaMemcpyHostToDevice, s->stream)) ||
-            !cuda_ok(s, cudaStreamSynchronize(s->stream))) {
-            free_state(s);
-            return GTQA_ERR_CUDA;
-        }
-    }
-    // |+>^N: Gamma[a][i][0][0][0] = 1/sqrt(2); lambda_e = (1, 0, ...)
-    const size_t H = (size_t)CHI * CHI * CHI * (s->D == 4 ? CHI : 1);
-    std::vector<unsigned char> g0(gel * eb, 0);
-    for (long long a = 0; a < N; ++a) {
-        for (int i = 0; i < 2; ++i) {
-            const size_t idx = a * 2 * H + i * H;
-            if (f32store(s)) reinterpret_cast<cf*>(g0.data())[idx] = cf{(float)M_SQRT1_2, 0.f};
-            else reinterpret_cast<cd*>(g0.data())[idx] = cd{M_SQRT1_2, 0.0};
-        }
-    }
-    std::vector<double> l0((size_t)s->m * CHI, 0.0);
-    for (long long e = 0; e < Mtot; ++e) l0[e * CHI] = 1.0;
-    std::vector<double> Jv(J ? J : (const double*)nullptr, J ? J + Mtot : (const double*)nullptr);
     std::vector<double> hv(N);   // h_a / degree of a, the share of every gate at a (App. F)
     for (long long a = 0; a < N; ++a) hv[a] = deg[a] > 0 ? h[a] / deg[a] : h[a];
     // the gates in the order they run, with what a gate needs to know of the graph
@@ -867,28 +824,93 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
         gmeta[q].a = make_int4(ed, v[0], v[1], bits);
         gmeta[q].b = make_int4(other[0], other[1], other[2], other[3]);
     }
-    Control ctl0;
-    std::memset(&ctl0, 0, sizeof(ctl0));
+    // One device allocation for the state, in three runs: what is copied from the host (one copy from
+    // one staging buffer), what starts as zero (one memset), and what every use writes first.  Some
+    // forty allocations, a dozen copies and the host-made |+> tensors took 0.33 ms at n = 16 and
+    // 6.8 ms at n = 12000, chi = 8 (with the destruction).
+    struct Part {
+        void** p;
+        size_t bytes;
+        const void* src;
+    };
+    std::vector<Part> copied, zeroed, scratch;
+    auto copy = [&](auto** p, const void* src, size_t count) { copied.push_back({(void**)p, count * sizeof(**p), src}); };
+    auto zero = [&](void** p, size_t bytes) { zeroed.push_back({p, bytes, nullptr}); };
+    auto raw = [&](void** p, size_t bytes) { scratch.push_back({p, bytes, nullptr}); };
+    const size_t M = (size_t)Mtot, V = (size_t)N, CC = (size_t)CHI * CHI;
+    copy(&s->edge_info, einfo.data(), M);
+    copy(&s->vert_edges, vedges.data(), V);
+    copy(&s->vert_inst, vinst.data(), V);
+    copy(&s->J, J, M);
+    copy(&s->h, hv.data(), V);
+    copy(&s->colour_edges, cedges.data(), M);
+    copy(&s->colour_off, coff.data(), (size_t)ncol + 1);
+    copy(&s->gates_meta, gmeta.data(), gmeta.size());
+    copy(&s->iso, iso.data(), iso.size());
+    copy(&s->inst_vbeg, vbeg.data(), (size_t)B + 1);
+    copy(&s->inst_m, minst.data(), (size_t)B);
+    if (s->plain) {
+        copy(&s->vslots4, v4.data(), V);
+        copy(&s->gate_bits, gbits.data(), M);
+    }
+    zero((void**)&s->ctl, sizeof(Control));
+    zero((void**)&s->stats, sizeof(double) * kStats);
+    zero((void**)&s->flags, sizeof(int) * 4);
+    zero((void**)&s->kdev, sizeof(int));
+    zero((void**)&s->acc, sizeof(double) * 6 * B);
+    zero((void**)&s->lam, sizeof(double) * M * CHI);
+    zero(&s->msg[0], mel * eb);
+    zero(&s->msg[1], mel * eb);
+    zero(&s->Gamma, gel * eb);
+    zero(&s->T, gel * eb);
+    raw((void**)&s->D0, mixed(s) ? mel * sizeof(cf) : 0);
+    raw((void**)&s->t0, mixed(s) ? 2 * M * sizeof(cd) : 0);
+    raw((void**)&s->X, M * 2 * CC * sizeof(cd));
+    raw((void**)&s->inst_done, sizeof(int) * B);
+    raw((void**)&s->inst_iters, sizeof(int) * B);
+    raw((void**)&s->inst_dist, sizeof(double) * B);
+    raw((void**)&s->rho, V * 4 * sizeof(cd));
+    raw((void**)&s->sign, V);
+    raw((void**)&s->rbuf, sizeof(double));
+    raw((void**)&s->cutbuf, M);
+    raw((void**)&s->xs, V);
+    raw((void**)&s->ps, V * sizeof(double));
+    if (s->plain) {
+        raw((void**)&s->pscratch, plain_scratch_entries(s->CHI, s->D, max_gates) * sizeof(cd));
+        raw((void**)&s->dm, mel * sizeof(cd));
+        raw((void**)&s->Fp, 2 * mel * sizeof(cd));
+    }
+    size_t total = 0;
+    auto layout = [&](std::vector<Part>& run) {
+        const size_t beg = total;
+        for (const Part& q : run) total += (std::max<size_t>(q.bytes, 1) + 255) / 256 * 256;
+        return beg;
+    };
+    layout(copied);
+    const size_t zbeg = layout(zeroed), rbeg = layout(scratch);
+    int rc = dalloc(s, (unsigned char**)&s->arena, total);
+    if (rc) {
+        free_state(s);
+        return rc;
+    }
+    std::vector<unsigned char> stage(zbeg);
+    size_t at = 0;
+    for (std::vector<Part>* run : {&copied, &zeroed, &scratch})
+        for (const Part& q : *run) {
+            *q.p = (unsigned char*)s->arena + at;
+            if (q.src && q.bytes) std::memcpy(stage.data() + at, q.src, q.bytes);
+            at += (std::max<size_t>(q.bytes, 1) + 255) / 256 * 256;
+        }
     cudaStream_t st = s->stream;
-    bool ok = cuda_ok(s, cudaMemcpyAsync(s->Gamma, g0.data(), g0.size(), cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemsetAsync(s->T, 0, gel * eb, st)) &&
-              cuda_ok(s, cudaMemsetAsync(s->msg[0], 0, mel * eb, st)) &&
-              cuda_ok(s, cudaMemsetAsync(s->msg[1], 0, mel * eb, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->lam, l0.data(), l0.size() * sizeof(double), cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->edge_info, einfo.data(), sizeof(int4) * Mtot, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->vert_edges, vedges.data(), sizeof(int4) * N, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->vert_inst, vinst.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->J, Jv.data(), sizeof(double) * Mtot, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->h, hv.data(), sizeof(double) * N, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->colour_edges, cedges.data(), sizeof(int) * Mtot, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->colour_off, coff.data(), sizeof(int) * (ncol + 1), cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->gates_meta, gmeta.data(), sizeof(GateMeta) * gmeta.size(), cudaMemcpyHostToDevice, st)) &&
-              (iso.empty() || cuda_ok(s, cudaMemcpyAsync(s->iso, iso.data(), sizeof(int) * iso.size(), cudaMemcpyHostToDevice, st))) &&
-              cuda_ok(s, cudaMemcpyAsync(s->inst_vbeg, vbeg.data(), sizeof(int) * (B + 1), cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->inst_m, minst.data(), sizeof(int) * B, cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemsetAsync(s->stats, 0, sizeof(double) * kStats, st)) &&
-              cuda_ok(s, cudaMemcpyAsync(s->ctl, &ctl0, sizeof(Control), cudaMemcpyHostToDevice, st)) &&
-              cuda_ok(s, cudaMemsetAsync(s->flags, 0, sizeof(int) * 4, st)) && cuda_ok(s, cudaStreamSynchronize(st));
+    bool ok = cuda_ok(s, cudaMemcpyAsync(s->arena, stage.data(), zbeg, cudaMemcpyHostToDevice, st)) &&
+              cuda_ok(s, cudaMemsetAsync((unsigned char*)s->arena + zbeg, 0, rbeg - zbeg, st));
+    if (ok) {
+        const size_t H = (size_t)CHI * CHI * CHI * (s->D == 4 ? CHI : 1);
+        const unsigned blocks = (unsigned)((std::max<size_t>(2 * V, M) + 255) / 256);
+        if (f32store(s)) plus_state_kernel<float><<<blocks, 256, 0, st>>>((cf*)s->Gamma, H, s->n, s->lam, CHI, s->m);
+        else plus_state_kernel<double><<<blocks, 256, 0, st>>>((cd*)s->Gamma, H, s->n, s->lam, CHI, s->m);
+        ok = cuda_ok(s, cudaGetLastError()) && cuda_ok(s, cudaStreamSynchronize(st));
+    }
     if (!ok) {
         free_state(s);
         return GTQA_ERR_CUDA;
