@@ -604,17 +604,21 @@ struct BPSm {
     // and meet by shuffles, or, where that does not divide, the sum in two halves over the
     // physical index i, added at use
     static constexpr int NPART = TB / CC;
+    // mixed mode, two lanes per fiber of one slot: the fiber-wise front (bp_front_fibers)
+    static constexpr bool FIBERS = Mode::mixed && CHI >= 4 && TB == 4 * CC;
+    static constexpr int NPT = FIBERS ? CC / 8 > 4 ? 4 : 2 : 1;   // partial sums of a message
     static constexpr bool HALVES = !(TB % CC == 0 && NPART <= 32 && (2 * CHI) % NPART == 0);
     static_assert(CHI % 2 == 0 && 3 * (CHI / 2) * (CHI / 2) * NS <= TB, "BP team too small for the overlap stage");
     // T, P and Q in the natural index order [i][j0][j1][j2] with one padding element after
     // every (i, j0) plane, so that a stride along slot 0 does not map to one bank
-    static constexpr int PS = CC + 1, H2P = 2 * CHI * PS;
-    C<TS> T[H2P];
+    // (two for the fiber-wise front: pairs of elements are loaded at once)
+    static constexpr int PS = CC + (FIBERS ? 2 : 1), H2P = 2 * CHI * PS;
+    alignas(16) C<TS> T[H2P];
     C<TS> P[NP][H2P];    // FP64: T x0 m0, T x1 m1; mixed: T x0 d0, T x1 d1, T x2 d2
-    C<TS> Q[3][H2P];     // per outgoing slot
-    C<TS> min[3][CC];    // incoming messages (mixed: m0 + delta)
-    C<TS> din[3][CC];    // mixed: incoming delta
-    C<TS> F[3][CC];      // the outgoing messages before normalisation
+    C<TS> Q[FIBERS ? 1 : 3][FIBERS ? 2 : H2P];   // per outgoing slot
+    alignas(16) C<TS> min[3][CC];   // incoming messages (mixed: m0 + delta)
+    alignas(16) C<TS> din[3][CC];   // mixed: incoming delta
+    C<TS> F[3 * NPT][CC];   // the outgoing messages before normalisation, [partial sum][slot]
     C<TS> F1[Mode::mixed ? 1 : 3][CC];   // FP64 mode with HALVES: the i = 1 half
     C<TS> prev[3][CC];   // outgoing messages of the previous sweep
     C<TS> D[3][CC];      // new - old, for the trace norm
@@ -627,6 +631,17 @@ struct BPSm {
     TS dsum[3];          // one instance: the team's distance summed over the rounds of a sweep
     int es[3], out_idx[3], in_idx[3];
     int cached;          // vertex held in the cache, -1 if none
+    // element r of the message out of slot k
+    __device__ __forceinline__ C<TS> out(int k, int r) const {
+        C<TS> f = F[k][r];
+        if constexpr (FIBERS) {
+            if (NPT == 4 || k == 2) f = f + F[3 + k][r];
+            if (NPT == 4 && k == 2) f = f + (F[6 + k][r] + F[9 + k][r]);
+        } else if constexpr (!Mode::mixed && HALVES) {
+            f = f + F1[k][r];
+        }
+        return f;
+    }
 };
 
 // Trace norm (sum of singular values) of the CHI x CHI matrix A (column-major, CHI^2/2 lanes; A is
@@ -682,7 +697,7 @@ __device__ void bp_prepare(const Ctx& c, int a, int tid, int team, int cur, BPSm
         }
     }
     const CT* Tg = (const CT*)c.T + (size_t)a * H2;
-    for (int t = tid; t < H2; t += TEAM) sm.T[t + t / CC] = ldcg(Tg + t);
+    for (int t = tid; t < H2; t += TEAM) sm.T[t + (t / CC) * (BPSm<CHI, Mode, TB>::PS - CC)] = ldcg(Tg + t);
     team_bar<TEAM>(team);
     const CT* src = (const CT*)c.msg[cur];
     for (int t = tid; t < 3 * CC; t += TEAM) {
@@ -707,35 +722,145 @@ __device__ void bp_prepare(const Ctx& c, int a, int tid, int team, int cur, BPSm
     team_bar<TEAM>(team);
 }
 
-// First part of the sweep for vertex a: incoming messages, the contractions, and the
-// traces of the three outgoing messages (left in sm.trs).
+// The contractions of a sweep, fiber by fiber (mixed mode, team of 4 CHI^2 lanes = two sets of one lane
+// per fiber).  Shared-memory loads bounded the element-wise form (two loads of 8 bytes per
+// complex product; at chi = 4 about 3800 of the 4400 cycles of a vertex's share of an SM).  Here a
+// lane loads a fiber of T or P once, in pairs, and forms its outputs from it, the message entries
+// are broadcasts to the whole warp, and a fiber of Q stays in registers until its overlap with
+// conj(T) is summed: about 140 load transactions per warp and vertex instead of 480 (chi = 4).
+//   P_k = T x_k delta_k: slot 0 by set 0, slot 1 by set 1, slot 2 by both (half of the outputs each);
+//   Q_0 = P_1 x_2 m_2 + m0_1 P_2 (set 0), Q_1 = P_0 x_2 m_2 + m0_0 P_2 (set 1),
+//   Q_2 = P_0 x_1 m_1 + m0_0 P_1 (both, half of the outputs each);
+//   F_s[j][j'] = sum Q_s[.., j@s, ..] conj(T[.., j'@s, ..]).
+template <int CHI>
+__device__ __forceinline__ void load_fiber(const cf* p, cf (&f)[CHI]) {
+#pragma unroll
+    for (int q = 0; q < CHI; q += 2) {
+        const float4 v = *reinterpret_cast<const float4*>(p + q);
+        f[q] = cf{v.x, v.y};
+        f[q + 1] = cf{v.z, v.w};
+    }
+}
+// outputs x0 and x0 + 1 of a fiber contracted with y[q][x]
+template <int CHI>
+__device__ __forceinline__ void fiber_pair(const cf (&in)[CHI], const cf* y, int x0, cf& a, cf& b) {
+#pragma unroll
+    for (int q = 0; q < CHI; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(y + q * CHI + x0);
+        a = cfma(in[q], cf{v.x, v.y}, a);
+        b = cfma(in[q], cf{v.z, v.w}, b);
+    }
+}
+// sum of ov[j'] over the CHI lanes of a fiber row (lane j' ends with ov[j']) and, where the two
+// physical indices share a warp (CHI = 4), over them
+template <int CHI>
+__device__ __forceinline__ cf fiber_sum(cf (&ov)[CHI]) {
+    float s[2 * CHI];
+#pragma unroll
+    for (int q = 0; q < CHI; ++q) {
+        s[2 * q] = ov[q].x;
+        s[2 * q + 1] = ov[q].y;
+    }
+    rs_level<CHI / 2, 2 * CHI>(s, 0xffffffffu, threadIdx.x & (CHI - 1));
+    if constexpr (CHI == 4) {
+        s[0] += __shfl_xor_sync(0xffffffffu, s[0], 16);
+        s[1] += __shfl_xor_sync(0xffffffffu, s[1], 16);
+    }
+    return cf{s[0], s[1]};
+}
 template <int CHI, class Mode, int TB>
-__device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<CHI, Mode, TB>& sm, bool have_pre,
-                         C<typename Mode::TS> pre) {
+__device__ __forceinline__ void bp_front_fibers(int tid, int team, BPSm<CHI, Mode, TB>& sm) {
+    using SM = BPSm<CHI, Mode, TB>;
+    constexpr int CC = CHI * CHI, NF = 2 * CC, S0 = SM::PS, S1 = CHI, HP = CHI * SM::PS, HALF = CHI / 2;
+    const int set = tid / NF, f = tid % NF, i = f / CC, u = (f / CHI) % CHI, v = f % CHI;
+    const cf z = cf{0.f, 0.f};
+    {   // P_0 or P_1
+        const int st = set ? S1 : S0, base = i * HP + u * (set ? S0 : S1) + v;
+        cf in[CHI];
+#pragma unroll
+        for (int q = 0; q < CHI; ++q) in[q] = sm.T[base + q * st];
+#pragma unroll
+        for (int x = 0; x < CHI; x += 2) {
+            cf a = z, b = z;
+            fiber_pair<CHI>(in, sm.din[set], x, a, b);
+            sm.P[set][base + x * st] = a;
+            sm.P[set][base + (x + 1) * st] = b;
+        }
+    }
+    {   // half of the outputs of P_2
+        const int base = i * HP + u * S0 + v * S1;
+        cf in[CHI];
+        load_fiber<CHI>(sm.T + base, in);
+#pragma unroll
+        for (int x = 0; x < HALF; x += 2) {
+            cf a = z, b = z;
+            fiber_pair<CHI>(in, sm.din[2], set * HALF + x, a, b);
+            *reinterpret_cast<float4*>(sm.P[2] + base + set * HALF + x) = float4{a.x, a.y, b.x, b.y};
+        }
+    }
+    team_bar<TB>(team);
+    const int j = u, a0 = v;   // message index and the index summed over the CHI neighbouring lanes
+    if (sm.es[set] >= 0) {   // the same for the set
+        // set 0: (j0, j1) = (j, a0), set 1: (a0, j)
+        const int base = i * HP + (set ? a0 : j) * S0 + (set ? j : a0) * S1;
+        cf in[CHI], q[CHI], p2[CHI];
+        load_fiber<CHI>((set ? sm.P[0] : sm.P[1]) + base, in);
+        load_fiber<CHI>(sm.P[2] + base, p2);
+        const float w = set ? sm.m0f[0][a0] : sm.m0f[1][a0];
+#pragma unroll
+        for (int b = 0; b < CHI; ++b) q[b] = w * p2[b];
+#pragma unroll
+        for (int b = 0; b < CHI; b += 2) fiber_pair<CHI>(in, sm.min[2], b, q[b], q[b + 1]);
+        cf ov[CHI];
+        const cf* Tb = sm.T + i * HP + a0 * (set ? S0 : S1);
+#pragma unroll
+        for (int jp = 0; jp < CHI; ++jp) {
+            cf t[CHI];
+            load_fiber<CHI>(Tb + jp * (set ? S1 : S0), t);
+            ov[jp] = z;
+#pragma unroll
+            for (int b = 0; b < CHI; ++b) ov[jp] = cfmac(t[b], q[b], ov[jp]);
+        }
+        const cf r = fiber_sum<CHI>(ov);
+        if (CHI != 4 || i == 0) sm.F[(CHI == 4 ? 0 : 3 * i) + set][j * CHI + a0] = r;
+    }
+    if (sm.es[2] >= 0) {
+        // j2 = j, j0 = a0, j1 = b in the set's half
+        const int base = i * HP + a0 * S0 + j;
+        cf in[CHI], q[HALF];
+#pragma unroll
+        for (int x = 0; x < CHI; ++x) in[x] = sm.P[0][base + x * S1];
+        const float w = sm.m0f[0][a0];
+#pragma unroll
+        for (int b = 0; b < HALF; ++b) q[b] = w * sm.P[1][base + (set * HALF + b) * S1];
+#pragma unroll
+        for (int b = 0; b < HALF; b += 2) fiber_pair<CHI>(in, sm.min[1], set * HALF + b, q[b], q[b + 1]);
+        cf ov[CHI];
+#pragma unroll
+        for (int jp = 0; jp < CHI; ++jp) ov[jp] = z;
+#pragma unroll
+        for (int b = 0; b < HALF; ++b) {
+            cf t[CHI];
+            load_fiber<CHI>(sm.T + i * HP + a0 * S0 + (set * HALF + b) * S1, t);
+#pragma unroll
+            for (int jp = 0; jp < CHI; ++jp) ov[jp] = cfmac(t[jp], q[b], ov[jp]);
+        }
+        const cf r = fiber_sum<CHI>(ov);
+        if (CHI != 4 || i == 0) sm.F[3 * (CHI == 4 ? set : i + 2 * set) + 2][j * CHI + a0] = r;
+    }
+    team_bar<TB>(team);
+}
+
+// The contractions of a sweep element by element (FP64 mode, and the shapes without a fiber-wise form).
+template <int CHI, class Mode, int TB>
+__device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, Mode, TB>& sm) {
     using TS = typename Mode::TS;
     using CT = C<TS>;
     using SM = BPSm<CHI, Mode, TB>;
     constexpr int TEAM = TB, CC = CHI * CHI, H = CHI * CHI * CHI, H2 = 2 * H;
     // strides in the padded shared-memory layout: slot 0, slot 1 (slot 2 has stride 1), i
     constexpr int S0 = SM::PS, S1 = CHI, HP = CHI * SM::PS;
-    if (sm.cached != a) bp_prepare<CHI, Mode, TB>(c, a, tid, team, cur, sm);
-    const CT* src = (const CT*)c.msg[cur];
     const CT z = CT{(TS)0, (TS)0};
-    // incoming messages (prefetched into `pre` by the caller when have_pre)
-    for (int t = tid; t < 3 * CC; t += TEAM) {
-        const int k = t / CC, r = t % CC;
-        const int in = sm.in_idx[k];
-        const CT lv = in >= 0 ? (have_pre ? pre : ldcg(src + (size_t)in * CC + r)) : z;
-        if constexpr (!Mode::mixed) {
-            sm.min[k][r] = in >= 0 ? lv : CT{(TS)(r == 0 ? 1 : 0), (TS)0};
-        } else {
-            const int j = r / CHI, jp = r % CHI;
-            const CT dv = lv;
-            sm.din[k][r] = dv;
-            sm.min[k][r] = CT{dv.x + ((j == jp) ? sm.m0f[k][j] : 0.f), dv.y};
-        }
-    }
-    team_bar<TEAM>(team);
     // first contractions along one slot: P_k[.., x@k, ..] = sum_q T[.., q@k, ..] y_k[q][x]
     //   FP64: y = m (k = 0, 1); mixed: y = delta (k = 0, 1, 2)
     constexpr int NP = SM::NP;
@@ -886,14 +1011,47 @@ __device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<C
         }
     }
     team_bar<TEAM>(team);
+}
+
+// First part of the sweep for vertex a: incoming messages, the contractions, and the
+// traces of the three outgoing messages (left in sm.trs).
+template <int CHI, class Mode, int TB>
+__device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<CHI, Mode, TB>& sm, bool have_pre,
+                         C<typename Mode::TS> pre) {
+    using TS = typename Mode::TS;
+    using CT = C<TS>;
+    using SM = BPSm<CHI, Mode, TB>;
+    constexpr int TEAM = TB, CC = CHI * CHI;
+    if (sm.cached != a) bp_prepare<CHI, Mode, TB>(c, a, tid, team, cur, sm);
+    const CT* src = (const CT*)c.msg[cur];
+    const CT z = CT{(TS)0, (TS)0};
+    // incoming messages (prefetched into `pre` by the caller when have_pre)
+    for (int t = tid; t < 3 * CC; t += TEAM) {
+        const int k = t / CC, r = t % CC;
+        const int in = sm.in_idx[k];
+        const CT lv = in >= 0 ? (have_pre ? pre : ldcg(src + (size_t)in * CC + r)) : z;
+        if constexpr (!Mode::mixed) {
+            sm.min[k][r] = in >= 0 ? lv : CT{(TS)(r == 0 ? 1 : 0), (TS)0};
+        } else {
+            const int j = r / CHI, jp = r % CHI;
+            const CT dv = lv;
+            sm.din[k][r] = dv;
+            sm.min[k][r] = CT{dv.x + ((j == jp) ? sm.m0f[k][j] : 0.f), dv.y};
+        }
+    }
+    team_bar<TEAM>(team);
+    if constexpr (SM::FIBERS) {
+        bp_front_fibers<CHI, Mode, TB>(tid, team, sm);
+    } else {
+        bp_front_elements<CHI, Mode, TB>(tid, team, sm);
+    }
     // traces of the outgoing messages (their reciprocals follow in FP64, bp_trace_rcp)
     if (tid < 3 * CC && tid % CC == 0) {
         const int k = tid / CC;
         CT trs = z;
 #pragma unroll
         for (int j = 0; j < CHI; ++j) {
-            trs = trs + sm.F[k][j * CHI + j];
-            if constexpr (!Mode::mixed && SM::HALVES) trs = trs + sm.F1[k][j * CHI + j];
+            trs = trs + sm.out(k, j * CHI + j);
         }
         sm.trs[k] = trs;
     }
@@ -938,8 +1096,7 @@ __device__ void bp_back(const Ctx& c, int tid, int team, int cur, bool exact, BP
         CT d = z;
         if (out >= 0) {
             const CT itr = sm.itr[k];
-            CT f = sm.F[k][r];
-            if constexpr (!Mode::mixed && BPSm<CHI, Mode, TB>::HALVES) f = f + sm.F1[k][r];
+            const CT f = sm.out(k, r);
             CT num = f;
             if constexpr (Mode::mixed) {
                 const int j = r / CHI, jp = r % CHI;

@@ -428,6 +428,78 @@ __device__ int jacobi_v32(const C<float>* A, C<float>* V, int g, unsigned gmask,
     return sweep;
 }
 
+// The same for a group of several warps (N = 16, 32): the columns go to the neighbouring pairs
+// through shared memory, in two buffers used in turn, so that a step has one barrier.  A, V: N^2
+// entries each; buf: 2 N^2 entries; nrm: 2 N floats.  V32 ends in V.
+template <int N, typename Group>
+__device__ int jacobi_v32_team(C<float>* A, C<float>* V, C<float>* buf, float* nrm, int g, const Group& grp,
+                               unsigned pair_mask, int keep) {
+    using CF = C<float>;
+    constexpr int NN = N * N, LAST = N / 2 - 1;
+    const int k = g / N, r = g % N;
+    // the slots (2 k: first column of pair k, 2 k + 1: second) that this pair's columns move to
+    const int da = (k == 0 ? 3 : 2 * (k - 1)) * N + r, db = (k == 0 ? 1 : (k == LAST ? 2 * LAST : 2 * (k + 1) + 1)) * N + r;
+    const int sa = 2 * k * N + r, sb = sa + N;
+    CF a = A[k * N + r], b = A[(N - 1 - k) * N + r];
+    CF va = CF{k == r ? 1.f : 0.f, 0.f}, vb = CF{N - 1 - k == r ? 1.f : 0.f, 0.f};
+    int sweep = 0, par = 0;
+    for (; sweep < 40; ++sweep) {
+        int big = 0;
+        float thr = 0.f;
+        for (int step = 0; step < N - 1; ++step) {
+            float s[4] = {norm2(a), norm2(b), fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x)};
+            group_sums<N>(s, pair_mask);
+            const float g2 = fmaf(s[2], s[2], s[3] * s[3]), ab = s[0] * s[1];
+            const bool rot = g2 > 1e-36f && g2 > 1e-12f * ab;
+            if (step == 0 && keep < N) {
+                if (r == 0) {
+                    nrm[2 * k] = s[0];
+                    nrm[2 * k + 1] = s[1];
+                }
+                grp.sync();
+                // a quarter of the keep-th largest squared norm
+                if (g < N) {
+                    const float x = nrm[g];
+                    int c = 0;
+                    for (int i = 0; i < N; ++i) c += nrm[i] >= x;
+                    nrm[N + g] = c >= keep ? 0.25f * x : 0.f;
+                }
+                grp.sync();
+                for (int j = 0; j < N; ++j) thr = fmaxf(thr, nrm[N + j]);
+                grp.sync();
+            }
+            const float mx = fmaxf(s[0], s[1]), lim = fminf(s[0], s[1]) >= thr ? ab : mx * mx;
+            if (rot && mx >= thr && g2 > 1e-6f * lim) big = 1;
+            const float d = s[1] - s[0];
+            const float tn = 2.f * fast_rcp(fabsf(d) + fast_sqrt(fmaf(d, d, 4.f * g2)));
+            const float tau = rot ? (d >= 0.f ? tn : -tn) : 0.f;
+            const float c = rot ? rsqrtf(fmaf(tau * tau, g2, 1.f)) : 1.f;
+            const CF se = CF{c * tau * s[2], c * tau * s[3]};
+            CF* bA = par ? buf : A;
+            CF* bV = par ? buf + NN : V;
+            par ^= 1;
+            if (step == 0 && sweep == 0) grp.sync();   // every lane has its columns of A
+            bA[da] = CF{fmaf(-se.x, b.x, fmaf(-se.y, b.y, c * a.x)), fmaf(-se.x, b.y, fmaf(se.y, b.x, c * a.y))};
+            bA[db] = CF{fmaf(se.x, a.x, fmaf(-se.y, a.y, c * b.x)), fmaf(se.x, a.y, fmaf(se.y, a.x, c * b.y))};
+            bV[da] = CF{fmaf(-se.x, vb.x, fmaf(-se.y, vb.y, c * va.x)), fmaf(-se.x, vb.y, fmaf(se.y, vb.x, c * va.y))};
+            bV[db] = CF{fmaf(se.x, va.x, fmaf(-se.y, va.y, c * vb.x)), fmaf(se.x, va.y, fmaf(se.y, va.x, c * vb.y))};
+            grp.sync();
+            a = bA[sa];
+            b = bA[sb];
+            va = bV[sa];
+            vb = bV[sb];
+        }
+        if (!grp.any(big)) {
+            ++sweep;
+            break;
+        }
+    }
+    grp.sync();
+    V[k * N + r] = va;
+    V[(N - 1 - k) * N + r] = vb;
+    return sweep;
+}
+
 // True if x (an updated squared norm) is negative, zero or below about half of ref, from the
 // raw bits only.
 __device__ __forceinline__ bool norm_collapsed(double x, double ref) {
@@ -613,7 +685,7 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 //      end once every pair was below `stop` (relative to its columns) before its pass.
 //      A pair with a larger K (nearly equal or not yet resolved columns) is rotated by
 //      FP64 Jacobi steps (only the steps of the schedule that hold such a pair) or, for N >= 16
-//      with many of them, by FP32 Jacobi on those columns of W rescaled to the largest of them,
+//      with many of them, by FP32 Jacobi on those and all shorter columns of W, rescaled,
 //      which resolves the columns that lay below the FP32 resolution of the first stage.
 //   A decomposition that is still open after MAXP passes goes to jacobi_polish.
 // Cores of whole anneals (n = 300, chi = 4): 1.3 passes on average in the mixed mode, 2.1 with
@@ -724,7 +796,9 @@ __device__ int svd32_unitary(C<double>* V, C<float>* A32, C<float>* V32, double*
         sw = jacobi_v32<N>(A32, V32, g, group_mask<LN>(), pair_mask, keep);
         grp.sync();
     } else {
-        sw = jacobi_svd<N, float>(A32, V32, g, grp, pair_mask, 1e-6f, 40, true, nullptr, 1e-3f);
+        sw = jacobi_v32_team<N>(A32, V32, reinterpret_cast<C<float>*>(V), reinterpret_cast<float*>(nrm), g, grp, pair_mask,
+                                keep);
+        grp.sync();
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) V[g + j * LN] = ccast<double>(V32[g + j * LN]);
@@ -869,7 +943,7 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
             cnt.pairs += nsteps * (N / 2);
             break;
         }
-        if (!(flags & 2u) || pass == 0) continue;   // the first pass only clears what it can
+        if (!(flags & 2u)) continue;
         const unsigned steps = grp.or_bits((mine & 2u) ? 1u << step : 0u);
         const int nst = __popc(steps);
         bool part = false;
@@ -879,7 +953,13 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
             cnt.pairs += nst * (N / 2);
         } else if constexpr (N >= 16) {
             ++second;
-            const unsigned cols = grp.or_bits((mine & 2u) ? (1u << p) | (1u << q) : 0u);
+            // the columns of those pairs, and every shorter one
+            unsigned cols = grp.or_bits((mine & 2u) ? (1u << p) | (1u << q) : 0u);
+            double longest = 0.0;
+            for (int j = 0; j < N; ++j)
+                if ((cols >> j) & 1u) longest = fmax(longest, nrm[j]);
+            for (int j = 0; j < N; ++j) cols |= nrm[j] <= longest ? 1u << j : 0u;
+            grp.sync();
             int e = 0;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
