@@ -29,6 +29,8 @@
 //          once per BP call in FP64.
 #pragma once
 
+#include <type_traits>
+
 #include "gtqa_common.cuh"
 
 namespace gtqa {
@@ -1218,7 +1220,14 @@ __device__ void bp_exact_pass(const Ctx& c, int cur_new, const int* need, BPSm<C
 }
 
 // ===========================================================================
-// regauge, edge part (team CHI^2): FP64 eigen/SVD, transforms X_a, X_b and lambda
+// regauge, edge part: FP64 eigen/SVD, transforms X_a, X_b and lambda
+//
+// A team is CHI^2 lanes, half of them per message, or CHI^2 / 2 lanes that take the two messages in
+// turn.  The three decompositions of an edge are the FP64 work: the wide team finishes an edge
+// sooner (two in turn instead of three) but leaves half of its lanes idle in the third one, and the
+// FP64 pipe charges a warp, not its lanes.  The narrow team runs once a sub-partition has more than
+// four wide warps' worth of edges (m > blocks x 512 / CHI^2): at 10 edges per block (n = 1000, chi = 4)
+// it is 9 us slower per regauge, at 165 (32 instances) a regauge is 15 % faster.
 // ===========================================================================
 template <int CHI>
 struct RGSm {
@@ -1241,9 +1250,10 @@ struct RGSm {
     double nrm[2][CHI];
 };
 
-template <int CHI, class Mode>
+template <int CHI, class Mode, int TEAM>
 __device__ void regauge_edge(const Ctx& c, int e, int tid, int team, int cur, RGSm<CHI>& sm) {
-    constexpr int TEAM = CHI * CHI, CC = CHI * CHI, GJ = CC / 2;
+    constexpr int CC = CHI * CHI, GJ = CC / 2;
+    static_assert(TEAM == CC || TEAM == GJ, "one or both messages at a time");
     // Hermitian parts of m_{a->b} (x = 0) and m_{b->a} (x = 1), column-major
     for (int t = tid; t < 2 * CC; t += TEAM) {
         const int x = t / CC, r = t % CC;
@@ -1271,16 +1281,19 @@ __device__ void regauge_edge(const Ctx& c, int e, int tid, int team, int cur, RG
     {
         // FP64 eigen-decompositions of the two Hermitian messages (the singular values of a
         // Hermitian matrix are the moduli of its eigenvalues)
-        const int x = tid / GJ, g = tid % GJ;
+        const int g = tid % GJ;
         WarpGroup grp{group_mask<GJ>()};
-        prune_noise<CHI>(sm.Am[x], g, grp);
-        const SvdCount cnt = refined_svd<CHI, !Mode::mixed>(
-            sm.Am[x], sm.Vm[x], sm.A32[x], sm.V32[x], sm.T1[x], sm.nrm[x], nullptr, g, grp, group_mask<CHI>(), c.eig_cut,
-            CHI, Mode::mixed ? 3e-7f : 1e-8f, Mode::mixed ? 1e-13 : 1e-15);
-        if (g == 0) {
-            atomicAdd(&c.stats[4], (double)cnt.passes);
-            atomicMax(&c.ctl->reg_sw_max, cnt.passes);
-            atomicMax(&c.ctl->reg_sw32_max, cnt.sweeps32);
+#pragma unroll 1
+        for (int x = tid / GJ; x < 2; x += TEAM / GJ) {
+            prune_noise<CHI>(sm.Am[x], g, grp);
+            const SvdCount cnt = refined_svd<CHI, !Mode::mixed>(
+                sm.Am[x], sm.Vm[x], sm.A32[x], sm.V32[x], sm.T1[x], sm.nrm[x], nullptr, g, grp, group_mask<CHI>(), c.eig_cut,
+                CHI, Mode::mixed ? 3e-7f : 1e-8f, Mode::mixed ? 1e-13 : 1e-15);
+            if (g == 0) {
+                atomicAdd(&c.stats[4], (double)cnt.passes);
+                atomicMax(&c.ctl->reg_sw_max, cnt.passes);
+                atomicMax(&c.ctl->reg_sw32_max, cnt.sweeps32);
+            }
         }
     }
     team_bar<TEAM>(team);
@@ -1438,18 +1451,196 @@ struct SmemSize {
     using S = Shape<CHI, V>;
     static constexpr int TPB = S::TPB;
     static constexpr size_t gate = sizeof(GateSm<CHI, Mode>) * (TPB / S::TG);
-    // per-team caches, block sums (64 doubles)
-    static constexpr size_t bp = sizeof(BPSm<CHI, Mode, S::TB>) * (TPB / S::TB) + 64 * sizeof(double);
-    static constexpr size_t rg = sizeof(RGSm<CHI>) * (TPB / S::TR);
+    // per-team caches, block sums (64 doubles), for the teams of the shape and the wide ones
+    static constexpr int WIDE_TB = !Mode::mixed && CHI <= 4 && S::TB == 64 ? 128 : S::TB;
+    static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
+    static constexpr size_t bp = mx(sizeof(BPSm<CHI, Mode, S::TB>) * (TPB / S::TB),
+                                    sizeof(BPSm<CHI, Mode, WIDE_TB>) * (TPB / WIDE_TB)) + 64 * sizeof(double);
+    static constexpr int rg_fit = (int)(190 * 1024 / sizeof(RGSm<CHI>));
+    static constexpr int rg_teams = TPB / (S::TR / 2) < rg_fit ? TPB / (S::TR / 2) : rg_fit;   // narrow regauge teams
+    static constexpr int rg_wide = TPB / S::TR < rg_fit ? TPB / S::TR : rg_fit;
+    static constexpr size_t rg = sizeof(RGSm<CHI>) * rg_teams;
     static constexpr size_t rv =
         sizeof(C<typename Mode::TS>) * (4 * CHI * CHI * CHI + 3 * CHI * CHI) * (TPB / S::TRV);
     static constexpr size_t init =
         (sizeof(double) * (6 * CHI + 4) + (Mode::mixed ? sizeof(cd) * (2 * CHI * CHI * CHI + 3 * CHI * CHI) : 0)) * S::NIT;
-    static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
     // bytes before the per-instance flags (which follow at this offset in the BP kernel)
     static constexpr size_t value = mx(mx((PH & PH_GATES) ? gate : 0, (PH & PH_BP) ? mx(bp, init) : 0),
                                        (PH & PH_REGAUGE) ? mx(rg, rv) : 0) + 16;
 };
+
+// The BP sweeps of one run (after bp_init_vertex) by vertex teams of TB lanes; false if a barrier gave up.
+template <int CHI, class Mode, unsigned PH, int V, int TB>
+__device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cur, unsigned char* smem) {
+    using S = Shape<CHI, V>;
+    const int team = threadIdx.x / TB, tid = threadIdx.x % TB;
+    const int tpb_teams = S::TPB / TB;
+    using CT_ = C<typename Mode::TS>;
+    using SMB = BPSm<CHI, Mode, TB>;
+    SMB& sm = reinterpret_cast<SMB*>(smem)[team];
+    double* bsum = reinterpret_cast<double*>(smem + sizeof(SMB) * tpb_teams);
+    // every block keeps its own copy of the per-instance state; all blocks take
+    // identical decisions from the same accumulators, so one barrier per sweep suffices
+    // (two when a sweep's lower bound falls under the threshold and the exact
+    // distance is computed afterwards)
+    int* done = reinterpret_cast<int*>(smem + SmemSize<CHI, Mode, PH, V>::value);
+    int* exnow = done + c.B;   // this sweep computes the exact distance inline
+    int* need = exnow + c.B;   // exact distance needed after the sweep
+    double* thr = reinterpret_cast<double*>(smem + SmemSize<CHI, Mode, PH, V>::value +
+                                            (3 * sizeof(int) * (size_t)c.B + 7) / 8 * 8);
+    double* thr_hi = thr + c.B;                               // bound that lets a sweep continue
+    float* thr3 = reinterpret_cast<float*>(thr_hi + c.B);     // inline-exact trigger
+    const double slack = Mode::mixed ? 1e-5 : 1e-12;   // rounding of the lower bound
+    for (int b = threadIdx.x; b < c.B; b += S::TPB) {
+        done[b] = 0;
+        exnow[b] = c.max_iter == 1;
+        need[b] = 0;
+        const double t = c.tol * (double)c.inst_m[b];
+        thr[b] = t;
+        thr_hi[b] = t / (1.0 - slack);
+        thr3[b] = (float)(3.0 * t);
+    }
+    if (tid == 0) sm.cached = -1;   // T and D0 changed in the init phase
+    if (tid < 3) sm.dsum[tid] = 0;
+    __syncthreads();
+    const int gteam = team * c.nblocks + blockIdx.x, nt = c.nblocks * tpb_teams;
+    const int inst0 = gteam < c.n ? c.vert_inst[gteam] : 0;   // the first round's vertex
+    SMB* all = reinterpret_cast<SMB*>(smem);
+    bool have_pre = false;
+    CT_ pre = CT_{0, 0};
+    int* sflag = reinterpret_cast<int*>(bsum + 48);   // [2]: need | open << 1, per sweep parity
+    if (threadIdx.x == 0) sflag[0] = sflag[1] = 0;
+    __syncthreads();
+    int it = 0;
+    for (; it < c.max_iter; ++it) {
+        double* acc = c.acc + (size_t)(it % 3) * c.B;
+        double* acc_next = c.acc + (size_t)((it + 1) % 3) * c.B;
+        double* ex = c.acc + (size_t)(3 + it % 3) * c.B;
+        double* ex_next = c.acc + (size_t)(3 + (it + 1) % 3) * c.B;
+        for (int b = blockIdx.x * S::TPB + threadIdx.x; b < c.B; b += c.nblocks * S::TPB) {
+            acc_next[b] = 0.0;
+            ex_next[b] = 0.0;
+        }
+        // rounds of one vertex per team; the block synchronises twice per round
+        for (int base = 0; base < c.n; base += nt) {
+            const int a = base + gteam;
+            int inst = 0;
+            bool act = false;
+            if (a < c.n) {
+                inst = base == 0 ? inst0 : c.vert_inst[a];
+                if (done[inst]) bp_copy_vertex<CHI, Mode>(c, a, tid, TB, cur);
+                else act = true;
+            }
+            if (act) bp_front<CHI, Mode, TB>(c, a, tid, team, cur, sm, base == 0 && have_pre, pre);
+            __syncthreads();
+            if (threadIdx.x < 32) bp_trace_rcp<CHI, Mode, TB>(all, tpb_teams);
+            __syncthreads();
+            if (act) bp_back<CHI, Mode, TB>(c, tid, team, cur, exnow[inst] != 0, sm, c.B == 1 ? nullptr : acc + inst);
+        }
+        cur ^= 1;
+        // one instance: the first warp sums the teams' distances between the block's
+        // barrier and its arrival at the grid barrier
+        if (!grid_sync_pre(gb, c.spin_limit, [&]() {
+                if (c.B != 1) return;
+                typename Mode::TS v = 0;
+                for (int q = threadIdx.x; q < 3 * tpb_teams; q += 32) v += all[q / 3].dsum[q % 3];
+    #pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (threadIdx.x == 0) atomicAdd(acc, (double)v);
+            }))
+            return false;
+        if (tid < 3) sm.dsum[tid] = 0;   // read by the first warp before the barrier
+        // the next sweep's incoming messages of this team's first vertex are loaded
+        // now, so that their latency overlaps the decision below
+        have_pre = false;
+        if (gteam < c.n && sm.cached == gteam && tid < 3 * CHI * CHI) {
+            const int in = sm.in_idx[tid / (CHI * CHI)];
+            if (in >= 0) pre = ldcg((const CT_*)c.msg[cur] + (size_t)in * CHI * CHI + tid % (CHI * CHI));
+            have_pre = true;
+        }
+        // stopping rule of App. B, per instance, evaluated identically by every block;
+        // the raw distance sums are kept and divided by |E| at the end
+        const bool last = it + 1 >= c.max_iter;
+        int open_local = 0, need_local = 0;
+        for (int b = threadIdx.x; b < c.B; b += S::TPB) {
+            if (done[b]) continue;
+            const double dsum = __ldcg(acc + b);
+            bool fin;
+            if (c.inst_m[b] == 0 || !(dsum == dsum)) {
+                fin = true;
+            } else if (exnow[b]) {
+                fin = last || dsum < thr[b];
+            } else if (!last && dsum >= thr_hi[b]) {
+                fin = false;   // the exact distance is at least the bound
+            } else {
+                need[b] = 1;
+                need_local = 1;
+                continue;
+            }
+            if (blockIdx.x == 0) {
+                c.inst_dist[b] = dsum;
+                c.inst_iters[b] = it + 1;
+                if (fin) c.inst_done[b] = 1;
+            }
+            if (fin) done[b] = 1;
+            else open_local = 1;
+            // the next sweep is exact inline when it is the last or when this
+            // sweep came within a factor 3 of the threshold
+            exnow[b] = (it + 2 >= c.max_iter) || (float)dsum < thr3[b];
+        }
+        // one block barrier for both flags (a word per sweep parity, reset one sweep ahead)
+        if (need_local | open_local) atomicOr(&sflag[it & 1], need_local | (open_local << 1));
+        __syncthreads();
+        const int fl = sflag[it & 1];
+        if (threadIdx.x == 0) sflag[(it + 1) & 1] = 0;
+        if (fl & 1) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) ++c.ctl->exact_passes;
+            bp_exact_pass<CHI, Mode, S::TPB, TB>(c, cur, need, sm, bsum + 32, ex);
+            if (!grid_sync(gb, c.spin_limit)) return false;
+            for (int b = threadIdx.x; b < c.B; b += S::TPB) {
+                if (!need[b]) continue;
+                need[b] = 0;
+                const double dsum = __ldcg(ex + b);
+                const bool fin = last || dsum < thr[b] || !(dsum == dsum);
+                if (blockIdx.x == 0) {
+                    c.inst_dist[b] = dsum;
+                    c.inst_iters[b] = it + 1;
+                    if (fin) c.inst_done[b] = 1;
+                }
+                if (fin) done[b] = 1;
+                else open_local = 1;
+                exnow[b] = 1;
+            }
+            if (!__syncthreads_or(open_local)) {
+                ++it;
+                break;
+            }
+        } else if (!(fl & 2)) {
+            ++it;
+            break;
+        }
+    }
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        int mi = 0, ncv = 0;
+        double md = 0.0;
+        for (int b = 0; b < c.B; ++b) {
+            const int mb = c.inst_m[b];
+            c.inst_dist[b] = mb > 0 ? c.inst_dist[b] / (double)mb : 0.0;
+            mi = c.inst_iters[b] > mi ? c.inst_iters[b] : mi;
+            md = c.inst_dist[b] > md ? c.inst_dist[b] : md;
+            if (!(c.inst_dist[b] < c.tol) && c.inst_m[b] > 0) ++ncv;
+        }
+        c.ctl->last_iters = mi;
+        c.ctl->last_dist = md;
+        c.ctl->not_conv = ncv;
+        c.ctl->sweeps_total += mi;
+        c.ctl->bp_calls += 1;
+        c.ctl->nc_calls += (ncv > 0) ? 1 : 0;
+        c.ctl->cur = cur;
+    }
+    return true;
+}
 
 template <int CHI, class Mode, unsigned PH, int V>
 __device__ __forceinline__ void anneal_body(const Ctx& c) {
@@ -1529,172 +1720,14 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
                 }
                 if (!grid_sync(gb, c.spin_limit)) return;
             }
-            const int team = threadIdx.x / S::TB, tid = threadIdx.x % S::TB;
-            const int tpb_teams = S::TPB / S::TB;
-            using CT_ = C<typename Mode::TS>;
-            using SMB = BPSm<CHI, Mode, S::TB>;
-            SMB& sm = reinterpret_cast<SMB*>(smem)[team];
-            double* bsum = reinterpret_cast<double*>(smem + sizeof(SMB) * tpb_teams);
-            // every block keeps its own copy of the per-instance state; all blocks take
-            // identical decisions from the same accumulators, so one barrier per sweep suffices
-            // (two when a sweep's lower bound falls under the threshold and the exact
-            // distance is computed afterwards)
-            int* done = reinterpret_cast<int*>(smem + SmemSize<CHI, Mode, PH, V>::value);
-            int* exnow = done + c.B;   // this sweep computes the exact distance inline
-            int* need = exnow + c.B;   // exact distance needed after the sweep
-            double* thr = reinterpret_cast<double*>(smem + SmemSize<CHI, Mode, PH, V>::value +
-                                                    (3 * sizeof(int) * (size_t)c.B + 7) / 8 * 8);
-            double* thr_hi = thr + c.B;                               // bound that lets a sweep continue
-            float* thr3 = reinterpret_cast<float*>(thr_hi + c.B);     // inline-exact trigger
-            const double slack = Mode::mixed ? 1e-5 : 1e-12;   // rounding of the lower bound
-            for (int b = threadIdx.x; b < c.B; b += S::TPB) {
-                done[b] = 0;
-                exnow[b] = c.max_iter == 1;
-                need[b] = 0;
-                const double t = c.tol * (double)c.inst_m[b];
-                thr[b] = t;
-                thr_hi[b] = t / (1.0 - slack);
-                thr3[b] = (float)(3.0 * t);
-            }
-            if (tid == 0) sm.cached = -1;   // T and D0 changed in the init phase
-            if (tid < 3) sm.dsum[tid] = 0;
-            __syncthreads();
-            const int gteam = team * c.nblocks + blockIdx.x, nt = c.nblocks * tpb_teams;
-            const int inst0 = gteam < c.n ? c.vert_inst[gteam] : 0;   // the first round's vertex
-            SMB* all = reinterpret_cast<SMB*>(smem);
-            bool have_pre = false;
-            CT_ pre = CT_{0, 0};
-            int* sflag = reinterpret_cast<int*>(bsum + 48);   // [2]: need | open << 1, per sweep parity
-            if (threadIdx.x == 0) sflag[0] = sflag[1] = 0;
-            __syncthreads();
-            int it = 0;
-            for (; it < c.max_iter; ++it) {
-                double* acc = c.acc + (size_t)(it % 3) * c.B;
-                double* acc_next = c.acc + (size_t)((it + 1) % 3) * c.B;
-                double* ex = c.acc + (size_t)(3 + it % 3) * c.B;
-                double* ex_next = c.acc + (size_t)(3 + (it + 1) % 3) * c.B;
-                for (int b = blockIdx.x * S::TPB + threadIdx.x; b < c.B; b += c.nblocks * S::TPB) {
-                    acc_next[b] = 0.0;
-                    ex_next[b] = 0.0;
-                }
-                // rounds of one vertex per team; the block synchronises twice per round
-                for (int base = 0; base < c.n; base += nt) {
-                    const int a = base + gteam;
-                    int inst = 0;
-                    bool act = false;
-                    if (a < c.n) {
-                        inst = base == 0 ? inst0 : c.vert_inst[a];
-                        if (done[inst]) bp_copy_vertex<CHI, Mode>(c, a, tid, S::TB, cur);
-                        else act = true;
-                    }
-                    if (act) bp_front<CHI, Mode, S::TB>(c, a, tid, team, cur, sm, base == 0 && have_pre, pre);
-                    __syncthreads();
-                    if (threadIdx.x < 32) bp_trace_rcp<CHI, Mode, S::TB>(all, tpb_teams);
-                    __syncthreads();
-                    if (act) bp_back<CHI, Mode, S::TB>(c, tid, team, cur, exnow[inst] != 0, sm, c.B == 1 ? nullptr : acc + inst);
-                }
-                cur ^= 1;
-                // one instance: the first warp sums the teams' distances between the block's
-                // barrier and its arrival at the grid barrier
-                if (!grid_sync_pre(gb, c.spin_limit, [&]() {
-                        if (c.B != 1) return;
-                        typename Mode::TS v = 0;
-                        for (int q = threadIdx.x; q < 3 * tpb_teams; q += 32) v += all[q / 3].dsum[q % 3];
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                        if (threadIdx.x == 0) atomicAdd(acc, (double)v);
-                    }))
-                    return;
-                if (tid < 3) sm.dsum[tid] = 0;   // read by the first warp before the barrier
-                // the next sweep's incoming messages of this team's first vertex are loaded
-                // now, so that their latency overlaps the decision below
-                have_pre = false;
-                if (gteam < c.n && sm.cached == gteam && tid < 3 * CHI * CHI) {
-                    const int in = sm.in_idx[tid / (CHI * CHI)];
-                    if (in >= 0) pre = ldcg((const CT_*)c.msg[cur] + (size_t)in * CHI * CHI + tid % (CHI * CHI));
-                    have_pre = true;
-                }
-                // stopping rule of App. B, per instance, evaluated identically by every block;
-                // the raw distance sums are kept and divided by |E| at the end
-                const bool last = it + 1 >= c.max_iter;
-                int open_local = 0, need_local = 0;
-                for (int b = threadIdx.x; b < c.B; b += S::TPB) {
-                    if (done[b]) continue;
-                    const double dsum = __ldcg(acc + b);
-                    bool fin;
-                    if (c.inst_m[b] == 0 || !(dsum == dsum)) {
-                        fin = true;
-                    } else if (exnow[b]) {
-                        fin = last || dsum < thr[b];
-                    } else if (!last && dsum >= thr_hi[b]) {
-                        fin = false;   // the exact distance is at least the bound
-                    } else {
-                        need[b] = 1;
-                        need_local = 1;
-                        continue;
-                    }
-                    if (blockIdx.x == 0) {
-                        c.inst_dist[b] = dsum;
-                        c.inst_iters[b] = it + 1;
-                        if (fin) c.inst_done[b] = 1;
-                    }
-                    if (fin) done[b] = 1;
-                    else open_local = 1;
-                    // the next sweep is exact inline when it is the last or when this
-                    // sweep came within a factor 3 of the threshold
-                    exnow[b] = (it + 2 >= c.max_iter) || (float)dsum < thr3[b];
-                }
-                // one block barrier for both flags (a word per sweep parity, reset one sweep ahead)
-                if (need_local | open_local) atomicOr(&sflag[it & 1], need_local | (open_local << 1));
-                __syncthreads();
-                const int fl = sflag[it & 1];
-                if (threadIdx.x == 0) sflag[(it + 1) & 1] = 0;
-                if (fl & 1) {
-                    if (blockIdx.x == 0 && threadIdx.x == 0) ++c.ctl->exact_passes;
-                    bp_exact_pass<CHI, Mode, S::TPB, S::TB>(c, cur, need, sm, bsum + 32, ex);
-                    if (!grid_sync(gb, c.spin_limit)) return;
-                    for (int b = threadIdx.x; b < c.B; b += S::TPB) {
-                        if (!need[b]) continue;
-                        need[b] = 0;
-                        const double dsum = __ldcg(ex + b);
-                        const bool fin = last || dsum < thr[b] || !(dsum == dsum);
-                        if (blockIdx.x == 0) {
-                            c.inst_dist[b] = dsum;
-                            c.inst_iters[b] = it + 1;
-                            if (fin) c.inst_done[b] = 1;
-                        }
-                        if (fin) done[b] = 1;
-                        else open_local = 1;
-                        exnow[b] = 1;
-                    }
-                    if (!__syncthreads_or(open_local)) {
-                        ++it;
-                        break;
-                    }
-                } else if (!(fl & 2)) {
-                    ++it;
-                    break;
-                }
-            }
-            __syncthreads();
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                int mi = 0, ncv = 0;
-                double md = 0.0;
-                for (int b = 0; b < c.B; ++b) {
-                    const int mb = c.inst_m[b];
-                    c.inst_dist[b] = mb > 0 ? c.inst_dist[b] / (double)mb : 0.0;
-                    mi = c.inst_iters[b] > mi ? c.inst_iters[b] : mi;
-                    md = c.inst_dist[b] > md ? c.inst_dist[b] : md;
-                    if (!(c.inst_dist[b] < c.tol) && c.inst_m[b] > 0) ++ncv;
-                }
-                c.ctl->last_iters = mi;
-                c.ctl->last_dist = md;
-                c.ctl->not_conv = ncv;
-                c.ctl->sweeps_total += mi;
-                c.ctl->bp_calls += 1;
-                c.ctl->nc_calls += (ncv > 0) ? 1 : 0;
-                c.ctl->cur = cur;
-            }
+            // FP64 at CHI <= 4 with at most one vertex per block: teams of four warps, one per
+            // sub-partition, halve a sweep's FP64 time (10.4 -> 5.6 us); with two or more vertices per
+            // block the pipes are as busy with teams of two
+            constexpr int WIDE = SmemSize<CHI, Mode, PH, V>::WIDE_TB;
+            bool ok;
+            if (WIDE != S::TB && c.n <= c.nblocks) ok = bp_sweeps<CHI, Mode, PH, V, WIDE>(c, gb, cur, smem);
+            else ok = bp_sweeps<CHI, Mode, PH, V, S::TB>(c, gb, cur, smem);
+            if (!ok) return;
         }
         if constexpr ((PH & PH_REGAUGE) != 0u) {
             if (c.rgate && blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1703,10 +1736,17 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
             }
             if (skip_regauge) continue;
             {
-                const int team = threadIdx.x / S::TR, tid = threadIdx.x % S::TR;
-                RGSm<CHI>& sm = reinterpret_cast<RGSm<CHI>*>(smem)[team];
-                const int gteam = team * c.nblocks + blockIdx.x, nt = c.nblocks * (S::TPB / S::TR);
-                for (int e = gteam; e < c.m; e += nt) regauge_edge<CHI, Mode>(c, e, tid, team, cur, sm);
+                using SZ = SmemSize<CHI, Mode, PH, V>;
+                auto edges = [&](auto lanes, int teams) {
+                    constexpr int TEAM = decltype(lanes)::value;
+                    const int team = threadIdx.x / TEAM, tid = threadIdx.x % TEAM;
+                    if (team >= teams) return;
+                    RGSm<CHI>& sm = reinterpret_cast<RGSm<CHI>*>(smem)[team];
+                    for (int e = team * c.nblocks + blockIdx.x; e < c.m; e += c.nblocks * teams)
+                        regauge_edge<CHI, Mode, TEAM>(c, e, tid, team, cur, sm);
+                };
+                if (c.m <= c.nblocks * (512 / S::TR)) edges(std::integral_constant<int, S::TR>{}, SZ::rg_wide);
+                else edges(std::integral_constant<int, S::TR / 2>{}, SZ::rg_teams);
                 if (!grid_sync(gb, c.spin_limit)) return;
             }
             {
