@@ -353,9 +353,9 @@ __device__ __forceinline__ float fast_rcp(float x) {
 // (460 cycles per step of N = 8, against about 700 through shared memory).  keep < N: pairs without
 // a column among the keep largest (norms within a factor 4 of the keep-th count) do not ask for
 // another sweep, and a kept column with a smaller one is judged by the kept column's norm, as in
-// refined_svd; that saves 0.6 to 1 of 4.6 to 5.3 sweeps of the gates.
-template <int N>
-__device__ int jacobi_v32(const C<float>* A, C<float>* V, int g, unsigned gmask, unsigned pair_mask, int keep) {
+// refined_svd; that saves 0.6 to 1 of 4.6 to 5.3 sweeps of the gates.  OUT: A ends as U S.
+template <int N, bool OUT = false>
+__device__ int jacobi_v32(C<float>* A, C<float>* V, int g, unsigned gmask, unsigned pair_mask, int keep) {
     using CF = C<float>;
     constexpr int LN = N * N / 2, LAST = N / 2 - 1;
     static_assert(LN <= 32, "the group lives in one warp");
@@ -425,13 +425,17 @@ __device__ int jacobi_v32(const C<float>* A, C<float>* V, int g, unsigned gmask,
     // after a whole sweep every column is back at its pair
     V[k * N + r] = va;
     V[(N - 1 - k) * N + r] = vb;
+    if constexpr (OUT) {
+        A[k * N + r] = a;
+        A[(N - 1 - k) * N + r] = b;
+    }
     return sweep;
 }
 
 // The same for a group of several warps (N = 16, 32): the columns go to the neighbouring pairs
 // through shared memory, in two buffers used in turn, so that a step has one barrier.  A, V: N^2
 // entries each; buf: 2 N^2 entries; nrm: 2 N floats.  V32 ends in V.
-template <int N, typename Group>
+template <int N, bool OUT, typename Group>
 __device__ int jacobi_v32_team(C<float>* A, C<float>* V, C<float>* buf, float* nrm, int g, const Group& grp,
                                unsigned pair_mask, int keep) {
     using CF = C<float>;
@@ -497,6 +501,10 @@ __device__ int jacobi_v32_team(C<float>* A, C<float>* V, C<float>* buf, float* n
     grp.sync();
     V[k * N + r] = va;
     V[(N - 1 - k) * N + r] = vb;
+    if constexpr (OUT) {
+        A[k * N + r] = a;
+        A[(N - 1 - k) * N + r] = b;
+    }
     return sweep;
 }
 
@@ -796,7 +804,7 @@ __device__ int svd32_unitary(C<double>* V, C<float>* A32, C<float>* V32, double*
         sw = jacobi_v32<N>(A32, V32, g, group_mask<LN>(), pair_mask, keep);
         grp.sync();
     } else {
-        sw = jacobi_v32_team<N>(A32, V32, reinterpret_cast<C<float>*>(V), reinterpret_cast<float*>(nrm), g, grp, pair_mask,
+        sw = jacobi_v32_team<N, false>(A32, V32, reinterpret_cast<C<float>*>(V), reinterpret_cast<float*>(nrm), g, grp, pair_mask,
                                 keep);
         grp.sync();
     }

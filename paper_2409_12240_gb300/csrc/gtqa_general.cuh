@@ -52,7 +52,7 @@ struct GenSm {
     C<R> Rf[2][S::NC][S::NC];  // R factors, [side][row][column]
     C<R> M[S::NM * S::NM];
     C<R> V[S::NM * S::NM];
-    C<R> T[sizeof(R) == 8 ? S::NM * S::NM : 1];   // scratch of refined_svd
+    C<R> T[sizeof(R) == 8 ? S::NM * S::NM : 2 * S::NM * S::NM];   // scratch of the SVD
     cf M32[sizeof(R) == 8 ? S::NM * S::NM : 1];
     cf V32[sizeof(R) == 8 ? S::NM * S::NM : 1];
     C<R> U[16];
@@ -74,14 +74,17 @@ __device__ __forceinline__ SvdCount core_svd(C<double>* M, C<double>* V, C<float
     return refined_svd<NM, true>(M, V, M32, V32, T, n2, relmask, g, grp, group_mask<NM>(), cut, chi, 1e-8f, 1e-15);
 }
 template <int NM, typename Group>
-__device__ __forceinline__ SvdCount core_svd(C<float>* M, C<float>* V, C<float>*, C<float>*, C<float>*, double* n2,
+__device__ __forceinline__ SvdCount core_svd(C<float>* M, C<float>* V, C<float>*, C<float>*, C<float>* T, double* n2,
                                              unsigned*, int g, const Group& grp, double, int) {
+    constexpr int LN = NM * NM / 2;
     SvdCount cnt;
-    int rot = 0;
-    cnt.sweeps32 = jacobi_svd<NM, float>(M, V, g, grp, group_mask<NM>(), 1e-6f, 60, true, &rot, 1e-3f);
+    if constexpr (LN <= 32) {
+        cnt.sweeps32 = jacobi_v32<NM, true>(M, V, g, group_mask<LN>(), group_mask<NM>(), NM);
+    } else {
+        cnt.sweeps32 = jacobi_v32_team<NM, true>(M, V, T, reinterpret_cast<float*>(n2), g, grp, group_mask<NM>(), NM);
+    }
     cnt.passes = cnt.sweeps32;
     cnt.pairs = cnt.sweeps32 * (NM - 1) * (NM / 2);
-    cnt.rot = rot;
     grp.sync();
     if (g < NM) {
         float s = 0.f;

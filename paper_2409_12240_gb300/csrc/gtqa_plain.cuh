@@ -609,6 +609,9 @@ __device__ __forceinline__ void plain_edge_svd(C<RC>* A, C<RC>* V, PlainEdgeSm<C
         prune_noise<CHI>(A, g, grp);
         refined_svd<CHI, true>(A, V, sm.A32[x], sm.V32[x], sm.T[x], sm.n2[x], nullptr, g, grp, group_mask<CHI>(), cut, CHI,
                                1e-8f, 1e-15);
+    } else if constexpr (CHI * CHI / 2 <= 32) {
+        jacobi_v32<CHI, true>(A, V, g, group_mask<CHI * CHI / 2>(), group_mask<CHI>(), CHI);
+        grp.sync();
     } else {
         jacobi_svd<CHI, RC>(A, V, g, grp, group_mask<CHI>(), (RC)1e-6, 60, true, nullptr, (RC)1e-3);
     }
@@ -983,7 +986,7 @@ struct PlainGateSm {
     C<R> U[4][CHI][S::NR];     // scaled reflectors, then the new tensors
     C<R> M[S::NM * S::NM];
     C<R> V[S::NM * S::NM];     // first the R factors [block][row][col]
-    C<R> T[sizeof(R) == 8 ? S::NM * S::NM : 1];
+    C<R> T[sizeof(R) == 8 ? S::NM * S::NM : (S::LS > 32 ? 2 * S::NM * S::NM : 1)];   // scratch of the SVD
     cf M32[sizeof(R) == 8 ? S::NM * S::NM : 1];
     cf V32[sizeof(R) == 8 ? S::NM * S::NM : 1];
     double lab[CHI];
@@ -1159,7 +1162,7 @@ struct Gate16Sm {
     static constexpr int CHI = 16, NM = 32, NR = 256;
     CR M[NM * NM];
     CR V[NM * NM];            // first the R factors [block][row][col]
-    CR T[NM * NM];            // scratch of the SVD; then Z [block][j][col]
+    CR T[(sizeof(R) == 8 ? 1 : 2) * NM * NM];   // scratch of the SVD; then Z [block][j][col]
     cf M32[sizeof(R) == 8 ? NM * NM : 1];
     cf V32[sizeof(R) == 8 ? NM * NM : 1];
     CR SU[4][CHI][CHI];       // u_j^H u_k, j < k
