@@ -174,6 +174,7 @@ struct GateMeta {
 template <int CHI, class Mode>
 struct GateSm {
     using TS = typename Mode::TS;
+    static constexpr int PB = CHI == 2 ? 2 : 8;   // four lanes each
     C<TS> U[4][CHI][CHI * CHI];   // [block][col][row]: scaled reflectors, then the new tensors
     cd M[4 * CHI * CHI];
     cd V[4 * CHI * CHI];       // first the R factors [block][row][col], then V
@@ -183,7 +184,7 @@ struct GateSm {
     double lab[CHI];
     double sig[2 * CHI];
     double isig[2 * CHI];      // 1 / sig
-    cd ph[4];
+    cd phases[PB * 4];         // diagonal gate phases of the team's next PB gates
     int perm[2 * CHI];
     int keep;
     unsigned relmask;          // columns that decide the stop of a closing polish
@@ -310,8 +311,31 @@ __device__ __forceinline__ int truncate_core(const double* n2, const int* perm, 
     return keep;
 }
 
+// The diagonal gate phases of gates first .. first + PB - 1 of the team's sequence (colour by colour,
+// every nt-th gate of a colour from gteam on), four lanes per gate: the FP64 sine and cosine (about 50
+// instructions) once per PB gates instead of once per gate.
 template <int CHI, class Mode>
-__device__ void gate_edge(const Ctx& c, const GateMeta& gm_, int tid, int team, GateSm<CHI, Mode>& sm, double tZ,
+__device__ void gate_phases(const Ctx& c, int first, int gteam, int nt, int tid, GateSm<CHI, Mode>& sm, double tZ) {
+    constexpr int PB = GateSm<CHI, Mode>::PB;
+    if (tid >= 4 * PB) return;
+    int r = first + tid / 4, idx = -1;
+    for (int col = 0; col < c.ncol && idx < 0; ++col) {
+        const int beg = c.colour_off[col] + gteam, end = c.colour_off[col + 1];
+        const int cnt = beg < end ? (end - beg + nt - 1) / nt : 0;
+        if (r < cnt) idx = beg + r * nt;
+        else r -= cnt;
+    }
+    if (idx < 0) return;
+    const int4 a = c.gates[idx].a;
+    const double ha = c.hd[a.y], hb = c.hd[a.z], Je = c.J[a.x];
+    const double za = 1.0 - 2.0 * ((tid >> 1) & 1), zb = 1.0 - 2.0 * (tid & 1);
+    double sn, cs;
+    sincos(-tZ * (Je * za * zb + ha * za + hb * zb), &sn, &cs);
+    sm.phases[tid] = cd{cs, sn};
+}
+
+template <int CHI, class Mode>
+__device__ void gate_edge(const Ctx& c, const GateMeta& gm_, const cd* ph, int tid, int team, GateSm<CHI, Mode>& sm,
                           double cX, double sX, bool pre, double cXp, double sXp) {
     using TS = typename Mode::TS;
     using CT = C<TS>;
@@ -343,14 +367,6 @@ __device__ void gate_edge(const Ctx& c, const GateMeta& gm_, int tid, int team, 
         w0 = lam_get(c.lam, CHI, e0, l / CHI) * lam_get(c.lam, CHI, e1, l % CHI);
         w1 = lam_get(c.lam, CHI, e0, (l + G) / CHI) * lam_get(c.lam, CHI, e1, l % CHI);
         if (tid < CHI) sm.lab[tid] = __ldcg(c.lam + (size_t)e * CHI + tid);
-        // the four diagonal gate phases
-        if (tid < 4) {
-            const double ha = c.hd[gm_.a.y], hb = c.hd[gm_.a.z], Je = c.J[e];
-            const double za = 1.0 - 2.0 * (tid >> 1), zb = 1.0 - 2.0 * (tid & 1);
-            double sn, cs;
-            sincos(-tZ * (Je * za * zb + ha * za + hb * zb), &sn, &cs);
-            sm.ph[tid] = cd{cs, sn};
-        }
 #pragma unroll
         for (int cc = 0; cc < CHI; ++cc) {
             y0[cc] = ccast<double>(t0[cc]);
@@ -365,7 +381,7 @@ __device__ void gate_edge(const Ctx& c, const GateMeta& gm_, int tid, int team, 
             y1[cc] = w1 * y1[cc];
         }
         if (tid == 0) sm.nrot = 0;
-        team_bar<TEAM>(team);   // lab and the phases; the previous edge's readers of sm are done
+        team_bar<TEAM>(team);   // lab; the previous edge's readers of sm are done
     }
 
     // ---- Householder QR of the four CHI^2 x CHI blocks; R (side a times lambda) goes to sm.V ----
@@ -386,7 +402,7 @@ __device__ void gate_edge(const Ctx& c, const GateMeta& gm_, int tid, int team, 
         cd acc = cd{0.0, 0.0};
         const int j0 = r > rp ? r : rp;
         for (int j = j0; j < CHI; ++j) acc = cfma(Ra[j], Rb[j], acc);
-        sm.M[t] = sm.ph[2 * ia + ib] * acc;
+        sm.M[t] = ph[2 * ia + ib] * acc;
     }
     team_bar<TEAM>(team);
     // rounding-level entries of the core (graded spectra of the early anneal) are zeroed first
@@ -1235,8 +1251,7 @@ struct RGSm {
     cd Vm[2][CHI * CHI];
     double w[2][CHI];
     double wq[2][CHI], wiq[2][CHI];   // w^{1/2} and w^{-1/2} of the kept eigenvalues, else 0
-    cd sq[2][CHI * CHI];
-    cd isq[2][CHI * CHI];
+    cd Y[2][CHI * CHI];               // scaled singular vectors of M
     cd M[CHI * CHI];
     cd VM[CHI * CHI];
     double sig[CHI];
@@ -1321,27 +1336,15 @@ __device__ void regauge_edge(const Ctx& c, int e, int tid, int team, int cur, RG
         sm.wq[x][k] = kept ? wk * isq : 0.0;
     }
     team_bar<TEAM>(team);
-    for (int t = tid; t < 2 * CC; t += TEAM) {
-        const int x = t / CC, r = t % CC;
-        const int j = r / CHI, jp = r % CHI;
-        cd s1 = cd{0.0, 0.0}, s2 = cd{0.0, 0.0};
-        for (int k = 0; k < CHI; ++k) {
-            const double isq = sm.wiq[x][k];
-            if (!(isq > 0.0)) continue;
-            const double sq = sm.wq[x][k];
-            const cd vv = sm.Vm[x][k * CHI + j] * conj(sm.Vm[x][k * CHI + jp]);
-            s1 = cfma(cd{sq, 0.0}, vv, s1);
-            s2 = cfma(cd{isq, 0.0}, vv, s2);
-        }
-        sm.sq[x][r] = s1;
-        sm.isq[x][r] = s2;
-    }
-    team_bar<TEAM>(team);
+    // with m_x = V_x w_x V_x^H:  M = (m_0^{1/2})^T m_1^{1/2} = conj(V_0) B V_1^H with
+    // B = w_0^{1/2} (V_0^T V_1) w_1^{1/2}, so the SVD of B gives U = conj(V_0) U', V = V_1 V', and the
+    // transforms are X_a = conj(V_0) w_0^{-1/2} U' ||S||^{1/2}, X_b = conj(V_1) w_1^{-1/2} conj(V') ||S||^{1/2}:
+    // a third of the products that forming m^{1/2} and m^{-1/2} takes
     for (int t = tid; t < CC; t += TEAM) {
         const int k = t % CHI, l = t / CHI;
         cd acc = cd{0.0, 0.0};
-        for (int j = 0; j < CHI; ++j) acc = cfma(sm.sq[0][j * CHI + k], sm.sq[1][j * CHI + l], acc);
-        sm.M[l * CHI + k] = acc;
+        for (int j = 0; j < CHI; ++j) acc = cfma(sm.Vm[0][k * CHI + j], sm.Vm[1][l * CHI + j], acc);
+        sm.M[l * CHI + k] = (sm.wq[0][k] * sm.wq[1][l]) * acc;
     }
     team_bar<TEAM>(team);
     if (tid < GJ) {
@@ -1381,20 +1384,20 @@ __device__ void regauge_edge(const Ctx& c, int e, int tid, int team, int cur, RG
         }
     }
     team_bar<TEAM>(team);
+    // w_x^{-1/2} U' ||S||^{1/2} (x = 0) and w_x^{-1/2} conj(V') ||S||^{1/2} (x = 1), [column][row]; 0 beyond
+    // the kept singular values
     for (int t = tid; t < 2 * CC; t += TEAM) {
-        const int x = t / CC, r = t % CC;
-        const int jpp = r / CHI, j = r % CHI;
+        const int x = t / CC, r = t % CC, j = r / CHI, k = r % CHI;
         const int pc = sm.perm[j];
-        const double s = sm.sig[pc];
+        const bool kept = sm.scal[0] > 0.0 && sm.sig[pc] > c.svd_cut * sm.sig[sm.perm[0]];
+        const double f = kept ? sm.wiq[x][k] * sm.scal[1] : 0.0;
+        sm.Y[x][r] = x == 0 ? (f * sm.isig[pc]) * sm.M[pc * CHI + k] : f * conj(sm.VM[pc * CHI + k]);
+    }
+    team_bar<TEAM>(team);
+    for (int t = tid; t < 2 * CC; t += TEAM) {
+        const int x = t / CC, r = t % CC, jpp = r / CHI, j = r % CHI;
         cd acc = cd{0.0, 0.0};
-        const bool kept = sm.scal[0] > 0.0 && s > c.svd_cut * sm.sig[sm.perm[0]];
-        if (kept) {
-            for (int jp = 0; jp < CHI; ++jp) {
-                const cd u = (x == 0) ? sm.isig[pc] * sm.M[pc * CHI + jp] : conj(sm.VM[pc * CHI + jp]);
-                acc = cfma(sm.isq[x][jp * CHI + jpp], u, acc);
-            }
-            acc = sm.scal[1] * acc;
-        }
+        for (int k = 0; k < CHI; ++k) acc = cfmac(sm.Vm[x][k * CHI + jpp], sm.Y[x][j * CHI + k], acc);
         c.X[((size_t)e * 2 + x) * CC + r] = acc;
     }
 }
@@ -1673,14 +1676,18 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
             const int team = threadIdx.x / S::TG, tid = threadIdx.x % S::TG;
             GateSm<CHI, Mode>& sm = reinterpret_cast<GateSm<CHI, Mode>*>(smem)[team];
             const int gteam = team * c.nblocks + blockIdx.x;
+            constexpr int PB = GateSm<CHI, Mode>::PB;
+            int seq = 0;   // gates this team has run in the layer
+            gate_phases<CHI, Mode>(c, 0, gteam, nteams_total_g, tid, sm, tZ);
             GateMeta next = {};
             if (c.ncol > 0 && c.colour_off[0] + gteam < c.colour_off[1]) next = c.gates[c.colour_off[0] + gteam];
             for (int col = 0; col < c.ncol; ++col) {
                 const int beg = c.colour_off[col], end = c.colour_off[col + 1];
-                for (int idx = beg + gteam; idx < end; idx += nteams_total_g) {
+                for (int idx = beg + gteam; idx < end; idx += nteams_total_g, ++seq) {
                     const GateMeta gm = next;
                     if (idx + nteams_total_g < end) next = c.gates[idx + nteams_total_g];
-                    gate_edge<CHI, Mode>(c, gm, tid, team, sm, tZ, cX, sX, pre, cXp, sXp);
+                    if (seq % PB == 0 && seq > 0) gate_phases<CHI, Mode>(c, seq, gteam, nteams_total_g, tid, sm, tZ);
+                    gate_edge<CHI, Mode>(c, gm, sm.phases + 4 * (seq % PB), tid, team, sm, cX, sX, pre, cXp, sXp);
                 }
                 if (col == c.ncol - 1)
                     for (int q = gteam; q < c.n_iso; q += nteams_total_g)

@@ -682,15 +682,16 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 // refinement below costs two or three N^3 products (N = 8: 130 to 200), all lanes busy and no
 // chain of steps, and one or two passes suffice:
 //   1. one-sided Jacobi on an FP32 copy (scaled by the exponent of its largest entry) gives V32;
-//   2. V = V32 is made unitary: V <- V (I - E/2), E = V^H V - I from an FP64 Gram product, the
-//      correction's product in FP32 (|E| ~ 1e-6, so its rounding lies near 1e-13); F64: twice,
-//      which leaves rounding level;
+//   2. V = V32 is made unitary: V <- V (I - E/2), E = V^H V - I in compensated FP32, the
+//      correction's product in FP32 (|E| ~ 1e-6, so its rounding lies near 1e-13); F64: once more
+//      with an FP64 Gram product, which leaves rounding level;
 //   3. W = A V in FP64;
 //   4. passes: the Gram matrix of W in FP64, every pair's rotation parameter (as in
 //      jacobi_polish: K_pq = tau gamma_pq) at once, and W <- W (I + K + K^2/2), V likewise, for
 //      all pairs with |K_pq| <= 1e-4.  K is antihermitian, so the factor is unitary up to
-//      |K|^4/4 < 3e-17, and the off-diagonals shrink to products of their sizes.  The passes
-//      end once every pair was below `stop` (relative to its columns) before its pass.
+//      |K|^4/4 < 3e-17, and the off-diagonals shrink to products of their sizes.  Without F64 the
+//      corrections are formed in FP32 where every kept column moves by less than 1e-3 of its length
+//      (12 FP64 instructions per warp instead of 64).  The passes end once every pair was below `stop` (relative to its columns) before its pass.
 //      A pair with a larger K (nearly equal or not yet resolved columns) is rotated by
 //      FP64 Jacobi steps (only the steps of the schedule that hold such a pair) or, for N >= 16
 //      with many of them, by FP32 Jacobi on those and all shorter columns of W, rescaled,
@@ -734,6 +735,61 @@ __device__ __forceinline__ C<double> gram(const C<double>* A, double* nrm, int g
         }
     grp.sync();
     return gam;
+}
+// acc + a b with the rounding errors of the product and of the sum collected in err (Dekker / Knuth
+// two-product and two-sum; the result acc + err has about twice the FP32 precision)
+__device__ __forceinline__ void dot2(float a, float b, float& acc, float& err) {
+    const float p = __fmul_rn(a, b), e = fmaf(a, b, -p);   // (intrinsics: not to be contracted)
+    const float t = __fadd_rn(acc, p), z = __fsub_rn(t, acc);
+    err += e + (__fsub_rn(acc, __fsub_rn(t, z)) + __fsub_rn(p, z));
+    acc = t;
+}
+// -(V^H V - I) / 2 of an FP32 matrix into L.  The entries are differences of about 1e-6 and are
+// needed to 1e-12: twice the FP32 precision in FP32 instructions (about 40 per complex product,
+// against 4 FP64 ones that take 64 cycles each).
+template <int N, typename Group>
+__device__ __forceinline__ void half_defect32(const C<float>* V, C<float>* L, int g, const Group& grp, bool has, int p,
+                                              int q) {
+    if (has) {
+        float x = 0.f, xe = 0.f, y = 0.f, ye = 0.f;
+        for (int i = 0; i < N; ++i) {
+            const int r = (i + g) & (N - 1);
+            const C<float> a = V[p * N + r], b = V[q * N + r];
+            dot2(a.x, b.x, x, xe);
+            dot2(a.x, b.y, y, ye);
+            dot2(a.y, b.y, x, xe);
+            dot2(-a.y, b.x, y, ye);
+        }
+        const C<float> e = C<float>{-0.5f * (x + xe), -0.5f * (y + ye)};
+        L[q * N + p] = e;
+        L[p * N + q] = conj(e);
+    }
+    if (g < N) {
+        float x = -1.f, xe = 0.f;
+        for (int r = 0; r < N; ++r) {
+            const C<float> a = V[g * N + r];
+            dot2(a.x, a.x, x, xe);
+            dot2(a.y, a.y, x, xe);
+        }
+        L[g * N + g] = C<float>{-0.5f * (x + xe), 0.f};
+    }
+    grp.sync();
+}
+// X <- X + X32 L with the product in FP32, X32 <- X rounded first.
+template <int N, typename Group>
+__device__ __forceinline__ void correct32(C<double>* X, C<float>* X32, const C<float>* L, int g, const Group& grp) {
+    constexpr int LN = N * N / 2;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) X32[g + j * LN] = ccast<float>(X[g + j * LN]);
+    grp.sync();
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int t = g + j * LN, q = t / N, r = t % N;
+        C<float> acc = C<float>{0.f, 0.f};
+        for (int p = 0; p < N; ++p) acc = cfma(X32[p * N + r], L[q * N + p], acc);
+        X[t] = X[t] + ccast<double>(acc);
+    }
+    grp.sync();
 }
 // V <- V + V32 L with the product in FP32, and V32 <- V rounded.
 template <int N, typename Group>
@@ -811,7 +867,9 @@ __device__ int svd32_unitary(C<double>* V, C<float>* A32, C<float>* V32, double*
 #pragma unroll
     for (int j = 0; j < 2; ++j) V[g + j * LN] = ccast<double>(V32[g + j * LN]);
     grp.sync();
-    for (int pass = 0; pass < (F64 ? 2 : 1); ++pass) {
+    half_defect32<N>(V32, A32, g, grp, has, p, q);
+    add_product32<N>(V, V32, A32, g, grp);
+    if constexpr (F64) {
         const C<double> e = gram<N>(V, nrm, g, grp, has, p, q);
         if (has) {
             const C<float> ef = ccast<float>(-0.5 * e);
@@ -864,7 +922,9 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         ++cnt.passes;
         cnt.pairs += NP;
         CF K = CF{0.f, 0.f};
-        unsigned flags = 0u;   // 1: a pair above stop, 2: one of those with a large K, 4: |K| > 1e-8, 8: any K
+        // 1: a pair above stop, 2: one of those with a large K, 4: |K| > 1e-8, 8: any K, 16: a K that moves
+        // the pair's shorter column by more than 1e-3 of its length
+        unsigned flags = 0u;
         if (has) {
             const double al = nrm[p], be = nrm[q];
             const long long la = __double_as_longlong(al), lb = __double_as_longlong(be);
@@ -902,6 +962,7 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                     } else {
                         flags |= 8u;
                         if (k2 > 1e-16f) flags |= 4u;
+                        if (k2 * fmaxf(an, bn) > 1e-6f * fminf(an, bn) && (rp && rq)) flags |= 16u;
                     }
                 }
             }
@@ -917,20 +978,25 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
             if (g < N) A32[g * N + g] = CF{0.f, 0.f};
             grp.sync();
             CF l[2];
+            // mixed mode: the corrections W L and V L in FP32, whose rounding is then below 1e-10 of every
+            // kept column (its storage is complex64); else in FP64
+            const bool low = !F64 && !(flags & 16u);
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int t = g + j * LN, c = t / N, r = t % N;
-                CD x = ccast<double>(A32[t]);
+                const CF k1 = A32[t];
                 CF k2 = CF{0.f, 0.f};
-                if (flags & 4u) {
+                if (flags & 4u)
                     for (int s = 0; s < N; ++s) k2 = cfma(A32[s * N + r], A32[c * N + s], k2);
-                    x = x + ccast<double>(0.5f * k2);
+                l[j] = k1 + 0.5f * k2;
+                if (!low) {
+                    CD x = ccast<double>(k1);
+                    if (flags & 4u) x = x + ccast<double>(0.5f * k2);
+                    T[t] = x;
                 }
-                l[j] = A32[t] + 0.5f * k2;
-                T[t] = x;
             }
             grp.sync();
-            mul64<N, true>(A, T, g, grp);
+            if (!low) mul64<N, true>(A, T, g, grp);
             if (F64 && (flags & 4u)) {
                 mul64<N, true>(V, T, g, grp);
             } else {
@@ -940,6 +1006,7 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                     if constexpr (F64) V32[g + j * LN] = ccast<float>(V[g + j * LN]);
                 }
                 grp.sync();
+                if (low) correct32<N>(A, reinterpret_cast<CF*>(T), A32, g, grp);
                 add_product32<N>(V, V32, A32, g, grp);
             }
         }

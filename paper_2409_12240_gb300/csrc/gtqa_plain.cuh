@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(512, 1) plain_bp_kernel(PlainBPArgs a) {
 template <int CHI, typename RC>
 struct PlainEdgeSm {
     static constexpr int CC = CHI * CHI;
-    C<RC> Am[2][CC], Vm[2][CC], sqm[2][CC], isq[2][CC], M[CC], VM[CC];
+    C<RC> Am[2][CC], Vm[2][CC], Y[2][CC], M[CC], VM[CC];
     C<RC> T[2][sizeof(RC) == 8 ? CC : 1];
     cf A32[2][sizeof(RC) == 8 ? CC : 1], V32[2][sizeof(RC) == 8 ? CC : 1];
     double n2[2][CHI];
@@ -676,29 +676,13 @@ __global__ void __launch_bounds__(CHI * CHI) plain_regauge_edge_kernel(PlainArgs
         sm.wq[x][k] = is > (RC)0 ? wk * is : (RC)0;
     }
     bar();
-    for (int t = tid; t < 2 * CC; t += NT) {
-        const int x = t / CC, r = t % CC;
-        const int j = r / CHI, jp = r % CHI;
-        C<RC> s1 = C<RC>{(RC)0, (RC)0}, s2 = C<RC>{(RC)0, (RC)0};
-        for (int k = 0; k < CHI; ++k) {
-            const RC is = sm.wiq[x][k];
-            if (!(is > (RC)0)) continue;
-            const RC sq = sm.wq[x][k];
-            const C<RC> vv = sm.Vm[x][k * CHI + j] * conj(sm.Vm[x][k * CHI + jp]);
-            s1.x = fma(sq, vv.x, s1.x);
-            s1.y = fma(sq, vv.y, s1.y);
-            s2.x = fma(is, vv.x, s2.x);
-            s2.y = fma(is, vv.y, s2.y);
-        }
-        sm.sqm[x][r] = s1;
-        sm.isq[x][r] = s2;
-    }
-    bar();
+    // with m_x = V_x w_x V_x^H: M = conj(V_0) B V_1^H, B = w_0^{1/2} (V_0^T V_1) w_1^{1/2}; with the SVD of
+    // B the transforms are conj(V_x) w_x^{-1/2} times its scaled singular vectors (as on the persistent path)
     for (int t = tid; t < CC; t += NT) {
         const int k = t % CHI, l = t / CHI;
         C<RC> acc = C<RC>{(RC)0, (RC)0};
-        for (int j = 0; j < CHI; ++j) acc = cfma(sm.sqm[0][j * CHI + k], sm.sqm[1][j * CHI + l], acc);
-        sm.M[l * CHI + k] = acc;
+        for (int j = 0; j < CHI; ++j) acc = cfma(sm.Vm[0][k * CHI + j], sm.Vm[1][l * CHI + j], acc);
+        sm.M[l * CHI + k] = (sm.wq[0][k] * sm.wq[1][l]) * acc;
     }
     bar();
     if (tid < GL) half_svd(sm.M, sm.VM, 0, tid, svd_cut);
@@ -728,17 +712,17 @@ __global__ void __launch_bounds__(CHI * CHI) plain_regauge_edge_kernel(PlainArgs
     }
     bar();
     for (int t = tid; t < 2 * CC; t += NT) {
-        const int x = t / CC, r = t % CC;
-        const int jpp = r / CHI, j = r % CHI;
+        const int x = t / CC, r = t % CC, j = r / CHI, k = r % CHI;
         const int pc = sm.perm[j];
+        const bool kept = sm.scal[0] > 0.0 && sm.sig[pc] > svd_cut * sm.sig[sm.perm[0]];
+        const RC f = kept ? sm.wiq[x][k] * sm.scal[1] : (RC)0;
+        sm.Y[x][r] = x == 0 ? (f * sm.isig[pc]) * sm.M[pc * CHI + k] : f * conj(sm.VM[pc * CHI + k]);
+    }
+    bar();
+    for (int t = tid; t < 2 * CC; t += NT) {
+        const int x = t / CC, r = t % CC, jpp = r / CHI, j = r % CHI;
         C<RC> acc = C<RC>{(RC)0, (RC)0};
-        if (sm.scal[0] > 0.0 && sm.sig[pc] > svd_cut * sm.sig[sm.perm[0]]) {
-            for (int jp = 0; jp < CHI; ++jp) {
-                const C<RC> u = (x == 0) ? sm.isig[pc] * sm.M[pc * CHI + jp] : conj(sm.VM[pc * CHI + jp]);
-                acc = cfma(sm.isq[x][jp * CHI + jpp], u, acc);
-            }
-            acc = sm.scal[1] * acc;
-        }
+        for (int k = 0; k < CHI; ++k) acc = cfmac(sm.Vm[x][k * CHI + jpp], sm.Y[x][j * CHI + k], acc);
         ((C<R>*)a.X)[((size_t)e * 2 + x) * CC + r] = ccast<R>(acc);
     }
 }
