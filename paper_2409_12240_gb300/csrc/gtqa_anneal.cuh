@@ -642,7 +642,7 @@ struct BPSm {
     C<TS> D[3][CC];      // new - old, for the trace norm
     cf D0f[3][CC];       // mixed: warm-start defect
     float m0f[3][CHI];   // mixed: warm-start diagonals
-    cd t0[3];            // mixed: traces of F0
+    cf t0h[3], t0l[3];   // mixed: traces of F0, as sums of two floats
     C<TS> trs[3];        // traces of the outgoing messages (mixed: of the correction terms)
     C<TS> itr[3];        // 1 / trace, formed in FP64
     TS dl[3];
@@ -734,7 +734,12 @@ __device__ void bp_prepare(const Ctx& c, int a, int tid, int team, int cur, BPSm
             const int k = t / CC, r = t % CC;
             sm.D0f[k][r] = sm.out_idx[k] >= 0 ? ldcg(c.D0 + (size_t)sm.out_idx[k] * CC + r) : cf{0.f, 0.f};
         }
-        if (tid < 3) sm.t0[tid] = sm.out_idx[tid] >= 0 ? ldcg(c.t0 + sm.out_idx[tid]) : cd{1.0, 0.0};
+        if (tid < 3) {
+            const cd t = sm.out_idx[tid] >= 0 ? ldcg(c.t0 + sm.out_idx[tid]) : cd{1.0, 0.0};
+            const cf h = ccast<float>(t);
+            sm.t0h[tid] = h;
+            sm.t0l[tid] = ccast<float>(t - ccast<double>(h));
+        }
     }
     if (tid == 0) sm.cached = a;
     team_bar<TEAM>(team);
@@ -1031,8 +1036,34 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
     team_bar<TEAM>(team);
 }
 
+// 1 / (t + d) for a complex t held as hi + lo: sums, products and the reciprocal carried as pairs of
+// floats (relative error about 1e-13) and rounded to FP32 once, so that the result is the FP32
+// rounding of the FP64 one.  In FP64 the same took one warp of the block 0.4 us per sweep (14
+// instructions of 64 cycles) between two block barriers.
+__device__ __forceinline__ void sum32(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float z = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+}
+__device__ __forceinline__ cf rcp_sum32(cf hi, cf lo, cf d) {
+    float x, xl, y, yl, h, e;
+    sum32(hi.x, d.x, h, e);
+    sum32(h, e + lo.x, x, xl);
+    sum32(hi.y, d.y, h, e);
+    sum32(h, e + lo.y, y, yl);
+    const float px = __fmul_rn(x, x), py = __fmul_rn(y, y);
+    float n, nl;
+    sum32(px, py, n, nl);
+    nl += (fmaf(x, x, -px) + 2.f * x * xl) + (fmaf(y, y, -py) + 2.f * y * yl);
+    if (!(n > 0.f)) return cf{0.f, 0.f};
+    const float r = __frcp_rn(n), rl = r * (fmaf(-n, r, 1.f) - nl * r);   // r + rl = 1 / (n + nl)
+    const float ax = __fmul_rn(x, r), ay = __fmul_rn(y, r);
+    return cf{ax + (fmaf(x, r, -ax) + (x * rl + xl * r)), -(ay + (fmaf(y, r, -ay) + (y * rl + yl * r)))};
+}
+
 // First part of the sweep for vertex a: incoming messages, the contractions, and the
-// traces of the three outgoing messages (left in sm.trs).
+// traces of the three outgoing messages with their reciprocals (left in sm.trs and sm.itr).  Only the
+// team's shared memory is written.
 template <int CHI, class Mode, int TB>
 __device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<CHI, Mode, TB>& sm, bool have_pre,
                          C<typename Mode::TS> pre) {
@@ -1063,35 +1094,22 @@ __device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<C
     } else {
         bp_front_elements<CHI, Mode, TB>(tid, team, sm);
     }
-    // traces of the outgoing messages (their reciprocals follow in FP64, bp_trace_rcp)
-    if (tid < 3 * CC && tid % CC == 0) {
-        const int k = tid / CC;
+    // traces of the outgoing messages and their reciprocals (reading R10: messages are divided by
+    // their complex trace)
+    if (tid < 3) {
         CT trs = z;
 #pragma unroll
-        for (int j = 0; j < CHI; ++j) {
-            trs = trs + sm.out(k, j * CHI + j);
+        for (int j = 0; j < CHI; ++j) trs = trs + sm.out(tid, j * CHI + j);
+        sm.trs[tid] = trs;
+        if constexpr (Mode::mixed) {
+            sm.itr[tid] = rcp_sum32(sm.t0h[tid], sm.t0l[tid], trs);
+        } else {
+            const double n2 = norm2(trs);
+            const double in2 = n2 > 0.0 ? nr_rcp(n2) : 0.0;
+            sm.itr[tid] = cd{trs.x * in2, -trs.y * in2};
         }
-        sm.trs[k] = trs;
     }
-}
-
-// Reciprocals of the complex traces of every team's outgoing messages in FP64 (reading
-// R10: messages are divided by their complex trace), one lane per message, by the first
-// warp of the block: FP64 instructions cost the same for 1 or 32 active lanes, so one
-// warp does this for all teams.  Mixed: the trace is t0 + tr Fd.
-template <int CHI, class Mode, int TB>
-__device__ void bp_trace_rcp(BPSm<CHI, Mode, TB>* all, int nteams) {
-    using TS = typename Mode::TS;
-    for (int l = threadIdx.x; l < 3 * nteams; l += 32) {
-        BPSm<CHI, Mode, TB>& sm = all[l / 3];
-        const int k = l % 3;
-        cd tr = ccast<double>(sm.trs[k]);
-        if constexpr (Mode::mixed) tr = tr + sm.t0[k];
-        const double n2 = norm2(tr);
-        // the mixed mode rounds the result to FP32, so one Newton step (relative error ~2^-44) suffices
-        const double in2 = n2 > 0.0 ? (Mode::mixed ? nr_rcp1(n2) : nr_rcp(n2)) : 0.0;
-        sm.itr[k] = ccast<TS>(cd{tr.x * in2, -tr.y * in2});
-    }
+    team_bar<TEAM>(team);
 }
 
 // Second part: new messages m' = F / tr F (mixed: delta' = (D0 + Fd - m0 tr Fd) / (t0 + tr Fd))
@@ -1514,8 +1532,52 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
     int* sflag = reinterpret_cast<int*>(bsum + 48);   // [2]: need | open << 1, per sweep parity
     if (threadIdx.x == 0) sflag[0] = sflag[1] = 0;
     __syncthreads();
+    // One instance: every thread takes the decision on a sweep itself, from the sum loaded right after
+    // the barrier.  In the mixed mode (AHEAD) it does so only once it has formed the next sweep's
+    // messages in shared memory, so that the load's latency and the decision lie behind that work
+    // (n = 1000, chi = 4: 5.05 -> 4.6 us per sweep with the team-wise reciprocals); a sweep that turns
+    // out not to be needed costs its first half, which is 1.9 us there but 31 us in FP64 mode, which
+    // therefore decides first.  Returns -1 if a barrier gave up, 1 to stop, 0 to go on.
+    constexpr bool AHEAD = Mode::mixed;
+    bool ex1 = c.max_iter == 1;   // the sweep under way computes the exact distance inline
+    auto decide = [&](int itd, double dsum) {
+        const bool last = itd + 1 >= c.max_iter;
+        bool fin = false;
+        if (c.inst_m[0] == 0 || !(dsum == dsum)) {
+            fin = true;
+        } else if (ex1) {
+            fin = last || dsum < thr[0];
+        } else if (last || dsum < thr_hi[0]) {   // a bound under the threshold: the exact distance decides
+            double* ex = c.acc + 3 + itd % 3;
+            if (blockIdx.x == 0 && threadIdx.x == 0) ++c.ctl->exact_passes;
+            if (threadIdx.x == 0) need[0] = 1;
+            __syncthreads();   // the teams are done with P and Q
+            bp_exact_pass<CHI, Mode, S::TPB, TB>(c, cur, need, sm, bsum + 32, ex);
+            if (!grid_sync(gb, c.spin_limit)) return -1;
+            dsum = __ldcg(ex);
+            fin = last || dsum < thr[0] || !(dsum == dsum);
+            ex1 = true;
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                c.inst_dist[0] = dsum;
+                c.inst_iters[0] = itd + 1;
+                if (fin) c.inst_done[0] = 1;
+            }
+            return fin ? 1 : 0;
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            c.inst_dist[0] = dsum;
+            c.inst_iters[0] = itd + 1;
+            if (fin) c.inst_done[0] = 1;
+        }
+        // the next sweep is exact inline when it is the last or when this one came within a factor 3
+        ex1 = itd + 2 >= c.max_iter || (float)dsum < thr3[0];
+        return fin ? 1 : 0;
+    };
+    const bool one = c.B == 1;
+    bool pend = false, stop = false;
+    double dprev = 0.0;
     int it = 0;
-    for (; it < c.max_iter; ++it) {
+    while (it < c.max_iter) {
         double* acc = c.acc + (size_t)(it % 3) * c.B;
         double* acc_next = c.acc + (size_t)((it + 1) % 3) * c.B;
         double* ex = c.acc + (size_t)(3 + it % 3) * c.B;
@@ -1524,46 +1586,65 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
             acc_next[b] = 0.0;
             ex_next[b] = 0.0;
         }
-        // rounds of one vertex per team; the block synchronises twice per round
+        // rounds of one vertex per team
         for (int base = 0; base < c.n; base += nt) {
             const int a = base + gteam;
             int inst = 0;
             bool act = false;
             if (a < c.n) {
                 inst = base == 0 ? inst0 : c.vert_inst[a];
-                if (done[inst]) bp_copy_vertex<CHI, Mode>(c, a, tid, TB, cur);
+                if (!one && done[inst]) bp_copy_vertex<CHI, Mode>(c, a, tid, TB, cur);
                 else act = true;
             }
             if (act) bp_front<CHI, Mode, TB>(c, a, tid, team, cur, sm, base == 0 && have_pre, pre);
-            __syncthreads();
-            if (threadIdx.x < 32) bp_trace_rcp<CHI, Mode, TB>(all, tpb_teams);
-            __syncthreads();
-            if (act) bp_back<CHI, Mode, TB>(c, tid, team, cur, exnow[inst] != 0, sm, c.B == 1 ? nullptr : acc + inst);
+            if (pend) {
+                pend = false;
+                const int r = decide(it - 1, dprev);
+                if (r < 0) return false;
+                if (r > 0) {
+                    stop = true;
+                    break;
+                }
+            }
+            if (act)
+                bp_back<CHI, Mode, TB>(c, tid, team, cur, one ? ex1 : exnow[inst] != 0, sm, one ? nullptr : acc + inst);
         }
+        if (stop) break;
         cur ^= 1;
         // one instance: the first warp sums the teams' distances between the block's
         // barrier and its arrival at the grid barrier
         if (!grid_sync_pre(gb, c.spin_limit, [&]() {
-                if (c.B != 1) return;
+                if (!one) return;
                 typename Mode::TS v = 0;
                 for (int q = threadIdx.x; q < 3 * tpb_teams; q += 32) v += all[q / 3].dsum[q % 3];
-    #pragma unroll
+#pragma unroll
                 for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                 if (threadIdx.x == 0) atomicAdd(acc, (double)v);
             }))
             return false;
+        if (one) dprev = __ldcg(acc);
         if (tid < 3) sm.dsum[tid] = 0;   // read by the first warp before the barrier
-        // the next sweep's incoming messages of this team's first vertex are loaded
-        // now, so that their latency overlaps the decision below
+        // the next sweep's incoming messages of this team's first vertex are loaded now
         have_pre = false;
         if (gteam < c.n && sm.cached == gteam && tid < 3 * CHI * CHI) {
             const int in = sm.in_idx[tid / (CHI * CHI)];
             if (in >= 0) pre = ldcg((const CT_*)c.msg[cur] + (size_t)in * CHI * CHI + tid % (CHI * CHI));
             have_pre = true;
         }
+        ++it;
+        if (one) {
+            if (AHEAD && it < c.max_iter) {
+                pend = true;
+                continue;
+            }
+            const int r = decide(it - 1, dprev);
+            if (r < 0) return false;
+            if (r > 0) break;
+            continue;
+        }
         // stopping rule of App. B, per instance, evaluated identically by every block;
         // the raw distance sums are kept and divided by |E| at the end
-        const bool last = it + 1 >= c.max_iter;
+        const bool last = it >= c.max_iter;
         int open_local = 0, need_local = 0;
         for (int b = threadIdx.x; b < c.B; b += S::TPB) {
             if (done[b]) continue;
@@ -1582,14 +1663,14 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
             }
             if (blockIdx.x == 0) {
                 c.inst_dist[b] = dsum;
-                c.inst_iters[b] = it + 1;
+                c.inst_iters[b] = it;
                 if (fin) c.inst_done[b] = 1;
             }
             if (fin) done[b] = 1;
             else open_local = 1;
             // the next sweep is exact inline when it is the last or when this
             // sweep came within a factor 3 of the threshold
-            exnow[b] = (it + 2 >= c.max_iter) || (float)dsum < thr3[b];
+            exnow[b] = (it + 1 >= c.max_iter) || (float)dsum < thr3[b];
         }
         // one block barrier for both flags (a word per sweep parity, reset one sweep ahead)
         if (need_local | open_local) atomicOr(&sflag[it & 1], need_local | (open_local << 1));
@@ -1607,19 +1688,15 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
                 const bool fin = last || dsum < thr[b] || !(dsum == dsum);
                 if (blockIdx.x == 0) {
                     c.inst_dist[b] = dsum;
-                    c.inst_iters[b] = it + 1;
+                    c.inst_iters[b] = it;
                     if (fin) c.inst_done[b] = 1;
                 }
                 if (fin) done[b] = 1;
                 else open_local = 1;
                 exnow[b] = 1;
             }
-            if (!__syncthreads_or(open_local)) {
-                ++it;
-                break;
-            }
+            if (!__syncthreads_or(open_local)) break;
         } else if (!(fl & 2)) {
-            ++it;
             break;
         }
     }
