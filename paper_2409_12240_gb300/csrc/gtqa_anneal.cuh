@@ -884,69 +884,103 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
     // strides in the padded shared-memory layout: slot 0, slot 1 (slot 2 has stride 1), i
     constexpr int S0 = SM::PS, S1 = CHI, HP = CHI * SM::PS;
     const CT z = CT{(TS)0, (TS)0};
-    // first contractions along one slot: P_k[.., x@k, ..] = sum_q T[.., q@k, ..] y_k[q][x]
-    //   FP64: y = m (k = 0, 1); mixed: y = delta (k = 0, 1, 2)
-    constexpr int NP = SM::NP;
     constexpr bool EVEN = H2 % TEAM == 0;   // whole tensors per team pass: slots fixed at compile time
     auto slot_stride = [](int k) { return k == 0 ? S0 : (k == 1 ? S1 : 1); };
-    // e: natural index of an element, pe: its padded position
-    auto p_elem = [&](int k, int e) {
-        const int pe = e + e / CC;
-        const int st = slot_stride(k);
-        const int x = k == 0 ? (e / CC) % CHI : (k == 1 ? (e / CHI) % CHI : e % CHI);
-        const int base = pe - x * st;
-        const CT* y = Mode::mixed ? sm.din[k] : sm.min[k];
-        CT acc = z;
+    if constexpr (!Mode::mixed) {
+        // the messages on the slots before s contracted into T, those after s (as m^H) into the other
+        // factor of the overlap: L_1 = T x_0 m_0, R_1 = T x_2 m_2^H, L_2 = L_1 x_1 m_1, R_0 = R_1 x_1 m_1^H;
+        // F_0 = <T, R_0>, F_1 = <L_1, R_1>, F_2 = <L_2, T>: seven tensor-sized products instead of
+        // the eight of two first and three second contractions
+        auto contract = [&](const CT* src, CT* dst, int k, bool adj, int e) {
+            const int pe = e + e / CC, st = slot_stride(k);
+            const int x = k == 0 ? (e / CC) % CHI : (k == 1 ? (e / CHI) % CHI : e % CHI);
+            const int base = pe - x * st;
+            const CT* y = sm.min[k];
+            CT acc = z;
 #pragma unroll
-        for (int q = 0; q < CHI; ++q) acc = cfma(sm.T[base + q * st], y[q * CHI + x], acc);
-        sm.P[k][pe] = acc;
-    };
-    if constexpr (EVEN) {
+            for (int q = 0; q < CHI; ++q)
+                acc = adj ? cfmac(y[x * CHI + q], src[base + q * st], acc) : cfma(src[base + q * st], y[q * CHI + x], acc);
+            dst[pe] = acc;
+        };
+        auto both = [&](const CT* s0, CT* d0, int k0, const CT* s1, CT* d1, int k1) {
+            if constexpr (EVEN) {
 #pragma unroll
-        for (int k = 0; k < NP; ++k)
+                for (int w = 0; w < H2 / TEAM; ++w) contract(s0, d0, k0, false, tid + w * TEAM);
 #pragma unroll
-            for (int w = 0; w < H2 / TEAM; ++w) p_elem(k, tid + w * TEAM);
+                for (int w = 0; w < H2 / TEAM; ++w) contract(s1, d1, k1, true, tid + w * TEAM);
+            } else {
+                for (int t = tid; t < 2 * H2; t += TEAM) {
+                    if (t < H2) contract(s0, d0, k0, false, t);
+                    else contract(s1, d1, k1, true, t - H2);
+                }
+            }
+            team_bar<TEAM>(team);
+        };
+        both(sm.T, sm.P[0], 0, sm.T, sm.P[1], 2);
+        both(sm.P[0], sm.Q[0], 1, sm.P[1], sm.Q[1], 1);
     } else {
-        for (int t = tid; t < NP * H2; t += TEAM) p_elem(t / H2, t % H2);
-    }
-    team_bar<TEAM>(team);
-    // second contractions per outgoing slot s (natural layout, slot-s index = j):
-    //   Q_0[i][j][a][b] = sum_q P_1[i][j][a][q] m_2[q][b]  (+ m0_1[a] P_2[i][j][a][b])
-    //   Q_1[i][a][j][b] = sum_q P_0[i][a][j][q] m_2[q][b]  (+ m0_0[a] P_2[i][a][j][b])
-    //   Q_2[i][a][b][j] = sum_q P_0[i][a][q][j] m_1[q][b]  (+ m0_0[a] P_1[i][a][b][j])
-    auto q_elem = [&](int s, int e) {
-        const int pe = e + e / CC;
-        const int j0 = (e / CC) % CHI, j1 = (e / CHI) % CHI, j2 = e % CHI;
-        CT acc = z;
-        if (s == 2) {
+        // first contractions along one slot: P_k[.., x@k, ..] = sum_q T[.., q@k, ..] y_k[q][x]
+        //   FP64: y = m (k = 0, 1); mixed: y = delta (k = 0, 1, 2)
+        constexpr int NP = SM::NP;
+        // e: natural index of an element, pe: its padded position
+        auto p_elem = [&](int k, int e) {
+            const int pe = e + e / CC;
+            const int st = slot_stride(k);
+            const int x = k == 0 ? (e / CC) % CHI : (k == 1 ? (e / CHI) % CHI : e % CHI);
+            const int base = pe - x * st;
+            const CT* y = Mode::mixed ? sm.din[k] : sm.min[k];
+            CT acc = z;
 #pragma unroll
-            for (int q = 0; q < CHI; ++q) acc = cfma(sm.P[0][pe - j1 * S1 + q * S1], sm.min[1][q * CHI + j1], acc);
+            for (int q = 0; q < CHI; ++q) acc = cfma(sm.T[base + q * st], y[q * CHI + x], acc);
+            sm.P[k][pe] = acc;
+        };
+        if constexpr (EVEN) {
+#pragma unroll
+            for (int k = 0; k < NP; ++k)
+#pragma unroll
+                for (int w = 0; w < H2 / TEAM; ++w) p_elem(k, tid + w * TEAM);
         } else {
-            const CT* Ps = (s == 0) ? sm.P[1] : sm.P[0];
+            for (int t = tid; t < NP * H2; t += TEAM) p_elem(t / H2, t % H2);
+        }
+        team_bar<TEAM>(team);
+        // second contractions per outgoing slot s (natural layout, slot-s index = j):
+        //   Q_0[i][j][a][b] = sum_q P_1[i][j][a][q] m_2[q][b]  (+ m0_1[a] P_2[i][j][a][b])
+        //   Q_1[i][a][j][b] = sum_q P_0[i][a][j][q] m_2[q][b]  (+ m0_0[a] P_2[i][a][j][b])
+        //   Q_2[i][a][b][j] = sum_q P_0[i][a][q][j] m_1[q][b]  (+ m0_0[a] P_1[i][a][b][j])
+        auto q_elem = [&](int s, int e) {
+            const int pe = e + e / CC;
+            const int j0 = (e / CC) % CHI, j1 = (e / CHI) % CHI, j2 = e % CHI;
+            CT acc = z;
+            if (s == 2) {
 #pragma unroll
-            for (int q = 0; q < CHI; ++q) acc = cfma(Ps[pe - j2 + q], sm.min[2][q * CHI + j2], acc);
-        }
-        if constexpr (Mode::mixed) {
-            const float w = (s == 0) ? sm.m0f[1][j1] : sm.m0f[0][j0];
-            const CT pv = (s == 2) ? sm.P[1][pe] : sm.P[2][pe];
-            acc = acc + w * pv;
-        }
-        sm.Q[s][pe] = acc;
-    };
-    if constexpr (EVEN) {
+                for (int q = 0; q < CHI; ++q) acc = cfma(sm.P[0][pe - j1 * S1 + q * S1], sm.min[1][q * CHI + j1], acc);
+            } else {
+                const CT* Ps = (s == 0) ? sm.P[1] : sm.P[0];
 #pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            if (sm.es[s] < 0) continue;
+                for (int q = 0; q < CHI; ++q) acc = cfma(Ps[pe - j2 + q], sm.min[2][q * CHI + j2], acc);
+            }
+            if constexpr (Mode::mixed) {
+                const float w = (s == 0) ? sm.m0f[1][j1] : sm.m0f[0][j0];
+                const CT pv = (s == 2) ? sm.P[1][pe] : sm.P[2][pe];
+                acc = acc + w * pv;
+            }
+            sm.Q[s][pe] = acc;
+        };
+        if constexpr (EVEN) {
 #pragma unroll
-            for (int w = 0; w < H2 / TEAM; ++w) q_elem(s, tid + w * TEAM);
+            for (int s = 0; s < 3; ++s) {
+                if (sm.es[s] < 0) continue;
+#pragma unroll
+                for (int w = 0; w < H2 / TEAM; ++w) q_elem(s, tid + w * TEAM);
+            }
+        } else {
+            for (int t = tid; t < 3 * H2; t += TEAM) {
+                const int s = t / H2;
+                if (sm.es[s] >= 0) q_elem(s, t % H2);
+            }
         }
-    } else {
-        for (int t = tid; t < 3 * H2; t += TEAM) {
-            const int s = t / H2;
-            if (sm.es[s] >= 0) q_elem(s, t % H2);
-        }
+        team_bar<TEAM>(team);
     }
-    team_bar<TEAM>(team);
     // overlaps with conj(T): F_s[j][j'] = sum over the 2 CHI^2 columns (i, u@o0, v@o1) of
     // Q_s[.., j@s, ..] conj(T[.., j'@s, ..]).  Mixed mode: a lane holds a 2 x 2 block of
     // (j, j') over a slice of the columns, so that every element it loads feeds two products;
@@ -998,13 +1032,15 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
             const int j = r / CHI, jp = r % CHI;
             const int ss = slot_stride(s);
             const int so = s == 0 ? S1 : S0, st2 = s == 2 ? S1 : 1;   // strides of the two other slots
+            const CT* X = s == 0 ? sm.T : (s == 1 ? sm.P[0] : sm.Q[0]);
+            const CT* Y = s == 0 ? sm.Q[1] : (s == 1 ? sm.P[1] : sm.T);
             CT acc = z;
 #pragma unroll
             for (int u = 0; u < CHI; ++u)
 #pragma unroll
                 for (int v = 0; v < CHI; ++v) {
                     const int off = i * HP + u * so + v * st2;
-                    acc = cfmac(sm.T[off + jp * ss], sm.Q[s][off + j * ss], acc);
+                    acc = cfmac(Y[off + jp * ss], X[off + j * ss], acc);
                 }
             if (i == 0) sm.F[s][r] = acc;
             else sm.F1[s][r] = acc;
@@ -1018,6 +1054,8 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
             if (sm.es[s] < 0) continue;
             const int ss = slot_stride(s);
             const int so = s == 0 ? S1 : S0, st2 = s == 2 ? S1 : 1;
+            const CT* X = s == 0 ? sm.T : (s == 1 ? sm.P[0] : sm.Q[0]);
+            const CT* Y = s == 0 ? sm.Q[1] : (s == 1 ? sm.P[1] : sm.T);
             CT acc = z;
 #pragma unroll
             for (int h = 0; h < PER; ++h) {
@@ -1025,7 +1063,7 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
 #pragma unroll
                 for (int v = 0; v < CHI; ++v) {
                     const int off = i * HP + u * so + v * st2;
-                    acc = cfmac(sm.T[off + jp * ss], sm.Q[s][off + j * ss], acc);
+                    acc = cfmac(Y[off + jp * ss], X[off + j * ss], acc);
                 }
             }
             acc.x = group_sum<NPART>(acc.x, group_mask<NPART>());
@@ -1804,12 +1842,13 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
                 }
                 if (!grid_sync(gb, c.spin_limit)) return;
             }
-            // FP64 at CHI <= 4 with at most one vertex per block: teams of four warps, one per
-            // sub-partition, halve a sweep's FP64 time (10.4 -> 5.6 us); with two or more vertices per
-            // block the pipes are as busy with teams of two
+            // FP64 at CHI <= 4 while a block's vertices all have a team of four warps: one warp per
+            // sub-partition halves a sweep's FP64 time where a block has one vertex (10.4 -> 5.6 us) and
+            // evens the sub-partitions out for an odd number; beyond that the teams of two keep every
+            // vertex resident
             constexpr int WIDE = SmemSize<CHI, Mode, PH, V>::WIDE_TB;
             bool ok;
-            if (WIDE != S::TB && c.n <= c.nblocks) ok = bp_sweeps<CHI, Mode, PH, V, WIDE>(c, gb, cur, smem);
+            if (WIDE != S::TB && c.n <= c.nblocks * (S::TPB / WIDE)) ok = bp_sweeps<CHI, Mode, PH, V, WIDE>(c, gb, cur, smem);
             else ok = bp_sweeps<CHI, Mode, PH, V, S::TB>(c, gb, cur, smem);
             if (!ok) return;
         }
