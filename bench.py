@@ -324,11 +324,11 @@ def gate_flops(chi: int, edges: int, pairs: int, rotations: int, mixed: bool = F
       core M (triangular R's)      sum_{r,r'} 10 (C - max(r, r')) + 26 per entry, 4 blocks
       singular values              3 N^2
       Q U / lambda (4 blocks)      4 C sum_k 16 (R-k) + 8 C R
-    plus per Jacobi pair examined 14 N (alpha, beta, gamma) and per rotation 40 N + 15.
-    Returns (FP64 flops, FP32 flops).  In the mixed mode the counted Jacobi sweeps are the
-    FP64 polish after the FP32 preconditioning sweeps (which are not counted), the
-    Newton-Schulz step (V^H V, V(3I - G)/2) and W = M V add 3 x 8 N^3 FP64 flops per
-    edge, and the last line (Q U / lambda) runs in FP32.
+    and the FP64 part of the core's SVD: W = M V (8 N^3), per pair examined 8 N (the Gram products
+    of a refinement pass), per pass 4 N^2 for the norms, per Jacobi rotation 40 N + 15; in FP64
+    mode also the unitarity Gram product (4 N^3) and W L and V L of every pass (16 N^3).
+    Returns (FP64 flops, FP32 flops).  In the mixed mode the corrections W L and V L and the last
+    line (Q U / lambda) run in FP32; the FP32 Jacobi sweeps are not counted.
     """
     C = storage_chi(chi)
     R, N = C * C, 2 * C
@@ -337,11 +337,12 @@ def gate_flops(chi: int, edges: int, pairs: int, rotations: int, mixed: bool = F
     core = 4 * sum(10 * (C - max(r, rp)) + 26 for r in range(C) for rp in range(C))
     sv = 3 * N * N
     back = 4 * C * sum(16 * (R - k) for k in range(C)) + 8 * C * R
-    jac = pairs * 14 * N + rotations * (40 * N + 15)
+    passes = pairs / (N * (N - 1) / 2)
+    svd = edges * 8 * N ** 3 + pairs * 8 * N + passes * 4 * N * N + rotations * (40 * N + 15)
     if not mixed:
-        return float(edges * (x + qr + core + sv + back) + jac), 0.0
-    ns = 3 * 8 * N ** 3
-    return float(edges * (x + qr + core + sv + ns) + jac), float(edges * back)
+        svd += edges * 4 * N ** 3 + passes * 16 * N ** 3
+        return float(edges * (x + qr + core + sv + back) + svd), 0.0
+    return float(edges * (x + qr + core + sv) + svd), float(edges * back + passes * 16 * N ** 3)
 
 
 def bp_sweep_flops(chi: int, vertices: int, mixed: bool) -> float:
@@ -396,14 +397,14 @@ def regauge_edge_flops(chi: int, mixed: bool) -> Tuple[float, float]:
 
 
 def regauge_flops_executed(chi: int, edges: int, svd_sweeps: int, mixed: bool) -> float:
-    """FP64 flops the regauge kernel issues: per counted Jacobi sweep (FP64 sweeps, or the FP64
-    polish sweeps of the mixed mode) (N - 1) N / 2 pairs of 14 N + 40 N + 15 flops at N = C;
-    per edge the Hermitian parts, roots, M and X (7 C^3 complex MACs), and in the mixed mode the
-    three Newton-Schulz steps and products (3 x 3 x 8 C^3)."""
+    """FP64 flops the regauge kernel issues: per counted refinement pass of an order-C decomposition
+    the Gram products 4 C^3 (and, in FP64 mode, the two corrections 16 C^3); per edge W = A V of the
+    three decompositions (3 x 8 C^3, and in FP64 mode their unitarity Gram products 3 x 4 C^3) and
+    the Hermitian parts, B and the two transforms (3 C^3 complex MACs)."""
     C = storage_chi(chi)
-    per_sweep = (C - 1) * C / 2 * (54 * C + 15)
-    fixed = 8 * 7 * C ** 3 + (3 * 3 * 8 * C ** 3 if mixed else 0)
-    return float(svd_sweeps * per_sweep + edges * fixed)
+    per_pass = 4 * C ** 3 + (0 if mixed else 16 * C ** 3)
+    fixed = 3 * 8 * C ** 3 + (0 if mixed else 3 * 4 * C ** 3) + 3 * 8 * C ** 3
+    return float(svd_sweeps * per_pass + edges * fixed)
 
 
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_n1000_chi4.json")

@@ -98,7 +98,7 @@ typedef struct gtqa_stats_t {
     int64_t bp_calls;        /* BP runs since creation (one per layer in gtqa_anneal) */
     int64_t bp_not_converged_calls; /* BP runs in which some instance reached max_iter */
     int64_t bp_exact_passes; /* separate passes computing the exact trace-norm distance of a sweep
-                                (persistent path: when a sweep's lower bound falls under tol) */
+                                (when a sweep's lower bound falls under tol) */
     int64_t regauge_svd_sweeps; /* FP64 refinement passes of the regauge's eigen-decompositions and SVDs
                                    (persistent path; work counter) */
     int32_t gate_svd_sweeps_max;      /* most FP64 refinement passes (and sweeps of a closing Jacobi polish)
@@ -137,8 +137,10 @@ void gtqa_options_init(gtqa_options* opt);
  * Anything else
  * returns GTQA_ERR_UNSUPPORTED.  On a plain-path state gtqa_autotune and gtqa_anneal_graph
  * return GTQA_ERR_UNSUPPORTED (there is no persistent launch to tune or capture), and so does
- * gtqa_apply_gates at chi > 8; every other call works as documented.  Its BP reads the
- * distance on the host after every sweep, and gtqa_anneal_policy reads R on the host.
+ * gtqa_apply_gates at chi > 8; every other call works as documented.  Its BP runs in one
+ * cooperative launch like the persistent path's; gtqa_anneal, gtqa_anneal_ex and
+ * gtqa_anneal_policy read the device status once at their end (they synchronise there, and
+ * return GTQA_ERR_NUMERIC if a BP distance was NaN), and gtqa_anneal_policy reads R on the host.
  */
 int gtqa_create(int32_t n, int32_t m, const int32_t* edges, const int32_t* colour,
                 const double* J, const double* h, int32_t chi,
@@ -218,7 +220,9 @@ int gtqa_set_grid(gtqa_state* s, const int32_t* grid);
  * BP and regauge 0, 1 and 2; variant 0 is the default of gtqa_create_batch.  For CHI <= 4
  * (threads per block, BP vertex team, regauge-vertex team) are (512, 64, 32), (256, 64, 32) and
  * (512, 128, 64); for CHI = 8 they are (256, 256, 128), (512, 256, 128) and (512, 512, 256).
- * The gate-edge team (2 CHI^2 threads) and the regauge-edge team (CHI^2) are fixed.
+ * The gate-edge team (2 CHI^2 threads) is fixed; the regauge-edge team has CHI^2 threads, or
+ * CHI^2 / 2 where m exceeds 512 / CHI^2 edges per block.  FP64 runs at CHI <= 4 whose vertices all have a
+ * team of 128 threads on the grid (n <= 4 x blocks of 512 threads) use such teams in variant 0 too.
  * GTQA_ERR_INVALID_ARG for an index out of range, GTQA_ERR_UNSUPPORTED when a variant's
  * shared memory does not fit on an SM (the state keeps its shapes) or for a plain-path state.
  * Drops a captured layer graph.
@@ -347,8 +351,7 @@ int gtqa_apply_single_qubit_gates(gtqa_state* s, int32_t k, const int32_t* verte
  *   u        float64 [k], host: the caller's uniform random numbers in [0, 1]
  *   x_out    int8 [n], host: +1 / -1 for the sampled qubits, 0 for the others
  *   p_out    float64 [k], host, nullable: the probability of each outcome given the earlier ones
- * For a batched state every step regauges all instances.  Synchronises the stream once (on a
- * plain-path state, see gtqa_create, also after every BP sweep).
+ * For a batched state every step regauges all instances.  Synchronises the stream once.
  */
 int gtqa_sample(gtqa_state* s, int32_t k, const int32_t* order, const double* u, double tol, int32_t max_iter,
                 int8_t* x_out, double* p_out);
