@@ -150,7 +150,8 @@ int gtqa_create(int32_t n, int32_t m, const int32_t* edges, const int32_t* colou
  * Create B independent instances that evolve together (one launch per phase covers
  * all of them).  Arrays are concatenations over instances: n[B], m[B]; edges (local
  * vertex ids per instance) sum(m) pairs; colour sum(m) or NULL; J sum(m); h sum(n).
- * BP convergence is tracked per instance: dist_b/|E_b| < tol.
+ * BP convergence is tracked per instance: dist_b/|E_b| < tol.  An instance in a batch follows its
+ * single run up to rounding (the batch's total size decides team widths, gtqa_set_shape).
  */
 int gtqa_create_batch(int32_t B, const int32_t* n, const int32_t* m, const int32_t* edges,
                       const int32_t* colour, const double* J, const double* h, int32_t chi,
@@ -204,8 +205,9 @@ int gtqa_anneal(gtqa_state* s, int32_t k_begin, int32_t k_end, int32_t K, double
  * state is snapshotted once (into device memory when a copy fits in free memory, else into host
  * memory), its contents and statistics are restored afterwards, and a layer graph captured by
  * gtqa_anneal_graph is dropped (the next call captures the new shapes).  grid_out (nullable,
- * 3 ints) receives the chosen grid sizes.  Results do not depend on the grid; across variants
- * they differ only in the rounding order of BP's contraction and distance sums.  Synchronises.
+ * 3 ints) receives the chosen grid sizes.  Results do not depend on the grid; across variants,
+ * and with the instance sizes at which a phase changes its team width (gtqa_create_batch), they
+ * differ only in the rounding order of BP's contraction and distance sums.  Synchronises.
  * Returns GTQA_ERR_UNSUPPORTED for a plain-path state (gtqa_create).
  */
 int gtqa_autotune(gtqa_state* s, double tau, double dt, double tol, int32_t max_iter, int32_t* grid_out);
@@ -221,8 +223,8 @@ int gtqa_set_grid(gtqa_state* s, const int32_t* grid);
  * (threads per block, BP vertex team, regauge-vertex team) are (512, 64, 32), (256, 64, 32) and
  * (512, 128, 64); for CHI = 8 they are (256, 256, 128), (512, 256, 128) and (512, 512, 256).
  * The gate-edge team (2 CHI^2 threads) is fixed; the regauge-edge team has CHI^2 threads, or
- * CHI^2 / 2 where m exceeds 512 / CHI^2 edges per block.  FP64 runs at CHI <= 4 whose vertices all have a
- * team of 128 threads on the grid (n <= 4 x blocks of 512 threads) use such teams in variant 0 too.
+ * CHI^2 / 2 where m exceeds 512 / CHI^2 edges per SM.  FP64 BP at CHI <= 4 uses teams of 128 threads
+ * up to one team per vertex on all SMs (n <= 4 per SM in blocks of 512 threads, 2 in blocks of 256).
  * GTQA_ERR_INVALID_ARG for an index out of range, GTQA_ERR_UNSUPPORTED when a variant's
  * shared memory does not fit on an SM (the state keeps its shapes) or for a plain-path state.
  * Drops a captured layer graph.

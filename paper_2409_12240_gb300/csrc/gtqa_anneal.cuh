@@ -68,8 +68,8 @@ struct Control {
     long long regauged;      // regauge-policy layers: regauged (BP and gauge finding ran)
     long long reg_skipped;   // and skipped (R at or below the threshold)
     long long exact_passes;  // separate exact-distance passes (bp_exact_pass) run by BP
-    int gate_sw_max;         // most FP64 Jacobi sweeps of one gate-core SVD (polish sweeps in the mixed mode)
-    int gate_sw32_max;       // mixed mode: most FP32 preconditioning sweeps of one gate-core SVD
+    int gate_sw_max;         // most FP64 refinement passes of one gate-core SVD (and sweeps of its closing polish)
+    int gate_sw32_max;       // most FP32 Jacobi sweeps of one gate-core SVD
     int reg_sw_max;          // the same for the regauge's eigen-decompositions and SVD
     int reg_sw32_max;
 };
@@ -118,6 +118,8 @@ struct Ctx {
     const double* rgate;      // regauge policy: the residual sum of this layer (null: always regauge)
     double rthr_sum;          // BP and regauge run only if *rgate > rthr_sum
     int nblocks;
+    int nsm;                  // SMs of the device: the team widths follow it, not the grid, so that a grid
+                              // chosen by gtqa_set_grid or gtqa_autotune does not change the rounding
     int bar_expect;           // arrivals per grid barrier (= nblocks; larger only in the timeout test)
     long long spin_limit;
 };
@@ -1298,7 +1300,7 @@ __device__ void bp_exact_pass(const Ctx& c, int cur_new, const int* need, BPSm<C
 // turn.  The three decompositions of an edge are the FP64 work: the wide team finishes an edge
 // sooner (two in turn instead of three) but leaves half of its lanes idle in the third one, and the
 // FP64 pipe charges a warp, not its lanes.  The narrow team runs once a sub-partition has more than
-// four wide warps' worth of edges (m > blocks x 512 / CHI^2): at 10 edges per block (n = 1000, chi = 4)
+// four wide warps' worth of edges (m > SMs x 512 / CHI^2): at 10 edges per block (n = 1000, chi = 4)
 // it is 9 us slower per regauge, at 165 (32 instances) a regauge is 15 % faster.
 // ===========================================================================
 template <int CHI>
@@ -1848,7 +1850,7 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
             // vertex resident
             constexpr int WIDE = SmemSize<CHI, Mode, PH, V>::WIDE_TB;
             bool ok;
-            if (WIDE != S::TB && c.n <= c.nblocks * (S::TPB / WIDE)) ok = bp_sweeps<CHI, Mode, PH, V, WIDE>(c, gb, cur, smem);
+            if (WIDE != S::TB && c.n <= c.nsm * (S::TPB / WIDE)) ok = bp_sweeps<CHI, Mode, PH, V, WIDE>(c, gb, cur, smem);
             else ok = bp_sweeps<CHI, Mode, PH, V, S::TB>(c, gb, cur, smem);
             if (!ok) return;
         }
@@ -1868,7 +1870,7 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
                     for (int e = team * c.nblocks + blockIdx.x; e < c.m; e += c.nblocks * teams)
                         regauge_edge<CHI, Mode, TEAM>(c, e, tid, team, cur, sm);
                 };
-                if (c.m <= c.nblocks * (512 / S::TR)) edges(std::integral_constant<int, S::TR>{}, SZ::rg_wide);
+                if (c.m <= c.nsm * (512 / S::TR)) edges(std::integral_constant<int, S::TR>{}, SZ::rg_wide);
                 else edges(std::integral_constant<int, S::TR / 2>{}, SZ::rg_teams);
                 if (!grid_sync(gb, c.spin_limit)) return;
             }

@@ -568,6 +568,7 @@ Ctx make_ctx(const gtqa_state* s) {
     c.svd_cut = s->svd_cutoff;
     c.eig_cut = s->eig_cutoff;
     c.nblocks = s->nblocks;
+    c.nsm = s->nblocks;
     c.bar_expect = s->nblocks + s->bar_extra;
     c.spin_limit = s->spin_limit;
     return c;

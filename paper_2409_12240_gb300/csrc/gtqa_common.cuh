@@ -516,8 +516,8 @@ __device__ __forceinline__ bool norm_collapsed(double x, double ref) {
 }
 
 // FP64 polish of a one-sided Jacobi SVD (same layout, pairing and rotations as
-// jacobi_svd<N, double>) for columns that are already nearly orthogonal, as after an
-// FP32 solve and an FP64 Newton-Schulz step.  Fewer FP64 instructions per step:
+// jacobi_svd<N, double>) for columns that are already nearly orthogonal, as
+// refined_svd leaves those that its passes do not close.  Fewer FP64 instructions per step:
 //  * the squared column norms are kept in nrm[N] (shared) and, in steps whose rotations are all
 //    small, updated as alpha' = alpha - tau |gamma|^2 and beta' = beta + tau |gamma|^2 (the two
 //    eigenvalues of the pair's 2x2 Gram matrix) instead of two reductions per step; after a

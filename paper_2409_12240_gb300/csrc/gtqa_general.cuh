@@ -8,7 +8,7 @@
 //   A_x = Q_x R_x                                  (Householder, FP64)
 //   M[(i_a, r), (i_b, r')] = sum_{i_a' i_b'} U[(i_a i_b), (i_a' i_b')]
 //                            sum_j R_a[r, (i_a', j)] lambda_j R_b[r', (i_b', j)]   (4 CHI x 4 CHI)
-//   M = U_s S V^H (one-sided Jacobi, FP64), truncated to chi as in App. D "Truncation",
+//   M = U_s S V^H (refined_svd; one-sided Jacobi in FP32 in the complex64 mode), truncated to chi as in App. D "Truncation",
 //   Gamma~_a[i_a][k][J] = (Q_a U_s)[(J), (i_a, k)] / w_a[J] and
 //   Gamma~_b[i_b][k][J] = (Q_b conj V)[(J), (i_b, k)] / w_b[J],
 // so that Theta' = Q_a M Q_b^T is the gate applied to the two-site tensor of App. E.

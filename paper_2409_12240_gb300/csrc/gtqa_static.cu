@@ -168,6 +168,7 @@ extern "C" int gtqa_bp_static(int32_t n, int32_t m, const int32_t* vert_edges, c
     c.tol = tol;
     c.max_iter = max_iter;
     c.nblocks = sms;
+    c.nsm = sms;
     c.bar_expect = sms;
     c.spin_limit = 1LL << 22;
     if (PhaseUnit<ModeFP64, PK_BP>::launch(kChi, 0, c, smem, st) != cudaSuccess) {
