@@ -95,7 +95,8 @@ struct Ctx {
     void* T;
     void* msg[2];
     cf* D0;                   // mixed: warm-start defect F(m0) - tr F(m0) m0, [2m][CHI^2]
-    cd* t0;                   // mixed: tr F(m0), [2m]
+    float4* t0;               // mixed: tr F(m0) as a sum of two complex floats, [2m]
+    float* m0f;               // mixed: the warm-start diagonal of each message, [2m][CHI]
     cd* X;                    // regauge transforms [m][2][CHI^2]
     double* acc;              // [3][B] per-sweep distance accumulators
     int* inst_done;
@@ -588,7 +589,11 @@ __device__ void bp_init_vertex(const Ctx& c, int a, int tid, int cur, bool warm,
             for (int q = 0; q < CHI; ++q) t0 += F[s * CC + q * CHI + q].x;
             const double m0 = (j == jp) ? wsm[3 * CHI + s * CHI + j] : 0.0;
             c.D0[(size_t)out[s] * CC + r] = ccast<float>(F[s * CC + r] - cd{t0 * m0, 0.0});
-            if (r == 0) c.t0[out[s]] = cd{t0, 0.0};
+            if (r == 0) {
+                const float h = (float)t0;
+                c.t0[out[s]] = make_float4(h, 0.f, (float)(t0 - (double)h), 0.f);
+            }
+            if (j == jp) c.m0f[(size_t)out[s] * CHI + j] = (float)m0;
         }
     }
 }
@@ -698,49 +703,73 @@ __device__ __forceinline__ TS trace_norm(C<TS>* A, int g, const WarpGroup& grp) 
     return s;
 }
 
+// The index of vertex a's outgoing message along slot k, -1 for a phantom slot, in two dependent loads.
+__device__ __forceinline__ int slot_edge(const Ctx& c, int a, int k) {
+    return reinterpret_cast<const int*>(c.vert_edges + a)[k];
+}
+__device__ __forceinline__ int slot_out(const Ctx& c, int a, int e) {
+    return e >= 0 ? 2 * e + (a == c.edge_info[e].x ? 0 : 1) : -1;
+}
+
+// Fills the team's cache for vertex a; out: its message index of slot tid (lanes 0..2).  `pre`
+// receives the lane's element of the incoming messages.  Where a sweep has several rounds this runs
+// in each, so everything is loaded at once, after the indices that the caller has fetched a round
+// ahead, and no FP64 instruction is left in it: m0 and t0 come as the floats that the init phase
+// stored.  (Formed here from lambda, by the first warp of each team, they put some 20 FP64
+// instructions per vertex on two of the four sub-partitions.)
 template <int CHI, class Mode, int TB>
-__device__ void bp_prepare(const Ctx& c, int a, int tid, int team, int cur, BPSm<CHI, Mode, TB>& sm) {
+__device__ __forceinline__ void bp_prepare(const Ctx& c, int a, int tid, int team, int cur, BPSm<CHI, Mode, TB>& sm,
+                                           int out, C<typename Mode::TS>& pre) {
     using TS = typename Mode::TS;
     using CT = C<TS>;
-    constexpr int TEAM = TB, CC = CHI * CHI, H2 = 2 * CHI * CHI * CHI;
+    constexpr int TEAM = TB, CC = CHI * CHI, H2 = 2 * CHI * CHI * CHI, NT = (H2 + TEAM - 1) / TEAM;
+    static_assert(3 * CC <= TEAM, "one message element per lane");
+    const CT* Tg = (const CT*)c.T + (size_t)a * H2;
+    CT tv[NT];
+#pragma unroll
+    for (int q = 0; q < NT; ++q)
+        if (H2 % TEAM == 0 || tid + q * TEAM < H2) tv[q] = ldcg(Tg + tid + q * TEAM);
     team_bar<TEAM>(team);   // the team may still be reading the previous vertex's cache
     if (tid < 3) {
-        const int4 ve = c.vert_edges[a];
-        const int e = tid == 0 ? ve.x : (tid == 1 ? ve.y : ve.z);
-        sm.es[tid] = e;
-        if (e >= 0) {
-            const int u = c.edge_info[e].x;
-            sm.out_idx[tid] = 2 * e + (a == u ? 0 : 1);
-            sm.in_idx[tid] = 2 * e + (a == u ? 1 : 0);
-        } else {
-            sm.out_idx[tid] = sm.in_idx[tid] = -1;
-        }
+        sm.es[tid] = out >= 0 ? out >> 1 : -1;
+        sm.out_idx[tid] = out;
+        sm.in_idx[tid] = out >= 0 ? out ^ 1 : -1;
     }
-    const CT* Tg = (const CT*)c.T + (size_t)a * H2;
-    for (int t = tid; t < H2; t += TEAM) sm.T[t + (t / CC) * (BPSm<CHI, Mode, TB>::PS - CC)] = ldcg(Tg + t);
     team_bar<TEAM>(team);
     const CT* src = (const CT*)c.msg[cur];
-    for (int t = tid; t < 3 * CC; t += TEAM) {
-        const int k = t / CC, r = t % CC;
-        const int out = sm.out_idx[k];
-        sm.prev[k][r] = out >= 0 ? ldcg(src + (size_t)out * CC + r) : CT{(TS)0, (TS)0};
+    const CT z = CT{(TS)0, (TS)0};
+    CT pv = z;
+    cf dv = cf{0.f, 0.f};
+    float mv = 0.f;
+    float4 t0 = make_float4(1.f, 0.f, 0.f, 0.f);
+    const int o = tid < 3 * CC ? sm.out_idx[tid / CC] : -1;
+    pre = z;
+    if (o >= 0) {
+        pre = ldcg(src + (size_t)(o ^ 1) * CC + tid % CC);
+        pv = ldcg(src + (size_t)o * CC + tid % CC);
+        if constexpr (Mode::mixed) dv = ldcg(c.D0 + (size_t)o * CC + tid % CC);
     }
     if constexpr (Mode::mixed) {
         if (tid < 3 * CHI) {
-            const int k = tid / CHI, j = tid % CHI;
-            double s = 0.0;
-            for (int q = 0; q < CHI; ++q) s += lam_get(c.lam, CHI, sm.es[k], q);
-            sm.m0f[k][j] = s > 0.0 ? (float)(lam_get(c.lam, CHI, sm.es[k], j) * nr_rcp(s)) : 0.f;
+            const int om = sm.out_idx[tid / CHI];
+            mv = om >= 0 ? __ldcg(c.m0f + (size_t)om * CHI + tid % CHI) : (tid % CHI == 0 ? 1.f : 0.f);
         }
-        for (int t = tid; t < 3 * CC; t += TEAM) {
-            const int k = t / CC, r = t % CC;
-            sm.D0f[k][r] = sm.out_idx[k] >= 0 ? ldcg(c.D0 + (size_t)sm.out_idx[k] * CC + r) : cf{0.f, 0.f};
-        }
+        if (tid < 3 && out >= 0) t0 = __ldcg(c.t0 + out);
+    }
+#pragma unroll
+    for (int q = 0; q < NT; ++q) {
+        const int t = tid + q * TEAM;
+        if (H2 % TEAM == 0 || t < H2) sm.T[t + (t / CC) * (BPSm<CHI, Mode, TB>::PS - CC)] = tv[q];
+    }
+    if (tid < 3 * CC) {
+        sm.prev[tid / CC][tid % CC] = pv;
+        if constexpr (Mode::mixed) sm.D0f[tid / CC][tid % CC] = dv;
+    }
+    if constexpr (Mode::mixed) {
+        if (tid < 3 * CHI) sm.m0f[tid / CHI][tid % CHI] = mv;
         if (tid < 3) {
-            const cd t = sm.out_idx[tid] >= 0 ? ldcg(c.t0 + sm.out_idx[tid]) : cd{1.0, 0.0};
-            const cf h = ccast<float>(t);
-            sm.t0h[tid] = h;
-            sm.t0l[tid] = ccast<float>(t - ccast<double>(h));
+            sm.t0h[tid] = cf{t0.x, t0.y};
+            sm.t0l[tid] = cf{t0.z, t0.w};
         }
     }
     if (tid == 0) sm.cached = a;
@@ -1103,15 +1132,18 @@ __device__ __forceinline__ cf rcp_sum32(cf hi, cf lo, cf d) {
 
 // First part of the sweep for vertex a: incoming messages, the contractions, and the
 // traces of the three outgoing messages with their reciprocals (left in sm.trs and sm.itr).  Only the
-// team's shared memory is written.
+// team's shared memory is written.  out: as in bp_prepare, read only where the cache holds another vertex.
 template <int CHI, class Mode, int TB>
 __device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<CHI, Mode, TB>& sm, bool have_pre,
-                         C<typename Mode::TS> pre) {
+                         C<typename Mode::TS> pre, int out) {
     using TS = typename Mode::TS;
     using CT = C<TS>;
     using SM = BPSm<CHI, Mode, TB>;
     constexpr int TEAM = TB, CC = CHI * CHI;
-    if (sm.cached != a) bp_prepare<CHI, Mode, TB>(c, a, tid, team, cur, sm);
+    if (sm.cached != a) {
+        bp_prepare<CHI, Mode, TB>(c, a, tid, team, cur, sm, out, pre);
+        have_pre = true;
+    }
     const CT* src = (const CT*)c.msg[cur];
     const CT z = CT{(TS)0, (TS)0};
     // incoming messages (prefetched into `pre` by the caller when have_pre)
@@ -1565,7 +1597,11 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
     if (tid < 3) sm.dsum[tid] = 0;
     __syncthreads();
     const int gteam = team * c.nblocks + blockIdx.x, nt = c.nblocks * tpb_teams;
-    const int inst0 = gteam < c.n ? c.vert_inst[gteam] : 0;   // the first round's vertex
+    // the first round's instance and, in lanes 0..2, its vertex's message index; with several rounds
+    // those of a vertex are fetched during the round before it
+    const bool rounds = c.n > nt;
+    int inst_a = gteam < c.n ? c.vert_inst[gteam] : 0;
+    int out_a = gteam < c.n && tid < 3 ? slot_out(c, gteam, slot_edge(c, gteam, tid)) : -1;
     SMB* all = reinterpret_cast<SMB*>(smem);
     bool have_pre = false;
     CT_ pre = CT_{0, 0};
@@ -1629,14 +1665,20 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
         // rounds of one vertex per team
         for (int base = 0; base < c.n; base += nt) {
             const int a = base + gteam;
-            int inst = 0;
+            const int inst = inst_a, out = out_a;
             bool act = false;
+            int an = gteam, en = -1;   // the next round's vertex (the first one again after the last round)
+            if (rounds && gteam < c.n) {
+                if (a + nt < c.n) an = a + nt;
+                inst_a = c.vert_inst[an];
+                if (tid < 3) en = slot_edge(c, an, tid);
+            }
             if (a < c.n) {
-                inst = base == 0 ? inst0 : c.vert_inst[a];
                 if (!one && done[inst]) bp_copy_vertex<CHI, Mode>(c, a, tid, TB, cur);
                 else act = true;
             }
-            if (act) bp_front<CHI, Mode, TB>(c, a, tid, team, cur, sm, base == 0 && have_pre, pre);
+            if (act) bp_front<CHI, Mode, TB>(c, a, tid, team, cur, sm, base == 0 && have_pre, pre, out);
+            if (rounds && gteam < c.n && tid < 3) out_a = slot_out(c, an, en);
             if (pend) {
                 pend = false;
                 const int r = decide(it - 1, dprev);

@@ -71,6 +71,7 @@ struct gtqa_state {
     void* msg[2] = {nullptr, nullptr};
     cf* D0 = nullptr;
     cd* t0 = nullptr;
+    float* m0f = nullptr;
     cd* X = nullptr;
     int4* edge_info = nullptr;
     int4* vert_edges = nullptr;
@@ -556,7 +557,8 @@ Ctx make_ctx(const gtqa_state* s) {
     c.msg[0] = s->msg[0];
     c.msg[1] = s->msg[1];
     c.D0 = s->D0;
-    c.t0 = s->t0;
+    c.t0 = reinterpret_cast<float4*>(s->t0);
+    c.m0f = s->m0f;
     c.X = s->X;
     c.acc = s->acc;
     c.inst_done = s->inst_done;
@@ -866,6 +868,7 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
     zero(&s->T, gel * eb);
     raw((void**)&s->D0, mixed(s) ? mel * sizeof(cf) : 0);
     raw((void**)&s->t0, mixed(s) ? 2 * M * sizeof(cd) : 0);
+    raw((void**)&s->m0f, mixed(s) && !s->plain ? 2 * M * CHI * sizeof(float) : 0);
     raw((void**)&s->X, M * 2 * CC * sizeof(cd));
     raw((void**)&s->inst_done, sizeof(int) * B);
     raw((void**)&s->inst_iters, sizeof(int) * B);
@@ -1321,6 +1324,7 @@ int gtqa_autotune(gtqa_state* s, double tau, double dt, double tol, int32_t max_
                              {s->msg[0], mel * eb, {}}, {s->msg[1], mel * eb, {}},
                              {s->X, sizeof(cd) * s->m * 2 * s->CHI * s->CHI, {}},
                              {s->D0, mixed(s) ? sizeof(cf) * mel : 0, {}}, {s->t0, mixed(s) ? sizeof(cd) * 2 * s->m : 0, {}},
+                             {s->m0f, mixed(s) ? sizeof(float) * 2 * s->m * s->CHI : 0, {}},
                              {s->stats, sizeof(double) * kStats, {}}, {s->ctl, sizeof(Control), {}},
                              {s->acc, sizeof(double) * 6 * s->B, {}}, {s->inst_done, sizeof(int) * s->B, {}},
                              {s->inst_iters, sizeof(int) * s->B, {}}, {s->inst_dist, sizeof(double) * s->B, {}}};
