@@ -219,7 +219,8 @@ int gtqa_set_grid(gtqa_state* s, const int32_t* grid);
 
 /*
  * Launch-shape variants (3 ints: gates, BP, regauge).  The gates kernel has variants 0 and 1,
- * BP and regauge 0, 1 and 2; variant 0 is the default of gtqa_create_batch.  For CHI <= 4
+ * BP and regauge 0, 1 and 2.  gtqa_create_batch takes variant 0, or at CHI = 8 variant 1 for a kernel
+ * with more items than blocks of 256 threads take in one round, where it fits.  For CHI <= 4
  * (threads per block, BP vertex team, regauge-vertex team) are (512, 64, 32), (256, 64, 32) and
  * (512, 128, 64); for CHI = 8 they are (256, 256, 128), (512, 256, 128) and (512, 512, 256).
  * The gate-edge team (2 CHI^2 threads) is fixed; the regauge-edge team has CHI^2 threads, or

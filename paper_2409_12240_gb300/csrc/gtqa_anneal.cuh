@@ -140,7 +140,7 @@ __device__ __forceinline__ double lam_get(const double* lam, int CHI, int e, int
 // team TG (one lane per element pair of the Jacobi SVD of the 2CHI x 2CHI core), the
 // regauge-edge team TR and the BP-init team TV are fixed by their algorithms; the block size
 // TPB, the BP vertex team TB and the regauge-vertex team TRV come in NSHAPE variants, which
-// gtqa_autotune times kernel by kernel.  Variant 0 is the default:
+// gtqa_autotune times kernel by kernel.  Variant 0 is the default, at CHI = 8 variant 1 on large instances:
 //   CHI <= 4: (TPB, TB, TRV) = (512, 64, 32), (256, 64, 32), (512, 128, 64)
 //   CHI  = 8:                  (256, 256, 128), (512, 256, 128), (512, 512, 256)
 constexpr int NSHAPE = 3;

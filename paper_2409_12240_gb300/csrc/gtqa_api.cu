@@ -745,8 +745,22 @@ int create_impl(int B, const int* n, const int* m, const int* edges, const int* 
         delete s;
         return GTQA_ERR_CUDA;
     }
+    // Variant 0, or at CHI = 8 blocks of 512 threads instead of 256 (variant 1, the same teams) for a
+    // kernel with more items than one round of the smaller blocks takes: two gates, one vertex or
+    // four edges per SM.  Per layer in mixed mode, gates / BP / regauge: n = 12000 9.11 / 4.27 / 1.59 ms
+    // in blocks of 256 and 7.73 / 3.72 / 1.54 in blocks of 512; n = 1000 1063 / 395 / 197 and
+    // 933 / 364 / 152 us; at n = 152 (one round) the smaller blocks are up to 2 % faster.  FP64 gates at
+    // n = 12000 15.8 and 14.8 ms; the FP64 BP of variant 1 does not fit on an SM.
+    long long items[PK_COUNT] = {0, N, Mtot};
+    {
+        std::vector<long long> of_colour(ncol, 0);
+        for (long long e = 0; e < Mtot; ++e) items[PK_GATES] = std::max(items[PK_GATES], ++of_colour[gcol[e]]);
+    }
+    const long long one_round[PK_COUNT] = {2LL * sms, sms, 4LL * sms};
     for (int pk = 0; pk < PK_COUNT && !s->plain; ++pk) {
-        const int src = apply_shape(s, pk, 0);
+        int src = GTQA_ERR_UNSUPPORTED;
+        if (s->CHI == 8 && items[pk] > one_round[pk]) src = apply_shape(s, pk, 1);
+        if (src == GTQA_ERR_UNSUPPORTED) src = apply_shape(s, pk, 0);
         if (src != GTQA_OK) {
             delete s;
             return src;

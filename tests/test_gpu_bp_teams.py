@@ -68,3 +68,24 @@ def test_instances_of_a_large_batch_follow_their_single_runs(chi, copies, precis
         for j in range(i, copies, 3):
             assert np.abs(rho[16 * j:16 * j + 16] - r1).max() < BOUND[precision]
             assert np.abs(lam[x.m * j:x.m * (j + 1)] - l1).max() < BOUND[precision]
+
+
+# chi = 8: blocks of 512 threads from the instance sizes on at which one round of the smaller blocks no
+# longer covers a kernel's items (two gates of a colour, one vertex, four edges per SM)
+@pytest.mark.parametrize("precision,n,variants", [(G.GTQA_MIXED, 152, [0, 0, 0]), (G.GTQA_MIXED, 154, [0, 1, 0]),
+                                                  (G.GTQA_MIXED, 1000, [1, 1, 1]), (G.GTQA_FP64, 1000, [1, 0, 1])])
+def test_chi8_block_size_follows_the_instance(precision, n, variants):
+    inst = make_instance(n, 4)
+    out = []
+    for shape in (None, [0, 0, 0]):
+        s = G.gtqa_create(inst.n, inst.edges, inst.J, inst.h, 8, inst.colour, G.gtqa_options_init(precision))
+        try:
+            t = G.gtqa_launch_shape(s)
+            assert [t[k]["variant"] for k in ("gates_kernel", "bp_kernel", "regauge_kernel")] == variants
+            if shape:
+                G.gtqa_set_shape(s, shape)
+            G.gtqa_anneal(s, 3, 5, 8, 0.3, 1e-12, 100)
+            out.append((G.gtqa_marginals(s)[0], G.gtqa_get_state(s)[1]))
+        finally:
+            G.gtqa_destroy(s)
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])   # the same teams
