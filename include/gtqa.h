@@ -224,7 +224,7 @@ int gtqa_set_grid(gtqa_state* s, const int32_t* grid);
  * (threads per block, BP vertex team, regauge-vertex team) are (512, 64, 32), (256, 64, 32) and
  * (512, 128, 64); for CHI = 8 they are (256, 256, 128), (512, 256, 128) and (512, 512, 256).
  * The gate-edge team (2 CHI^2 threads) is fixed; the regauge-edge team has CHI^2 threads, or
- * CHI^2 / 2 where m exceeds 512 / CHI^2 edges per SM.  FP64 BP at CHI <= 4 uses teams of 128 threads
+ * CHI^2 / 2 where m exceeds 512 / CHI^2 edges per SM.  FP64 BP at CHI = 4 uses teams of 128 threads
  * up to one team per vertex on all SMs (n <= 4 per SM in blocks of 512 threads, 2 in blocks of 256).
  * GTQA_ERR_INVALID_ARG for an index out of range, GTQA_ERR_UNSUPPORTED when a variant's
  * shared memory does not fit on an SM (the state keeps its shapes) or for a plain-path state.

@@ -1167,18 +1167,20 @@ __device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<C
         bp_front_elements<CHI, Mode, TB>(tid, team, sm);
     }
     // traces of the outgoing messages and their reciprocals (reading R10: messages are divided by
-    // their complex trace)
-    if (tid < 3) {
+    // their complex trace).  In FP64 some 20 instructions of one warp: the teams of a block take warps on
+    // different sub-partitions (a team of two warps has two of them, every other team the same two)
+    const int k = Mode::mixed ? tid : tid - 32 * (TEAM == 64 ? (team >> 1) & 1 : team % (TEAM / 32));
+    if (k >= 0 && k < 3) {
         CT trs = z;
 #pragma unroll
-        for (int j = 0; j < CHI; ++j) trs = trs + sm.out(tid, j * CHI + j);
-        sm.trs[tid] = trs;
+        for (int j = 0; j < CHI; ++j) trs = trs + sm.out(k, j * CHI + j);
+        sm.trs[k] = trs;
         if constexpr (Mode::mixed) {
-            sm.itr[tid] = rcp_sum32(sm.t0h[tid], sm.t0l[tid], trs);
+            sm.itr[k] = rcp_sum32(sm.t0h[k], sm.t0l[k], trs);
         } else {
             const double n2 = norm2(trs);
             const double in2 = n2 > 0.0 ? nr_rcp(n2) : 0.0;
-            sm.itr[tid] = cd{trs.x * in2, -trs.y * in2};
+            sm.itr[k] = cd{trs.x * in2, -trs.y * in2};
         }
     }
     team_bar<TEAM>(team);
@@ -1545,7 +1547,7 @@ struct SmemSize {
     static constexpr int TPB = S::TPB;
     static constexpr size_t gate = sizeof(GateSm<CHI, Mode>) * (TPB / S::TG);
     // per-team caches, block sums (64 doubles), for the teams of the shape and the wide ones
-    static constexpr int WIDE_TB = !Mode::mixed && CHI <= 4 && S::TB == 64 ? 128 : S::TB;
+    static constexpr int WIDE_TB = !Mode::mixed && CHI == 4 && S::TB == 64 ? 128 : S::TB;
     static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
     static constexpr size_t bp = mx(sizeof(BPSm<CHI, Mode, S::TB>) * (TPB / S::TB),
                                     sizeof(BPSm<CHI, Mode, WIDE_TB>) * (TPB / WIDE_TB)) + 64 * sizeof(double);
@@ -1616,14 +1618,19 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
     // therefore decides first.  Returns -1 if a barrier gave up, 1 to stop, 0 to go on.
     constexpr bool AHEAD = Mode::mixed;
     bool ex1 = c.max_iter == 1;   // the sweep under way computes the exact distance inline
+    const double thr3d = thr3[0];
+    // Distances and thresholds are not negative, so their bits compare like the values (a NaN lies above
+    // the infinities): every thread decides, and an FP64 comparison of 16 warps is 0.12 us of the pipe.
+    auto less = [](double x, double y) { return __double_as_longlong(x) < __double_as_longlong(y); };
+    auto isnan_d = [](double x) { return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL; };
     auto decide = [&](int itd, double dsum) {
         const bool last = itd + 1 >= c.max_iter;
         bool fin = false;
-        if (c.inst_m[0] == 0 || !(dsum == dsum)) {
+        if (c.inst_m[0] == 0 || isnan_d(dsum)) {
             fin = true;
         } else if (ex1) {
-            fin = last || dsum < thr[0];
-        } else if (last || dsum < thr_hi[0]) {   // a bound under the threshold: the exact distance decides
+            fin = last || less(dsum, thr[0]);
+        } else if (last || less(dsum, thr_hi[0])) {   // a bound under the threshold: the exact distance decides
             double* ex = c.acc + 3 + itd % 3;
             if (blockIdx.x == 0 && threadIdx.x == 0) ++c.ctl->exact_passes;
             if (threadIdx.x == 0) need[0] = 1;
@@ -1631,7 +1638,7 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
             bp_exact_pass<CHI, Mode, S::TPB, TB>(c, cur, need, sm, bsum + 32, ex);
             if (!grid_sync(gb, c.spin_limit)) return -1;
             dsum = __ldcg(ex);
-            fin = last || dsum < thr[0] || !(dsum == dsum);
+            fin = last || less(dsum, thr[0]) || isnan_d(dsum);
             ex1 = true;
             if (blockIdx.x == 0 && threadIdx.x == 0) {
                 c.inst_dist[0] = dsum;
@@ -1646,7 +1653,7 @@ __device__ __forceinline__ bool bp_sweeps(const Ctx& c, GridBarrier& gb, int& cu
             if (fin) c.inst_done[0] = 1;
         }
         // the next sweep is exact inline when it is the last or when this one came within a factor 3
-        ex1 = itd + 2 >= c.max_iter || (float)dsum < thr3[0];
+        ex1 = itd + 2 >= c.max_iter || less(dsum, thr3d);
         return fin ? 1 : 0;
     };
     const bool one = c.B == 1;
@@ -1886,7 +1893,7 @@ __device__ __forceinline__ void anneal_body(const Ctx& c) {
                 }
                 if (!grid_sync(gb, c.spin_limit)) return;
             }
-            // FP64 at CHI <= 4 while a block's vertices all have a team of four warps: one warp per
+            // FP64 at CHI = 4 while a block's vertices all have a team of four warps: one warp per
             // sub-partition halves a sweep's FP64 time where a block has one vertex (10.4 -> 5.6 us) and
             // evens the sub-partitions out for an odd number; beyond that the teams of two keep every
             // vertex resident
