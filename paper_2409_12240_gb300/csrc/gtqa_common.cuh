@@ -691,7 +691,9 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 //      all pairs with |K_pq| <= 1e-4.  K is antihermitian, so the factor is unitary up to
 //      |K|^4/4 < 3e-17, and the off-diagonals shrink to products of their sizes.  Without F64 the
 //      corrections are formed in FP32 where every kept column moves by less than 1e-3 of its length
-//      (12 FP64 instructions per warp instead of 64).  The passes end once every pair was below `stop` (relative to its columns) before its pass.
+//      (12 FP64 instructions per warp instead of 64).  A pair is open, and asks for another pass, while
+//      its cosine is above `stop` or, unless the cosine is below tol, its |K| above 1e-8 (1e-4 without
+//      F64): columns of nearly the same length take a large rotation at a small cosine.
 //      A pair with a larger K (nearly equal or not yet resolved columns) is rotated by
 //      FP64 Jacobi steps (only the steps of the schedule that hold such a pair) or, for N >= 16
 //      with many of them, by FP32 Jacobi on those and all shorter columns of W, rescaled,
@@ -915,15 +917,16 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
     }
     cnt.sweeps32 = svd32_unitary<N, F64>(V, A32, V32, nrm, g, grp, pair_mask, keep_rank);
     mul64<N, false>(A, V, g, grp);
-    const float stop2 = stop * stop, cut2 = (float)(0.25 * cut * cut);
+    const float stop2 = stop * stop, cut2 = (float)(0.25 * cut * cut), tol2 = (float)(tol * tol);
+    constexpr float OPEN2 = F64 ? 1e-16f : KMAX2;
     int second = 0;   // FP32 runs on a part of the columns
     for (int pass = 0;; ++pass) {
         const CD gam = gram<N>(A, nrm, g, grp, has, p, q);
         ++cnt.passes;
         cnt.pairs += NP;
         CF K = CF{0.f, 0.f};
-        // 1: a pair above stop, 2: one of those with a large K, 4: |K| > 1e-8, 8: any K, 16: a K that moves
-        // the pair's shorter column by more than 1e-3 of its length
+        // 1: an open pair, 2: one of those with a large K, 32: and with a cosine above stop, 4: |K| > 1e-8,
+        // 8: any K, 16: a K that moves the pair's shorter column by more than 1e-3 of its length
         unsigned flags = 0u;
         if (has) {
             const double al = nrm[p], be = nrm[q];
@@ -948,17 +951,22 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                 const float gx = (float)(gam.x * gsc), gy = (float)(gam.y * gsc);
                 const float g2 = fmaf(gx, gx, gy * gy);
                 const float lim = rp && rq ? an * bn : fmaxf(an, bn) * fmaxf(an, bn);
-                const bool open = g2 > stop2 * 1.152921504606847e18f * lim;
-                if (open) flags |= 1u;
+                const bool wide = g2 > stop2 * 1.152921504606847e18f * lim;
+                if (wide) flags |= 1u;
                 if (g2 > 0.f) {
                     const float g2n = g2 * 8.673617379884035e-19f;
                     const float tn = 2.f * 9.313225746154785e-10f * __frcp_rn(fabsf(dn) + sqrtf(fmaf(dn, dn, 4.f * g2n)));
                     const float t = dn >= 0.f ? tn : -tn;
                     K = CF{t * gx, t * gy};
                     const float k2 = norm2(K);
+                    // Columns of nearly the same length: the rotation is gamma over the difference of the
+                    // squared lengths, which may be of order one where the cosine is far below `stop`
+                    // (a cosine of 1e-9 between lengths equal to 1e-9 leaves the kept triplets open).  Such a
+                    // pair is open until K is small or the cosine is rounding.
+                    if (k2 > OPEN2 && g2 > tol2 * 1.152921504606847e18f * lim) flags |= 1u;
                     if (!(k2 <= KMAX2)) {
                         K = CF{0.f, 0.f};
-                        if (open) flags |= 2u;
+                        if (flags & 1u) flags |= wide ? 34u : 2u;
                     } else {
                         flags |= 8u;
                         if (k2 > 1e-16f) flags |= 4u;
@@ -1013,7 +1021,8 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         if (!(flags & 1u)) break;
         if (pass + 1 >= MAXP) {
             int nsteps = 0;
-            cnt.passes += jacobi_polish<N, Group, true>(A, V, nrm, g, grp, pair_mask, tol, stop, 60, &cnt.rot, keep_rank,
+            // to the resolution of the rotations: `stop` would leave pairs of close lengths open
+            cnt.passes += jacobi_polish<N, Group, true>(A, V, nrm, g, grp, pair_mask, tol, 16.0 * tol, 60, &cnt.rot, keep_rank,
                                                         relmask, &nsteps);
             cnt.pairs += nsteps * (N / 2);
             break;
@@ -1022,14 +1031,15 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         const unsigned steps = grp.or_bits((mine & 2u) ? 1u << step : 0u);
         const int nst = __popc(steps);
         bool part = false;
-        if constexpr (N >= 16) part = nst > N / 4 && second < 3;
+        if constexpr (N >= 16)   // FP32 resolves nothing below a cosine of 1e-7
+            part = second < 3 && __popc(grp.or_bits((mine & 32u) ? 1u << step : 0u)) > N / 4;
         if (!part) {
             jacobi_polish<N, Group, true>(A, V, nrm, g, grp, pair_mask, tol, stop, 1, &cnt.rot, N, nullptr, nullptr, steps);
             cnt.pairs += nst * (N / 2);
         } else if constexpr (N >= 16) {
             ++second;
             // the columns of those pairs, and every shorter one
-            unsigned cols = grp.or_bits((mine & 2u) ? (1u << p) | (1u << q) : 0u);
+            unsigned cols = grp.or_bits((mine & 32u) ? (1u << p) | (1u << q) : 0u);
             double longest = 0.0;
             for (int j = 0; j < N; ++j)
                 if ((cols >> j) & 1u) longest = fmax(longest, nrm[j]);

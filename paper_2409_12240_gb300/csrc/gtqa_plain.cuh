@@ -488,7 +488,9 @@ __device__ RC plain_trace_norm(const C<R>* dm, unsigned char* base, int g, const
         cf* A32 = reinterpret_cast<cf*>(T + CC);
         double* nrm = reinterpret_cast<double*>(A32 + 2 * CC);
         prune_noise<CHI>(A, g, grp);
-        refined_svd<CHI, true>(A, V, A32, A32 + CC, T, nrm, nullptr, g, grp, group_mask<CHI>(), 1e-16, CHI, 1e-8f, 1e-15);
+        // tol 1e-8: the sum of the values depends on a cosine that is left only in second order, so pairs
+        // of close lengths (a traceless difference has them) need no rotation beyond that
+        refined_svd<CHI, true>(A, V, A32, A32 + CC, T, nrm, nullptr, g, grp, group_mask<CHI>(), 1e-16, CHI, 1e-8f, 1e-8);
         if (g == 0)
             for (int q = 0; q < CHI; ++q) s += nr_sqrt(nrm[q]);
     } else {

@@ -1,0 +1,153 @@
+"""Decompositions with singular values that are close but not equal: at the truncation cut, where the
+kept triplets depend on resolving the pair, and in the regauge, against the oracle's LAPACK."""
+import numpy as np
+import pytest
+
+from oracle import gtqa_oracle as O
+from paper_2409_12240_gb300 import gtqa as G
+
+pytestmark = pytest.mark.gpu
+
+
+def two_centres(C, D, gap, seed):
+    """Two joined vertices of degree D with their leaves, and a state whose joining bond (edge 0), after
+    the gate exp(-i theta Z Z) with tan(theta) = 0.6, has 2 C singular values of which the C-th
+    and the (C+1)-th differ by the relative gap (a list: that many values after the C-th lie at
+    these distances).  The blocks of the two sides by physical index have orthonormal columns, so
+    the gate splits every value v into v cos(theta) and v sin(theta); a unitary on the bond mixes
+    the columns."""
+    rng = np.random.default_rng(seed)
+    edges = [(0, 1)]
+    for v in (0, 1):
+        for _ in range(D - 1):
+            edges.append((v, 2 + len(edges) - 1))
+    n, m = 2 * D, len(edges)
+    gaps = np.atleast_1d(gap)
+    half = C // 2
+    value = np.concatenate([np.linspace(1.0, 0.7, half) if half > 1 else [1.0], np.linspace(0.1, 0.05, C - half)])
+    value[half:half + gaps.size] = 0.6 * value[half - 1] * (1.0 - gaps)
+    value = value[:C]
+    unitary = lambda r, c: np.linalg.qr(rng.standard_normal((r, c)) + 1j * rng.standard_normal((r, c)))[0]  # noqa: E731
+    R = C ** (D - 1)
+    mix = unitary(C, C)
+    bond = np.linspace(1.0, 0.4, C)
+    bond /= np.linalg.norm(bond)
+    side = (lambda u: u @ mix), (lambda u: (u * value) @ mix.conj() / bond)
+    Gam = np.zeros((n, 2) + (C,) * D, dtype=np.complex128)
+    lam = np.full((m, C), C ** -0.5)
+    lam[0] = bond
+    for v in (0, 1):
+        for i in range(2):
+            block = side[v](unitary(R, C)) * C ** (0.5 * (D - 1))   # rows over the leaves' weights
+            Gam[v, i] = np.moveaxis(block.reshape((C,) * (D - 1) + (C,)), -1, 0)
+    Gam[2:].reshape(n - 2, 2, C, -1)[..., 0] = rng.standard_normal((n - 2, 2, C)) + 1j * rng.standard_normal((n - 2, 2, C))
+    colour = [0] + 2 * list(range(1, D))
+    return n, np.array(edges), np.array(colour), Gam, lam
+
+
+THETA = float(np.arctan(0.6))
+SHAPES = [(2, 3), (4, 3), (8, 3), (16, 3), (2, 4), (4, 4)]
+# A state's error is a decomposition's backward error over the relative gap: at most some 100 units of
+# 1e-16 (inner products and rotations of up to 64 terms) in the library, and as much in the oracle.
+# Mixed: the stated 1e-4, with the oracle on the same complex64 tensors.
+CASES = [(G.GTQA_FP64, d, max(1e-12, 2e-14 / d)) for d in (1e-3, 1e-5, 1e-7, 1e-9)]
+CASES += [(G.GTQA_MIXED, d, 1e-4) for d in (1e-3, 1e-5)]
+
+
+def both_sides(C, D, precision, state, update):
+    """(library, oracle) normalised state vector and bond weights of edge 0 after `update`."""
+    n, edges, colour, Gam, lam = state
+    if precision == G.GTQA_MIXED:
+        Gam = Gam.astype(np.complex64).astype(np.complex128)
+    m = len(edges)
+    J = np.zeros(m)
+    J[0] = 1.0
+    st = O.from_padded(n, edges, Gam, lam)
+    s = G.gtqa_create(n, edges, J, np.zeros(n), C, colour, G.gtqa_options_init(precision))
+    try:
+        G.gtqa_set_state(s, Gam, lam, O.messages_to_padded(st, O.reconstructed_messages(st), C))
+        st = update(s, st, colour, J)
+        Gg, lg, _ = G.gtqa_get_state(s)
+    finally:
+        G.gtqa_destroy(s)
+    got = O.from_padded(n, edges, Gg, lg)
+    out = []
+    for x in (got, st):
+        psi = O.to_statevector(x)
+        out.append((psi / np.linalg.norm(psi), np.pad(x.lam[0], (0, C - x.lam[0].size))))
+    return out
+
+
+@pytest.mark.parametrize("seed", [1, 2])
+@pytest.mark.parametrize("precision,gap,bound", CASES)
+@pytest.mark.parametrize("C,D", SHAPES)
+def test_gate_with_close_values_at_the_cut(C, D, precision, gap, bound, seed):
+    def layer(s, st, colour, J):
+        G.gtqa_trotter_split(s, THETA, 0.0, 0.0)
+        O.trotter_layer(st, colour, J, np.zeros(st.n), THETA, 0.0, C)
+        return st
+
+    (a, la), (b, lb) = both_sides(C, D, precision, two_centres(C, D, gap, seed), layer)
+    assert np.abs(la - lb).max() < (1e-12 if precision == G.GTQA_FP64 else 1e-6)
+    assert np.linalg.norm(a - b) < bound
+
+
+@pytest.mark.parametrize("gap", [1e-5, 1e-7, 1e-9])
+@pytest.mark.parametrize("C,D", [(2, 3), (4, 3), (8, 3), (4, 4)])
+def test_arbitrary_gate_with_close_values_at_the_cut(C, D, gap):
+    z = np.array([1.0, -1.0])
+    U = np.diag(np.exp(-1j * THETA * np.kron(z, z)))
+
+    def gate(s, st, colour, J):
+        G.gtqa_apply_gates(s, [0], U[None])
+        O.apply_gates(st, [(0, U)], C)
+        return st
+
+    (a, la), (b, lb) = both_sides(C, D, G.GTQA_FP64, two_centres(C, D, gap, 3), gate)
+    assert np.abs(la - lb).max() < 1e-12
+    assert np.linalg.norm(a - b) < max(1e-12, 2e-14 / gap)
+
+
+@pytest.mark.parametrize("C", [4, 8, 16])
+def test_gate_with_several_close_values_at_the_cut(C):
+    """Three values next to the cut within 3e-6 of each other."""
+    def layer(s, st, colour, J):
+        G.gtqa_trotter_split(s, THETA, 0.0, 0.0)
+        O.trotter_layer(st, colour, J, np.zeros(st.n), THETA, 0.0, C)
+        return st
+
+    (a, la), (b, lb) = both_sides(C, 3, G.GTQA_FP64, two_centres(C, 3, [1e-6, 3e-6], 4), layer)
+    assert np.abs(la - lb).max() < 1e-12
+    assert np.linalg.norm(a - b) < 2e-14 / 1e-6
+
+
+@pytest.mark.parametrize("gap", [1e-5, 1e-7, 1e-9])
+@pytest.mark.parametrize("C,D", SHAPES)
+def test_regauge_of_messages_with_close_eigenvalues(C, D, gap):
+    """Eigenvalues in pairs of the relative gap.  lambda is backward stable whatever the gap; the
+    state vector does not depend on the gauge."""
+    n, edges, colour, Gam, lam = two_centres(C, D, 1e-3, 5)
+    rng = np.random.default_rng(6)
+    st = O.from_padded(n, edges, Gam, lam)
+    msgs = {}
+    for key in O.reconstructed_messages(st):
+        w = np.repeat(np.linspace(1.0, 0.3, C // 2), 2)
+        w[1::2] *= 1.0 - gap
+        q = np.linalg.qr(rng.standard_normal((C, C)) + 1j * rng.standard_normal((C, C)))[0]
+        msgs[key] = (q * (w / w.sum())) @ q.conj().T
+    s = G.gtqa_create(n, edges, np.zeros(len(edges)), np.zeros(n), C, colour)
+    try:
+        G.gtqa_set_state(s, Gam, lam, O.messages_to_padded(st, msgs, C))
+        G.gtqa_bp_sweep(s, 0.0, 1, 0)   # T from Gamma; one sweep replaces the messages
+        G.gtqa_set_state(s, Gam, lam, O.messages_to_padded(st, msgs, C))
+        G.gtqa_regauge(s)
+        Gg, lg, _ = G.gtqa_get_state(s)
+    finally:
+        G.gtqa_destroy(s)
+    want = O.vidal_gauge(st, O.symmetric_gauge(st), msgs)
+    ref = O.to_padded(want, C, D)[1]
+    assert np.abs(lg - ref).max() < 1e-12
+    got = O.from_padded(n, edges, Gg, lg)
+    assert np.abs(O.local_orthogonality_residual(got) - O.local_orthogonality_residual(want)) < 1e-11
+    a, b = O.to_statevector(got), O.to_statevector(want)
+    assert np.linalg.norm(a / np.linalg.norm(a) - b / np.linalg.norm(b)) < 1e-11
