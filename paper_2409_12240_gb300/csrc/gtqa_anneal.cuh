@@ -651,7 +651,7 @@ struct BPSm {
     float m0f[3][CHI];   // mixed: warm-start diagonals
     cf t0h[3], t0l[3];   // mixed: traces of F0, as sums of two floats
     C<TS> trs[3];        // traces of the outgoing messages (mixed: of the correction terms)
-    C<TS> itr[3];        // 1 / trace, formed in FP64
+    C<TS> itr[3];        // 1 / trace (mixed: from pairs of floats, rcp_sum32)
     TS dl[3];
     TS dsum[3];          // one instance: the team's distance summed over the rounds of a sweep
     int es[3], out_idx[3], in_idx[3];
@@ -1122,14 +1122,22 @@ __device__ __forceinline__ cf rcp_sum32(cf hi, cf lo, cf d) {
     sum32(h, e + lo.x, x, xl);
     sum32(hi.y, d.y, h, e);
     sum32(h, e + lo.y, y, yl);
+    if (x == 0.f && y == 0.f) return cf{0.f, 0.f};
+    // scaled by a power of two to between 1 and 4, so that the squares stay in range for every trace
+    // that complex64 holds (a vertex tensor may carry any factor)
+    const int ex = max(__float_as_int(x) & 0x7f800000, __float_as_int(y) & 0x7f800000);
+    const float sc = __int_as_float(min(max(0x7f000000 - ex, 0x00800000), 0x7e800000));
+    x *= sc;
+    xl *= sc;
+    y *= sc;
+    yl *= sc;
     const float px = __fmul_rn(x, x), py = __fmul_rn(y, y);
     float n, nl;
     sum32(px, py, n, nl);
     nl += (fmaf(x, x, -px) + 2.f * x * xl) + (fmaf(y, y, -py) + 2.f * y * yl);
-    if (!(n > 0.f)) return cf{0.f, 0.f};
     const float r = __frcp_rn(n), rl = r * (fmaf(-n, r, 1.f) - nl * r);   // r + rl = 1 / (n + nl)
     const float ax = __fmul_rn(x, r), ay = __fmul_rn(y, r);
-    return cf{ax + (fmaf(x, r, -ax) + (x * rl + xl * r)), -(ay + (fmaf(y, r, -ay) + (y * rl + yl * r)))};
+    return cf{sc * (ax + (fmaf(x, r, -ax) + (x * rl + xl * r))), -sc * (ay + (fmaf(y, r, -ay) + (y * rl + yl * r)))};
 }
 
 // First part of the sweep for vertex a: incoming messages, the contractions, and the
