@@ -415,6 +415,12 @@ __device__ void plain_bp_item(const PlainBPArgs& a, int item, int cur, int tid, 
     }
 }
 
+// sqrt of a squared norm, 0 for 0; a NaN stays one, so that the distance reports it
+template <typename R>
+__device__ __forceinline__ R norm_root(R x) {
+    return x == x ? nr_sqrt(x) : x;
+}
+
 // (B): message o from its two halves; returns the Frobenius norm of new - old
 template <int CHI, typename R, typename RC>
 __device__ RC plain_bp_finish(const PlainBPArgs& a, int o, int cur, int lane) {
@@ -471,7 +477,7 @@ __device__ RC plain_bp_finish(const PlainBPArgs& a, int o, int cur, int lane) {
         }
     }
     d2 = group_sum<32>(d2, 0xffffffffu);
-    return nr_sqrt(d2);
+    return norm_root(d2);
 }
 
 // (C): trace norm of new - old of message o (group of CC / 2 lanes)
@@ -492,7 +498,7 @@ __device__ RC plain_trace_norm(const C<R>* dm, unsigned char* base, int g, const
         // of close lengths (a traceless difference has them) need no rotation beyond that
         refined_svd<CHI, true>(A, V, A32, A32 + CC, T, nrm, nullptr, g, grp, group_mask<CHI>(), 1e-16, CHI, 1e-8f, 1e-8);
         if (g == 0)
-            for (int q = 0; q < CHI; ++q) s += nr_sqrt(nrm[q]);
+            for (int q = 0; q < CHI; ++q) s += norm_root(nrm[q]);
     } else {
         jacobi_svd<CHI, RC, Group, false>(A, nullptr, g, grp, group_mask<CHI>(), (RC)1e-6, 60, false);
         grp.sync();
@@ -500,7 +506,7 @@ __device__ RC plain_trace_norm(const C<R>* dm, unsigned char* base, int g, const
             for (int q = 0; q < CHI; ++q) {
                 RC n2 = (RC)0;
                 for (int r = 0; r < CHI; ++r) n2 += norm2(A[q * CHI + r]);
-                s += nr_sqrt(n2);
+                s += norm_root(n2);
             }
     }
     grp.sync();
