@@ -361,7 +361,8 @@ __device__ void plain_bp_item(const PlainBPArgs& a, int item, int cur, int tid, 
         int dim = 1;
         if (e >= 0) {
             dim = 0;
-            for (int q = 0; q < CHI; ++q) dim = __ldcg(a.p.lam + (size_t)e * CHI + q) > 0.0 ? q + 1 : dim;
+            // (a NaN counts: its index must reach the distance, which reports it)
+            for (int q = 0; q < CHI; ++q) dim = __ldcg(a.p.lam + (size_t)e * CHI + q) <= 0.0 ? dim : q + 1;
         }
         tm.dim[tid] = dim;
         tm.dim[4 + tid] = e < 0 ? -1 : 2 * e + (a.p.edge_info[e].x == v ? 0 : 1);
@@ -1277,7 +1278,7 @@ __global__ void __launch_bounds__(512, 1) ising16_gate_kernel(PlainGateArgs c) {
     if (tid == 0) sm.nrot = 0;
     __syncthreads();
     int nc = 0;   // the bond's current dimension
-    for (int j = 0; j < CHI; ++j) nc = sm.lab[j] > 0.0 ? j + 1 : nc;
+    for (int j = 0; j < CHI; ++j) nc = sm.lab[j] <= 0.0 ? nc : j + 1;   // (a NaN counts)
     nc = nc > 0 ? nc : 1;
     double w2[2];
 #pragma unroll 1

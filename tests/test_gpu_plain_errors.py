@@ -7,7 +7,8 @@ from paper_2409_12240_gb300 import gtqa as G
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(2, 4, G.GTQA_FP64), (4, 4, G.GTQA_FP64), (4, 4, G.GTQA_MIXED), (2, 3, G.GTQA_C64), (4, 3, G.GTQA_C64)]
+SHAPES = [(2, 4, G.GTQA_FP64), (4, 4, G.GTQA_FP64), (4, 4, G.GTQA_MIXED), (2, 3, G.GTQA_C64), (4, 3, G.GTQA_C64),
+          (8, 3, G.GTQA_C64), (16, 3, G.GTQA_FP64), (16, 3, G.GTQA_MIXED), (16, 3, G.GTQA_C64)]
 
 
 def plain_state(chi, degree, precision):
