@@ -75,6 +75,12 @@ struct PlainShape {
     static constexpr size_t vertex_smem = sizeof(C<R>) * (PH + CC);
 };
 
+// Whether an earlier launch on this state failed (a NaN distance, a barrier that gave up).  The host reads
+// the status once per call, so the BP runs and regauges behind a failed launch leave by themselves: a
+// barrier that gave up leaves a count that is no multiple of the grid, and messages half written.  The
+// load is issued at a kernel's start and used where it waits or writes first, so that it costs no latency.
+__device__ __forceinline__ bool run_failed(const Control* ctl) { return __ldcg(&ctl->err) != 0; }
+
 __device__ __forceinline__ int plain_slot_edge(const int4& v, int k) {
     return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
 }
@@ -522,6 +528,7 @@ __global__ void __launch_bounds__(512, 1) plain_bp_kernel(PlainBPArgs a) {
     __shared__ double bsum;
     __shared__ int flags[8];
     Control* ctl = a.p.ctl;
+    if (threadIdx.x == 0) flags[0] = run_failed(ctl);   // one value per block: another one may give up meanwhile
     GridBarrier gb = grid_barrier_init(a.bar, &ctl->err, (unsigned)a.bar_expect);
     int cur = *(volatile int*)&ctl->cur;
     const int team = threadIdx.x / NT, tid = threadIdx.x % NT;
@@ -541,6 +548,10 @@ __global__ void __launch_bounds__(512, 1) plain_bp_kernel(PlainBPArgs a) {
         }
         for (int item = team * a.nblocks + blockIdx.x; item < 2 * a.p.n; item += a.nblocks * S::TEAMS)
             plain_bp_item<CHI, D, R, RC>(a, item, cur, tid, team, tm);
+        if (it == 0) {
+            __syncthreads();
+            if (flags[0]) return;
+        }
         if (!grid_sync(gb, a.spin_limit)) return;
         if (threadIdx.x == 0) bsum = 0.0;
         __syncthreads();
@@ -640,6 +651,7 @@ __global__ void __launch_bounds__(CHI * CHI) plain_regauge_edge_kernel(PlainArgs
         if constexpr (GL <= 32) plain_edge_svd<CHI, RC>(A, V, sm, x, g, WarpGroup{group_mask<GL>()}, cut);
         else plain_edge_svd<CHI, RC>(A, V, sm, x, g, TeamGroup<GL>{x, &sm.flag[x]}, cut);
     };
+    const bool failed = run_failed(a.ctl);
     const C<R>* msg = (const C<R>*)a.msg[a.ctl->cur];
     // mixed mode: the messages hold delta = m - m0, m0 = diag(lambda_e)/sum(lambda_e) (read before
     // this kernel overwrites lambda_e)
@@ -705,6 +717,7 @@ __global__ void __launch_bounds__(CHI * CHI) plain_regauge_edge_kernel(PlainArgs
     }
     bar();
     for (int cc = tid; cc < CHI; cc += NT) sm.perm[desc_rank(sm.sig, CHI, cc)] = cc;
+    if (failed) return;
     bar();
     if (tid == 0) {
         RC tot = 0.0;
@@ -783,10 +796,12 @@ __global__ void __launch_bounds__(PlainShape<CHI, D, R, R>::NT) plain_regauge_ve
     C<R>* Xs = buf + S::PH;
     const int v = blockIdx.x >> 1;
     const int4 sl = a.vslots[v];
+    const bool failed = run_failed(a.ctl);
     const C<R>* T = (const C<R>*)a.T + (size_t)blockIdx.x * S::H;
     for (int t = threadIdx.x; t < S::H; t += NT) buf[t + t / CC] = T[t];
     __syncthreads();
     plain_regauge_slot<CHI, D, R, 0>(buf, Xs, a, sl, v, threadIdx.x);
+    if (failed) return;
     C<R>* g = (C<R>*)a.Gamma + (size_t)blockIdx.x * S::H;
     for (int t = threadIdx.x; t < S::H; t += NT) g[t] = buf[t + t / CC];
 }

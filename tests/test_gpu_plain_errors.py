@@ -1,4 +1,6 @@
-"""Errors inside a run of the plain path are reported."""
+"""Errors inside a run of the plain path are reported and end the run."""
+import time
+
 import numpy as np
 import pytest
 
@@ -37,3 +39,22 @@ def test_nan_is_reported(chi, degree, precision, call):
         assert err.value.code == G.GTQA_ERR_NUMERIC
     finally:
         G.gtqa_destroy(s)
+
+
+@pytest.mark.parametrize("chi,degree,precision", SHAPES)
+def test_layers_after_a_barrier_that_gave_up_do_not_run(chi, degree, precision):
+    """One barrier waits for an arrival that does not come and gives up; forty layers take no longer
+    over it than one."""
+    took = {}
+    for layers in (1, 40):
+        _, s = plain_state(chi, degree, precision)
+        try:
+            G.gtqa_debug_barrier(s, 100000, 1)
+            t = time.perf_counter()
+            with pytest.raises(G.GTQAError) as err:
+                G.gtqa_anneal(s, 1, layers, 40, 0.3, 1e-6, 20)
+            took[layers] = time.perf_counter() - t
+            assert err.value.code == G.GTQA_ERR_TIMEOUT
+        finally:
+            G.gtqa_destroy(s)
+    assert took[40] < 5 * took[1] + 0.1
