@@ -907,9 +907,17 @@ __device__ __forceinline__ void bp_front_fibers(int tid, int team, BPSm<CHI, Mod
     team_bar<TB>(team);
 }
 
+// The warp of a team that takes a stage of one warp's work: those of a block's teams spread over the
+// sub-partitions (a team of two warps has two of them, every other team the same two).
+template <int TEAM>
+__device__ __forceinline__ int lone_warp(int team) {
+    return TEAM == 64 ? (team >> 1) & 1 : team % (TEAM / 32);
+}
+
 // The contractions of a sweep element by element (FP64 mode, and the shapes without a fiber-wise form).
+// lone: no block has a second vertex.
 template <int CHI, class Mode, int TB>
-__device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, Mode, TB>& sm) {
+__device__ __forceinline__ void bp_front_elements(int tid, int team, bool lone, BPSm<CHI, Mode, TB>& sm) {
     using TS = typename Mode::TS;
     using CT = C<TS>;
     using SM = BPSm<CHI, Mode, TB>;
@@ -919,6 +927,8 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
     const CT z = CT{(TS)0, (TS)0};
     constexpr bool EVEN = H2 % TEAM == 0;   // whole tensors per team pass: slots fixed at compile time
     auto slot_stride = [](int k) { return k == 0 ? S0 : (k == 1 ? S1 : 1); };
+    // a stage of no more than one warp's work: the teams of a block take warps on different sub-partitions
+    const int wt = (tid + TEAM - 32 * lone_warp<TEAM>(team)) % TEAM;
     if constexpr (!Mode::mixed) {
         // the messages on the slots before s contracted into T, those after s (as m^H) into the other
         // factor of the overlap: L_1 = T x_0 m_0, R_1 = T x_2 m_2^H, L_2 = L_1 x_1 m_1, R_0 = R_1 x_1 m_1^H;
@@ -942,9 +952,30 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
 #pragma unroll
                 for (int w = 0; w < H2 / TEAM; ++w) contract(s1, d1, k1, true, tid + w * TEAM);
             } else {
-                for (int t = tid; t < 2 * H2; t += TEAM) {
-                    if (t < H2) contract(s0, d0, k0, false, t);
-                    else contract(s1, d1, k1, true, t - H2);
+                // CHI = 2, 16 elements each.  As two branches of one warp the contractions would be issued
+                // one after the other.  Where a block has several vertices they fill one warp in one
+                // instruction stream (m or m^H by index and sign: half the FP64 instructions), for
+                // a lone vertex two warps (no selects: 7.5 -> 7.4 us per sweep at n = 100).
+                static_assert(H2 == 16 && TEAM >= 64, "two contractions in one warp, or in two");
+                auto one = [&](const CT* src, CT* dst, int k, bool adj, int e) {
+                    const int pe = e + e / CC, st = slot_stride(k);
+                    const int x = k == 0 ? (e / CC) % CHI : (k == 1 ? (e / CHI) % CHI : e % CHI);
+                    const int base = pe - x * st;
+                    CT acc = z;
+#pragma unroll
+                    for (int q = 0; q < CHI; ++q) {
+                        CT m = sm.min[k][adj ? x * CHI + q : q * CHI + x];
+                        if (adj) m.y = __longlong_as_double(__double_as_longlong(m.y) ^ LLONG_MIN);
+                        acc = cfma(m, src[base + q * st], acc);
+                    }
+                    dst[pe] = acc;
+                };
+                if (lone) {
+                    if (tid < H2) one(s0, d0, k0, false, tid);
+                    else if (tid >= 32 && tid < 32 + H2) one(s1, d1, k1, true, tid - 32);
+                } else if (wt < 2 * H2) {
+                    const bool adj = wt >= H2;
+                    one(adj ? s1 : s0, adj ? d1 : d0, adj ? k1 : k0, adj, wt % H2);
                 }
             }
             team_bar<TEAM>(team);
@@ -1058,7 +1089,7 @@ __device__ __forceinline__ void bp_front_elements(int tid, int team, BPSm<CHI, M
             }
         }
     } else if constexpr (SM::HALVES) {
-        for (int t = tid; t < 2 * 3 * CC; t += TEAM) {
+        for (int t = wt; t < 2 * 3 * CC; t += TEAM) {
             const int i = t / (3 * CC), rem = t % (3 * CC);
             const int s = rem / CC, r = rem % CC;
             if (sm.es[s] < 0) continue;
@@ -1174,12 +1205,11 @@ __device__ void bp_front(const Ctx& c, int a, int tid, int team, int cur, BPSm<C
     if constexpr (SM::FIBERS) {
         bp_front_fibers<CHI, Mode, TB>(tid, team, sm);
     } else {
-        bp_front_elements<CHI, Mode, TB>(tid, team, sm);
+        bp_front_elements<CHI, Mode, TB>(tid, team, c.n <= c.nblocks, sm);
     }
     // traces of the outgoing messages and their reciprocals (reading R10: messages are divided by
-    // their complex trace).  In FP64 some 20 instructions of one warp: the teams of a block take warps on
-    // different sub-partitions (a team of two warps has two of them, every other team the same two)
-    const int k = Mode::mixed ? tid : tid - 32 * (TEAM == 64 ? (team >> 1) & 1 : team % (TEAM / 32));
+    // their complex trace).  In FP64 some 20 instructions of one warp
+    const int k = Mode::mixed ? tid : tid - 32 * lone_warp<TEAM>(team);
     if (k >= 0 && k < 3) {
         CT trs = z;
 #pragma unroll
