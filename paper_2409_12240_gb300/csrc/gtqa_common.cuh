@@ -693,7 +693,8 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 //      corrections are formed in FP32 where every kept column moves by less than 1e-3 of its length
 //      (12 FP64 instructions per warp instead of 64).  A pair is open, and asks for another pass, while
 //      its cosine is above `stop` or, unless the cosine is below tol, its |K| above 1e-8 (1e-4 without
-//      F64): columns of nearly the same length take a large rotation at a small cosine.
+//      F64): columns of nearly the same length take a large rotation at a small cosine.  With F64 the
+//      columns that do not count set the end too, where they are long and not orthogonal to each other.
 //      A pair with a larger K (nearly equal or not yet resolved columns) is rotated by
 //      FP64 Jacobi steps (only the steps of the schedule that hold such a pair) or, for N >= 16
 //      with many of them, by FP32 Jacobi on those and all shorter columns of W, rescaled,
@@ -926,30 +927,31 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         cnt.pairs += NP;
         CF K = CF{0.f, 0.f};
         // 1: an open pair, 2: one of those with a large K, 32: and with a cosine above stop, 4: |K| > 1e-8,
-        // 8: any K, 16: a K that moves the pair's shorter column by more than 1e-3 of its length
+        // 8: any K, 16: a K that moves the pair's shorter column by more than 1e-3 of its length; from bit 8 on:
+        // sizes of K and c (below)
         unsigned flags = 0u;
         if (has) {
             const double al = nrm[p], be = nrm[q];
-            const long long la = __double_as_longlong(al), lb = __double_as_longlong(be);
-            // positive doubles compare as integers; + 2 in the exponent: times 4
-            const long long a4 = la + (2ll << 52), b4 = lb + (2ll << 52);
-            long long lmax = 0;
+            // the upper words of positive doubles compare as integers; + 2 in the exponent: times 4
+            const int ha = __double2hiint(al), hb = __double2hiint(be), a4 = ha + (2 << 20), b4 = hb + (2 << 20);
+            int hmax = 0, next = INT_MAX;   // longest column; shortest one clearly longer than the pair's
             int ca = 0, cb = 0;
             for (int j = 0; j < N; ++j) {
-                const long long x = __double_as_longlong(nrm[j]);
+                const int x = __double2hiint(nrm[j]);
                 ca += x > a4;
                 cb += x > b4;
-                lmax = x > lmax ? x : lmax;
+                hmax = max(hmax, x);
+                if (F64) next = x > max(a4, b4) ? min(next, x) : next;
             }
-            const double sc = inv_exp2((int)((la > lb ? la : lb) >> 52));
+            const double sc = inv_exp2(max(ha, hb) >> 20);
             const float an = (float)(al * sc), bn = (float)(be * sc);
-            const float top = (float)(__longlong_as_double(lmax) * sc);
+            const float top = (float)(__hiloint2double(hmax, 0) * sc);
             const bool rp = ca < keep_rank && an >= cut2 * top, rq = cb < keep_rank && bn >= cut2 * top;
+            const double gsc = sc * 1073741824.0;   // gamma times 2^30: |gamma|^2 stays in the FP32 range
+            const float gx = (float)(gam.x * gsc), gy = (float)(gam.y * gsc);
+            const float g2 = fmaf(gx, gx, gy * gy);
             if ((rp || rq) && sc > 0.0) {
                 const float dn = (float)((be - al) * sc);
-                const double gsc = sc * 1073741824.0;   // gamma times 2^30: |gamma|^2 stays in the FP32 range
-                const float gx = (float)(gam.x * gsc), gy = (float)(gam.y * gsc);
-                const float g2 = fmaf(gx, gx, gy * gy);
                 const float lim = rp && rq ? an * bn : fmaxf(an, bn) * fmaxf(an, bn);
                 const bool wide = g2 > stop2 * 1.152921504606847e18f * lim;
                 if (wide) flags |= 1u;
@@ -963,7 +965,13 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                     // squared lengths, which may be of order one where the cosine is far below `stop`
                     // (a cosine of 1e-9 between lengths equal to 1e-9 leaves the kept triplets open).  Such a
                     // pair is open until K is small or the cosine is rounding.
-                    if (k2 > OPEN2 && g2 > tol2 * 1.152921504606847e18f * lim) flags |= 1u;
+                    const bool above = g2 > tol2 * 1.152921504606847e18f * lim;
+                    if (k2 > OPEN2 && above) flags |= 1u;
+                    // bit 8 + i: a |K| of at least 2^(-30 - 3 i) between a column that counts and another one
+                    if (F64 && above && !(rp && rq)) {
+                        const int i = max(0, (72 - (__float_as_int(k2) >> 23)) / 6);
+                        if (i < 8) flags |= (0xffu << i & 0xffu) << 8;
+                    }
                     if (!(k2 <= KMAX2)) {
                         K = CF{0.f, 0.f};
                         if (flags & 1u) flags |= wide ? 34u : 2u;
@@ -973,10 +981,24 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                         if (k2 * fmaxf(an, bn) > 1e-6f * fminf(an, bn) && (rp && rq)) flags |= 16u;
                     }
                 }
+            } else if (F64) {
+                // two columns that do not count, and c, their product over the squared length of the shortest
+                // column that is clearly longer (exponents only): bit 16 + i for c of at least 2^(-20 + 3 i)
+                const int i = ((__float_as_int(g2) >> 23) - 141 - 2 * ((next >> 20) - (max(ha, hb) >> 20))) / 6;
+                if (i > 0) flags |= ((1u << min(i, 8)) - 1u) << 16;
             }
         }
-        const unsigned mine = flags;
+        unsigned mine = flags;
         flags = grp.or_bits(flags);
+        // A rotation K of a column that counts against one of those two leaves K c against the other, so a
+        // pass gains a factor c there instead of squaring: open while K c is above rounding (about 2^-50),
+        // and from the fourth pass on two such columns with c above 2^-11 are rotated themselves (a Jacobi
+        // step costs a third of a pass, so at first passes are cheaper: arbitrary gates 20 % slower).
+        if (F64 && ((flags >> 8) & (flags >> 16) & 0xffu)) {
+            const bool late = pass >= 3;
+            flags |= late && (flags & 1u << 19) ? 3u : 1u;
+            if (late && (mine & 1u << 19)) mine |= 2u;
+        }
         if (flags & 8u) {
             // I + K + K^2/2 on W (FP64) and V (FP64, or the correction in FP32)
             if (has) {

@@ -151,3 +151,51 @@ def test_regauge_of_messages_with_close_eigenvalues(C, D, gap):
     assert np.abs(O.local_orthogonality_residual(got) - O.local_orthogonality_residual(want)) < 1e-11
     a, b = O.to_statevector(got), O.to_statevector(want)
     assert np.linalg.norm(a / np.linalg.norm(a) - b / np.linalg.norm(b)) < 1e-11
+
+
+# seeds whose discarded columns the FP32 first stage leaves far from orthogonal, and a few others
+LONG = [(2, 0, s) for s in (1957, 2316, 1404, 0, 1)] + [(2, 1, s) for s in (1335, 1593, 1685, 0, 1)]
+LONG += [(4, 0, s) for s in (1888, 1348, 2030, 0, 1)] + [(4, 1, s) for s in (1301, 2087, 2887, 0, 1)]
+
+
+@pytest.mark.parametrize("C,kind,seed", LONG)
+def test_arbitrary_gate_with_long_discarded_columns(C, kind, seed):
+    """A gate sum_k s_k P_k x P_k (Pauli matrices P_k, and a unitary on every leg) on two tensors whose
+    columns P_k a_j are orthonormal: the core has the singular values s_k value_j, here with discarded
+    ones up to half as long as the kept ones.  Bound: 100 units of 1e-16 in the library and as much in
+    LAPACK, over a gap at the cut of at least a sixth."""
+    D, rng = 3, np.random.default_rng(seed)
+    unitary = lambda r, c: np.linalg.qr(rng.standard_normal((r, c)) + 1j * rng.standard_normal((r, c)))[0]  # noqa: E731
+    if kind == 0:
+        value = np.sort(rng.uniform(0.5, 1.0, C))[::-1]
+        sk = np.concatenate([[1.0], rng.uniform(0.2, 0.45, 3)])
+    else:
+        value = np.concatenate([np.linspace(1.0, 0.8, C // 2) if C > 2 else [1.0], 0.3 * rng.uniform(0.5, 1.0, C - C // 2)])
+        sk = np.concatenate([[1.0, 0.7], rng.uniform(0.2, 0.35, 2)])
+    n, edges, colour, Gam, lam = two_centres(C, D, 1e-3, 0)
+    mix = unitary(C, C)
+    side = (lambda u: u @ mix), (lambda u: (u * value) @ mix.conj() / lam[0])
+    for v in (0, 1):
+        q = unitary(C * C, 2 * C)
+        for i in range(2):
+            Gam[v, i] = np.moveaxis((side[v](q[:, i * C:(i + 1) * C]) * C).reshape((C,) * D), -1, 0)
+    pauli = [np.eye(2), np.array([[0, 1], [1, 0]]), np.array([[0, -1j], [1j, 0]]), np.diag([1.0, -1.0])]
+    U = sum(sk[k] * np.kron(pauli[k], pauli[k]) for k in range(4))
+    legs = [unitary(2, 2) for _ in range(4)]
+    U = np.kron(legs[0], legs[1]) @ U @ np.kron(legs[2], legs[3])
+    s = G.gtqa_create(n, edges, np.zeros(len(edges)), np.zeros(n), C, colour)
+    try:
+        st = O.from_padded(n, edges, Gam, lam)
+        G.gtqa_set_state(s, Gam, lam, O.messages_to_padded(st, O.reconstructed_messages(st), C))
+        G.gtqa_apply_gates(s, [0], U[None])
+        new, lnew, _ = G.gtqa_get_state(s)
+    finally:
+        G.gtqa_destroy(s)
+    # the two-site tensor, rows (i, J) of each side weighted with the leaves' 1 / C
+    A, B = [np.moveaxis(Gam[v], 1, -1).reshape(2, -1, C) / C for v in (0, 1)]
+    theta = np.einsum("abcd,cpj,j,dqj->apbq", U.reshape(2, 2, 2, 2), A, lam[0], B).reshape(2 * C * C, -1)
+    u, x, vh = np.linalg.svd(theta)
+    want = (u[:, :C] * x[:C]) @ vh[:C] / np.linalg.norm(x[:C])
+    A, B = [np.moveaxis(new[v], 1, -1).reshape(-1, C) / C for v in (0, 1)]
+    assert x[C - 1] - x[C] > x[0] / 6
+    assert np.linalg.norm((A * lnew[0]) @ B.T - want) < 1.2e-13
