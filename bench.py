@@ -17,7 +17,7 @@ warm-up is timed.
     python bench.py [--gpus N] [--steps S] [--warmup W] [--precision fp64|mixed]
     python bench.py --impl reference ...     # the CPU oracle on the same workload
 
-Prints one JSON line (rank 0).  Under torchrun every rank runs its own replica of
+Prints one JSON line (rank 0); the record with every table goes to stderr.  Under torchrun every rank runs its own replica of
 the workload (no collective on the data path) and the slowest rank's time counts.
 """
 from __future__ import annotations
@@ -407,6 +407,25 @@ def regauge_flops_executed(chi: int, edges: int, svd_sweeps: int, mixed: bool) -
     return float(svd_sweeps * per_pass + edges * fixed)
 
 
+# records with a table per leg, layer or kernel: of these the line has the single values only
+DETAILED = ("batched", "fp64_path", "scale", "whole_anneal", "roofline_other_kernels", "cpu_baseline")
+
+
+def summary_line(out: dict) -> dict:
+    """The record without its tables, short enough for a reader that keeps a few thousand characters
+    of output (the whole record is some 22000 long; it goes to stderr as {"details": ...})."""
+    def values(d, depth):
+        kept = {}
+        for k, v in d.items():
+            if isinstance(v, dict) and depth:
+                kept[k] = values(v, depth - 1)
+            elif v is None or isinstance(v, (bool, int, float)) or (isinstance(v, str) and len(v) <= 24):
+                kept[k] = v
+        return {k: v for k, v in kept.items() if v != {}}
+
+    return {k: values(v, 1) if k in DETAILED and isinstance(v, dict) else v for k, v in out.items()}
+
+
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_n1000_chi4.json")
 TRAFFIC_SOURCES = [os.path.join(ROOT, "paper_2409_12240_gb300", "csrc", f) for f in ("gtqa_anneal.cuh", "gtqa_common.cuh")]
 
@@ -758,7 +777,8 @@ def run_gtqa(a):
         "final_marginals": {"mean_abs_z": float(np.mean(np.abs(main["rho"][:, 0, 0].real - main["rho"][:, 1, 1].real))),
                             "E": energy(inst, main["sign"])},
     }
-    print(json.dumps(out))
+    print(json.dumps({"details": out}), file=sys.stderr)
+    print(json.dumps(summary_line(out)))
     if dist:
         dist.destroy_process_group()
 
