@@ -57,7 +57,8 @@ extern "C" {
 
 /* arithmetic modes */
 #define GTQA_FP64 0   /* complex128 everywhere */
-#define GTQA_MIXED 1  /* complex64 tensors and BP contractions; FP64 QR/SVD, gauge roots, normalisation.
+#define GTQA_MIXED 1  /* complex64 tensors and BP contractions; FP64 QR/SVD and gauge roots; normalisation from
+                         pairs of floats (1e-13 relative, any trace that complex64 holds; FP64 on plain-path states).
                          Messages are held as m0 + delta: m0 = diag(lambda)/sum(lambda) (exact),
                          delta in complex64; get/set_state convert to and from complex128. */
 #define GTQA_C64 2    /* complex64 with every step in FP32, including the QR/SVD, gauge roots and

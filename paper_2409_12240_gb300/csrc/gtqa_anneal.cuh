@@ -22,8 +22,9 @@
 // Precision modes:
 //   FP64   complex128 tensors and messages, FP64 arithmetic throughout.
 //   Mixed  complex64 Gamma, T and message corrections; the simple update's QR and
-//          SVD, the regauge's eigen/SVD and square roots, and the message
-//          normalisation in FP64.  Messages are kept as m = m0 + delta with m0 the
+//          SVD and the regauge's eigen/SVD and square roots in FP64 (first stage and
+//          small corrections of the SVDs in FP32), the message normalisation from
+//          pairs of floats (1e-13).  Messages are kept as m = m0 + delta with m0 the
 //          warm start (exact, from lambda) and delta in complex64; each sweep
 //          contracts only delta in FP32, and the warm-start part F(m0) is contracted
 //          once per BP call in FP64.

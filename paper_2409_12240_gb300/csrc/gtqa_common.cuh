@@ -1,6 +1,6 @@
 // Small device-side toolkit shared by the GTQA kernels: complex arithmetic,
-// thread-team synchronisation, butterfly reductions and the batched one-sided
-// Jacobi SVD used for every small matrix decomposition of the method.
+// thread-team synchronisation, butterfly reductions and the small matrix decompositions of the
+// method: one-sided Jacobi SVDs (FP32, FP64) and the FP64 SVD refined from an FP32 one.
 #pragma once
 
 #include <climits>
@@ -538,16 +538,15 @@ __device__ __forceinline__ bool norm_collapsed(double x, double ref) {
 // size of the rotation of the kept column) rather than sqrt(alpha_p beta_q).  The kept
 // columns then converge as with keep_rank = N, while rotations among discarded columns, which
 // leave the kept subspace unchanged, no longer force a confirming sweep.
-// PARTIAL: every pair is rotated in the first sweep; a later sweep runs only the steps of the
+// The first sweep runs first_steps (all by default); a later sweep runs only the steps of the
 // round-robin schedule in which the previous sweep made a rotation above quad_tol.  A pair
 // whose rotation in a sweep stayed below quad_tol is orthogonal after it to about quad_tol
 // times the largest rotation of that sweep (the rotations of its columns with the others
 // reintroduce only products of their sizes), which is the accuracy of the quadratic stop, so
-// those steps need no second pass.  Otherwise every pair is rotated in each sweep that runs.
-// first_steps: the steps that the first sweep runs (all by default).
+// those steps need no second pass.
 // Returns the sweeps run (partial ones included); *nsteps (if given, group lane 0) counts the
 // steps run, of N / 2 pairs each.
-template <int N, typename Group, bool PARTIAL = false>
+template <int N, typename Group>
 __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, const Group& grp, unsigned pair_mask,
                              double tol, double quad_tol, int max_sweeps, int* nrot, int keep_rank = N,
                              unsigned* relmask = nullptr, int* nsteps = nullptr, unsigned first_steps = ~0u) {
@@ -587,10 +586,9 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
     unsigned steps = ((1u << (N - 1)) - 1u) & first_steps;   // steps this sweep runs
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
-        int big = 0;
         unsigned bigsteps = 0u;   // this lane's steps with a rotation above quad_tol
         for (int step = 0; step < N - 1; ++step) {
-            if (PARTIAL && !((steps >> step) & 1u)) continue;   // the same for the whole group
+            if (!((steps >> step) & 1u)) continue;   // the same for the whole group
             int bstep = 0;   // this lane's pair rotated by more than quad_tol
             if (nsteps && g == 0) ++*nsteps;
             int p, q;
@@ -655,17 +653,11 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
                     nrm[q] = nq;
                 }
             }
-            big |= bstep;
             if (bstep) bigsteps |= 1u << step;
             grp.sync();
         }
-        if constexpr (PARTIAL) {
-            steps = grp.or_bits(bigsteps);
-            if (!steps) {
-                ++sweep;
-                break;
-            }
-        } else if (!grp.any(big)) {
+        steps = grp.or_bits(bigsteps);
+        if (!steps) {
             ++sweep;
             break;
         }
@@ -689,7 +681,10 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 //   4. passes: the Gram matrix of W in FP64, every pair's rotation parameter (as in
 //      jacobi_polish: K_pq = tau gamma_pq) at once, and W <- W (I + K + K^2/2), V likewise, for
 //      all pairs with |K_pq| <= 1e-4.  K is antihermitian, so the factor is unitary up to
-//      |K|^4/4 < 3e-17, and the off-diagonals shrink to products of their sizes.  Without F64 the
+//      ||K||^4/4 and the FP32 rounding of K^2: V^H V - I stays below 4e-15 (N = 8), 1e-14 (16) and 2e-14 (32)
+//      on clustered spectra, whose K are the largest, and near 1e-15 elsewhere.  (Taking V's defect out in the
+//      next pass leaves 1e-15 everywhere for 1.5 % of an FP64 anneal: not done, FP64 Jacobi sweeps
+//      accumulate 3e-15 to 8e-15.)  The off-diagonals shrink to products of their sizes.  Without F64 the
 //      corrections are formed in FP32 where every kept column moves by less than 1e-3 of its length
 //      (12 FP64 instructions per warp instead of 64).  A pair is open, and asks for another pass, while
 //      its cosine is above `stop` or, unless the cosine is below tol, its |K| above 1e-8 (1e-4 without
@@ -700,9 +695,9 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 //      with many of them, by FP32 Jacobi on those and all shorter columns of W, rescaled,
 //      which resolves the columns that lay below the FP32 resolution of the first stage.
 //   A decomposition that is still open after MAXP passes goes to jacobi_polish.
-// Cores of whole anneals (n = 300, chi = 4): 1.3 passes on average in the mixed mode, 2.1 with
-// F64, Jacobi steps in 2 % of the gates; slow early anneals with spectra graded over 12 orders:
-// 3.3 and 3.9.  Orthogonality of the kept columns after it: 2e-10 (stop 1e-5) and 1e-15 (F64).
+// Cores of whole anneals (n = 300, chi = 4): 1.3 passes on average in the mixed mode, 2.2 with
+// F64; chi = 8 2.0 and 3.1, chi = 16 (F64) 2.0.  Orthogonality of the kept columns after it: 2e-10
+// (stop 1e-5) and 1e-15 (F64).  Kept triplets with a relative gap d to the first discarded one: 1e-16 / d (F64).
 // ---------------------------------------------------------------------------
 // The pair of columns of lane g: the N (N - 1) / 2 pairs in the order of the Jacobi schedule
 // (lane g: pair g % (N / 2) of step g / (N / 2)); false for the lanes that are left over.
@@ -1044,7 +1039,7 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         if (pass + 1 >= MAXP) {
             int nsteps = 0;
             // to the resolution of the rotations: `stop` would leave pairs of close lengths open
-            cnt.passes += jacobi_polish<N, Group, true>(A, V, nrm, g, grp, pair_mask, tol, 16.0 * tol, 60, &cnt.rot, keep_rank,
+            cnt.passes += jacobi_polish<N>(A, V, nrm, g, grp, pair_mask, tol, 16.0 * tol, 60, &cnt.rot, keep_rank,
                                                         relmask, &nsteps);
             cnt.pairs += nsteps * (N / 2);
             break;
@@ -1056,7 +1051,7 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         if constexpr (N >= 16)   // FP32 resolves nothing below a cosine of 1e-7
             part = second < 3 && __popc(grp.or_bits((mine & 32u) ? 1u << step : 0u)) > N / 4;
         if (!part) {
-            jacobi_polish<N, Group, true>(A, V, nrm, g, grp, pair_mask, tol, stop, 1, &cnt.rot, N, nullptr, nullptr, steps);
+            jacobi_polish<N>(A, V, nrm, g, grp, pair_mask, tol, stop, 1, &cnt.rot, N, nullptr, nullptr, steps);
             cnt.pairs += nst * (N / 2);
         } else if constexpr (N >= 16) {
             ++second;

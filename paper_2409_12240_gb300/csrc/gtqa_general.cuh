@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kerne
         const unsigned gm = group_mask<G>();
         if constexpr (QREG) {
             // rows in registers, as in the Ising gates; the reflectors stay scaled (sqrt(tau) v) in
-            // sm.X, R in sm.R
+            // sm.X, R in sm.Rf
             CR y0[NC], y1[NC];
 #pragma unroll
             for (int cc = 0; cc < NC; ++cc) {
@@ -210,8 +210,7 @@ __global__ void __launch_bounds__(GenShape<CHI, D>::TEAM, 1) general_gates_kerne
                     Xc[r1] = cfms(u1, d, y1);
                 }
                 __syncwarp(gm);
-                // column k: R above the diagonal and on it, the scaled reflector below and in sm.Rf's
-                // column for the diagonal entry
+                // column k of R into sm.Rf, the scaled reflector (its entry k included) into sm.X
                 for (int r = l; r < NC; r += G)
                     if (r <= k) sm.Rf[x][r][k] = r < k ? Xk[r] : CR{-nrm * ph.x, -nrm * ph.y};
                 __syncwarp(gm);

@@ -1067,7 +1067,7 @@ __global__ void __launch_bounds__(PlainGateShape<CHI, D>::TEAM) plain_ising_kern
         bar();
     }
     qr_steps<CHI, G, 0>(y0, y1, &sm.U[blk][0][0], l, gm);
-    // rows l and, where the group is smaller than CHI, l + G of R
+    static_assert(G >= CHI, "lane l holds row l of R");
 #pragma unroll
     for (int cc = 0; cc < CHI; ++cc) {
         const R lb = x == 0 ? (R)sm.lab[cc] : (R)1;
