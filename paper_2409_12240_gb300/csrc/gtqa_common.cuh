@@ -689,14 +689,15 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 //      (12 FP64 instructions per warp instead of 64).  A pair is open, and asks for another pass, while
 //      its cosine is above `stop` or, unless the cosine is below tol, its |K| above 1e-8 (1e-4 without
 //      F64): columns of nearly the same length take a large rotation at a small cosine.  With F64 the
-//      columns that do not count set the end too, where they are long and not orthogonal to each other.
+//      products of the columns that do not count enter K and the end too, where they are long and
+//      not orthogonal to each other.
 //      A pair with a larger K (nearly equal or not yet resolved columns) is rotated by
 //      FP64 Jacobi steps (only the steps of the schedule that hold such a pair) or, for N >= 16
 //      with many of them, by FP32 Jacobi on those and all shorter columns of W, rescaled,
 //      which resolves the columns that lay below the FP32 resolution of the first stage.
 //   A decomposition that is still open after MAXP passes goes to jacobi_polish.
-// Cores of whole anneals (n = 300, chi = 4): 1.3 passes on average in the mixed mode, 2.2 with
-// F64; chi = 8 2.0 and 3.1, chi = 16 (F64) 2.0.  Orthogonality of the kept columns after it: 2e-10
+// Cores of whole anneals (n = 300, chi = 4): 1.3 passes on average in the mixed mode, 2.1 with
+// F64; chi = 8 2.0 and 2.8, chi = 16 (F64) 1.9.  Orthogonality of the kept columns after it: 2e-10
 // (stop 1e-5) and 1e-15 (F64).  Kept triplets with a relative gap d to the first discarded one: 1e-16 / d (F64).
 // ---------------------------------------------------------------------------
 // The pair of columns of lane g: the N (N - 1) / 2 pairs in the order of the Jacobi schedule
@@ -925,6 +926,12 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
         // 8: any K, 16: a K that moves the pair's shorter column by more than 1e-3 of its length; from bit 8 on:
         // sizes of K and c (below)
         unsigned flags = 0u;
+        // F64: which columns of the pair count, their difference (scaled by the longer one), that scale
+        // against the longest column's, and the product of two columns that do not count
+        bool rp = false, rq = false;
+        float dn = 0.f;
+        int down = 0;
+        CF cross = CF{0.f, 0.f};
         if (has) {
             const double al = nrm[p], be = nrm[q];
             // the upper words of positive doubles compare as integers; + 2 in the exponent: times 4
@@ -941,12 +948,14 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
             const double sc = inv_exp2(max(ha, hb) >> 20);
             const float an = (float)(al * sc), bn = (float)(be * sc);
             const float top = (float)(__hiloint2double(hmax, 0) * sc);
-            const bool rp = ca < keep_rank && an >= cut2 * top, rq = cb < keep_rank && bn >= cut2 * top;
+            rp = ca < keep_rank && an >= cut2 * top;
+            rq = cb < keep_rank && bn >= cut2 * top;
+            down = (hmax >> 20) - (max(ha, hb) >> 20);
             const double gsc = sc * 1073741824.0;   // gamma times 2^30: |gamma|^2 stays in the FP32 range
             const float gx = (float)(gam.x * gsc), gy = (float)(gam.y * gsc);
             const float g2 = fmaf(gx, gx, gy * gy);
             if ((rp || rq) && sc > 0.0) {
-                const float dn = (float)((be - al) * sc);
+                dn = (float)((be - al) * sc);
                 const float lim = rp && rq ? an * bn : fmaxf(an, bn) * fmaxf(an, bn);
                 const bool wide = g2 > stop2 * 1.152921504606847e18f * lim;
                 if (wide) flags |= 1u;
@@ -978,18 +987,24 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                 }
             } else if (F64) {
                 // two columns that do not count, and c, their product over the squared length of the shortest
-                // column that is clearly longer (exponents only): bit 16 + i for c of at least 2^(-20 + 3 i)
-                const int i = ((__float_as_int(g2) >> 23) - 141 - 2 * ((next >> 20) - (max(ha, hb) >> 20))) / 6;
-                if (i > 0) flags |= ((1u << min(i, 8)) - 1u) << 16;
+                // column that is clearly longer (exponents only): bit 16 + i for c of at least 2^(-20 + 3 i),
+                // bit 24 + i for c^2
+                const int e = (__float_as_int(g2) >> 23) - 187 - 2 * ((next >> 20) - (max(ha, hb) >> 20));
+                if (e >= -40) flags |= ((1u << min((e + 46) / 6, 8)) - 1u) << 16;
+                if (e >= -20) flags |= ((1u << min((e + 23) / 3, 8)) - 1u) << 24;
+                const float f = __int_as_float(max(127 - down, 0) << 23);
+                cross = CF{f * gx, f * gy};
             }
         }
         unsigned mine = flags;
         flags = grp.or_bits(flags);
         // A rotation K of a column that counts against one of those two leaves K c against the other, so a
-        // pass gains a factor c there instead of squaring: open while K c is above rounding (about 2^-50),
-        // and from the fourth pass on two such columns with c above 2^-11 are rotated themselves (a Jacobi
-        // step costs a third of a pass, so at first passes are cheaper: arbitrary gates 20 % slower).
-        if (F64 && ((flags >> 8) & (flags >> 16) & 0xffu)) {
+        // pass would gain a factor c there instead of squaring.  Where K c is above rounding (about 2^-50)
+        // the rotations take that term along (below), which leaves K c^2; open while that is above
+        // rounding, and from the fourth pass on two such columns with c above 2^-11 are rotated themselves.
+        // (Further passes alone instead: 2.19 passes per gate for 2.11, FP64 anneals 2 to 4 % longer.)
+        const bool coupled = F64 && ((flags >> 8) & (flags >> 16) & 0xffu);
+        if (F64 && ((flags >> 8) & (flags >> 24) & 0xffu)) {
             const bool late = pass >= 3;
             flags |= late && (flags & 1u << 19) ? 3u : 1u;
             if (late && (mine & 1u << 19)) mine |= 2u;
@@ -1001,6 +1016,28 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
                 A32[p * N + q] = CF{-K.x, K.y};
             }
             if (g < N) A32[g * N + g] = CF{0.f, 0.f};
+            if (coupled) {
+                // K_qp of a kept column p and another one q solves gamma_qp + (|a_q|^2 - |a_p|^2) K_qp +
+                // sum_r a_q^H a_r K_rp = 0, r over the others: one step of that sum from the K above
+                if (has) {
+                    V32[q * N + p] = cross;
+                    V32[p * N + q] = conj(cross);
+                }
+                if (g < N) V32[g * N + g] = CF{0.f, 0.f};
+                grp.sync();
+                if (rp != rq && norm2(K) > 0.f) {
+                    const int kept = rp ? p : q, other = rp ? q : p;
+                    CF sum = CF{0.f, 0.f};
+                    for (int r = 0; r < N; ++r) sum = cfma(V32[r * N + other], A32[kept * N + r], sum);
+                    const float f = __int_as_float(min(97 + down, 254) << 23) / (rp ? -dn : dn);
+                    K = rp ? K - conj(f * sum) : K + f * sum;
+                }
+                grp.sync();
+                if (has) {
+                    A32[q * N + p] = K;
+                    A32[p * N + q] = CF{-K.x, K.y};
+                }
+            }
             grp.sync();
             CF l[2];
             // mixed mode: the corrections W L and V L in FP32, whose rounding is then below 1e-10 of every
