@@ -681,8 +681,8 @@ __device__ int jacobi_polish(C<double>* A, C<double>* V, double* nrm, int g, con
 //   4. passes: the Gram matrix of W in FP64, every pair's rotation parameter (as in
 //      jacobi_polish: K_pq = tau gamma_pq) at once, and W <- W (I + K + K^2/2), V likewise, for
 //      all pairs with |K_pq| <= 1e-4.  K is antihermitian, so the factor is unitary up to
-//      ||K||^4/4 and the FP32 rounding of K^2: V^H V - I stays below 4e-15 (N = 8), 1e-14 (16) and 2e-14 (32)
-//      on clustered spectra, whose K are the largest, and near 1e-15 elsewhere.  (Taking V's defect out in the
+//      ||K||^4/4 and the FP32 rounding of K^2: V^H V - I stays below 4e-15 (N = 8), 1e-14 (16) and 4e-14 (32)
+//      on clustered and graded spectra, whose K are the largest, and near 1e-15 elsewhere.  (Taking V's defect out in the
 //      next pass leaves 1e-15 everywhere for 1.5 % of an FP64 anneal: not done, FP64 Jacobi sweeps
 //      accumulate 3e-15 to 8e-15.)  The off-diagonals shrink to products of their sizes.  Without F64 the
 //      corrections are formed in FP32 where every kept column moves by less than 1e-3 of its length
@@ -1018,19 +1018,22 @@ __device__ SvdCount refined_svd(C<double>* A, C<double>* V, C<float>* A32, C<flo
             if (g < N) A32[g * N + g] = CF{0.f, 0.f};
             if (coupled) {
                 // K_qp of a kept column p and another one q solves gamma_qp + (|a_q|^2 - |a_p|^2) K_qp +
-                // sum_r a_q^H a_r K_rp = 0, r over the others: one step of that sum from the K above
+                // sum_r a_q^H a_r K_rp = 0, r over the others: one step of that sum from the K above.  Only
+                // where q is clearly the shorter one, as it is against every column that is kept (two equal
+                // columns may lie on both sides of the line between those that count and the others)
                 if (has) {
                     V32[q * N + p] = cross;
                     V32[p * N + q] = conj(cross);
                 }
                 if (g < N) V32[g * N + g] = CF{0.f, 0.f};
                 grp.sync();
-                if (rp != rq && norm2(K) > 0.f) {
+                if (rp != rq && fabsf(dn) > 0.5f && norm2(K) > 0.f) {
                     const int kept = rp ? p : q, other = rp ? q : p;
                     CF sum = CF{0.f, 0.f};
                     for (int r = 0; r < N; ++r) sum = cfma(V32[r * N + other], A32[kept * N + r], sum);
                     const float f = __int_as_float(min(97 + down, 254) << 23) / (rp ? -dn : dn);
-                    K = rp ? K - conj(f * sum) : K + f * sum;
+                    const CF next = rp ? K - conj(f * sum) : K + f * sum;
+                    if (norm2(next) <= KMAX2) K = next;
                 }
                 grp.sync();
                 if (has) {

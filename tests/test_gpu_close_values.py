@@ -158,20 +158,11 @@ LONG = [(2, 0, s) for s in (1957, 2316, 1404, 0, 1)] + [(2, 1, s) for s in (1335
 LONG += [(4, 0, s) for s in (1888, 1348, 2030, 0, 1)] + [(4, 1, s) for s in (1301, 2087, 2887, 0, 1)]
 
 
-@pytest.mark.parametrize("C,kind,seed", LONG)
-def test_arbitrary_gate_with_long_discarded_columns(C, kind, seed):
-    """A gate sum_k s_k P_k x P_k (Pauli matrices P_k, and a unitary on every leg) on two tensors whose
-    columns P_k a_j are orthonormal: the core has the singular values s_k value_j, here with discarded
-    ones up to half as long as the kept ones.  Bound: 100 units of 1e-16 in the library and as much in
-    LAPACK, over a gap at the cut of at least a sixth."""
-    D, rng = 3, np.random.default_rng(seed)
+def pauli_gate(C, value, sk, rng):
+    """A state and a gate sum_k s_k P_k x P_k (Pauli matrices P_k, and a unitary on every leg) whose core has
+    the singular values s_k value_j: the columns P_k a_j of the two tensors are orthonormal."""
+    D = 3
     unitary = lambda r, c: np.linalg.qr(rng.standard_normal((r, c)) + 1j * rng.standard_normal((r, c)))[0]  # noqa: E731
-    if kind == 0:
-        value = np.sort(rng.uniform(0.5, 1.0, C))[::-1]
-        sk = np.concatenate([[1.0], rng.uniform(0.2, 0.45, 3)])
-    else:
-        value = np.concatenate([np.linspace(1.0, 0.8, C // 2) if C > 2 else [1.0], 0.3 * rng.uniform(0.5, 1.0, C - C // 2)])
-        sk = np.concatenate([[1.0, 0.7], rng.uniform(0.2, 0.35, 2)])
     n, edges, colour, Gam, lam = two_centres(C, D, 1e-3, 0)
     mix = unitary(C, C)
     side = (lambda u: u @ mix), (lambda u: (u * value) @ mix.conj() / lam[0])
@@ -182,7 +173,13 @@ def test_arbitrary_gate_with_long_discarded_columns(C, kind, seed):
     pauli = [np.eye(2), np.array([[0, 1], [1, 0]]), np.array([[0, -1j], [1j, 0]]), np.diag([1.0, -1.0])]
     U = sum(sk[k] * np.kron(pauli[k], pauli[k]) for k in range(4))
     legs = [unitary(2, 2) for _ in range(4)]
-    U = np.kron(legs[0], legs[1]) @ U @ np.kron(legs[2], legs[3])
+    return n, edges, colour, Gam, lam, np.kron(legs[0], legs[1]) @ U @ np.kron(legs[2], legs[3])
+
+
+def kept_part(C, n, edges, colour, Gam, lam, U):
+    """Distance of the gate's two-site tensor, rows (i, J) of each side weighted with the leaves' 1 / C, from
+    LAPACK's truncation of it, the largest defect of the new tensors' orthonormal columns, and the
+    relative gap at the cut."""
     s = G.gtqa_create(n, edges, np.zeros(len(edges)), np.zeros(n), C, colour)
     try:
         st = O.from_padded(n, edges, Gam, lam)
@@ -191,11 +188,38 @@ def test_arbitrary_gate_with_long_discarded_columns(C, kind, seed):
         new, lnew, _ = G.gtqa_get_state(s)
     finally:
         G.gtqa_destroy(s)
-    # the two-site tensor, rows (i, J) of each side weighted with the leaves' 1 / C
     A, B = [np.moveaxis(Gam[v], 1, -1).reshape(2, -1, C) / C for v in (0, 1)]
     theta = np.einsum("abcd,cpj,j,dqj->apbq", U.reshape(2, 2, 2, 2), A, lam[0], B).reshape(2 * C * C, -1)
     u, x, vh = np.linalg.svd(theta)
     want = (u[:, :C] * x[:C]) @ vh[:C] / np.linalg.norm(x[:C])
     A, B = [np.moveaxis(new[v], 1, -1).reshape(-1, C) / C for v in (0, 1)]
-    assert x[C - 1] - x[C] > x[0] / 6
-    assert np.linalg.norm((A * lnew[0]) @ B.T - want) < 1.2e-13
+    defect = max(np.abs(X.conj().T @ X - np.eye(C)).max() for X in (A, B))
+    return np.linalg.norm((A * lnew[0]) @ B.T - want), defect, (x[C - 1] - x[C]) / x[0]
+
+
+@pytest.mark.parametrize("C,kind,seed", LONG)
+def test_arbitrary_gate_with_long_discarded_columns(C, kind, seed):
+    """Discarded values up to half as large as the kept ones.  Bound: 100 units of 1e-16 in the library and
+    as much in LAPACK, over a gap at the cut of at least a sixth."""
+    rng = np.random.default_rng(seed)
+    if kind == 0:
+        value = np.sort(rng.uniform(0.5, 1.0, C))[::-1]
+        sk = np.concatenate([[1.0], rng.uniform(0.2, 0.45, 3)])
+    else:
+        value = np.concatenate([np.linspace(1.0, 0.8, C // 2) if C > 2 else [1.0], 0.3 * rng.uniform(0.5, 1.0, C - C // 2)])
+        sk = np.concatenate([[1.0, 0.7], rng.uniform(0.2, 0.35, 2)])
+    err, _, gap = kept_part(C, *pauli_gate(C, value, sk, rng))
+    assert gap > 1.0 / 6.0
+    assert err < 1.2e-13
+
+
+@pytest.mark.parametrize("seed", range(12))
+@pytest.mark.parametrize("C", [2, 4, 8])
+def test_arbitrary_gate_with_equal_pairs_of_values(C, seed):
+    """Pairs of equal values in steps of two, so that columns lie exactly at the factors by which the
+    refinement tells long from short ones.  Bound: 100 units of 1e-16 (orthonormality; and the kept part,
+    whose gap is as large as the smallest kept value)."""
+    pairs = 0.5 ** (4 * np.arange((C + 1) // 2))
+    err, defect, gap = kept_part(C, *pauli_gate(C, np.repeat(pairs, 2)[:C], 0.5 ** np.arange(4), np.random.default_rng(seed)))
+    assert defect < 1e-14
+    assert err < 2e-14 / min(gap, 0.05)
